@@ -97,6 +97,12 @@ struct lgf_ctx {
     bool accel32 = false;     // FP64 iterations take the accelerator's transforms in FP32
     bool gu32 = false;        // FP32 phase: g builder and update in one persistent launch
     unsigned* gu_sync = nullptr;  // its queue, epoch and per-plane flags
+    // FP64 iterations run on 64-bit fixed point (lgf_kfx.cuh) while the stored links
+    // are within its range; `wide` links (a snapshot of anything else) take the FP64
+    // kernels.  g64, AH64 and Fs64 hold the fixed-point g, parts and Re Tr meanwhile.
+    longlong2* UX = nullptr;  // [4][6][V]
+    longlong2* GX = nullptr;  // [6][V]
+    bool wide = false, graph_wide = false;
     void* Fd = nullptr;       // [4][V] double2 (the FP32 phase uses the front half as float2)
     double2* AH64 = nullptr;  // [4][4][V] packed anti-Hermitian parts of the links
     double* Fs64 = nullptr;   // [V] Re Tr of the four links of a site
@@ -175,45 +181,91 @@ template <typename T> const Shape& shape_of(const lgf_ctx* c);
 template <> const Shape& shape_of<double>(const lgf_ctx* c) { return c->sh64; }
 template <> const Shape& shape_of<float>(const lgf_ctx* c) { return c->sh32; }
 
-// one FP64 iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, update,
-// Delta+FFT(x,y)
-// Delta, theta and F of the FP64 links with the forward x,y transform: in FP64, or
-// in FP32 into the front half of Fd when the accelerator runs in FP32
+longlong2* as_fx(double2* p) { return reinterpret_cast<longlong2*>(p); }
+long long* as_fx(double* p) { return reinterpret_cast<long long*>(p); }
+
+// Delta, theta and F of the FP64 loop's links with the forward x,y transform: in
+// FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
 void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist)
 {
-    if (c->accel32 && !c->plain)
-        launch_delta64_f32(c->lat, c->sh64, s, c->AH64, c->Fs64, reinterpret_cast<float2*>(c->Fd), c->partials, ctl,
-                           hist);
-    else
-        launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, reinterpret_cast<double2*>(c->Fd),
-                             c->partials, ctl, hist, !c->plain);
+    double2* Fd = reinterpret_cast<double2*>(c->Fd);
+    float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
+    const bool f32 = c->accel32 && !c->plain;
+    if (!c->wide) {
+        if (f32)
+            launch_fx_delta<float>(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), Fd32, c->partials, ctl, hist,
+                                   true);
+        else
+            launch_fx_delta<double>(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), Fd, c->partials, ctl, hist,
+                                    !c->plain);
+    } else if (f32) {
+        launch_delta64_f32(c->lat, c->sh64, s, c->AH64, c->Fs64, Fd32, c->partials, ctl, hist);
+    } else {
+        launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, Fd, c->partials, ctl, hist, !c->plain);
+    }
 }
 
-// the accelerator and the g builder of an FP64 iteration: FP64 transforms, or FP32
-// transforms (z,t kernel of the FP32 phase, FP32 inverse x,y with the FP64
-// Gram-Schmidt writing the FP64 g)
-void launch_accel_g64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
+// the z,t part of the accelerator in an FP64 iteration
+void launch_zt64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
+{
+    if (c->accel32)
+        launch_zt<float>(c->lat32, c->sh32, c->tb, s, reinterpret_cast<float2*>(c->Fd), ctl);
+    else
+        launch_zt<double>(c->lat, c->sh64, c->tb, s, reinterpret_cast<double2*>(c->Fd), ctl);
+}
+
+// the inverse x,y transform (FP64, or FP32 with the FP64 Gram-Schmidt) and g
+void launch_g64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
-    if (c->accel32) {
-        float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
-        launch_zt<float>(c->lat32, c->sh32, c->tb, s, Fd32, ctl);
+    float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
+    if (!c->wide) {
+        if (c->accel32)
+            launch_fx_xyinv_g<float>(c->lat32, c->sh32, s, Fd32, as_fx(c->g64), ctl);
+        else
+            launch_fx_xyinv_g<double>(c->lat, c->sh64, s, Fd, as_fx(c->g64), ctl);
+    } else if (c->accel32) {
         launch_xyinv_g32_64(c->lat32, c->sh32, s, Fd32, c->g64, ctl);
     } else {
-        launch_zt<double>(c->lat, c->sh64, c->tb, s, Fd, ctl);
         launch_xyinv_g<double>(c->lat, c->sh64, c->tb, s, Fd, c->g64, ctl);
     }
 }
 
-void launch_body64(lgf_ctx* c, cudaStream_t s, double2* G)
+void launch_update64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
+{
+    if (!c->wide)
+        launch_fx_update(c->lat, s, c->UX, c->GX, as_fx(c->g64), ctl, as_fx(c->AH64), as_fx(c->Fs64));
+    else
+        launch_update<double>(c->lat, s, c->U64, c->G64, c->g64, ctl, c->AH64, c->Fs64);
+}
+
+// start of an FP64 loop on the stored links (without Delta), and its end
+void launch_start64(lgf_ctx* c, cudaStream_t s)
+{
+    if (!c->wide)
+        launch_fx_start(c->lat, s, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64), as_fx(c->Fs64));
+    else
+        launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
+}
+void launch_finish64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
+{
+    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->GX, c->U64, c->G64, ctl, c->mixed);
+}
+
+// one FP64 iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, update,
+// Delta+FFT(x,y)
+void launch_body64(lgf_ctx* c, cudaStream_t s)
 {
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
-    const Lat& d = c->lat;
-    if (c->plain)
-        launch_build_g<double>(d, s, Fd, c->g64, c->ctl);
-    else
-        launch_accel_g64(c, s, c->ctl);
-    launch_update<double>(d, s, c->U64, G, c->g64, c->ctl, c->AH64, c->Fs64);
+    if (!c->plain) {
+        launch_zt64(c, s, c->ctl);
+        launch_g64(c, s, c->ctl);
+    } else if (!c->wide) {
+        launch_fx_build_g(c->lat, s, Fd, as_fx(c->g64), c->ctl);
+    } else {
+        launch_build_g<double>(c->lat, s, Fd, c->g64, c->ctl);
+    }
+    launch_update64(c, s, c->ctl);
     launch_delta64(c, s, c->ctl, c->hist);
 }
 
@@ -301,13 +353,13 @@ int add_while(cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps, cudaGraph_t
 }
 
 // FP64 loop: one iteration per body run
-int add_loop64(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps, double2* G)
+int add_loop64(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps)
 {
     cudaGraph_t body;
     cudaGraphConditionalHandle h;
     CKR(add_while(graph, deps, &body, &h));
     CK(cudaStreamBeginCaptureToGraph(c->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    launch_body64(c, c->cap, G);
+    launch_body64(c, c->cap);
     launch_loop_ctl(c->cap, c->ctl, h);
     CK(cudaGetLastError());
     cudaGraph_t out;
@@ -345,18 +397,24 @@ int append_fix(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps
         CKR(capture_end(c, deps));
         CKR(add_loop32(c, graph, deps));
         CKR(capture_begin(c, graph, deps));
-        launch_switch(c->cap, c->lat, c->G32, c->g64, c->U64, c->G64, c->ctl);
-        launch_ah_init<double>(c->lat, c->cap, c->U64, c->AH64, c->Fs64);
-        launch_delta64(c, c->cap, c->ctl, c->hist);
-        CKR(capture_end(c, deps));
-        CKR(add_loop64(c, graph, deps, c->G64));
+        if (!c->wide) {
+            launch_fx_project(c->lat, c->cap, c->G32, c->g64, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64),
+                              as_fx(c->Fs64), c->ctl);
+        } else {
+            launch_switch(c->cap, c->lat, c->G32, c->g64, c->U64, c->G64, c->ctl);
+            launch_start64(c, c->cap);
+        }
     } else {
         CKR(capture_begin(c, graph, deps));
-        launch_ah_init<double>(c->lat, c->cap, c->U64, c->AH64, c->Fs64);
-        launch_delta64(c, c->cap, c->ctl, c->hist);
-        CKR(capture_end(c, deps));
-        CKR(add_loop64(c, graph, deps, c->track ? c->G64 : nullptr));
+        launch_start64(c, c->cap);
     }
+    launch_delta64(c, c->cap, c->ctl, c->hist);
+    CKR(capture_end(c, deps));
+    CKR(add_loop64(c, graph, deps));
+    CKR(capture_begin(c, graph, deps));
+    launch_finish64(c, c->cap, c->ctl);
+    CKR(capture_end(c, deps));
+    c->graph_wide = c->wide;
     return LGF_OK;
 }
 
@@ -372,8 +430,15 @@ int instantiate(cudaGraph_t graph, cudaGraphExec_t* exec)
     return LGF_OK;
 }
 
+void drop_graph(lgf_ctx* c)
+{
+    if (c->exec) cudaGraphExecDestroy(c->exec);
+    c->exec = nullptr;
+}
+
 int build_graph(lgf_ctx* c)
 {
+    if (c->exec && c->graph_wide != c->wide) drop_graph(c);
     if (c->exec) return LGF_OK;
     cudaGraph_t graph;
     CK(cudaGraphCreate(&graph, 0));
@@ -384,12 +449,6 @@ int build_graph(lgf_ctx* c)
         return r;
     }
     return instantiate(graph, &c->exec);
-}
-
-void drop_graph(lgf_ctx* c)
-{
-    if (c->exec) cudaGraphExecDestroy(c->exec);
-    c->exec = nullptr;
 }
 
 // ---------------------------------------------------------------- set-up
@@ -505,6 +564,9 @@ int create_impl(const int dims[4], int flags, lgf_ctx* c)
     CKR(alloc(&c->Fd, 4 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->AH64, 16 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->Fs64, Vs * sizeof(double)));
+    CK(fx_prepare(d));
+    CKR(alloc((void**)&c->UX, 24 * Vs * sizeof(longlong2)));
+    if (c->track) CKR(alloc((void**)&c->GX, 6 * Vs * sizeof(longlong2)));
     if (c->mixed) {
         CKR(alloc((void**)&c->U32, 24 * Vs * sizeof(float2)));
         CKR(alloc((void**)&c->U32b, 24 * Vs * sizeof(float2)));
@@ -538,7 +600,7 @@ void free_all(lgf_ctx* c)
     if (c->exec) cudaGraphExecDestroy(c->exec);
     void* ptrs[] = {c->U64, c->G64, c->g64, c->U32, c->G32, c->g32, c->Fd, c->partials, c->ctl, c->ctl_stage,
                     c->hist, c->err, c->stage, c->tables, c->mult, c->AH64, c->Fs64, c->U32b, c->AH32, c->Fs32, c->dGp, c->dGud, c->dQ, c->dGgs, c->dFA, c->dFB,
-                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync};
+                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX, c->GX};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->host_ctl) cudaFreeHost(c->host_ctl);
@@ -999,6 +1061,7 @@ int lgf_set_links(lgf_ctx* c, const double* U, int on_device)
     memcpy(&ef, &e[2], sizeof ef);
     if (!(eu < 1e-12) || !(ed < 1e-12)) return LGF_ERR_NOT_SU3;
     if (!(ef < kForm8Tol)) return LGF_ERR_NOT_SU3;  // 8-real form only (0 otherwise)
+    c->wide = false;
     c->have_links = true;
     return LGF_OK;
 }
@@ -1019,6 +1082,7 @@ int lgf_fix(lgf_ctx* c, double alpha, double theta_tol, int max_iter, int* iters
     c->last_iters = r.iter;
     c->last_iters32 = r.iter_phase0;
     c->last_hist = r.iter + 1;
+    if (r.bad) c->wide = true;  // the stored links are NaN now
     if (iters) *iters = r.iter;
     if (F) *F = r.F;
     if (theta) *theta = r.theta;
@@ -1083,9 +1147,16 @@ int lgf_load_links(lgf_ctx* c, const void* src)
 {
     if (!c || !src) return LGF_ERR_ARG;
     CK(cudaMemcpyAsync(c->U64, src, lgf_links_state_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
+    // a snapshot is not checked: whether its links are in the fixed-point range
+    int* wide = reinterpret_cast<int*>(c->err);
+    CK(cudaMemsetAsync(wide, 0, sizeof(int), c->stream));
+    launch_check_range(c->lat, c->stream, c->U64, wide);
     if (c->track) launch_identity_rows64(c->stream, c->V, c->G64);
     CK(cudaGetLastError());
+    int h = 0;
+    CK(cudaMemcpyAsync(&h, wide, sizeof h, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    c->wide = h != 0;
     c->have_links = true;
     return LGF_OK;
 }
@@ -1275,32 +1346,19 @@ int lgf_time_kernels(lgf_ctx* c, double alpha, int n_iter, int precision, double
         launch_mixed_prep(s, c->V, c->lat.ne, c->U64, c->U32, c->G32, c->ctl_stage);
         launch_start32(c, s, c->ctl_stage, nullptr);
     } else {
-        launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
+        launch_start64(c, s);
     }
     for (int it = 0; it < n_iter && rc == LGF_OK; it++) {
         cudaEventRecord(ev[0], s);
         if (precision == 64) {
             // the kernels lgf_fix runs (the accelerator in FP32 when so set)
-            double2* Fd = reinterpret_cast<double2*>(c->Fd);
-            float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
-            if (c->accel32)
-                launch_delta64_f32(c->lat, c->sh64, s, c->AH64, c->Fs64, Fd32, c->partials, c->ctl_stage, nullptr);
-            else
-                launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, Fd, c->partials, c->ctl_stage,
-                                     nullptr, true);
+            launch_delta64(c, s, c->ctl_stage, nullptr);
             cudaEventRecord(ev[1], s);
-            if (c->accel32)
-                launch_zt<float>(c->lat32, c->sh32, c->tb, s, Fd32, c->ctl_stage);
-            else
-                launch_zt<double>(c->lat, c->sh64, c->tb, s, Fd, c->ctl_stage);
+            launch_zt64(c, s, c->ctl_stage);
             cudaEventRecord(ev[2], s);
-            if (c->accel32)
-                launch_xyinv_g32_64(c->lat32, c->sh32, s, Fd32, c->g64, c->ctl_stage);
-            else
-                launch_xyinv_g<double>(c->lat, c->sh64, c->tb, s, Fd, c->g64, c->ctl_stage);
+            launch_g64(c, s, c->ctl_stage);
             cudaEventRecord(ev[3], s);
-            launch_update<double>(c->lat, s, c->U64, c->track ? c->G64 : nullptr, c->g64, c->ctl_stage, c->AH64,
-                                  c->Fs64);
+            launch_update64(c, s, c->ctl_stage);
         } else {
             // FP32 phase.  Fused: FFT(x,y) alone, then z,t, IFFT(x,y) + g, and the update
             // fused with Delta, theta and F (links alternate between the two buffers).
@@ -1342,6 +1400,10 @@ int lgf_time_kernels(lgf_ctx* c, double alpha, int n_iter, int precision, double
     }
     for (int i = 0; i < 5; i++) cudaEventDestroy(ev[i]);
     if (rc != LGF_OK) return rc;
+    if (precision == 64) {
+        launch_finish64(c, s, c->ctl_stage);
+        CK(cudaStreamSynchronize(s));
+    }
     CK(cudaGetLastError());
     // median over the iterations: a launch delayed by the host (the events bracket
     // the enqueue as well as the kernel) shows up as an outlier, not in the median
@@ -1499,6 +1561,11 @@ int lgf_batch_fix(lgf_batch* b, double alpha, double theta_tol, int max_iter, in
         if (b->exec) cudaGraphExecDestroy(b->exec);
         b->exec = nullptr;
     }
+    for (lgf_ctx* c : b->ctx)
+        if (b->exec && c->graph_wide != c->wide) {
+            cudaGraphExecDestroy(b->exec);
+            b->exec = nullptr;
+        }
     CKR(batch_build(b));
     for (lgf_ctx* c : b->ctx) {
         *c->host_ctl = initial_ctl(c, alpha, theta_tol, max_iter);
@@ -1517,6 +1584,7 @@ int lgf_batch_fix(lgf_batch* b, double alpha, double theta_tol, int max_iter, in
         c->last_iters = r.iter;
         c->last_iters32 = r.iter_phase0;
         c->last_hist = r.iter + 1;
+        if (r.bad) c->wide = true;
         const int st = status_of(r);
         if (iters) iters[i] = r.iter;
         if (F) F[i] = r.F;
@@ -1623,6 +1691,7 @@ int lgf_set_unit_links(lgf_ctx* c)
 {
     if (!c) return LGF_ERR_ARG;
     if (c->lat.ne == 4) return LGF_ERR_STATE;  // the 8-real form cannot hold the unit matrix
+    c->wide = false;
     launch_unit_links(c->stream, c->lat, c->U64);
     if (c->track) launch_identity_rows64(c->stream, c->V, c->G64);
     CK(cudaGetLastError());

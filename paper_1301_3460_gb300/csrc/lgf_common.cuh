@@ -16,6 +16,7 @@ namespace lgf {
 template <typename T> struct vec2;
 template <> struct vec2<double> { using type = double2; };
 template <> struct vec2<float> { using type = float2; };
+template <> struct vec2<long long> { using type = longlong2; };  // fixed point (lgf_fx.cuh)
 template <typename T> using vec2_t = typename vec2<T>::type;
 
 template <typename T> struct cx {
@@ -259,6 +260,7 @@ struct Ctl {
     int stall;             // FP32 phase ends after this many iterations without a new smallest theta (0: never) ...
     int stall_near;        // ... or after this many once theta_best < near_floor
     double near_floor;
+    int bad;               // an entry of g was not finite (fixed-point iterations): theta and F become NaN
     int fault;             // a kernel gave up waiting for its own asynchronous copies (loop stopped)
 };
 

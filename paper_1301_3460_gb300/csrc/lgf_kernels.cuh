@@ -22,8 +22,11 @@
 // its eight real degrees of freedom; the accelerator is real and even in k, so
 // it maps each packed real pair to a real pair and the packing commutes with it.
 #pragma once
+#include <type_traits>
+
 #include "lgf_common.cuh"
 #include "lgf_dft.cuh"
+#include "lgf_fx.cuh"
 
 namespace lgf {
 
@@ -233,8 +236,10 @@ static __device__ void reduce_theta_F(double th, double f, double* __restrict__ 
     a = block_sum(a, scratch);
     b = block_sum(b, scratch);
     if (threadIdx.x == 0) {
-        const double theta = a / (3.0 * (double)V);
-        const double F = b / (12.0 * (double)V);
+        // fixed-point links cannot hold the NaN of a g that is not finite
+        const double nan = ld_flag(&ctl->bad) ? __hiloint2double(0x7ff80000, 0) : 0.0;
+        const double theta = a / (3.0 * (double)V) + nan;
+        const double F = b / (12.0 * (double)V) + nan;
         ctl->theta = theta;
         ctl->F = F;
         const int it = ctl->iter;
@@ -648,6 +653,42 @@ __device__ __forceinline__ void reunit_rows(cx<double>* X /* 6 in */, cx<double>
     complete_row2(g, g + 6);
 }
 
+// g of site s from its orthonormal rows 0,1: the nine entries in the form g is
+// stored in.  Row 2 = conj(r0 x r1) in that form's own arithmetic, from the rounded
+// rows, so that the stored g is unitary to that rounding; fixed point sets
+// Ctl::bad when an entry is not finite.
+template <typename TG>
+__device__ __forceinline__ void store_g(vec2_t<TG>* __restrict__ g, int V, int s, const cx<double>* gm, const Ctl* ctl)
+{
+    if constexpr (std::is_same_v<TG, fx>) {
+        cfx r[6], r2[3];
+        cdig rd[6];
+        bool bad = false;
+#pragma unroll
+        for (int e = 0; e < 6; e++) {
+            r[e] = cfx{d2fx(gm[e].re, &bad), d2fx(gm[e].im, &bad)};
+            rd[e] = digits(r[e]);
+            stx(g + (size_t)e * V + s, r[e]);
+        }
+        fx_row2(rd, rd + 3, r2);
+#pragma unroll
+        for (int e = 0; e < 3; e++) stx(g + (size_t)(6 + e) * V + s, r2[e]);
+        if (bad) const_cast<Ctl*>(ctl)->bad = 1;
+    } else {
+        cx<TG> gs[9];
+        if constexpr (sizeof(TG) == 4) {
+#pragma unroll
+            for (int e = 0; e < 6; e++) gs[e] = mk<TG>(d2f_int(gm[e].re), d2f_int(gm[e].im));
+        } else {
+#pragma unroll
+            for (int e = 0; e < 6; e++) gs[e] = gm[e];
+        }
+        complete_row2(gs, gs + 6);
+#pragma unroll
+        for (int e = 0; e < 9; e++) st<TG>(g + (size_t)e * V + s, gs[e]);
+    }
+}
+
 // One xy-plane by one block: inverse transform along y (columns read from Fd)
 // and x (rows of the plane tile sm), then g = reunit(1 + alpha/2 Delta~) by row
 // Gram-Schmidt in FP64 whatever T is; g stored as TG.
@@ -688,22 +729,10 @@ __device__ __forceinline__ void xyinv_g_plane(const Lat& d, const vec2_t<T>* __r
             X[4] = mk<double>(1.0, h * f3.y);
             X[5] = mk<double>(h * f2.x, h * f2.y);
         }
-        // Gram-Schmidt in FP64; row 2 = conj(r0 x r1) in the precision g is
-        // stored in (for an FP32 g, from the rounded rows, so that the stored g
-        // is unitary to FP32 rounding)
+        // Gram-Schmidt in FP64
         cx<double> gm[6];
         gram_schmidt01(X, gm);
-        cx<TG> gs[9];
-        if constexpr (sizeof(TG) == 4) {
-#pragma unroll
-            for (int e = 0; e < 6; e++) gs[e] = mk<TG>(d2f_int(gm[e].re), d2f_int(gm[e].im));
-        } else {
-#pragma unroll
-            for (int e = 0; e < 6; e++) gs[e] = mk<TG>((TG)gm[e].re, (TG)gm[e].im);
-        }
-        complete_row2(gs, gs + 6);
-#pragma unroll
-        for (int e = 0; e < 9; e++) st<TG>(g + (size_t)e * V + s0 + xy, gs[e]);
+        store_g<TG>(g, V, s0 + xy, gm, ctl);
     }
 }
 
@@ -739,12 +768,7 @@ __global__ void __launch_bounds__(256) k_build_g(Lat d, const vec2_t<T>* __restr
     X[5] = mk<double>(h * (double)f2.x, h * (double)f2.y);
     cx<double> gm[6];
     gram_schmidt01(X, gm);
-    cx<TG> gs[9];
-#pragma unroll
-    for (int e = 0; e < 6; e++) gs[e] = mk<TG>((TG)gm[e].re, (TG)gm[e].im);
-    complete_row2(gs, gs + 6);
-#pragma unroll
-    for (int e = 0; e < 9; e++) st<TG>(g + (size_t)e * V + s, gs[e]);
+    store_g<TG>(g, V, s, gm, ctl);
 }
 
 // ---------------------------------------------------------------- k_update

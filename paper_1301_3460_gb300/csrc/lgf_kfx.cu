@@ -1,0 +1,94 @@
+// The FP64 iterations on 64-bit fixed point: launchers of lgf_kfx.cuh and the g
+// builders that store a fixed-point g.
+#include "lgf_kfx.cuh"
+#include "lgf_launch_impl.cuh"
+
+namespace lgf {
+
+namespace {
+inline unsigned blocks(long n, int nt) { return (unsigned)((n + nt - 1) / nt); }
+}  // namespace
+
+cudaError_t fx_prepare(const Lat& d)
+{
+    int dev = 0, optin = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev))) return e;
+    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
+    if ((size_t)optin < plane_smem_bytes(d, sizeof(double2)) + 1024) return cudaErrorInvalidValue;
+    if ((e = allow_max_smem(k_delta_fx<true, 32, double>, optin))) return e;
+    if ((e = allow_max_smem(k_delta_fx<true, 128, double>, optin))) return e;
+    if ((e = allow_max_smem(k_delta_fx<true, 32, float>, optin))) return e;
+    if ((e = allow_max_smem(k_delta_fx<true, 128, float>, optin))) return e;
+    if ((e = allow_max_smem(k_xyinv_g<double, fx, 32>, optin))) return e;
+    if ((e = allow_max_smem(k_xyinv_g<double, fx, 128>, optin))) return e;
+    if ((e = allow_max_smem(k_xyinv_g<float, fx, 32>, optin))) return e;
+    return allow_max_smem(k_xyinv_g<float, fx, 128>, optin);
+}
+
+void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
+                     longlong2* AH, fx* Fs)
+{
+    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, U, G, AH, Fs);
+}
+void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
+                       const double2* G64, longlong2* U, longlong2* G, longlong2* AH, fx* Fs, Ctl* ctl)
+{
+    k_switch_gs<<<blocks(d.V, 256), 256, 0, s>>>(d.V, G32, Gs, ctl);
+    k_fx_project<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, Gs, U, G, AH, Fs, ctl);
+    k_phase_switch<<<1, 1, 0, s>>>(ctl);
+}
+void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
+                      const Ctl* ctl, bool always)
+{
+    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl, always ? 1 : 0);
+}
+void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
+                      longlong2* AH, fx* Fs)
+{
+    k_update_fx<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+}
+
+template <typename TF>
+void launch_fx_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const fx* Fs,
+                     vec2_t<TF>* Fd, double* partials, Ctl* ctl, double2* hist, bool fft)
+{
+    const size_t sm = plane_smem_bytes(d, sizeof(vec2_t<TF>));
+    if (!fft)
+        k_delta_fx<false, 128, TF><<<d.nplanes, sh64.nt_xy, 0, s>>>(d, AH, Fs, Fd, partials, ctl, hist);
+    else if (small_plane<double>(d))
+        k_delta_fx<true, 32, TF><<<d.nplanes, sh64.nt_xy, sm, s>>>(d, AH, Fs, Fd, partials, ctl, hist);
+    else
+        k_delta_fx<true, 128, TF><<<d.nplanes, sh64.nt_xy, sm, s>>>(d, AH, Fs, Fd, partials, ctl, hist);
+}
+
+template <typename TF>
+void launch_fx_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const vec2_t<TF>* Fd, longlong2* g,
+                       const Ctl* ctl)
+{
+    const size_t sm = plane_smem_bytes(d, sizeof(vec2_t<TF>));
+    if (small_plane<TF>(d))
+        k_xyinv_g<TF, fx, 32><<<d.nplanes, sh.nt_xy, sm, s>>>(d, Fd, g, ctl);
+    else
+        k_xyinv_g<TF, fx, 128><<<d.nplanes, sh.nt_xy, sm, s>>>(d, Fd, g, ctl);
+}
+
+void launch_fx_build_g(const Lat& d, cudaStream_t s, const double2* Fd, longlong2* g, const Ctl* ctl)
+{
+    k_build_g<double, fx><<<blocks(d.V, 256), 256, 0, s>>>(d, Fd, g, ctl);
+}
+
+void launch_check_range(const Lat& d, cudaStream_t s, const double2* U64, int* wide)
+{
+    k_check_range<<<blocks(4L * d.V, 256), 256, 0, s>>>(d, U64, wide);
+}
+
+template void launch_fx_delta<double>(const Lat&, const Shape&, cudaStream_t, const longlong2*, const fx*, double2*,
+                                      double*, Ctl*, double2*, bool);
+template void launch_fx_delta<float>(const Lat&, const Shape&, cudaStream_t, const longlong2*, const fx*, float2*,
+                                     double*, Ctl*, double2*, bool);
+template void launch_fx_xyinv_g<double>(const Lat&, const Shape&, cudaStream_t, const double2*, longlong2*,
+                                        const Ctl*);
+template void launch_fx_xyinv_g<float>(const Lat&, const Shape&, cudaStream_t, const float2*, longlong2*, const Ctl*);
+
+}  // namespace lgf
