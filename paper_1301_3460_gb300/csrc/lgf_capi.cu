@@ -101,8 +101,9 @@ struct lgf_ctx {
     // are within its range; `wide` links (a snapshot of anything else) take the FP64
     // kernels.  g64, AH64 and Fs64 hold the fixed-point g, parts and Re Tr meanwhile.
     longlong2* UX = nullptr;  // [4][6][V]
-    longlong2* GX = nullptr;  // [6][V]
     bool wide = false, graph_wide = false;
+    void* fxt_mem = nullptr;  // multipliers and exponents of the integer transform
+    FxtBuf fxt{};
     void* Fd = nullptr;       // [4][V] double2 (the FP32 phase uses the front half as float2)
     double2* AH64 = nullptr;  // [4][4][V] packed anti-Hermitian parts of the links
     double* Fs64 = nullptr;   // [V] Re Tr of the four links of a site
@@ -184,6 +185,10 @@ template <> const Shape& shape_of<float>(const lgf_ctx* c) { return c->sh32; }
 longlong2* as_fx(double2* p) { return reinterpret_cast<longlong2*>(p); }
 long long* as_fx(double* p) { return reinterpret_cast<long long*>(p); }
 
+// whether the FP64 loop's transforms run on integers: the default form (the
+// TMA-staged z,t kernel and the FP32 accelerator have their own)
+bool use_fxt(const lgf_ctx* c) { return !c->wide && !c->plain && !c->accel32 && !c->sh64.zt_tma; }
+
 // Delta, theta and F of the FP64 loop's links with the forward x,y transform: in
 // FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
 void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist)
@@ -191,7 +196,10 @@ void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist)
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
     float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
     const bool f32 = c->accel32 && !c->plain;
-    if (!c->wide) {
+    if (use_fxt(c)) {
+        launch_fxt_delta(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), as_fx(Fd), c->fxt, c->partials, ctl,
+                         hist);
+    } else if (!c->wide) {
         if (f32)
             launch_fx_delta<float>(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), Fd32, c->partials, ctl, hist,
                                    true);
@@ -208,7 +216,9 @@ void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist)
 // the z,t part of the accelerator in an FP64 iteration
 void launch_zt64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
-    if (c->accel32)
+    if (use_fxt(c))
+        launch_fxt_zt(c->lat, c->sh64, s, as_fx(reinterpret_cast<double2*>(c->Fd)), c->fxt, ctl);
+    else if (c->accel32)
         launch_zt<float>(c->lat32, c->sh32, c->tb, s, reinterpret_cast<float2*>(c->Fd), ctl);
     else
         launch_zt<double>(c->lat, c->sh64, c->tb, s, reinterpret_cast<double2*>(c->Fd), ctl);
@@ -219,7 +229,9 @@ void launch_g64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
     float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
-    if (!c->wide) {
+    if (use_fxt(c)) {
+        launch_fxt_xyinv_g(c->lat, c->sh64, s, as_fx(Fd), as_fx(c->g64), c->fxt, ctl);
+    } else if (!c->wide) {
         if (c->accel32)
             launch_fx_xyinv_g<float>(c->lat32, c->sh32, s, Fd32, as_fx(c->g64), ctl);
         else
@@ -234,7 +246,7 @@ void launch_g64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 void launch_update64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
     if (!c->wide)
-        launch_fx_update(c->lat, s, c->UX, c->GX, as_fx(c->g64), ctl, as_fx(c->AH64), as_fx(c->Fs64));
+        launch_fx_update(c->lat, s, c->UX, c->G64, as_fx(c->g64), ctl, as_fx(c->AH64), as_fx(c->Fs64));
     else
         launch_update<double>(c->lat, s, c->U64, c->G64, c->g64, ctl, c->AH64, c->Fs64);
 }
@@ -243,13 +255,13 @@ void launch_update64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 void launch_start64(lgf_ctx* c, cudaStream_t s)
 {
     if (!c->wide)
-        launch_fx_start(c->lat, s, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64), as_fx(c->Fs64));
+        launch_fx_start(c->lat, s, c->U64, c->UX, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
     else
         launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
 }
 void launch_finish64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
-    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->GX, c->U64, c->G64, ctl, c->mixed);
+    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->U64, c->G64, ctl, c->mixed);
 }
 
 // one FP64 iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, update,
@@ -398,8 +410,8 @@ int append_fix(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps
         CKR(add_loop32(c, graph, deps));
         CKR(capture_begin(c, graph, deps));
         if (!c->wide) {
-            launch_fx_project(c->lat, c->cap, c->G32, c->g64, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64),
-                              as_fx(c->Fs64), c->ctl);
+            launch_fx_project(c->lat, c->cap, c->G32, c->g64, c->U64, c->G64, c->UX, as_fx(c->AH64), as_fx(c->Fs64),
+                              c->fxt.fe, c->ctl);
         } else {
             launch_switch(c->cap, c->lat, c->G32, c->g64, c->U64, c->G64, c->ctl);
             launch_start64(c, c->cap);
@@ -517,6 +529,11 @@ int build_tables(lgf_ctx* c)
     CK(cudaDeviceSynchronize());
     c->tb.mult64 = m64;
     c->tb.mult32 = m32;
+    CKR(alloc(&c->fxt_mem, fxt_bytes(c->lat)));
+    c->fxt = fxt_carve(c->lat, c->fxt_mem);
+    launch_fxt_tables(c->lat, nullptr, m64, c->fxt);
+    CK(cudaGetLastError());
+    CK(cudaDeviceSynchronize());
     return LGF_OK;
 }
 
@@ -566,7 +583,6 @@ int create_impl(const int dims[4], int flags, lgf_ctx* c)
     CKR(alloc((void**)&c->Fs64, Vs * sizeof(double)));
     CK(fx_prepare(d));
     CKR(alloc((void**)&c->UX, 24 * Vs * sizeof(longlong2)));
-    if (c->track) CKR(alloc((void**)&c->GX, 6 * Vs * sizeof(longlong2)));
     if (c->mixed) {
         CKR(alloc((void**)&c->U32, 24 * Vs * sizeof(float2)));
         CKR(alloc((void**)&c->U32b, 24 * Vs * sizeof(float2)));
@@ -600,7 +616,7 @@ void free_all(lgf_ctx* c)
     if (c->exec) cudaGraphExecDestroy(c->exec);
     void* ptrs[] = {c->U64, c->G64, c->g64, c->U32, c->G32, c->g32, c->Fd, c->partials, c->ctl, c->ctl_stage,
                     c->hist, c->err, c->stage, c->tables, c->mult, c->AH64, c->Fs64, c->U32b, c->AH32, c->Fs32, c->dGp, c->dGud, c->dQ, c->dGgs, c->dFA, c->dFB,
-                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX, c->GX};
+                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX, c->fxt_mem};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->host_ctl) cudaFreeHost(c->host_ctl);
@@ -719,16 +735,28 @@ template <typename T> int time_shape(lgf_ctx* c, const Shape& sh, int which, flo
         if (which == 0) {
             // the plane kernels of the precision's iteration: FP64 Delta + FFT(x,y) and
             // IFFT(x,y) + g; FP32 FFT(x,y) and IFFT(x,y) + g
-            if constexpr (sizeof(T) == 8)
+            if constexpr (sizeof(T) == 8) {
+                if (use_fxt(c)) {
+                    launch_fxt_delta(c->lat, sh, s, as_fx(c->AH64), as_fx(c->Fs64), as_fx(reinterpret_cast<double2*>(c->Fd)),
+                                     c->fxt, c->partials, c->ctl_stage, nullptr);
+                    launch_fxt_xyinv_g(c->lat, sh, s, as_fx(reinterpret_cast<double2*>(c->Fd)), as_fx(c->g64), c->fxt, c->ctl_stage);
+                    continue;
+                }
                 launch_delta<double>(c->lat, sh, c->tb, s, c->AH64, c->Fs64, reinterpret_cast<double2*>(c->Fd),
                                      c->partials, c->ctl_stage, nullptr, true);
-            else if (c->fused32)
+            } else if (c->fused32)
                 launch_xy_fft<float>(c->lat32, sh, c->tb, s, reinterpret_cast<float2*>(c->Fd), false);
             else
                 launch_delta<float>(c->lat32, sh, c->tb, s, c->AH32, c->Fs32, reinterpret_cast<float2*>(c->Fd),
                                     c->partials, c->ctl_stage, nullptr, true);
             launch_xyinv_g<T>(lat_of<T>(c), sh, c->tb, s, Fd, g_of<T>(c), c->ctl_stage);
         } else {
+            if constexpr (sizeof(T) == 8) {
+                if (use_fxt(c) && !sh.zt_tma) {
+                    launch_fxt_zt(c->lat, sh, s, as_fx(reinterpret_cast<double2*>(c->Fd)), c->fxt, c->ctl_stage);
+                    continue;
+                }
+            }
             launch_zt<T>(lat_of<T>(c), sh, c->tb, s, Fd, c->ctl_stage);
         }
     }
@@ -797,7 +825,7 @@ int autotune_ctx(lgf_ctx* c)
 {
     if (!c->have_links) return LGF_ERR_STATE;
     CKR(reset_stage_ctl(c, 0.08));
-    launch_ah_init<double>(c->lat, c->stream, c->U64, c->AH64, c->Fs64);
+    launch_start64(c, c->stream);
     CKR(autotune_prec<double>(c));
     if (c->mixed) {
         launch_mixed_prep(c->stream, c->V, c->lat.ne, c->U64, c->U32, c->G32, c->ctl_stage);

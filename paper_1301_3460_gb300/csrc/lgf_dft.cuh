@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "lgf_common.cuh"
+#include "lgf_fx.cuh"
 
 namespace lgf {
 
@@ -151,6 +152,46 @@ __host__ __device__ constexpr double cos384(int m)
 }
 __host__ __device__ constexpr double sin384(int m) { return cos384(96 - m); }
 
+// round(2^62 cos(2 pi m / 384)) for 0 <= m <= 96: the roots of the fixed-point
+// transforms (evaluated with 200 bits)
+__host__ __device__ constexpr fx cos384xq(int m)
+{
+    constexpr fx t[97] = {
+    4611686018427387904ll, 4611068688496516515ll, 4609216863978052423ll, 4606131040650197959ll,
+    4601812044662475904ll, 4596261032314549277ll, 4589479489746651964ll, 4581469232541713033ll,
+    4572232405239281286ll, 4561771480761380163ll, 4550089259750446721ll, 4537188869819531930ll,
+    4523073764714963030ll, 4507747723391692126ll, 4491214849001578570ll, 4473479567794875989ll,
+    4454546627935218059ll, 4434421098228420290ll, 4413108366765438139ll, 4390614139479844773ll,
+    4366944438620214675ll, 4342105601137822079ll, 4316104276990085883ll, 4288947427360215242ll,
+    4260642322793532497ll, 4231196541250972386ll, 4200617966080278656ll, 4168914783905441250ll,
+    4136095482434939102ll, 4102168848189375341ll, 4067143964149113252ll, 4031030207322542809ll,
+    3993837246235628775ll, 3955575038343412514ll, 3916253827364160492ll, 3875884140536873200ll,
+    3834476785802888710ll, 3792042848912335440ll, 3748593690456208775ll, 3704140942824866152ll,
+    3658696507093754878ll, 3612272549837206457ll, 3564881499871150442ll, 3516536044925619868ll,
+    3467249128247939127ll, 3417033945137503676ll, 3365903939413079316ll, 3313872799813566826ll,
+    3260954456333195553ll, 3207163076492127117ll, 3152513061543467682ll, 3097019042617704261ll,
+    3040695876805597297ll, 2983558643180578204ll, 2925622638761716784ll, 2866903374418339332ll,
+    2807416570717393844ll, 2747178153714674114ll, 2686204250691029488ll, 2624511185834701810ll,
+    2562115475870945497ll, 2499033825640100800ll, 2435283123625304105ll, 2370880437431032621ll,
+    2305843009213693952ll, 2240188251065483894ll, 2173933740352748318ll, 2107097215010097159ll,
+    2039696568791530406ll, 1971749846479847467ll, 1903275239055622476ll, 1834291078827038919ll,
+    1764815834521887442ll, 1694868106343040831ll, 1624466620988729937ll, 1553630226638953726ll,
+    1482377887909365732ll, 1410728680773987865ll, 1338701787458110889ll, 1266316491302748871ll,
+    1193592171602022505ll, 1120548298414853464ll, 1047204427352358823ll, 973580194342341097ll,
+    899695310372275547ll, 825569556212202211ll, 751222777118935442ll, 676674877523008785ll, 601945815699777620ll,
+    527055598426106234ll, 452024275624069880ll, 376871934993105809ll, 301618696632050392ll, 226284707652502141ll,
+    150890136784952761ll, 75455168979130296ll, 0ll};
+    return t[m];
+}
+__host__ __device__ constexpr fx cos384x(int m)
+{
+    m %= 384;
+    if (m < 0) m += 384;
+    if (m > 192) m = 384 - m;
+    return m <= 96 ? cos384xq(m) : -cos384xq(192 - m);
+}
+__host__ __device__ constexpr fx sin384x(int m) { return cos384x(96 - m); }
+
 __host__ __device__ constexpr int imod(int a, int n) { return ((a % n) + n) % n; }
 
 // b^-1 mod n for coprime b, n (small n: by search)
@@ -188,6 +229,32 @@ template <typename T, bool INV> __host__ __device__ __forceinline__ cx<T> mul_ni
     else return cx<T>{z.im, -z.re};
 }
 
+// ---------------------------------------------------------------- fixed-point products
+
+// Transforms of integers (T = fx): values of up to 2^62 in magnitude, roots x 2^62
+// in digits (lgf_fx.cuh), every product rounded to nearest.  Against the doubles'
+// relative 2^-53 the absolute error of one product is 2^-1 or less, so a line
+// scaled to fill 57 bits keeps more precision than FP64 arithmetic does.
+
+// root x 2^62 -> digits (a value of exactly 2^62 is exact in its high digit)
+__host__ __device__ constexpr dig xdigits(fx v)
+{
+    return dig{(int)(v >> 32) + (int)((unsigned)v >> 31), (int)(unsigned)v};
+}
+// w b for a root w (digits of its real and imaginary part)
+__host__ __device__ __forceinline__ cx<fx> xcmul(dig wr, dig wi, dig nwi, cx<fx> b)
+{
+    const dig br = digits(b.re), bi = digits(b.im);
+    facc r = fmul<2>(br, wr), i = fmul<2>(br, wi);
+    fmac(r, bi, nwi);
+    fmac(i, bi, wr);
+    return cx<fx>{fval<2>(r), fval<2>(i)};
+}
+// c x for a real c
+__host__ __device__ __forceinline__ fx xrmul(dig c, fx x) { return fval<2>(fmul<2>(digits(x), c)); }
+// x / 2, ties to even (a fixed rounding direction would add up over the lattice)
+__host__ __device__ __forceinline__ fx xhalf(fx x) { return (x + ((x >> 1) & 1)) >> 1; }
+
 // ---------------------------------------------------------------- butterflies
 
 // x0 = a + w b, x1 = a - w b with w = w_N^E (exp(-2 pi i E/N) forward,
@@ -208,6 +275,25 @@ __host__ __device__ __forceinline__ void bfly2(cx<T> a, cx<T> b, cx<T>& x0, cx<T
         x1 = a + b;
     } else if constexpr (4 * e == 3 * N) {
         const cx<T> wb = mul_ni<T, !INV>(b);  // w = +i forward
+        x0 = a + wb;
+        x1 = a - wb;
+    } else if constexpr (std::is_same_v<T, fx>) {
+        static_assert(384 % N == 0, "roots of unity of order dividing 384");
+        constexpr int m = e * (384 / N);
+        cx<fx> wb;
+        if constexpr (m % 96 == 48) {
+            // odd multiples of an eighth of a turn: two real products
+            constexpr dig c = xdigits(cos384x(48));
+            constexpr bool cneg = cos384x(m) < 0, sneg = (sin384x(m) < 0) == INV;  // signs of Re w, Im w
+            // w = (+-1 +- i) sqrt(1/2)
+            const fx sr = cneg ? -b.re : b.re, si = cneg ? -b.im : b.im;
+            const fx tr = sneg ? -b.re : b.re, ti = sneg ? -b.im : b.im;
+            wb = cx<fx>{xrmul(c, sr - ti), xrmul(c, tr + si)};
+        } else {
+            constexpr fx wi = INV ? sin384x(m) : -sin384x(m);
+            constexpr dig dr = xdigits(cos384x(m)), di = xdigits(wi), dn = xdigits(-wi);
+            wb = xcmul(dr, di, dn, b);
+        }
         x0 = a + wb;
         x1 = a - wb;
     } else {
@@ -240,6 +326,17 @@ template <typename T, bool INV> __host__ __device__ __forceinline__ void dft3(cx
 {
     // X1 = c -+ i h (x1 - x2), X2 = c +- i h (x1 - x2), c = x0 - (x1 + x2)/2,
     // h = sqrt(3)/2 (upper signs forward)
+    if constexpr (std::is_same_v<T, fx>) {
+        constexpr dig h = xdigits(3993837246235628775ll);  // round(2^62 sqrt(3)/2)
+        const cx<fx> t1 = v[1] + v[2], t2 = v[1] - v[2];
+        const cx<fx> c = cx<fx>{v[0].re - xhalf(t1.re), v[0].im - xhalf(t1.im)};
+        const fx sr = xrmul(h, t2.re), si = xrmul(h, t2.im);
+        v[0] = v[0] + t1;
+        const cx<fx> w = INV ? cx<fx>{-si, sr} : cx<fx>{si, -sr};
+        v[1] = c + w;
+        v[2] = c - w;
+        return;
+    } else {
     constexpr T h = (T)0.866025403784438646763723170752936183;
     const cx<T> t1 = v[1] + v[2], t2 = v[1] - v[2];
     const cx<T> c = cx<T>{fma((T)-0.5, t1.re, v[0].re), fma((T)-0.5, t1.im, v[0].im)};
@@ -247,6 +344,7 @@ template <typename T, bool INV> __host__ __device__ __forceinline__ void dft3(cx
     constexpr T s = INV ? -h : h;  // X1 = c + s (t2_i, -t2_r)
     v[1] = cx<T>{fma(s, t2.im, c.re), fma(-s, t2.re, c.im)};
     v[2] = cx<T>{fma(-s, t2.im, c.re), fma(s, t2.re, c.im)};
+    }
 }
 
 template <typename T, bool INV> __host__ __device__ __forceinline__ void dft4(cx<T>* v)
@@ -355,13 +453,30 @@ template <typename T, int L, int NL = line_lanes<T>(L)> __host__ __device__ __fo
 // tau < T, chosen among T compile-time constants
 template <typename T, int L, int Tl, int E, bool INV> __host__ __device__ __forceinline__ cx<T> lane_root(int tau)
 {
-    cx<T> w = cx<T>{(T)1, (T)0};
-    sfor<1, Tl>([&](auto t) {
-        constexpr int m = imod(t.value * E * (384 / L), 384);
-        constexpr T c = (T)cos384(m), sn = (T)(INV ? sin384(m) : -sin384(m));
-        if (tau == t.value) w = cx<T>{c, sn};
-    });
-    return w;
+    if constexpr (std::is_same_v<T, fx>) {
+        cx<fx> w = cx<fx>{1ll << 62, 0};  // x 2^62
+        sfor<1, Tl>([&](auto t) {
+            constexpr int m = imod(t.value * E * (384 / L), 384);
+            constexpr fx c = cos384x(m), sn = INV ? sin384x(m) : -sin384x(m);
+            if (tau == t.value) w = cx<fx>{c, sn};
+        });
+        return w;
+    } else {
+        cx<T> w = cx<T>{(T)1, (T)0};
+        sfor<1, Tl>([&](auto t) {
+            constexpr int m = imod(t.value * E * (384 / L), 384);
+            constexpr T c = (T)cos384(m), sn = (T)(INV ? sin384(m) : -sin384(m));
+            if (tau == t.value) w = cx<T>{c, sn};
+        });
+        return w;
+    }
+}
+
+// v times a root from lane_root
+template <typename T> __host__ __device__ __forceinline__ cx<T> mul_root(cx<T> v, cx<T> w)
+{
+    if constexpr (std::is_same_v<T, fx>) return xcmul(digits(w.re), digits(w.im), digits(-w.im), v);
+    else return cmul(v, w);
 }
 
 // steps 1-2 of the forward line transform in one lane (step 1 alone for T = 1)
@@ -371,7 +486,7 @@ __host__ __device__ __forceinline__ void line_fwd_local(cx<T>* v, int tau)
     constexpr int Tl = NL, R = L / Tl;
     dft<T, R, false>(v);
     if constexpr (Tl > 1) {
-        sfor<1, R>([&](auto r) { v[r.value] = cmul(v[r.value], lane_root<T, L, Tl, r.value, false>(tau)); });
+        sfor<1, R>([&](auto r) { v[r.value] = mul_root<T>(v[r.value], lane_root<T, L, Tl, r.value, false>(tau)); });
     }
 }
 
@@ -381,7 +496,7 @@ __host__ __device__ __forceinline__ void line_inv_local(cx<T>* v, int tau)
 {
     constexpr int Tl = NL, R = L / Tl;
     if constexpr (Tl > 1) {
-        sfor<1, R>([&](auto r) { v[r.value] = cmul(v[r.value], lane_root<T, L, Tl, r.value, true>(tau)); });
+        sfor<1, R>([&](auto r) { v[r.value] = mul_root<T>(v[r.value], lane_root<T, L, Tl, r.value, true>(tau)); });
     }
     dft<T, R, true>(v);
 }
@@ -403,6 +518,8 @@ __host__ __device__ __forceinline__ float sflip(float x, unsigned m)
     return m ? -x : x;
 #endif
 }
+
+__host__ __device__ __forceinline__ fx sflip(fx x, unsigned m) { return m ? -x : x; }
 
 // One radix-2 stage across lanes for lane bit h, o the partner lane's value
 // (partner tau ^ h).  Forward (decimation in frequency): the low lane keeps
@@ -441,7 +558,7 @@ template <typename T, int R, bool INV> __host__ __device__ __forceinline__ void 
     } else if (h == 4) {
         const cx<T> w = lane_root<T, 8, 4, 1, INV>((tau & 4) ? (tau & 3) : 0);
 #pragma unroll
-        for (int r = 0; r < R; r++) v[r] = cmul(v[r], w);
+        for (int r = 0; r < R; r++) v[r] = mul_root<T>(v[r], w);
     }
 }
 

@@ -661,18 +661,15 @@ template <typename TG>
 __device__ __forceinline__ void store_g(vec2_t<TG>* __restrict__ g, int V, int s, const cx<double>* gm, const Ctl* ctl)
 {
     if constexpr (std::is_same_v<TG, fx>) {
-        cfx r[6], r2[3];
         cdig rd[6];
         bool bad = false;
 #pragma unroll
         for (int e = 0; e < 6; e++) {
-            r[e] = cfx{d2fx(gm[e].re, &bad), d2fx(gm[e].im, &bad)};
-            rd[e] = digits(r[e]);
-            stx(g + (size_t)e * V + s, r[e]);
+            rd[e] = digits(cfx{d2fx<kFxG>(gm[e].re, &bad), d2fx<kFxG>(gm[e].im, &bad)});
+            std_(g + (size_t)e * V + s, rd[e]);
         }
-        fx_row2(rd, rd + 3, r2);
 #pragma unroll
-        for (int e = 0; e < 3; e++) stx(g + (size_t)(6 + e) * V + s, r2[e]);
+        for (int j = 0; j < 3; j++) std_(g + (size_t)(6 + j) * V + s, digits(fx_row2<2>(rd, rd + 3, j)));
         if (bad) const_cast<Ctl*>(ctl)->bad = 1;
     } else {
         cx<TG> gs[9];

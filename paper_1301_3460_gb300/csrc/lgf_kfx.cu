@@ -1,6 +1,6 @@
 // The FP64 iterations on 64-bit fixed point: launchers of lgf_kfx.cuh and the g
 // builders that store a fixed-point g.
-#include "lgf_kfx.cuh"
+#include "lgf_fxt.cuh"
 #include "lgf_launch_impl.cuh"
 
 namespace lgf {
@@ -23,30 +23,85 @@ cudaError_t fx_prepare(const Lat& d)
     if ((e = allow_max_smem(k_xyinv_g<double, fx, 32>, optin))) return e;
     if ((e = allow_max_smem(k_xyinv_g<double, fx, 128>, optin))) return e;
     if ((e = allow_max_smem(k_xyinv_g<float, fx, 32>, optin))) return e;
-    return allow_max_smem(k_xyinv_g<float, fx, 128>, optin);
+    if ((e = allow_max_smem(k_xyinv_g<float, fx, 128>, optin))) return e;
+    if ((e = allow_max_smem(k_delta_fxt<32>, optin))) return e;
+    if ((e = allow_max_smem(k_delta_fxt<128>, optin))) return e;
+    if ((e = allow_max_smem(k_zt_fxt<32>, optin))) return e;
+    if ((e = allow_max_smem(k_zt_fxt<128>, optin))) return e;
+    if ((e = allow_max_smem(k_xyinv_fxt<32>, optin))) return e;
+    return allow_max_smem(k_xyinv_fxt<128>, optin);
 }
 
-void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
-                     longlong2* AH, fx* Fs)
+size_t fxt_bytes(const Lat& d)
 {
-    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, U, G, AH, Fs);
+    return sizeof(FxExp) + ((size_t)d.nplanes + 4 * (size_t)d.P + (size_t)d.P * d.L[2]) * sizeof(int) +
+           (size_t)d.V * sizeof(fx);
 }
-void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
-                       const double2* G64, longlong2* U, longlong2* G, longlong2* AH, fx* Fs, Ctl* ctl)
+FxtBuf fxt_carve(const Lat& d, void* p)
+{
+    FxtBuf b;
+    b.mx = reinterpret_cast<fx*>(p);
+    b.fe = reinterpret_cast<FxExp*>(b.mx + d.V);
+    b.pexp = reinterpret_cast<int*>(b.fe + 1);
+    b.bexp = b.pexp + d.nplanes;
+    b.me = b.bexp + 4 * (size_t)d.P;
+    return b;
+}
+void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const FxtBuf& b)
+{
+    k_make_mult_fx<<<blocks((long)d.P * d.L[2], 128), 128, 0, s>>>(d, m64, b.mx, b.me);
+}
+void launch_fxt_delta(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* AH, const fx* Fs, longlong2* Fd,
+                      const FxtBuf& b, double* partials, Ctl* ctl, double2* hist)
+{
+    const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
+    if (small_plane<double>(d))
+        k_delta_fxt<32><<<d.nplanes, sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.pexp, b.fe, partials, ctl, hist);
+    else
+        k_delta_fxt<128><<<d.nplanes, sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.pexp, b.fe, partials, ctl, hist);
+}
+void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl)
+{
+    const size_t sm = pencil_smem_bytes(d, sh.xw, sizeof(longlong2)) + (size_t)sh.xw * d.L[2] * sizeof(int);
+    const dim3 grid(d.L[0] / sh.xw, d.L[1], 4);
+    if (short_zt_lines(d))
+        k_zt_fxt<32><<<grid, sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.mx, b.me, b.pexp, b.bexp, b.fe);
+    else
+        k_zt_fxt<128><<<grid, sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.mx, b.me, b.pexp, b.bexp, b.fe);
+}
+void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* Fd, longlong2* g,
+                        const FxtBuf& b, const Ctl* ctl)
+{
+    const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
+    int xs = 0;
+    while ((1 << xs) < sh.xw) xs++;
+    if (small_plane<double>(d))
+        k_xyinv_fxt<32><<<d.nplanes, sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.bexp, b.fe);
+    else
+        k_xyinv_fxt<128><<<d.nplanes, sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.bexp, b.fe);
+}
+
+void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, longlong2* U, longlong2* AH, fx* Fs,
+                     FxExp* fe)
+{
+    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, U, AH, Fs, fe);
+}
+void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64, double2* G64,
+                       longlong2* U, longlong2* AH, fx* Fs, FxExp* fe, Ctl* ctl)
 {
     k_switch_gs<<<blocks(d.V, 256), 256, 0, s>>>(d.V, G32, Gs, ctl);
-    k_fx_project<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, Gs, U, G, AH, Fs, ctl);
+    k_fx_project<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, Gs, U, AH, Fs, fe, ctl);
     k_phase_switch<<<1, 1, 0, s>>>(ctl);
 }
-void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
-                      const Ctl* ctl, bool always)
+void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, double2* U64, double2* G64, const Ctl* ctl,
+                      bool always)
 {
-    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl, always ? 1 : 0);
+    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, U64, G64, ctl, always ? 1 : 0);
 }
-void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
+void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, double2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, fx* Fs)
 {
-    k_update_fx<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+    k_update_fx<<<blocks(d.V, 64), 64, 0, s>>>(d, U, G, g, ctl, AH, Fs);
 }
 
 template <typename TF>

@@ -80,18 +80,31 @@ void launch_delta64_f32(const Lat& d, const Shape& sh64, cudaStream_t s, const d
 void launch_xyinv_g32_64(const Lat& d, const Shape& sh32, cudaStream_t s, const float2* Fd, double2* g,
                          const Ctl* ctl);
 
-// FP64 iterations on 64-bit fixed point (lgf_kfx.cuh): links, G and g on the grid
-// 2^-61, packed parts and Re Tr on 2^-57.  start: from the stored links; project:
-// the end of the FP32 phase (links rebuilt on the input's orbit, phase switched);
-// finish: back to the stored FP64 links and G.  TF: precision of the transforms.
+// FP64 iterations on 64-bit fixed point (lgf_kfx.cuh): links on the grid 2^-61, g on
+// 2^-62, packed parts and Re Tr on 2^-58; G in FP64.  start: from the stored links;
+// project: the end of the FP32 phase (links rebuilt on the input's orbit, phase
+// switched); finish: back to the stored FP64 links.  TF: precision of the transforms.
+struct FxExp;
+// buffers of the integer transform (lgf_fxt.cuh): multipliers and exponents, carved
+// from fxt_bytes(d) of device memory
+struct FxtBuf {
+    long long* mx = nullptr;  // [V]
+    FxExp* fe = nullptr;
+    int* pexp = nullptr;      // [planes]
+    int* bexp = nullptr;      // [pencils], at most 4 P
+    int* me = nullptr;        // [t-lines]
+};
+size_t fxt_bytes(const Lat& d);
+FxtBuf fxt_carve(const Lat& d, void* p);
+void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const FxtBuf& b);
 cudaError_t fx_prepare(const Lat& d);
-void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
-                     longlong2* AH, long long* Fs);
-void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
-                       const double2* G64, longlong2* U, longlong2* G, longlong2* AH, long long* Fs, Ctl* ctl);
-void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
-                      const Ctl* ctl, bool always);
-void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
+void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, longlong2* U, longlong2* AH, long long* Fs,
+                     FxExp* fe);
+void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64, double2* G64,
+                       longlong2* U, longlong2* AH, long long* Fs, FxExp* fe, Ctl* ctl);
+void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, double2* U64, double2* G64, const Ctl* ctl,
+                      bool always);
+void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, double2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, long long* Fs);
 template <typename TF>
 void launch_fx_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
@@ -99,6 +112,13 @@ void launch_fx_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const long
 template <typename TF>
 void launch_fx_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const vec2_t<TF>* Fd, longlong2* g,
                        const Ctl* ctl);
+// the iteration's transforms on integers: Delta + x,y forward; z,t with the
+// multiplier; x,y inverse + g
+void launch_fxt_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
+                      longlong2* Fd, const FxtBuf& b, double* partials, Ctl* ctl, double2* hist);
+void launch_fxt_zt(const Lat& d, const Shape& sh64, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl);
+void launch_fxt_xyinv_g(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* Fd, longlong2* g,
+                        const FxtBuf& b, const Ctl* ctl);
 void launch_fx_build_g(const Lat& d, cudaStream_t s, const double2* Fd, longlong2* g, const Ctl* ctl);
 // *wide set when a stored link is not within 1e-3 of SU(3)
 void launch_check_range(const Lat& d, cudaStream_t s, const double2* U64, int* wide);
