@@ -49,27 +49,32 @@ __device__ __forceinline__ void block_or(unsigned o, unsigned* s)
     if ((threadIdx.x & 31) == 0 && o) atomicOr(s, o);
 }
 
-// right shift by r >= 0, rounded to nearest
+// Right shift by r >= 0, rounded to nearest, ties away from zero: a tie rule that
+// favours one sign would add up over the lattice into the lowest momenta, which
+// the accelerator amplifies by up to p2max/p2min (at 64 x 16^3 ties up cost six times the
+// error of an FP64 transform; this is below it).
 struct RShift {
     fx rnd;
     int r;
 };
+__device__ __forceinline__ fx shift_round(fx v, fx rnd, int r) { return (v + rnd + (v >> 63)) >> r; }
 __device__ __forceinline__ RShift rshift(int r)
 {
     r = r < 0 ? 0 : (r > 62 ? 62 : r);
     return RShift{r > 0 ? 1ll << (r - 1) : 0ll, r};
 }
-__device__ __forceinline__ fx apply(RShift s, fx v) { return (v + s.rnd) >> s.r; }
+__device__ __forceinline__ fx apply(RShift s, fx v) { return s.r ? shift_round(v, s.rnd, s.r) : v; }
 __device__ __forceinline__ cfx apply(RShift s, cfx v) { return cfx{apply(s, v.re), apply(s, v.im)}; }
 // The bits to reserve for values that are aligned to others before a pass over lines
 // of L points: at least B + 1, so that the common exponent lies above every
 // exponent and each alignment is a right shift of one bit or more.
 __device__ __forceinline__ int align_top(unsigned o, int L) { return max(top_bits(o), fx_bits_rt(L) + 1); }
-// the alignment: a right shift of the value's own by r >= 1, rounded to nearest
+// the alignment: a right shift of the value's own by r >= 1
 __device__ __forceinline__ cfx rshift1(cfx v, int r)
 {
-    r = r > 62 ? 61 : r - 1;
-    return cfx{((v.re >> r) + 1) >> 1, ((v.im >> r) + 1) >> 1};
+    r = r > 62 ? 62 : r;
+    const fx rnd = 1ll << (r - 1);
+    return cfx{shift_round(v.re, rnd, r), shift_round(v.im, rnd, r)};
 }
 
 // Delta (as k_delta_fx), theta and F, then the forward transform along x and y.
