@@ -187,7 +187,10 @@ long long* as_fx(double* p) { return reinterpret_cast<long long*>(p); }
 
 // whether the FP64 loop's transforms run on integers: the default form (the
 // TMA-staged z,t kernel and the FP32 accelerator have their own)
-bool use_fxt(const lgf_ctx* c) { return !c->wide && !c->plain && !c->accel32 && !c->sh64.zt_tma; }
+bool use_fxt(const lgf_ctx* c)
+{
+    return !c->wide && !c->plain && !c->accel32 && !c->sh64.zt_tma && fxt_fits(c->lat, c->sh64);
+}
 
 // Delta, theta and F of the FP64 loop's links with the forward x,y transform: in
 // FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
@@ -752,7 +755,7 @@ template <typename T> int time_shape(lgf_ctx* c, const Shape& sh, int which, flo
             launch_xyinv_g<T>(lat_of<T>(c), sh, c->tb, s, Fd, g_of<T>(c), c->ctl_stage);
         } else {
             if constexpr (sizeof(T) == 8) {
-                if (use_fxt(c) && !sh.zt_tma) {
+                if (use_fxt(c) && !sh.zt_tma && fxt_fits(c->lat, sh)) {
                     launch_fxt_zt(c->lat, sh, s, as_fx(reinterpret_cast<double2*>(c->Fd)), c->fxt, c->ctl_stage);
                     continue;
                 }

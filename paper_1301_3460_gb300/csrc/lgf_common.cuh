@@ -205,7 +205,7 @@ struct Lat {
     int ne;        // complex entries stored per link: 6 (rows 0,1; row 2 rebuilt on load),
                    // 9 (row 2 kept as written, the rebuild done once when stored) or
                    // 4 (the 8-real form, FP64 only: u01, u02, u10, phases of u00 and u20)
-    FastDiv dLx, dLy, dP;  // division by Lx, Ly and Lx*Ly
+    FastDiv dLx, dLy, dP, dLz;  // division by Lx, Ly, Lx*Ly and Lz
 };
 
 // the division helpers of a lattice descriptor (call after L is set)
@@ -214,6 +214,7 @@ inline void lat_set_divisors(Lat& d)
     d.dLx = make_fastdiv((unsigned)d.L[0]);
     d.dLy = make_fastdiv((unsigned)d.L[1]);
     d.dP = make_fastdiv((unsigned)(d.L[0] * d.L[1]));
+    d.dLz = make_fastdiv((unsigned)d.L[2]);
 }
 
 __device__ __forceinline__ int site_shift(const Lat& d, int s, int c_mu, int mu, int dir)

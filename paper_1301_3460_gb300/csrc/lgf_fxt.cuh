@@ -1,16 +1,29 @@
-// The 4D transform of the FP64 iterations on 64-bit integers: the same passes and
-// tiles as k_delta, k_zt and k_xyinv_g (lgf_kernels.cuh), with block floating
-// point in place of FP64.
+// The 4D transform of the FP64 iterations on 64-bit integers, in block floating point:
+// Delta and the forward x,y transform per xy-plane, z,t with the accelerator per
+// pencil, the inverse x,y transform and g per plane, each in a shared-memory tile as
+// k_delta, k_zt and k_xyinv_g (lgf_kernels.cuh) do it in FP64.
 //
-// Every pass takes values of at most 2^B in magnitude, B = 62 - ceil(log2 L), so a
-// line of L points cannot overflow, and its rounding errors (about one unit) are
-// 2^-57 of the largest value for L = 32, below FP64's own (a line of 32 random
-// values: 0.9 units rms against 58 for the FP64 codelet).  Between passes the
+// A line of L = A B points is transformed in two steps, A-point codelets with the
+// twiddles w_L^(n2 k1) and B-point codelets (Cooley-Tukey: n = B n1 + n2, k = k1 +
+// A k2), in place, so that a thread holds at most 8 complex integers (16 beyond 64
+// points): 80 registers and 24 warps per SM, and 3 to 5 thousand instructions per
+// kernel.  Whole 32-point lines in registers, as the FP64 kernels have them, take 168
+// registers and 12,000 unrolled instructions in the z,t kernel and wait for
+// instruction fetches (32^4: 178/220/215 us against the figures at the kernels).
+// In place, frequency k of a line lands on position (k mod A) B + k / A; the fields
+// stay in that order between the kernels, the multiplier table is laid out in it,
+// and the inverse (B-point, twiddles, A-point) takes it back.  An inverse runs the
+// forward codelets with real and imaginary part exchanged on the way in and out.
+//
+// Every line transform takes values of at most 2^B in magnitude, B = 62 - ceil(log2
+// L), so that L points cannot overflow, and its rounding errors (about one unit)
+// are 2^-57 of the largest value for L = 32, below FP64's own (a line of 32 random
+// values: 0.9 units rms against 58 for the FP64 codelet).  Between transforms the
 // values are shifted so that the largest fills B bits again: the bits in use are
 // the OR of the values' magnitudes, gathered per tile in shared memory (per line
 // for the accelerated t-lines, whose multipliers differ by orders of magnitude).
 // A transform does not lower the largest value by more than half a bit, so after
-// the first pass right shifts (rounded to nearest) are enough.  A value is
+// the first one right shifts (rounded to nearest) are enough.  A value is
 // the integer times 2^E; E is kept per xy-plane after the Delta kernel (pexp), per
 // z,t pencil after the accelerator (bexp), and the consumer aligns them to the
 // largest magnitude exponent of all planes (FxExp::amax1) or pencils (amax2).
@@ -49,39 +62,110 @@ __device__ __forceinline__ void block_or(unsigned o, unsigned* s)
     if ((threadIdx.x & 31) == 0 && o) atomicOr(s, o);
 }
 
-// Right shift by r >= 0, rounded to nearest, ties away from zero: a tie rule that
+// Right shift by r >= 1, rounded to nearest, ties away from zero: a tie rule that
 // favours one sign would add up over the lattice into the lowest momenta, which
-// the accelerator amplifies by up to p2max/p2min (at 64 x 16^3 ties up cost six times the
-// error of an FP64 transform; this is below it).
+// the accelerator amplifies by up to p2max/p2min (at 64 x 16^3 ties up cost six times
+// the error of an FP64 transform; this is below it).
 struct RShift {
     fx rnd;
     int r;
 };
-__device__ __forceinline__ fx shift_round(fx v, fx rnd, int r) { return (v + rnd + (v >> 63)) >> r; }
 __device__ __forceinline__ RShift rshift(int r)
 {
-    r = r < 0 ? 0 : (r > 62 ? 62 : r);
-    return RShift{r > 0 ? 1ll << (r - 1) : 0ll, r};
+    r = r < 1 ? 1 : (r > 62 ? 62 : r);
+    return RShift{1ll << (r - 1), r};
 }
-__device__ __forceinline__ fx apply(RShift s, fx v) { return s.r ? shift_round(v, s.rnd, s.r) : v; }
+__device__ __forceinline__ fx apply(RShift s, fx v) { return (v + s.rnd + (v >> 63)) >> s.r; }
 __device__ __forceinline__ cfx apply(RShift s, cfx v) { return cfx{apply(s, v.re), apply(s, v.im)}; }
 // The bits to reserve for values that are aligned to others before a pass over lines
 // of L points: at least B + 1, so that the common exponent lies above every
 // exponent and each alignment is a right shift of one bit or more.
 __device__ __forceinline__ int align_top(unsigned o, int L) { return max(top_bits(o), fx_bits_rt(L) + 1); }
-// the alignment: a right shift of the value's own by r >= 1
-__device__ __forceinline__ cfx rshift1(cfx v, int r)
+
+// factors of a line length (B = 1: one codelet)
+template <int L> struct Fac {
+    static constexpr int A = L <= 8 ? L : L == 12 || L == 16 || L == 24 || L == 32 ? 4 : L == 48 || L == 64 ? 8 : 16;
+    static constexpr int B = L / A;
+};
+__host__ __device__ inline int fac_a(int L) { return L <= 8 ? L : L <= 32 ? 4 : L <= 64 ? 8 : 16; }
+// storage position of frequency k
+__host__ __device__ inline int fac_pos(int k, int L) { return (k % fac_a(L)) * (L / fac_a(L)) + k / fac_a(L); }
+
+// blocks of 256 threads; three per SM (80 registers) up to 32 points
+constexpr int kFxtThreads = 256;
+template <int LMAX> constexpr int kFxtMinBlocks = LMAX <= 32 ? 3 : 2;
+
+// One step over nlines lines: N-point codelets on the columns c = 0 .. NC-1 of each
+// line, elements at positions c CS + i IS; with TW the results are multiplied by
+// w^(c i) (tw: the length's roots).  ld(line) gives a functor position -> value,
+// st(line) one (position, value); end(line, pos, v, N) sees a column's results first
+// (pos(i): the position of the i-th).
+// Consecutive threads take consecutive lines of one column.
+template <int N, int NC, int CS, int IS, bool TW, typename LD, typename END, typename ST>
+__device__ __forceinline__ void fx_step(int nlines, const longlong2* __restrict__ tw, LD ld, END end, ST st)
 {
-    r = r > 62 ? 62 : r;
-    const fx rnd = 1ll << (r - 1);
-    return cfx{shift_round(v.re, rnd, r), shift_round(v.im, rnd, r)};
+    const float inv = 1.0f / (float)nlines;
+    const int n = NC * nlines;
+#pragma unroll 1
+    for (int i0 = threadIdx.x; i0 < n; i0 += blockDim.x) {
+        // i0 / nlines, exact: (i0 + 1/2) / nlines is at least 1 / (2 nlines) from an integer
+        const int c = NC == 1 ? 0 : (int)(((float)i0 + 0.5f) * inv), l = i0 - c * nlines;
+        cfx v[N];
+        auto get = ld(l);
+#pragma unroll
+        for (int i = 0; i < N; i++) v[i] = get(c * CS + i * IS);
+        dft<fx, N, false>(v);
+        if constexpr (TW) {
+#pragma unroll
+            for (int i = 1; i < N; i++) {
+                const longlong2 w = __ldg(tw + c * i);
+                const cdig d = unpack(w);
+                v[i] = xcmul(d.re, d.im, digits(-value(d.im)), v[i]);
+            }
+        }
+        end(l, [=](int i) { return c * CS + i * IS; }, v, std::integral_constant<int, N>{});
+        auto put = st(l);
+#pragma unroll
+        for (int i = 0; i < N; i++) put(c * CS + i * IS, v[i]);
+    }
 }
 
+struct NoEnd {
+    template <typename POS, typename NN> __device__ __forceinline__ void operator()(int, POS, cfx*, NN) const {}
+};
+
+// A line transform (forward, or inverse when inv): first loads through ld, last
+// stores through st after end, the values between the two steps in place through
+// mid(line) -> pointer-like functors (mld, mst).
+template <int LMAX, bool INV, typename LD, typename MLD, typename MST, typename END, typename ST>
+__device__ __forceinline__ void fx_lines(int len, int nlines, const longlong2* __restrict__ tw, LD ld, MLD mld, MST mst,
+                                         END end, ST st)
+{
+    with_length<LMAX>(len, [&](auto Lc) {
+        constexpr int L = decltype(Lc)::value, A = Fac<L>::A, B = Fac<L>::B;
+        if constexpr (B == 1) {
+            fx_step<A, 1, 0, 1, false>(nlines, tw, ld, end, st);
+        } else if constexpr (!INV) {
+            fx_step<A, B, 1, B, true>(nlines, tw, ld, NoEnd{}, mst);
+            __syncthreads();
+            fx_step<B, A, B, 1, false>(nlines, tw, mld, end, st);
+        } else {
+            fx_step<B, A, B, 1, true>(nlines, tw, ld, NoEnd{}, mst);
+            __syncthreads();
+            fx_step<A, B, 1, B, false>(nlines, tw, mld, end, st);
+        }
+    });
+}
+
+__device__ __forceinline__ cfx swapped(longlong2 v) { return cfx{v.y, v.x}; }
+
 // Delta (as k_delta_fx), theta and F, then the forward transform along x and y.
+// tw: roots of unity of the four lengths, one after the other.
 template <int LMAX>
-__global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double, LMAX>) k_delta_fxt(
+__global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_delta_fxt(
     Lat d, const longlong2* __restrict__ AH, const fx* __restrict__ Fs, longlong2* __restrict__ Fd,
-    int* __restrict__ pexp, FxExp* fe, double* __restrict__ partials, Ctl* ctl, double2* hist)
+    const longlong2* __restrict__ tw, int* __restrict__ pexp, FxExp* fe, double* __restrict__ partials, Ctl* ctl,
+    double2* hist)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
@@ -92,7 +176,6 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
     __syncthreads();
     const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1];
     const int plane = blockIdx.x;
-    const int s0 = plane * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
     double th = 0.0, fsum = 0.0;
     unsigned o = 0;
@@ -105,55 +188,51 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
     });
     block_or(o, s_or);
     reduce_theta_F(th, fsum, partials, ctl, hist, V);
-    __syncthreads();
-    // x: to B bits (Delta shrinks by orders of magnitude over a fix: left shifts here)
+    longlong2* out = Fd + plane * P;
     int E = -kFxSum;
-    {
-        const int sh = fx_bits_rt(Lx) - top_bits(s_or[0]);
+#pragma unroll 1
+    for (int pass = 0; pass < 2; pass++) {
+        __syncthreads();
+        // x rows, then y columns, each to B + 1 bits before a shift by one (Delta shrinks
+        // by orders of magnitude over a fix: a left shift in the first pass)
+        const int len = pass ? Ly : Lx, estr = pass ? rsx : 1;
+        const int sh = fx_bits_rt(len) + 1 - top_bits(s_or[pass]);
         const int l = sh > 0 ? sh : 0;
-        const RShift rs = rshift(-sh);
-        E -= sh;
+        const RShift rs = rshift(1 - (sh < 0 ? sh : 0));
+        E += rs.r - l;
         o = 0;
-        with_length<LMAX>(Lx, [&](auto Lc) {
-            constexpr int L = decltype(Lc)::value;
-            auto row = [&](int ln) {
-                const int f = (int)fdiv((unsigned)ln, d.dLy), y = ln - f * Ly;
-                return sm + f * fs + y * rsx;
-            };
-            lines_pass<fx, L, false>(
-                4 * Ly,
-                [&](int ln, int e) {
-                    const cfx v = ldv<fx>(row(ln) + e);
+        auto line = [&](int ln) {
+            const int f = (int)fdiv((unsigned)ln, pass ? d.dLx : d.dLy), c = ln - f * (pass ? Lx : Ly);
+            return sm + f * fs + (pass ? c : c * rsx);
+        };
+        fx_lines<LMAX, false>(
+            len, pass ? 4 * Lx : 4 * Ly, tw + (pass ? Lx : 0),
+            [&](int ln) {
+                const longlong2* p = line(ln);
+                return [=](int e) {
+                    const cfx v = ldv<fx>(p + e * estr);
                     return apply(rs, cfx{v.re << l, v.im << l});
-                },
-                [&](int ln, int e, cfx v) {
-                    or_bits(o, v);
-                    st<fx>(row(ln) + e, v);
-                });
-        });
-        block_or(o, s_or + 1);
-    }
-    __syncthreads();
-    {
-        const RShift rs = rshift(top_bits(s_or[1]) - fx_bits_rt(Ly));
-        E += rs.r;
-        o = 0;
-        longlong2* out = Fd + s0;
-        with_length<LMAX>(Ly, [&](auto Lc) {
-            constexpr int L = decltype(Lc)::value;
-            lines_pass<fx, L, false>(
-                4 * Lx,
-                [&](int ln, int e) {
-                    const int f = (int)fdiv((unsigned)ln, d.dLx), x = ln - f * Lx;
-                    return apply(rs, ldv<fx>(sm + (f * fs + e * rsx + x)));
-                },
-                [&](int ln, int e, cfx v) {
-                    const int f = (int)fdiv((unsigned)ln, d.dLx), x = ln - f * Lx;
-                    or_bits(o, v);
-                    st<fx>(out + (f * V + e * Lx + x), v);
-                });
-        });
-        block_or(o, s_or + 2);
+                };
+            },
+            [&](int ln) {
+                const longlong2* p = line(ln);
+                return [=](int e) { return ldv<fx>(p + e * estr); };
+            },
+            [&](int ln) {
+                longlong2* p = line(ln);
+                return [=](int e, cfx v) { st<fx>(p + e * estr, v); };
+            },
+            [&](int, auto, const cfx* v, auto N) {
+#pragma unroll
+                for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
+            },
+            [&](int ln) {
+                const int f = (int)fdiv((unsigned)ln, pass ? d.dLx : d.dLy), c = ln - f * (pass ? Lx : Ly);
+                longlong2* p = pass ? out + (f * V + c) : sm + f * fs + c * rsx;
+                const int str = pass ? Lx : 1;
+                return [=](int e, cfx v) { st<fx>(p + e * str, v); };
+            });
+        block_or(o, s_or + pass + 1);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -162,12 +241,21 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
     }
 }
 
-// z,t pencils (as k_zt): the multiplier p2max/(p2 V) of a t-line is kept as integers
-// mx (digits, x 2^62) times 2^me, the largest of the line in [1/2, 1).
+// z,t pencils (as k_zt): z forward, t forward and the accelerator, t inverse, z inverse
+// in the tile [t][kz][xi].  The multiplier p2max/(p2 V) of a t-line is kept as
+// integers mx (digits, x 2^62) times 2^me, the largest of the line in [1/2, 1); every
+// accelerated t-line has an exponent of its own (lexp).  Shared memory after the
+// tile: the pencil's multipliers, lexp and the lines' magnitude bits [kz][xi].
+inline size_t fxt_pencil_smem(const Lat& d, int xw)
+{
+    return pencil_smem_bytes(d, xw, sizeof(longlong2)) + (size_t)xw * d.L[2] * 2 * sizeof(int);
+}
+
 template <int LMAX>
-__global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double, LMAX>) k_zt_fxt(
-    Lat d, int xw, longlong2* __restrict__ Fd, const Ctl* ctl, const fx* __restrict__ mx, const int* __restrict__ me,
-    const int* __restrict__ pexp, int* __restrict__ bexp, FxExp* fe)
+__global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_zt_fxt(
+    Lat d, int xw, longlong2* __restrict__ Fd, const Ctl* ctl, const longlong2* __restrict__ tw,
+    const fx* __restrict__ mx, const int* __restrict__ me, const int* __restrict__ pexp, int* __restrict__ bexp,
+    FxExp* fe)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
@@ -181,121 +269,158 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
     const int c0 = x0 + Lx * ky;
     longlong2* g = Fd + (size_t)blockIdx.z * d.V + c0;
     fx* m64 = reinterpret_cast<fx*>(sm + Lt * rs);
-    int* lexp = reinterpret_cast<int*>(m64 + xw * Lz * Lt);  // [kz][xi]
+    int* lexp = reinterpret_cast<int*>(m64 + xw * Lz * Lt);       // [kz][xi]
+    unsigned* lor = reinterpret_cast<unsigned*>(lexp + xw * Lz);  // [kz][xi]
     if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
     if (threadIdx.x == 2) s_az = kExpNone;
-    block_copy<8, fx>(
-        xw * Lz * Lt,
-        [&](int i) {
-            const int zt = i >> xs, xi = i & (xw - 1);
-            return __ldg(mx + c0 + (xi + P * zt));
-        },
-        [&](int i, fx v) { m64[i] = v; });
-    __syncthreads();
-    const int lane = (int)threadIdx.x & 31;
-    // z forward: planes aligned to the largest
-    const int Ez = __ldg(&fe->amax1) - fx_bits_rt(Lz);
-    unsigned o = 0;
-    with_length<LMAX>(Lz, [&](auto Lc) {
-        constexpr int L = decltype(Lc)::value;
-        lines_pass<fx, L, false>(
-            xw * Lt,
-            [&](int l, int e) {
-                const int tt = l >> xs, xi = l & (xw - 1);
-                const int p = e + L * tt;
-                return rshift1(ldv<fx>(g + (xi + P * p)), Ez - __ldg(pexp + p));
-            },
-            [&](int l, int e, cfx v) {
-                const int tt = l >> xs, xi = l & (xw - 1);
-                or_bits(o, v);
-                st<fx>(sm + tt * rs + e * xw + xi, v);
+    for (int i = threadIdx.x; i < xw * Lz; i += blockDim.x) lor[i] = 0u;
+    // the planes' values, aligned to B + 1 bits of the largest, and the multipliers
+    int E = __ldg(&fe->amax1) - fx_bits_rt(Lz) - 1;
+    {
+        const FastDiv dz = d.dLz;
+        block_copy<4, longlong2>(
+            xw * Lz * Lt, [&](int i) { return g[(i & (xw - 1)) + P * (i >> xs)]; },
+            [&](int i, longlong2 v) {
+                const int zt = i >> xs, t = (int)fdiv((unsigned)zt, dz), z = zt - t * Lz;
+                const int r = E - __ldg(pexp + zt);
+                const cfx w = r > 0 ? apply(rshift(r), cfx{v.x, v.y}) : cfx{v.x, v.y};
+                st<fx>(sm + t * rs + (z << xs) + (i & (xw - 1)), w);
             });
-    });
-    block_or(o, s_or);
+        block_copy<4, fx>(
+            xw * Lz * Lt, [&](int i) { return __ldg(mx + c0 + ((i & (xw - 1)) + P * (i >> xs))); },
+            [&](int i, fx v) { m64[i] = v; });
+    }
+    auto zline = [&](int l) { return sm + (l >> xs) * rs + (l & (xw - 1)); };
+    auto tline = [&](int l) { return sm + l; };
+    auto mload = [&](auto line, int str) {
+        return [=](int l) {
+            const longlong2* p = line(l);
+            return [=](int e) { return ldv<fx>(p + e * str); };
+        };
+    };
+    auto mstore = [&](auto line, int str) {
+        return [=](int l) {
+            longlong2* p = line(l);
+            return [=](int e, cfx v) { st<fx>(p + e * str, v); };
+        };
+    };
+    const longlong2 *twz = tw + d.L[0] + d.L[1], *twt = twz + Lz;
+    // z forward
+    unsigned o = 0;
     __syncthreads();
-    // t forward, accelerator, t inverse: lines (xi, kz), each with an exponent of its own
+    {
+        const RShift r1 = rshift(1);
+        E += 1;
+        fx_lines<LMAX, false>(
+            Lz, xw * Lt, twz,
+            [&](int l) {
+                const longlong2* p = zline(l);
+                return [=](int e) { return apply(r1, ldv<fx>(p + (e << xs))); };
+            },
+            mload(zline, xw), mstore(zline, xw),
+            [&](int, auto, const cfx* v, auto N) {
+#pragma unroll
+                for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
+            },
+            mstore(zline, xw));
+        block_or(o, s_or);
+    }
+    __syncthreads();
+    // t forward and the multipliers (storage order: position by position)
     {
         const RShift rt = rshift(top_bits(s_or[0]) - fx_bits_rt(Lt));
-        const int Et = Ez + rt.r;
-        int amax = kExpNone;
-        with_length<LMAX>(Lt, [&](auto Lc) {
-            constexpr int L = decltype(Lc)::value;
-            constexpr int Tl = line_lanes<fx>(L), R = L / Tl, W = 32 / Tl, B = fx_bits(L);
-            const int tau = lane / W, w = lane - tau * W;
-            const int step = ((int)blockDim.x >> 5) * W, nlines = xw * Lz;
-            for (int l0 = ((int)threadIdx.x >> 5) * W; l0 < nlines; l0 += step) {
-                const int l = l0 + w;
-                const bool ok = l < nlines;
-                const int lc = ok ? l : l0;
-                const int ml = __ldg(me + c0 + ((lc & (xw - 1)) + P * (lc >> xs)));
-                cfx v[R];
-#pragma unroll
-                for (int j = 0; j < R; j++) v[j] = apply(rt, ldv<fx>(sm + line_pos_x<fx, L>(tau, j) * rs + lc));
-                line_fwd<fx, L>(v, tau);
+        E += rt.r;
+        fx_lines<LMAX, false>(
+            Lt, xw * Lz, twt,
+            [&](int l) {
+                const longlong2* p = tline(l);
+                return [=](int e) { return apply(rt, ldv<fx>(p + e * rs)); };
+            },
+            mload(tline, rs), mstore(tline, rs),
+            [&](int l, auto pos, cfx* v, auto N) {
+                const fx* mp = m64 + l;
+                const int ms = xw * Lz;
                 unsigned b = 0;
 #pragma unroll
-                for (int r = 0; r < R; r++) {
-                    const fx mw = m64[lc + xw * Lz * line_pos_k<fx, L>(tau, r)];
+                for (int j = 0; j < decltype(N)::value; j++) {
+                    const fx mw = mp[pos(j) * ms];
                     const dig m = dig{(int)(mw >> 32), (int)mw};
-                    v[r] = cfx{xrmul(m, v[r].re), xrmul(m, v[r].im)};
-                    or_bits(b, v[r]);
+                    v[j] = cfx{xrmul(m, v[j].re), xrmul(m, v[j].im)};
+                    or_bits(b, v[j]);
                 }
+                atomicOr(lor + l, b);
+            },
+            mstore(tline, rs));
+    }
+    __syncthreads();
+    // t inverse, every line scaled to B bits by itself
+    {
+        int amax = kExpNone;
+        const int B1 = fx_bits_rt(Lt) + 1;
+        fx_lines<LMAX, true>(
+            Lt, xw * Lz, twt,
+            [&](int l) {
+                const longlong2* p = tline(l);
+                const int sh = B1 - top_bits(lor[l]), sl = sh > 0 ? sh : 0;
+                const RShift r = rshift(1 - (sh < 0 ? sh : 0));
+                return [=](int e) {
+                    const cfx v = swapped(p[e * rs]);
+                    return apply(r, cfx{v.re << sl, v.im << sl});
+                };
+            },
+            mload(tline, rs), mstore(tline, rs),
+            [&](int l, auto, const cfx* v, auto N) {
+                unsigned b = 0;
 #pragma unroll
-                for (int h = 1; h < Tl; h <<= 1) b |= __shfl_xor_sync(0xffffffffu, b, h * W);
-                const int sh = B - top_bits(b), sl = sh > 0 ? sh : 0;
-                const RShift sr = rshift(-sh);
-#pragma unroll
-                for (int r = 0; r < R; r++) v[r] = apply(sr, cfx{v[r].re << sl, v[r].im << sl});
-                line_inv<fx, L>(v, tau);
-                b = 0;
-#pragma unroll
-                for (int j = 0; j < R; j++) or_bits(b, v[j]);
-                const int El = Et + ml - sh;
-                if (ok) {
-#pragma unroll
-                    for (int j = 0; j < R; j++) st<fx>(sm + line_pos_x<fx, L>(tau, j) * rs + l, v[j]);
-                    if (tau == 0) lexp[l] = El;
-                    amax = max(amax, El + align_top(b, Lz));
-                }
-            }
-        });
+                for (int j = 0; j < decltype(N)::value; j++) or_bits(b, v[j]);
+                const int sh = B1 - top_bits(lor[l]);
+                const int El = E + __ldg(me + c0 + ((l & (xw - 1)) + P * (l >> xs))) + 1 - sh;
+                lexp[l] = El;
+                amax = max(amax, El + align_top(b, Lz));
+            },
+            [&](int l) {
+                longlong2* p = tline(l);
+                return [=](int e, cfx v) { p[e * rs] = make_longlong2(v.im, v.re); };
+            });
         amax = __reduce_max_sync(0xffffffffu, amax);
-        if (lane == 0) atomicMax(&s_az, amax);
+        if ((threadIdx.x & 31) == 0) atomicMax(&s_az, amax);
     }
     __syncthreads();
     // z inverse, back to Fd
     {
-        const int Eo = s_az - fx_bits_rt(Lz);
+        E = s_az - fx_bits_rt(Lz);
         o = 0;
-        with_length<LMAX>(Lz, [&](auto Lc) {
-            constexpr int L = decltype(Lc)::value;
-            lines_pass<fx, L, true>(
-                xw * Lt,
-                [&](int l, int e) {
-                    const int tt = l >> xs, xi = l & (xw - 1);
-                    return rshift1(ldv<fx>(sm + tt * rs + e * xw + xi), Eo - lexp[e * xw + xi]);
-                },
-                [&](int l, int e, cfx v) {
-                    const int tt = l >> xs, xi = l & (xw - 1);
-                    or_bits(o, v);
-                    st<fx>(g + (xi + P * (e + L * tt)), v);
-                });
-        });
+        fx_lines<LMAX, true>(
+            Lz, xw * Lt, twz,
+            [&](int l) {
+                const longlong2* p = zline(l);
+                const int* ep = lexp + (l & (xw - 1));
+                return [=](int e) { return apply(rshift(E - ep[e << xs]), swapped(p[e << xs])); };
+            },
+            mload(zline, xw), mstore(zline, xw),
+            [&](int, auto, const cfx* v, auto N) {
+#pragma unroll
+                for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
+            },
+            [&](int l) {
+                longlong2* p = g + ((l & (xw - 1)) + P * Lz * (l >> xs));
+                return [=](int e, cfx v) { p[e * P] = make_longlong2(v.im, v.re); };
+            });
         block_or(o, s_or + 1);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            bexp[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = Eo;
-            atomicMax(&fe->amax2, Eo + align_top(s_or[1], d.L[1]));
-        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        bexp[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = E;
+        atomicMax(&fe->amax2, E + align_top(s_or[1], d.L[1]));
     }
 }
 
 // inverse along y and x, then g = reunit(1 + alpha/2 Delta~) in FP64, stored in fixed
 // point.  xs: log2 of the pencils' width.
 template <int LMAX>
-__global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double, LMAX>) k_xyinv_fxt(
+__global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
     Lat d, int xs, const longlong2* __restrict__ Fd, longlong2* __restrict__ g, const Ctl* ctl,
-    const int* __restrict__ bexp, FxExp* fe)
+    const longlong2* __restrict__ tw, const int* __restrict__ bexp, FxExp* fe)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
@@ -303,42 +428,62 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
     if (ld_flag(&ctl->phase_done)) return;
     if (threadIdx.x == 0) s_or = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
-    __syncthreads();
     const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1];
     const int s0 = blockIdx.x * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
     const int nxc = Lx >> xs;
-    int E = __ldg(&fe->amax2) - fx_bits_rt(Ly);
-    unsigned o = 0;
-    with_length<LMAX>(Ly, [&](auto Lc) {
-        constexpr int L = decltype(Lc)::value;
-        lines_pass<fx, L, true>(
-            4 * Lx,
-            [&](int l, int e) {
-                const int f = (int)fdiv((unsigned)l, d.dLx), x = l - f * Lx;
-                const int Eb = __ldg(bexp + (f * L + e) * nxc + (x >> xs));
-                return rshift1(ldv<fx>(Fd + (s0 + f * V + e * Lx + x)), E - Eb);
-            },
-            [&](int l, int e, cfx v) {
-                const int f = (int)fdiv((unsigned)l, d.dLx), x = l - f * Lx;
-                or_bits(o, v);
-                st<fx>(sm + (f * fs + e * rsx + x), v);
-            });
-    });
-    block_or(o, &s_or);
-    __syncthreads();
-    const RShift rx = rshift(top_bits(s_or) - fx_bits_rt(Lx));
-    E += rx.r;
-    with_length<LMAX>(Lx, [&](auto Lc) {
-        constexpr int L = decltype(Lc)::value;
-        auto row = [&](int ln) {
-            const int f = (int)fdiv((unsigned)ln, d.dLy), y = ln - f * Ly;
-            return sm + f * fs + y * rsx;
+    int E = __ldg(&fe->amax2) - fx_bits_rt(Ly) - 1;
+    // the plane, aligned to B + 1 bits of the largest pencil
+    block_copy<4, longlong2>(
+        4 * P,
+        [&](int i) {
+            const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P;
+            return Fd[s0 + f * V + xy];
+        },
+        [&](int i, longlong2 v) {
+            const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P, y = (int)fdiv((unsigned)xy, d.dLx), x = xy - y * Lx;
+            const int r = E - __ldg(bexp + (f * Ly + y) * nxc + (x >> xs));
+            const cfx w = r > 0 ? apply(rshift(r), cfx{v.x, v.y}) : cfx{v.x, v.y};
+            st<fx>(sm + (f * fs + y * rsx + x), w);
+        });
+#pragma unroll 1
+    for (int pass = 0; pass < 2; pass++) {
+        __syncthreads();
+        // y columns, then x rows
+        const int len = pass ? Lx : Ly, estr = pass ? 1 : rsx;
+        const RShift rs = rshift(pass ? top_bits(s_or) - fx_bits_rt(Lx) : 1);
+        E += rs.r;
+        unsigned o = 0;
+        auto line = [&](int ln) {
+            const int f = (int)fdiv((unsigned)ln, pass ? d.dLy : d.dLx), c = ln - f * (pass ? Ly : Lx);
+            return sm + f * fs + (pass ? c * rsx : c);
         };
-        lines_pass<fx, L, true>(
-            4 * Ly, [&](int ln, int e) { return apply(rx, ldv<fx>(row(ln) + e)); },
-            [&](int ln, int e, cfx v) { st<fx>(row(ln) + e, v); });
-    });
+        fx_lines<LMAX, true>(
+            len, pass ? 4 * Ly : 4 * Lx, tw + (pass ? 0 : Lx),
+            [&](int ln) {
+                const longlong2* p = line(ln);
+                return [=](int e) { return apply(rs, swapped(p[e * estr])); };
+            },
+            [&](int ln) {
+                const longlong2* p = line(ln);
+                return [=](int e) { return ldv<fx>(p + e * estr); };
+            },
+            [&](int ln) {
+                longlong2* p = line(ln);
+                return [=](int e, cfx v) { st<fx>(p + e * estr, v); };
+            },
+            [&](int, auto, const cfx* v, auto N) {
+                if (pass == 0) {
+#pragma unroll
+                    for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
+                }
+            },
+            [&](int ln) {
+                longlong2* p = line(ln);
+                return [=](int e, cfx v) { p[e * estr] = make_longlong2(v.im, v.re); };
+            });
+        if (pass == 0) block_or(o, &s_or);
+    }
     __syncthreads();
     // alpha/2 2^E (a field too large for FP64 gives infinity, as FP64 arithmetic does)
     const double h = scalbn(0.5 * ctl->alpha, E);
@@ -362,7 +507,7 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
 }
 
 // the multipliers p2max/(p2(k) V) of every momentum as mx 2^(me - 62), me per t-line
-// (one thread each), mx in digits
+// (one thread each), mx in digits; both in the storage order of the transform
 static __global__ void k_make_mult_fx(Lat d, const double* __restrict__ m64, fx* __restrict__ mx, int* __restrict__ me)
 {
     const int nl = d.P * d.L[2];
@@ -371,8 +516,25 @@ static __global__ void k_make_mult_fx(Lat d, const double* __restrict__ m64, fx*
     double top = 0.0;
     for (int t = 0; t < d.L[3]; t++) top = fmax(top, m64[l + nl * t]);
     const int e = ilogb(top) + 1;  // top 2^-e in [1/2, 1)
-    me[l] = e;
-    for (int t = 0; t < d.L[3]; t++) mx[l + nl * t] = word(digits(__double2ll_rn(scalbn(m64[l + nl * t], 62 - e))));
+    int c[4];
+    site_coords(d, l, c);
+    const int q = fac_pos(c[0], d.L[0]) + d.L[0] * (fac_pos(c[1], d.L[1]) + d.L[1] * fac_pos(c[2], d.L[2]));
+    me[q] = e;
+    for (int t = 0; t < d.L[3]; t++)
+        mx[q + nl * fac_pos(t, d.L[3])] = word(digits(__double2ll_rn(scalbn(m64[l + nl * t], 62 - e))));
+}
+
+// roots of unity exp(-2 pi i m / L_mu), x 2^62 in digits, of the four lengths
+static __global__ void k_make_roots_fx(Lat d, longlong2* __restrict__ tw)
+{
+    for (int mu = 0; mu < 4; mu++) {
+        const int L = d.L[mu], step = 384 / L;
+        for (int m = threadIdx.x; m < L; m += blockDim.x) {
+            const cfx w = cfx{cos384x(m * step), -sin384x(m * step)};
+            tw[m] = make_longlong2(word(digits(w.re)), word(digits(w.im)));
+        }
+        tw += L;
+    }
 }
 
 }  // namespace lgf

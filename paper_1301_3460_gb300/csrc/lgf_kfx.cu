@@ -32,15 +32,18 @@ cudaError_t fx_prepare(const Lat& d)
     return allow_max_smem(k_xyinv_fxt<128>, optin);
 }
 
+bool fxt_fits(const Lat& d, const Shape& sh) { return fxt_pencil_smem(d, sh.xw) <= 226 * 1024; }
+
 size_t fxt_bytes(const Lat& d)
 {
     return sizeof(FxExp) + ((size_t)d.nplanes + 4 * (size_t)d.P + (size_t)d.P * d.L[2]) * sizeof(int) +
-           (size_t)d.V * sizeof(fx);
+           (size_t)d.V * sizeof(fx) + (size_t)(d.L[0] + d.L[1] + d.L[2] + d.L[3]) * sizeof(longlong2);
 }
 FxtBuf fxt_carve(const Lat& d, void* p)
 {
     FxtBuf b;
-    b.mx = reinterpret_cast<fx*>(p);
+    b.tw = reinterpret_cast<longlong2*>(p);
+    b.mx = reinterpret_cast<fx*>(b.tw + d.L[0] + d.L[1] + d.L[2] + d.L[3]);
     b.fe = reinterpret_cast<FxExp*>(b.mx + d.V);
     b.pexp = reinterpret_cast<int*>(b.fe + 1);
     b.bexp = b.pexp + d.nplanes;
@@ -50,24 +53,25 @@ FxtBuf fxt_carve(const Lat& d, void* p)
 void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const FxtBuf& b)
 {
     k_make_mult_fx<<<blocks((long)d.P * d.L[2], 128), 128, 0, s>>>(d, m64, b.mx, b.me);
+    k_make_roots_fx<<<1, 128, 0, s>>>(d, b.tw);
 }
 void launch_fxt_delta(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* AH, const fx* Fs, longlong2* Fd,
                       const FxtBuf& b, double* partials, Ctl* ctl, double2* hist)
 {
     const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
     if (small_plane<double>(d))
-        k_delta_fxt<32><<<d.nplanes, sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.pexp, b.fe, partials, ctl, hist);
+        k_delta_fxt<32><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
     else
-        k_delta_fxt<128><<<d.nplanes, sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.pexp, b.fe, partials, ctl, hist);
+        k_delta_fxt<128><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
 }
 void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl)
 {
-    const size_t sm = pencil_smem_bytes(d, sh.xw, sizeof(longlong2)) + (size_t)sh.xw * d.L[2] * sizeof(int);
+    const size_t sm = fxt_pencil_smem(d, sh.xw);
     const dim3 grid(d.L[0] / sh.xw, d.L[1], 4);
     if (short_zt_lines(d))
-        k_zt_fxt<32><<<grid, sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.mx, b.me, b.pexp, b.bexp, b.fe);
+        k_zt_fxt<32><<<grid, 2 * sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
     else
-        k_zt_fxt<128><<<grid, sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.mx, b.me, b.pexp, b.bexp, b.fe);
+        k_zt_fxt<128><<<grid, 2 * sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
 }
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* Fd, longlong2* g,
                         const FxtBuf& b, const Ctl* ctl)
@@ -76,9 +80,9 @@ void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const lon
     int xs = 0;
     while ((1 << xs) < sh.xw) xs++;
     if (small_plane<double>(d))
-        k_xyinv_fxt<32><<<d.nplanes, sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.bexp, b.fe);
+        k_xyinv_fxt<32><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
     else
-        k_xyinv_fxt<128><<<d.nplanes, sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.bexp, b.fe);
+        k_xyinv_fxt<128><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
 }
 
 void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, longlong2* U, longlong2* AH, fx* Fs,

@@ -88,6 +88,7 @@ struct FxExp;
 // buffers of the integer transform (lgf_fxt.cuh): multipliers and exponents, carved
 // from fxt_bytes(d) of device memory
 struct FxtBuf {
+    longlong2* tw = nullptr;  // [Lx + Ly + Lz + Lt] roots of unity
     long long* mx = nullptr;  // [V]
     FxExp* fe = nullptr;
     int* pexp = nullptr;      // [planes]
@@ -95,6 +96,9 @@ struct FxtBuf {
     int* me = nullptr;        // [t-lines]
 };
 size_t fxt_bytes(const Lat& d);
+// whether a pencil of this shape fits into shared memory (the tile budget leaves no
+// room for the lines' exponents in a few shapes of 16 columns)
+bool fxt_fits(const Lat& d, const Shape& sh);
 FxtBuf fxt_carve(const Lat& d, void* p);
 void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const FxtBuf& b);
 cudaError_t fx_prepare(const Lat& d);
