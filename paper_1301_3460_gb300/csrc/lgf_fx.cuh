@@ -106,6 +106,7 @@ template <int S> __host__ __device__ __forceinline__ fx fval(facc a)
     if constexpr (S == 0) return a.hh + (a.m >> 32);
     else return (a.hh << S) + (a.m >> (32 - S));
 }
+__host__ __device__ __forceinline__ facc fzero() { return facc{0, 0}; }
 // p - n (p holds the rounding term)
 __host__ __device__ __forceinline__ facc fsub(facc p, facc n) { return facc{p.hh - n.hh, p.m - n.m}; }
 
@@ -126,6 +127,9 @@ __device__ __forceinline__ cdig3 with_diff(cfx a) { return cdig3{digits(a.re), d
 template <int S> __device__ __forceinline__ cfx fx_mul(const cdig3* a, const cdig3* b, int j)
 {
     facc p = fmul<S>(a[0].re, b[j].re), q = fmul<0>(a[0].im, b[j].im), r = fmul<S>(a[0].s, b[j].s);
+    // three roundings toward minus infinity: Im starts low by half a unit, so that
+    // the mean error of both parts is zero
+    if constexpr (S == 0) r.m -= 1ll << 31;
 #pragma unroll
     for (int k = 1; k < 3; k++) {
         fmac(p, a[k].re, b[3 * k + j].re);
@@ -169,6 +173,98 @@ template <int S, typename D> __device__ __forceinline__ cfx fx_row2(const D* r0,
 {
     const int a = j == 0 ? 1 : j == 1 ? 2 : 0, b = j == 0 ? 2 : j == 1 ? 0 : 1;
     return fx_det2c<S>(r0[a], r1[b], r0[b], r1[a]);
+}
+
+// ---------------------------------------------------------------- Gram-Schmidt
+
+// Rows 0,1 of g = reunit(X), X = 1 + A with A anti-Hermitian, on integers: X comes
+// x 2^(61-q) with components below 2^(q-1) (2^60 as integers), the rows leave x 2^62.
+// X X^dag = 1 + A A^dag, so both norms that are divided by are at least 1.  About 170
+// mad.wide.s32 per site against 70 FP64 operations (2 per clock and SM); errors
+// near 2^(q-60), FP64's 2^-53.
+
+// sum of products with a run-time scale: 2^S (hh 2^32 + m) / 2^32, rounded
+__device__ __forceinline__ fx fval_rt(facc a, int S) { return (a.hh << S) + ((a.m + (1ll << (31 - S))) >> (32 - S)); }
+
+// |x|^2 of a row of three complex numbers (digits, x 2^(61-q)), x 2^(61-2q).  The
+// squares of the low digits, dropped elsewhere, are added here to 15 bits: they are
+// all positive, and a norm that is low at every site would shrink the links a
+// little in every iteration.
+__device__ __forceinline__ fx fx_norm2(const cdig* x)
+{
+    fx hh = 0, hl = 1ll << 27;
+    unsigned ll = 0;
+    auto add = [&](dig v) {
+        hh = madw(v.h, v.h, hh);
+        hl = madw(v.h, v.l, hl);
+        const int t = v.l >> 17;
+        ll += (unsigned)(t * t);
+    };
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        add(x[j].re);
+        add(x[j].im);
+    }
+    return (hh << 3) + ((hl + 2 * (fx)ll) >> 28);
+}
+
+// 1/sqrt(n) x 2^62 of n >= 1 given x 2^(61-2q), q <= 5: y0 from the FP32 reciprocal
+// square root (22 bits), then one third-order step y0 (1 + d/2 + 3/8 d^2), d = 1 -
+// n y0^2 (the binomial series of (1 - d)^(-1/2); next term 5/16 d^3 < 2^-62)
+__device__ __forceinline__ fx fx_rsqrt(fx n, int q)
+{
+    const float nf = fmaf((float)(int)(n >> 32), 0x1p32f, (float)(unsigned)n) * __int_as_float((127 - 61 + 2 * q) << 23);
+    const int y0 = __float2int_rn(rsqrtf(nf) * 0x1p30f);
+    const dig nd = digits(n), yy = digits(mulw(y0, y0));  // y0^2 x 2^60
+    // n y0^2 x 2^62: product x 2^(121-2q), all four partial products
+    facc t = facc{mulw(nd.h, yy.h), madw(nd.h, yy.l, mulw(nd.l, yy.h))};
+    t.m += mulw(nd.l, yy.l) >> 32;
+    const fx d = (1ll << 62) - fval_rt(t, 5 + 2 * q);
+    const int ds = (int)(d >> 12);  // x 2^50, |d| < 2^-20
+    const fx c = (d >> 1) + ((mulw(ds, ds) >> 38) * 3 >> 3);
+    const dig cd = digits(c);
+    return ((fx)y0 << 32) + ((mulw(y0, cd.h) << 2) + (mulw(y0, cd.l) >> 30));
+}
+
+// g: rows 0,1 in digits x 2^62
+__device__ __forceinline__ void fx_gram_schmidt(const cfx* X, int q, cdig* g)
+{
+    cdig x0[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) x0[j] = digits(X[j]);
+    const dig y = digits(fx_rsqrt(fx_norm2(x0), q));
+    auto scale = [&](dig v, dig w) {  // x 2^(61-q) times x 2^62 -> x 2^62
+        facc a = fzero();
+        fmac(a, v, w);
+        return digits(fval_rt(a, 3 + q));
+    };
+#pragma unroll
+    for (int j = 0; j < 3; j++) g[j] = cdig{scale(x0[j].re, y), scale(x0[j].im, y)};
+    // <r0, X1> = sum conj(r0_j) X1_j, x 2^(61-q)
+    cdig x1[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) x1[j] = digits(X[3 + j]);
+    facc pr = fmul<2>(x1[0].re, g[0].re), pi = fmul<2>(x1[0].im, g[0].re), n = fmul<0>(x1[0].re, g[0].im);
+    fmac(pr, x1[0].im, g[0].im);
+#pragma unroll
+    for (int j = 1; j < 3; j++) {
+        fmac(pr, x1[j].re, g[j].re);
+        fmac(pi, x1[j].im, g[j].re);
+        fmac(n, x1[j].re, g[j].im);
+        fmac(pr, x1[j].im, g[j].im);
+    }
+    const cdig ip = digits(cfx{fval<2>(pr), fval<2>(fsub(pi, n))});
+    // v = X1 - ip r0
+    cdig v[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        facc re = fmul<2>(ip.re, g[j].re), im = fmul<2>(ip.re, g[j].im), m = fmul<0>(ip.im, g[j].im);
+        fmac(im, ip.im, g[j].re);
+        v[j] = digits(cfx{X[3 + j].re - fval<2>(fsub(re, m)), X[3 + j].im - fval<2>(im)});
+    }
+    const dig z = digits(fx_rsqrt(fx_norm2(v), q));
+#pragma unroll
+    for (int j = 0; j < 3; j++) g[3 + j] = cdig{scale(v[j].re, z), scale(v[j].im, z)};
 }
 
 __device__ __forceinline__ cfx ldx(const longlong2* p)

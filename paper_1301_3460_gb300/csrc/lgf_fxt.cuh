@@ -91,9 +91,11 @@ __host__ __device__ inline int fac_a(int L) { return L <= 8 ? L : L <= 32 ? 4 : 
 // storage position of frequency k
 __host__ __device__ inline int fac_pos(int k, int L) { return (k % fac_a(L)) * (L / fac_a(L)) + k / fac_a(L); }
 
-// blocks of 256 threads; three per SM (80 registers) up to 32 points
-constexpr int kFxtThreads = 256;
-template <int LMAX> constexpr int kFxtMinBlocks = LMAX <= 32 ? 3 : 2;
+// Blocks of up to 256 threads, three per SM (80 registers), for lines up to 32 points;
+// longer lines (128 registers): up to 512 threads, which a tile too large for two
+// blocks per SM gets.
+template <int LMAX> constexpr int kFxtThreads = LMAX <= 32 ? 256 : 512;
+template <int LMAX> constexpr int kFxtMinBlocks = LMAX <= 32 ? 3 : 1;
 
 // One step over nlines lines: N-point codelets on the columns c = 0 .. NC-1 of each
 // line, elements at positions c CS + i IS; with TW the results are multiplied by
@@ -162,7 +164,7 @@ __device__ __forceinline__ cfx swapped(longlong2 v) { return cfx{v.y, v.x}; }
 // Delta (as k_delta_fx), theta and F, then the forward transform along x and y.
 // tw: roots of unity of the four lengths, one after the other.
 template <int LMAX>
-__global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_delta_fxt(
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delta_fxt(
     Lat d, const longlong2* __restrict__ AH, const fx* __restrict__ Fs, longlong2* __restrict__ Fd,
     const longlong2* __restrict__ tw, int* __restrict__ pexp, FxExp* fe, double* __restrict__ partials, Ctl* ctl,
     double2* hist)
@@ -252,7 +254,7 @@ inline size_t fxt_pencil_smem(const Lat& d, int xw)
 }
 
 template <int LMAX>
-__global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_zt_fxt(
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_zt_fxt(
     Lat d, int xw, longlong2* __restrict__ Fd, const Ctl* ctl, const longlong2* __restrict__ tw,
     const fx* __restrict__ mx, const int* __restrict__ me, const int* __restrict__ pexp, int* __restrict__ bexp,
     FxExp* fe)
@@ -415,18 +417,19 @@ __global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_zt_fxt(
     }
 }
 
-// inverse along y and x, then g = reunit(1 + alpha/2 Delta~) in FP64, stored in fixed
-// point.  xs: log2 of the pencils' width.
+// inverse along y and x, then g = reunit(1 + alpha/2 Delta~) stored in fixed point, by
+// the integer Gram-Schmidt (in FP64 where alpha/2 Delta~ exceeds 16: far beyond any
+// step that converges).  xs: log2 of the pencils' width.
 template <int LMAX>
-__global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
     Lat d, int xs, const longlong2* __restrict__ Fd, longlong2* __restrict__ g, const Ctl* ctl,
     const longlong2* __restrict__ tw, const int* __restrict__ bexp, FxExp* fe)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or;
+    __shared__ unsigned s_or[2];
     if (ld_flag(&ctl->phase_done)) return;
-    if (threadIdx.x == 0) s_or = 0u;
+    if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
     const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1];
     const int s0 = blockIdx.x * P;
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
         __syncthreads();
         // y columns, then x rows
         const int len = pass ? Lx : Ly, estr = pass ? 1 : rsx;
-        const RShift rs = rshift(pass ? top_bits(s_or) - fx_bits_rt(Lx) : 1);
+        const RShift rs = rshift(pass ? top_bits(s_or[0]) - fx_bits_rt(Lx) : 1);
         E += rs.r;
         unsigned o = 0;
         auto line = [&](int ln) {
@@ -473,20 +476,60 @@ __global__ void __launch_bounds__(kFxtThreads, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
                 return [=](int e, cfx v) { st<fx>(p + e * estr, v); };
             },
             [&](int, auto, const cfx* v, auto N) {
-                if (pass == 0) {
 #pragma unroll
-                    for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
-                }
+                for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
             },
             [&](int ln) {
                 longlong2* p = line(ln);
                 return [=](int e, cfx v) { p[e * estr] = make_longlong2(v.im, v.re); };
             });
-        if (pass == 0) block_or(o, &s_or);
+        block_or(o, s_or + pass);
     }
     __syncthreads();
-    // alpha/2 2^E (a field too large for FP64 gives infinity, as FP64 arithmetic does)
-    const double h = scalbn(0.5 * ctl->alpha, E);
+    // |alpha/2 Delta~| <= alpha/2 2^(E + top) < 2^(q-1); ha = alpha/2 = hm 2^(he-62) exactly
+    const double ha = 0.5 * ctl->alpha;
+    const int he = ilogb(ha) + 1;
+    const int q = max(1, he + E + top_bits(s_or[1]) + 1);
+    if (ha < 1e30 && q <= 5) {
+        // X x 2^(61-q) = f hm 2^(he - 62 + E + 61 - q)
+        const dig hm = digits(__double2ll_rn(scalbn(ha, 62 - he)));
+        const dig hm3 = digits(__double2ll_rn(scalbn(ha * (2.0 / 3.0), 62 - he)));
+        const int sh = he + E + 61 - q, sl = sh > 0 ? sh : 0;
+        const RShift sr = rshift(-sh);
+        const fx one = 1ll << (61 - q);
+        auto scaled = [&](dig m, fx f) { return apply(sr, xrmul(m, f)); };
+        auto scaledl = [&](dig m, fx f) { return xrmul(m, f) << sl; };
+        for (int xy = threadIdx.x; xy < P; xy += blockDim.x) {
+            const int y = (int)fdiv((unsigned)xy, d.dLx), x = xy - y * Lx;
+            const int i = y * rsx + x;
+            const cfx f0 = ldv<fx>(sm + i), f1 = ldv<fx>(sm + fs + i), f2 = ldv<fx>(sm + 2 * fs + i),
+                      f3 = ldv<fx>(sm + 3 * fs + i);
+            cfx X[6];
+            if (sh < 0) {
+                X[0] = cfx{one, scaled(hm3, f3.re)};
+                X[1] = cfx{scaled(hm, f0.re), scaled(hm, f0.im)};
+                X[2] = cfx{scaled(hm, f1.re), scaled(hm, f1.im)};
+                X[4] = cfx{one, scaled(hm3, f3.im)};
+                X[5] = cfx{scaled(hm, f2.re), scaled(hm, f2.im)};
+            } else {
+                X[0] = cfx{one, scaledl(hm3, f3.re)};
+                X[1] = cfx{scaledl(hm, f0.re), scaledl(hm, f0.im)};
+                X[2] = cfx{scaledl(hm, f1.re), scaledl(hm, f1.im)};
+                X[4] = cfx{one, scaledl(hm3, f3.im)};
+                X[5] = cfx{scaledl(hm, f2.re), scaledl(hm, f2.im)};
+            }
+            X[3] = cfx{-X[1].re, X[1].im};  // -conj(Delta01)
+            cdig r[6];
+            fx_gram_schmidt(X, q, r);
+#pragma unroll
+            for (int e = 0; e < 6; e++) std_(g + (size_t)e * V + s0 + xy, r[e]);
+#pragma unroll
+            for (int j = 0; j < 3; j++) std_(g + (size_t)(6 + j) * V + s0 + xy, digits(fx_row2<2>(r, r + 3, j)));
+        }
+        return;
+    }
+    // a field too large for FP64 gives infinity, as FP64 arithmetic does
+    const double h = scalbn(ha, E);
     const double h3 = h * (2.0 / 3.0);
     for (int xy = threadIdx.x; xy < P; xy += blockDim.x) {
         const int y = (int)fdiv((unsigned)xy, d.dLx), x = xy - y * Lx;

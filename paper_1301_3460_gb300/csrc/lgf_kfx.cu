@@ -55,23 +55,30 @@ void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const Fx
     k_make_mult_fx<<<blocks((long)d.P * d.L[2], 128), 128, 0, s>>>(d, m64, b.mx, b.me);
     k_make_roots_fx<<<1, 128, 0, s>>>(d, b.tw);
 }
+// threads: twice the shape's (its tiles were sized for FP64 lines in one thread), 512
+// where one tile fills an SM's shared memory
+static int fxt_threads(int nt, size_t smem, bool lines32)
+{
+    return !lines32 && smem > 113 * 1024 ? 512 : 2 * nt;
+}
+
 void launch_fxt_delta(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* AH, const fx* Fs, longlong2* Fd,
                       const FxtBuf& b, double* partials, Ctl* ctl, double2* hist)
 {
     const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
     if (small_plane<double>(d))
-        k_delta_fxt<32><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
+        k_delta_fxt<32><<<d.nplanes, fxt_threads(sh.nt_xy, sm, true), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
     else
-        k_delta_fxt<128><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
+        k_delta_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
 }
 void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl)
 {
     const size_t sm = fxt_pencil_smem(d, sh.xw);
     const dim3 grid(d.L[0] / sh.xw, d.L[1], 4);
     if (short_zt_lines(d))
-        k_zt_fxt<32><<<grid, 2 * sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
+        k_zt_fxt<32><<<grid, fxt_threads(sh.nt_zt, sm, true), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
     else
-        k_zt_fxt<128><<<grid, 2 * sh.nt_zt, sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
+        k_zt_fxt<128><<<grid, fxt_threads(sh.nt_zt, sm, false), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
 }
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* Fd, longlong2* g,
                         const FxtBuf& b, const Ctl* ctl)
@@ -80,9 +87,9 @@ void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const lon
     int xs = 0;
     while ((1 << xs) < sh.xw) xs++;
     if (small_plane<double>(d))
-        k_xyinv_fxt<32><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
+        k_xyinv_fxt<32><<<d.nplanes, fxt_threads(sh.nt_xy, sm, true), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
     else
-        k_xyinv_fxt<128><<<d.nplanes, 2 * sh.nt_xy, sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
+        k_xyinv_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
 }
 
 void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, longlong2* U, longlong2* AH, fx* Fs,
