@@ -101,9 +101,9 @@ struct lgf_ctx {
     // are within its range; `wide` links (a snapshot of anything else) take the FP64
     // kernels.  g64, AH64 and Fs64 hold the fixed-point g, parts and Re Tr meanwhile.
     longlong2* UX = nullptr;  // [4][6][V]
+    longlong2* GX = nullptr;  // [6][V]
     bool wide = false, graph_wide = false;
-    void* fxt_mem = nullptr;  // multipliers and exponents of the integer transform
-    FxtBuf fxt{};
+    FxtBuf fxt{};             // the integer transform's tables and exponents (in mult)
     void* Fd = nullptr;       // [4][V] double2 (the FP32 phase uses the front half as float2)
     double2* AH64 = nullptr;  // [4][4][V] packed anti-Hermitian parts of the links
     double* Fs64 = nullptr;   // [V] Re Tr of the four links of a site
@@ -249,7 +249,7 @@ void launch_g64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 void launch_update64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
     if (!c->wide)
-        launch_fx_update(c->lat, s, c->UX, c->G64, as_fx(c->g64), ctl, as_fx(c->AH64), as_fx(c->Fs64));
+        launch_fx_update(c->lat, s, c->UX, c->GX, as_fx(c->g64), ctl, as_fx(c->AH64), as_fx(c->Fs64));
     else
         launch_update<double>(c->lat, s, c->U64, c->G64, c->g64, ctl, c->AH64, c->Fs64);
 }
@@ -258,13 +258,13 @@ void launch_update64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 void launch_start64(lgf_ctx* c, cudaStream_t s)
 {
     if (!c->wide)
-        launch_fx_start(c->lat, s, c->U64, c->UX, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
+        launch_fx_start(c->lat, s, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
     else
         launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
 }
 void launch_finish64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
-    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->U64, c->G64, ctl, c->mixed);
+    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->GX, c->U64, c->G64, ctl, c->mixed);
 }
 
 // one FP64 iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, update,
@@ -413,8 +413,8 @@ int append_fix(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps
         CKR(add_loop32(c, graph, deps));
         CKR(capture_begin(c, graph, deps));
         if (!c->wide) {
-            launch_fx_project(c->lat, c->cap, c->G32, c->g64, c->U64, c->G64, c->UX, as_fx(c->AH64), as_fx(c->Fs64),
-                              c->fxt.fe, c->ctl);
+            launch_fx_project(c->lat, c->cap, c->G32, c->g64, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64),
+                              as_fx(c->Fs64), c->fxt.fe, c->ctl);
         } else {
             launch_switch(c->cap, c->lat, c->G32, c->g64, c->U64, c->G64, c->ctl);
             launch_start64(c, c->cap);
@@ -524,19 +524,18 @@ int build_tables(lgf_ctx* c)
     CK(cudaMemcpy(c->tables, h.data(), bytes, cudaMemcpyHostToDevice));
     // p2max/(p2(k) V) for every momentum, in both precisions
     const size_t Vs = (size_t)c->V;
-    CKR(alloc(&c->mult, Vs * (sizeof(double) + sizeof(float))));
+    const size_t fxt_off = (Vs * (sizeof(double) + sizeof(float)) + 255) / 256 * 256;
+    CKR(alloc(&c->mult, fxt_off + fxt_bytes(c->lat)));
     double* m64 = reinterpret_cast<double*>(c->mult);
     float* m32 = reinterpret_cast<float*>(m64 + Vs);
     launch_make_mult(nullptr, c->lat, c->tb, m64, m32);
+    // the integer transform's multipliers, roots and exponents, in the same allocation
+    c->fxt = fxt_carve(c->lat, reinterpret_cast<unsigned char*>(c->mult) + fxt_off);
+    launch_fxt_tables(c->lat, nullptr, m64, c->fxt);
     CK(cudaGetLastError());
     CK(cudaDeviceSynchronize());
     c->tb.mult64 = m64;
     c->tb.mult32 = m32;
-    CKR(alloc(&c->fxt_mem, fxt_bytes(c->lat)));
-    c->fxt = fxt_carve(c->lat, c->fxt_mem);
-    launch_fxt_tables(c->lat, nullptr, m64, c->fxt);
-    CK(cudaGetLastError());
-    CK(cudaDeviceSynchronize());
     return LGF_OK;
 }
 
@@ -585,7 +584,8 @@ int create_impl(const int dims[4], int flags, lgf_ctx* c)
     CKR(alloc((void**)&c->AH64, 16 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->Fs64, Vs * sizeof(double)));
     CK(fx_prepare(d));
-    CKR(alloc((void**)&c->UX, 24 * Vs * sizeof(longlong2)));
+    CKR(alloc((void**)&c->UX, (c->track ? 30 : 24) * Vs * sizeof(longlong2)));
+    if (c->track) c->GX = c->UX + 24 * Vs;
     if (c->mixed) {
         CKR(alloc((void**)&c->U32, 24 * Vs * sizeof(float2)));
         CKR(alloc((void**)&c->U32b, 24 * Vs * sizeof(float2)));
@@ -619,7 +619,7 @@ void free_all(lgf_ctx* c)
     if (c->exec) cudaGraphExecDestroy(c->exec);
     void* ptrs[] = {c->U64, c->G64, c->g64, c->U32, c->G32, c->g32, c->Fd, c->partials, c->ctl, c->ctl_stage,
                     c->hist, c->err, c->stage, c->tables, c->mult, c->AH64, c->Fs64, c->U32b, c->AH32, c->Fs32, c->dGp, c->dGud, c->dQ, c->dGgs, c->dFA, c->dFB,
-                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX, c->fxt_mem};
+                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->host_ctl) cudaFreeHost(c->host_ctl);

@@ -6,10 +6,9 @@
 // iterations therefore run on 64-bit integers: links and G hold a real x as
 // x 2^61 (range +-4, resolution 4.3e-19; FP64 resolves 1.1e-16 near 1), g as x 2^62.
 //
-// Digits.  A value is h 2^32 + l with h, l signed 32-bit digits, and is kept in
-// memory as that pair (l in the low word, h in the high one: the plain integer
-// plus its own bit 31 in the upper half), so that a loaded word needs no work to
-// be multiplied.
+// Digits.  For products a value is split into h 2^32 + l with h, l signed 32-bit
+// digits: l is the low word, h the high word plus the low word's top bit (one
+// instruction).  Constant tables hold the pairs themselves.
 //
 // Products.  Every partial product of two digits is one signed mad.wide.s32.  A
 // sum of products keeps two accumulators: hh = sum h h' and m = sum (h l' + l h'),
@@ -52,15 +51,12 @@ __host__ __device__ __forceinline__ dig digits(fx v)
 __host__ __device__ __forceinline__ cdig digits(cfx v) { return cdig{digits(v.re), digits(v.im)}; }
 __host__ __device__ __forceinline__ fx value(dig d) { return ((fx)d.h << 32) + d.l; }
 
-// digit pairs in memory
+// digit pairs in a table
 __device__ __forceinline__ cdig unpack(longlong2 v)
 {
     return cdig{dig{(int)(v.x >> 32), (int)v.x}, dig{(int)(v.y >> 32), (int)v.y}};
 }
 __device__ __forceinline__ fx word(dig d) { return ((fx)d.h << 32) | (unsigned)d.l; }
-__device__ __forceinline__ cdig ldd(const longlong2* p) { return unpack(__ldg(p)); }
-__device__ __forceinline__ void std_(longlong2* p, cdig v) { *p = make_longlong2(word(v.re), word(v.im)); }
-
 // sum of products of digit pairs
 struct facc {
     fx hh, m;
@@ -114,47 +110,44 @@ __host__ __device__ __forceinline__ facc fsub(facc p, facc n) { return facc{p.hh
 //   a b:        Re = p - q, Im = r - p - q,  r = (Re a + Im a) bs
 //   a conj(b):  Re = p + q, Im = p - q - r,  r = (Re a - Im a) bs
 // (p = Re a Re b, q = Im a Im b; sums over the row inside each).  The sums of a
-// row's entries obey the same bound as its six reals above.
+// row's entries obey the same bound as its six reals above, so each of the three
+// accumulators stays within 64 bits; their differences would not, and are taken
+// between the rounded values.
 struct cdig3 {
     dig re, im, s;
 };
-__device__ __forceinline__ cdig3 with_sum(cdig a) { return cdig3{a.re, a.im, digits(value(a.re) + value(a.im))}; }
-__device__ __forceinline__ cdig3 with_diff(cdig a) { return cdig3{a.re, a.im, digits(value(a.re) - value(a.im))}; }
 __device__ __forceinline__ cdig3 with_sum(cfx a) { return cdig3{digits(a.re), digits(a.im), digits(a.re + a.im)}; }
 __device__ __forceinline__ cdig3 with_diff(cfx a) { return cdig3{digits(a.re), digits(a.im), digits(a.re - a.im)}; }
 
-// row a of a left factor (three entries, sums) times column j of the 3x3 b
-template <int S> __device__ __forceinline__ cfx fx_mul(const cdig3* a, const cdig3* b, int j)
+struct pqr {
+    fx p, q, r;
+};
+// the three sums over a row a and three entries b[0], b[BS], b[2 BS], x 2^S
+template <int S, int BS> __device__ __forceinline__ pqr fx_pqr(const cdig3* a, const cdig3* b)
 {
-    facc p = fmul<S>(a[0].re, b[j].re), q = fmul<0>(a[0].im, b[j].im), r = fmul<S>(a[0].s, b[j].s);
-    // three roundings toward minus infinity: Im starts low by half a unit, so that
-    // the mean error of both parts is zero
+    facc p = fmul<S>(a[0].re, b[0].re), q = fmul<S>(a[0].im, b[0].im), r = fmul<S>(a[0].s, b[0].s);
+    // S = 0 rounds toward minus infinity; r starts low by half a unit, so that the
+    // mean error of r - p - q is zero
     if constexpr (S == 0) r.m -= 1ll << 31;
 #pragma unroll
     for (int k = 1; k < 3; k++) {
-        fmac(p, a[k].re, b[3 * k + j].re);
-        fmac(q, a[k].im, b[3 * k + j].im);
-        fmac(r, a[k].s, b[3 * k + j].s);
+        fmac(p, a[k].re, b[BS * k].re);
+        fmac(q, a[k].im, b[BS * k].im);
+        fmac(r, a[k].s, b[BS * k].s);
     }
-    if constexpr (S == 0) {
-        const fx x = fval<0>(p), y = fval<0>(q);
-        return cfx{x - y, fval<0>(r) - x - y};
-    } else {
-        return cfx{fval<S>(fsub(p, q)), fval<S>(facc{r.hh - p.hh - q.hh, r.m - p.m - q.m + (1ll << (31 - S))})};
-    }
+    return pqr{fval<S>(p), fval<S>(q), fval<S>(r)};
 }
-
-// row a (three entries, differences) times row j of conj(b): sum_k a_k conj(b_jk)
-template <int S> __device__ __forceinline__ cfx fx_mul_dag(const cdig3* a, const cdig3* b, int j)
+// row a of a left factor (three entries, sums) times column j of the 3x3 b
+template <int S> __device__ __forceinline__ cfx fx_mul(const cdig3* a, const cdig3* b, int j)
 {
-    facc p = fmul<S>(a[0].re, b[3 * j].re), q = fmul<0>(a[0].im, b[3 * j].im), r = fmul<0>(a[0].s, b[3 * j].s);
-#pragma unroll
-    for (int k = 1; k < 3; k++) {
-        fmac(p, a[k].re, b[3 * j + k].re);
-        fmac(q, a[k].im, b[3 * j + k].im);
-        fmac(r, a[k].s, b[3 * j + k].s);
-    }
-    return cfx{fval<S>(facc{p.hh + q.hh, p.m + q.m}), fval<S>(facc{p.hh - q.hh - r.hh, p.m - q.m - r.m})};
+    const pqr v = fx_pqr<S, 3>(a, b + j);
+    return cfx{v.p - v.q, v.r - v.p - v.q};
+}
+// row a (three entries, differences) times row b of a conjugated factor
+template <int S> __device__ __forceinline__ cfx fx_mul_dag(const cdig3* a, const cdig3* b)
+{
+    const pqr v = fx_pqr<S, 1>(a, b);
+    return cfx{v.p + v.q, v.p - v.q - v.r};
 }
 
 // conj(a b - c d)
@@ -226,8 +219,8 @@ __device__ __forceinline__ fx fx_rsqrt(fx n, int q)
     return ((fx)y0 << 32) + ((mulw(y0, cd.h) << 2) + (mulw(y0, cd.l) >> 30));
 }
 
-// g: rows 0,1 in digits x 2^62
-__device__ __forceinline__ void fx_gram_schmidt(const cfx* X, int q, cdig* g)
+// r: rows 0,1 x 2^62, g: their digits
+__device__ __forceinline__ void fx_gram_schmidt(const cfx* X, int q, cfx* r, cdig* g)
 {
     cdig x0[3];
 #pragma unroll
@@ -236,10 +229,13 @@ __device__ __forceinline__ void fx_gram_schmidt(const cfx* X, int q, cdig* g)
     auto scale = [&](dig v, dig w) {  // x 2^(61-q) times x 2^62 -> x 2^62
         facc a = fzero();
         fmac(a, v, w);
-        return digits(fval_rt(a, 3 + q));
+        return fval_rt(a, 3 + q);
     };
 #pragma unroll
-    for (int j = 0; j < 3; j++) g[j] = cdig{scale(x0[j].re, y), scale(x0[j].im, y)};
+    for (int j = 0; j < 3; j++) {
+        r[j] = cfx{scale(x0[j].re, y), scale(x0[j].im, y)};
+        g[j] = digits(r[j]);
+    }
     // <r0, X1> = sum conj(r0_j) X1_j, x 2^(61-q)
     cdig x1[3];
 #pragma unroll
@@ -264,7 +260,10 @@ __device__ __forceinline__ void fx_gram_schmidt(const cfx* X, int q, cdig* g)
     }
     const dig z = digits(fx_rsqrt(fx_norm2(v), q));
 #pragma unroll
-    for (int j = 0; j < 3; j++) g[3 + j] = cdig{scale(v[j].re, z), scale(v[j].im, z)};
+    for (int j = 0; j < 3; j++) {
+        r[3 + j] = cfx{scale(v[j].re, z), scale(v[j].im, z)};
+        g[3 + j] = digits(r[3 + j]);
+    }
 }
 
 __device__ __forceinline__ cfx ldx(const longlong2* p)

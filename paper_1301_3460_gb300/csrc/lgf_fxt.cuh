@@ -519,12 +519,13 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
                 X[5] = cfx{scaledl(hm, f2.re), scaledl(hm, f2.im)};
             }
             X[3] = cfx{-X[1].re, X[1].im};  // -conj(Delta01)
-            cdig r[6];
-            fx_gram_schmidt(X, q, r);
+            cfx r[6];
+            cdig rd[6];
+            fx_gram_schmidt(X, q, r, rd);
 #pragma unroll
-            for (int e = 0; e < 6; e++) std_(g + (size_t)e * V + s0 + xy, r[e]);
+            for (int e = 0; e < 6; e++) stx(g + (size_t)e * V + s0 + xy, r[e]);
 #pragma unroll
-            for (int j = 0; j < 3; j++) std_(g + (size_t)(6 + j) * V + s0 + xy, digits(fx_row2<2>(r, r + 3, j)));
+            for (int j = 0; j < 3; j++) stx(g + (size_t)(6 + j) * V + s0 + xy, fx_row2<2>(rd, rd + 3, j));
         }
         return;
     }

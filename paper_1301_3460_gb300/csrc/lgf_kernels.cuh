@@ -665,11 +665,12 @@ __device__ __forceinline__ void store_g(vec2_t<TG>* __restrict__ g, int V, int s
         bool bad = false;
 #pragma unroll
         for (int e = 0; e < 6; e++) {
-            rd[e] = digits(cfx{d2fx<kFxG>(gm[e].re, &bad), d2fx<kFxG>(gm[e].im, &bad)});
-            std_(g + (size_t)e * V + s, rd[e]);
+            const cfx v = cfx{d2fx<kFxG>(gm[e].re, &bad), d2fx<kFxG>(gm[e].im, &bad)};
+            rd[e] = digits(v);
+            stx(g + (size_t)e * V + s, v);
         }
 #pragma unroll
-        for (int j = 0; j < 3; j++) std_(g + (size_t)(6 + j) * V + s, digits(fx_row2<2>(rd, rd + 3, j)));
+        for (int j = 0; j < 3; j++) stx(g + (size_t)(6 + j) * V + s, fx_row2<2>(rd, rd + 3, j));
         if (bad) const_cast<Ctl*>(ctl)->bad = 1;
     } else {
         cx<TG> gs[9];

@@ -92,27 +92,27 @@ void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const lon
         k_xyinv_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
 }
 
-void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, longlong2* U, longlong2* AH, fx* Fs,
-                     FxExp* fe)
+void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
+                     longlong2* AH, fx* Fs, FxExp* fe)
 {
-    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, U, AH, Fs, fe);
+    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, U, G, AH, Fs, fe);
 }
-void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64, double2* G64,
-                       longlong2* U, longlong2* AH, fx* Fs, FxExp* fe, Ctl* ctl)
+void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
+                       const double2* G64, longlong2* U, longlong2* G, longlong2* AH, fx* Fs, FxExp* fe, Ctl* ctl)
 {
     k_switch_gs<<<blocks(d.V, 256), 256, 0, s>>>(d.V, G32, Gs, ctl);
-    k_fx_project<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, Gs, U, AH, Fs, fe, ctl);
+    k_fx_project<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, Gs, U, G, AH, Fs, fe, ctl);
     k_phase_switch<<<1, 1, 0, s>>>(ctl);
 }
-void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, double2* U64, double2* G64, const Ctl* ctl,
-                      bool always)
+void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
+                      const Ctl* ctl, bool always)
 {
-    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, U64, G64, ctl, always ? 1 : 0);
+    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl, always ? 1 : 0);
 }
-void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, double2* G, const longlong2* g, Ctl* ctl,
+void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, fx* Fs)
 {
-    k_update_fx<<<blocks(d.V, 64), 64, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+    k_update_fx<<<blocks(d.V, kUpdThreads), kUpdThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
 }
 
 template <typename TF>

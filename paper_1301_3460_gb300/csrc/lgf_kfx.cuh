@@ -1,8 +1,9 @@
 // The FP64 iterations on 64-bit fixed point (lgf_fx.cuh): start and end of a
 // loop, the update and the Delta stencil.  Arrays of a loop:
-//   UX   [mu=4][6][V]  rows 0,1 of every link, x 2^61 in digits (whatever form the
+//   UX   [mu=4][6][V]  rows 0,1 of every link, x 2^61 (whatever form the
 //                      context stores its FP64 links in)
-//   gX   [9][V]        g, x 2^62 in digits
+//   GX   [6][V]        rows 0,1 of G, x 2^61 (null: not tracked)
+//   gX   [9][V]        g, x 2^62
 //   AHX  [mu=4][4][V]  packed anti-Hermitian parts of the links, x 2^58; the
 //                      fourth entry holds 2 Im w00 - Im w11 - Im w22 and 2 Im w11
 //                      - Im w00 - Im w22 (3/2 of the packed traceless diagonal:
@@ -34,15 +35,15 @@ __device__ __forceinline__ void fx_ah(const cfx* w, const cdig* wd, cfx* a, fx& 
     retr += to_sum(w[0].re + w[4].re) + w2[2].re;
 }
 
-// Row 2 of a link from the digits of its rows 0,1 and its packed part: the
+// Row 2 of a link from its rows 0,1 (w, digits r) and its packed part: the
 // off-diagonal entries of the part are w02 - conj(w20) and w12 - conj(w21), its
 // diagonal gives Im w22, so only Re w22 is multiplied out (60 of 72 integer
 // products less, for 48 bytes read; the same values as fx_ah's row 2).
-__device__ __forceinline__ void fx_row2_from_part(const cdig* r, const longlong2* part, cfx* r2)
+__device__ __forceinline__ void fx_row2_from_part(const cfx* w, const cdig3* r, const longlong2* part, cfx* r2)
 {
-    const fx w02r = to_sum(value(r[2].re)), w02i = to_sum(value(r[2].im));
-    const fx w12r = to_sum(value(r[5].re)), w12i = to_sum(value(r[5].im));
-    const fx s0 = to_sum(value(r[0].im)), s1 = to_sum(value(r[4].im));
+    const fx w02r = to_sum(w[2].re), w02i = to_sum(w[2].im);
+    const fx w12r = to_sum(w[5].re), w12i = to_sum(w[5].im);
+    const fx s0 = to_sum(w[0].im), s1 = to_sum(w[4].im);
     r2[0] = cfx{w02r - part[0].x, part[0].y - w02i};
     r2[1] = cfx{w12r - part[1].x, part[1].y - w12i};
     // part[2].x = 3 s0 - (s0 + s1 + Im w22)
@@ -54,30 +55,26 @@ __device__ __forceinline__ void fx_row2_from_part(const cdig* r, const longlong2
     for (int j = 0; j < 3; j++) r2[j] = cfx{r2[j].re << (kFxBits - kFxSum), r2[j].im << (kFxBits - kFxSum)};
 }
 
-// Rows 0,1 of w = ga u gb^dag: A = rows 0,1 of ga times u (at 2^-59, unshifted), then
-// times gb^dag.  u: digits of rows 0,1; u2: row 2; gb: digits of all three rows.
-__device__ __forceinline__ void fx_link_gug(const cdig3* ga, const cdig* u, const cfx* u2, const cdig* gb, cfx* w)
+// A = rows 0,1 of ga times u (at 2^-59, unshifted), kept with their differences for the
+// product with gb^dag
+__device__ __forceinline__ void fx_left(const cdig3* ga, const cdig3* ud, cdig3* A)
 {
-    cdig3 A[6];
-    {
-        cdig3 ud[9];
-#pragma unroll
-        for (int e = 0; e < 6; e++) ud[e] = with_sum(u[e]);
-#pragma unroll
-        for (int j = 0; j < 3; j++) ud[6 + j] = with_sum(u2[j]);
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            A[j] = with_diff(fx_mul<0>(ga, ud, j));
-            A[3 + j] = with_diff(fx_mul<0>(ga + 3, ud, j));
-        }
-    }
-    cdig3 b[9];
-#pragma unroll
-    for (int e = 0; e < 9; e++) b[e] = with_sum(gb[e]);
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-        w[j] = fx_mul_dag<4>(A, b, j);
-        w[3 + j] = fx_mul_dag<4>(A + 3, b, j);
+        A[j] = with_diff(fx_mul<0>(ga, ud, j));
+        A[3 + j] = with_diff(fx_mul<0>(ga + 3, ud, j));
+    }
+}
+// rows 0,1 of w = A gb^dag; gb(e): entry e of gb
+template <typename GB> __device__ __forceinline__ void fx_right(const cdig3* A, GB gb, cfx* w)
+{
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        cdig3 b[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) b[k] = with_sum(gb(3 * j + k));
+        w[j] = fx_mul_dag<4>(A, b);
+        w[3 + j] = fx_mul_dag<4>(A + 3, b);
     }
 }
 
@@ -89,7 +86,7 @@ __device__ __forceinline__ void fx_store_link(longlong2* __restrict__ U, longlon
 #pragma unroll
     for (int e = 0; e < 6; e++) {
         wd[e] = digits(w[e]);
-        std_(U + (size_t)(mu * 6 + e) * V + s, wd[e]);
+        stx(U + (size_t)(mu * 6 + e) * V + s, w[e]);
     }
     cfx a[4];
     fx_ah(w, wd, a, f);
@@ -97,62 +94,134 @@ __device__ __forceinline__ void fx_store_link(longlong2* __restrict__ U, longlon
     for (int k = 0; k < 4; k++) stx(AH + (size_t)(mu * 4 + k) * V + s, a[k]);
 }
 
-// The update of one site: U'_mu(x) = g(x) U_mu(x) g^dag(x+mu) in place, the
-// packed parts and Re Tr of the new links, G(x) <- g(x) G(x).  G stays in FP64: its
-// 96 operations per site run on the FP64 pipe beside the integer products.
-//
-// Bound (32^4): 1630 mad.wide.s32 per site (24 per clock and SM with distinct
-// operands: 0.23 ms) and 1560 B/site of HBM traffic (0.24 ms).  One direction per
-// pass of a rolled loop keeps the code in the instruction cache.
-__device__ __forceinline__ void fx_update_site(const Lat& d, longlong2* __restrict__ U, double2* __restrict__ G,
-                                               const longlong2* __restrict__ g, longlong2* __restrict__ AH,
-                                               fx* __restrict__ Fs, int s)
+// G(x) <- g(x) G(x): rows 0,1 (m on entry), G's row 2 rebuilt
+__device__ __forceinline__ void fx_gauge_accumulate(longlong2* __restrict__ G, int V, int s, const cdig3* gx,
+                                                    const cfx* m)
 {
-    const int V = d.V;
-    int c[4];
-    site_coords(d, s, c);
-    cdig3 gx[6];
+    cdig3 md[9];
 #pragma unroll
-    for (int e = 0; e < 6; e++) gx[e] = with_sum(ldd(g + (size_t)e * V + s));
-    fx f = 0;
-#pragma unroll 1
-    for (int mu = 0; mu < 4; mu++) {
-        const int cm = mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3];
-        const int sn = site_shift(d, s, cm, mu, +1);
-        cdig u[6], gn[9];
-        longlong2 part[3];
+    for (int e = 0; e < 6; e++) md[e] = with_sum(m[e]);
 #pragma unroll
-        for (int e = 0; e < 6; e++) u[e] = unpack(U[(size_t)(mu * 6 + e) * V + s]);
+    for (int j = 0; j < 3; j++) md[6 + j] = with_sum(fx_row2<3>(md, md + 3, j));
 #pragma unroll
-        for (int k = 0; k < 3; k++) part[k] = AH[(size_t)(mu * 4 + 1 + k) * V + s];
+    for (int i = 0; i < 2; i++)
 #pragma unroll
-        for (int e = 0; e < 9; e++) gn[e] = ldd(g + (size_t)e * V + sn);
-        cfx u2[3], w[6];
-        fx_row2_from_part(u, part, u2);
-        fx_link_gug(gx, u, u2, gn, w);
-        fx_store_link(U, AH, V, mu, s, w, f);
-    }
-    Fs[s] = f;
-    if (G != nullptr) {
-        cx<double> gd[6];
-#pragma unroll
-        for (int e = 0; e < 6; e++) gd[e] = mk<double>(fx2d(value(gx[e].re), kFxG), fx2d(value(gx[e].im), kFxG));
-        gauge_accumulate<double>(G, V, s, gd);
-    }
+        for (int j = 0; j < 3; j++) stx(G + (size_t)(3 * i + j) * V + s, fx_mul<2>(gx + 3 * i, md, j));
 }
 
-static __global__ void __launch_bounds__(64, 6) k_update_fx(Lat d, longlong2* __restrict__ U,
-                                                            double2* __restrict__ G,
-                                                             const longlong2* __restrict__ g, Ctl* ctl,
-                                                             longlong2* __restrict__ AH, fx* __restrict__ Fs)
+// 16 bytes to the thread's own slot in shared memory, past L1 (streamed data) or
+// through it (g, read by up to five sites)
+template <bool L1> __device__ __forceinline__ void cp_async16(longlong2* dst, const longlong2* src)
 {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(dst);
+    if (L1) asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+    else asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest group of this thread's copies have arrived
+__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+
+// The update of every site, one thread each: U'_mu(x) = g(x) U_mu(x) g^dag(x+mu) in
+// place, the packed parts and Re Tr of the new links, G(x) <- g(x) G(x).
+//
+// Bound: 1632 (+ 234 with G) mad.wide.s32 per site, which issue at 24 to 32 per clock
+// and SM with distinct operands (32^4: 0.21 to 0.28 ms), and 1560 B/site of HBM
+// traffic (0.24 ms).  A thread holds some 120 registers, so 16 warps per SM: too few to
+// wait out the loads.  Each direction's inputs are therefore copied to slots in shared
+// memory of the thread's own (no barrier) one direction ahead: the link and its part as
+// soon as the current ones are in registers, g(x+mu) as soon as it has been used; g(x)
+// waits in shared memory too.  32^4, with G: 447 us with loads where they are used (455
+// with G in FP64), 323 us like this; without G 357 and 281 us.
+constexpr int kUpdThreads = 128;
+static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, longlong2* __restrict__ U,
+                                                                     longlong2* __restrict__ G,
+                                                                     const longlong2* __restrict__ g, Ctl* ctl,
+                                                                     longlong2* __restrict__ AH, fx* __restrict__ Fs)
+{
+    __shared__ longlong2 slots[24 * kUpdThreads];  // per thread: link and part (9), g(x+mu) (9), rows 0,1 of g(x) (6)
+    constexpr int NT = kUpdThreads;
     if (ld_flag(&ctl->phase_done)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->iter += 1;
         if (ctl->phase == 0) ctl->iter_phase0 += 1;
     }
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < d.V) fx_update_site(d, U, G, g, AH, Fs, s);
+    const int V = d.V;
+    const int s = blockIdx.x * NT + threadIdx.x;
+    if (s >= V) return;
+    longlong2 *su = slots + threadIdx.x, *sn = su + 9 * NT, *sx = sn + 9 * NT;
+    int nb[4];
+    {
+        int c[4];
+        site_coords(d, s, c);
+#pragma unroll
+        for (int mu = 0; mu < 4; mu++) nb[mu] = site_shift(d, s, c[mu], mu, +1);
+    }
+    auto fetch_u = [&](int mu) {
+#pragma unroll
+        for (int e = 0; e < 6; e++) cp_async16<false>(su + e * NT, U + (size_t)(mu * 6 + e) * V + s);
+#pragma unroll
+        for (int k = 0; k < 3; k++) cp_async16<false>(su + (6 + k) * NT, AH + (size_t)(mu * 4 + 1 + k) * V + s);
+    };
+    auto fetch_g = [&](int site) {
+#pragma unroll
+        for (int e = 0; e < 9; e++) cp_async16<true>(sn + e * NT, g + (size_t)e * V + site);
+    };
+    fetch_u(0);
+    cp_async_commit();
+    fetch_g(nb[0]);
+    cp_async_commit();
+#pragma unroll
+    for (int e = 0; e < 6; e++) sx[e * NT] = __ldg(g + (size_t)e * V + s);
+    auto load_gx = [&](cdig3* gx) {
+#pragma unroll
+        for (int e = 0; e < 6; e++) gx[e] = with_sum(ldv<fx>(sx + e * NT));
+    };
+    fx f = 0;
+#pragma unroll 1
+    for (int mu = 0; mu < 4; mu++) {
+        cfx u[9], w[6];
+        cdig3 A[6];
+        cp_async_wait1();
+        {
+            cdig3 ud[9];
+            longlong2 part[3];
+#pragma unroll
+            for (int e = 0; e < 6; e++) u[e] = ldv<fx>(su + e * NT);
+#pragma unroll
+            for (int k = 0; k < 3; k++) part[k] = su[(6 + k) * NT];
+#pragma unroll
+            for (int e = 0; e < 6; e++) ud[e] = with_sum(u[e]);
+            fx_row2_from_part(u, ud, part, u + 6);
+            // the slots are free: the next direction's link, G after the last one
+            if (mu < 3) {
+                fetch_u(mu + 1);
+            } else if (G != nullptr) {
+#pragma unroll
+                for (int e = 0; e < 6; e++) cp_async16<false>(su + e * NT, G + (size_t)e * V + s);
+            }
+            cp_async_commit();
+#pragma unroll
+            for (int e = 6; e < 9; e++) ud[e] = with_sum(u[e]);
+            cdig3 gx[6];
+            load_gx(gx);
+            fx_left(gx, ud, A);
+        }
+        cp_async_wait1();
+        fx_right(A, [&](int e) { return ldv<fx>(sn + e * NT); }, w);
+        if (mu < 3) fetch_g(mu == 0 ? nb[1] : mu == 1 ? nb[2] : nb[3]);
+        cp_async_commit();
+        fx_store_link(U, AH, V, mu, s, w, f);
+    }
+    Fs[s] = f;
+    if (G != nullptr) {
+        cp_async_wait1();
+        cdig3 gx[6];
+        cfx m[6];
+        load_gx(gx);
+#pragma unroll
+        for (int e = 0; e < 6; e++) m[e] = ldv<fx>(su + e * NT);
+        fx_gauge_accumulate(G, V, s, gx, m);
+    }
 }
 
 // magnitude exponents of the integer transform's fields (lgf_fxt.cuh)
@@ -162,10 +231,11 @@ struct FxExp {
     int amax2;  // over the pencils, after the accelerator (reset by the Delta kernel)
 };
 
-// Start of a loop: the links' rows 0,1 on the grid, rounded to nearest, with their
-// packed parts and Re Tr.
+// Start of a loop: the links' rows 0,1 (and G's) on the grid, rounded to nearest, with
+// the links' packed parts and Re Tr.
 static __global__ void __launch_bounds__(128) k_fx_start(Lat d, const double2* __restrict__ U64,
-                                                         longlong2* __restrict__ U, longlong2* __restrict__ AH,
+                                                         const double2* __restrict__ G64, longlong2* __restrict__ U,
+                                                         longlong2* __restrict__ G, longlong2* __restrict__ AH,
                                                          fx* __restrict__ Fs, FxExp* fe)
 {
     const int V = d.V;
@@ -183,14 +253,22 @@ static __global__ void __launch_bounds__(128) k_fx_start(Lat d, const double2* _
         fx_store_link(U, AH, V, mu, s, w, f);
     }
     Fs[s] = f;
+    if (G != nullptr) {
+#pragma unroll
+        for (int e = 0; e < 6; e++) {
+            const double2 v = G64[(size_t)e * V + s];
+            stx(G + (size_t)e * V + s, cfx{__double2ll_rn(v.x * 0x1p61), __double2ll_rn(v.y * 0x1p61)});
+        }
+    }
 }
 
 // Start of the FP64 loop after the FP32 phase: the links rebuilt on the input's
 // gauge orbit, U_mu(x) = Gs(x) U_in,mu(x) Gs^dag(x+mu), and G(x) <- Gs(x) G(x),
 // straight onto the grid (Gs: [9][V], re-orthonormalised in FP64).
 static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2* __restrict__ U64,
-                                                           double2* __restrict__ G, const double2* __restrict__ Gs,
-                                                           longlong2* __restrict__ U, longlong2* __restrict__ AH,
+                                                           const double2* __restrict__ G64,
+                                                           const double2* __restrict__ Gs, longlong2* __restrict__ U,
+                                                           longlong2* __restrict__ G, longlong2* __restrict__ AH,
                                                            fx* __restrict__ Fs, FxExp* fe, const Ctl* ctl)
 {
     if (ld_flag(&ctl->nan_seen)) return;
@@ -203,7 +281,7 @@ static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2*
     bool bad = false;
     auto load_gs = [&](int site, int e) {
         const cx<double> v = ld<double>(Gs + (size_t)e * V + site);
-        return digits(cfx{d2fx<kFxG>(v.re, &bad), d2fx<kFxG>(v.im, &bad)});
+        return cfx{d2fx<kFxG>(v.re, &bad), d2fx<kFxG>(v.im, &bad)};
     };
     cdig3 gx[6];
 #pragma unroll
@@ -212,39 +290,41 @@ static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2*
 #pragma unroll 1
     for (int mu = 0; mu < 4; mu++) {
         const int cm = mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3];
-        cdig u[6], gn[9];
-        {
-            cx<double> ud[9];
-            load_link<double>(U64, V, d.ne, mu, s, ud);
-#pragma unroll
-            for (int e = 0; e < 6; e++)
-                u[e] = digits(cfx{d2fx<kFxBits>(ud[e].re, &bad), d2fx<kFxBits>(ud[e].im, &bad)});
-        }
         const int sn = site_shift(d, s, cm, mu, +1);
+        cfx w[6];
+        cdig3 A[6];
+        {
+            cx<double> u[9];
+            cdig3 ud[9];
+            load_link<double>(U64, V, d.ne, mu, s, u);
 #pragma unroll
-        for (int e = 0; e < 9; e++) gn[e] = load_gs(sn, e);
-        cfx u2[3], w[6];
+            for (int e = 0; e < 6; e++) ud[e] = with_sum(cfx{d2fx<kFxBits>(u[e].re, &bad), d2fx<kFxBits>(u[e].im, &bad)});
 #pragma unroll
-        for (int j = 0; j < 3; j++) u2[j] = fx_row2<3>(u, u + 3, j);
-        fx_link_gug(gx, u, u2, gn, w);
+            for (int j = 0; j < 3; j++) ud[6 + j] = with_sum(fx_row2<3>(ud, ud + 3, j));
+            fx_left(gx, ud, A);
+        }
+        fx_right(A, [&](int e) { return load_gs(sn, e); }, w);
         fx_store_link(U, AH, V, mu, s, w, f);
     }
     Fs[s] = f;
     if (G != nullptr) {
-        cx<double> gd[6];
+        cfx m[6];
 #pragma unroll
-        for (int e = 0; e < 6; e++) gd[e] = ld<double>(Gs + (size_t)e * V + s);
-        gauge_accumulate<double>(G, V, s, gd);
+        for (int e = 0; e < 6; e++) {
+            const double2 v = G64[(size_t)e * V + s];
+            m[e] = cfx{d2fx<kFxBits>(v.x, &bad), d2fx<kFxBits>(v.y, &bad)};
+        }
+        fx_gauge_accumulate(G, V, s, gx, m);
     }
     if (bad) const_cast<Ctl*>(ctl)->bad = 1;
 }
 
-// End of a loop: links back to FP64 in the context's form (links and G NaN when an
-// entry of g was not finite).  Nothing is written when no update was made (always:
-// the start's links are not the stored ones, mixed mode), nor after a NaN in the
-// FP32 phase.
+// End of a loop: links and G back to FP64 in the context's form (NaN when an entry of g
+// was not finite).  Nothing is written when no update was made (always: the start's
+// links are not the stored ones, mixed mode), nor after a NaN in the FP32 phase.
 static __global__ void __launch_bounds__(128) k_fx_finish(Lat d, const longlong2* __restrict__ U,
-                                                          double2* __restrict__ U64, double2* __restrict__ G,
+                                                          const longlong2* __restrict__ G,
+                                                          double2* __restrict__ U64, double2* __restrict__ G64,
                                                           const Ctl* ctl, int always)
 {
     const bool bad = ld_flag(&ctl->bad) != 0;
@@ -254,19 +334,19 @@ static __global__ void __launch_bounds__(128) k_fx_finish(Lat d, const longlong2
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= V) return;
     const cx<double> nan = mk<double>(__hiloint2double(0x7ff80000, 0), __hiloint2double(0x7ff80000, 0));
+    auto back = [&](cfx v) { return bad ? nan : mk<double>(fx2d(v.re, kFxBits), fx2d(v.im, kFxBits)); };
 #pragma unroll 1
     for (int mu = 0; mu < 4; mu++) {
         cx<double> w[9];
 #pragma unroll
-        for (int e = 0; e < 6; e++) {
-            const cdig v = ldd(U + (size_t)(mu * 6 + e) * V + s);
-            w[e] = bad ? nan : mk<double>(fx2d(value(v.re), kFxBits), fx2d(value(v.im), kFxBits));
-        }
+        for (int e = 0; e < 6; e++) w[e] = back(ldx(U + (size_t)(mu * 6 + e) * V + s));
         if (d.ne != 6) complete_row2(w, w + 6);
         store_link<double>(U64, V, d.ne, mu, s, w);
     }
-    if (bad && G != nullptr)
-        for (int e = 0; e < 6; e++) st<double>(G + (size_t)e * V + s, nan);
+    if (G != nullptr) {
+#pragma unroll
+        for (int e = 0; e < 6; e++) st<double>(G64 + (size_t)e * V + s, back(ldx(G + (size_t)e * V + s)));
+    }
 }
 
 // Delta of the sites of one xy-plane from the fixed-point parts: the stencil's 56

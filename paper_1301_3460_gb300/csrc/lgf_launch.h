@@ -80,8 +80,8 @@ void launch_delta64_f32(const Lat& d, const Shape& sh64, cudaStream_t s, const d
 void launch_xyinv_g32_64(const Lat& d, const Shape& sh32, cudaStream_t s, const float2* Fd, double2* g,
                          const Ctl* ctl);
 
-// FP64 iterations on 64-bit fixed point (lgf_kfx.cuh): links on the grid 2^-61, g on
-// 2^-62, packed parts and Re Tr on 2^-58; G in FP64.  start: from the stored links;
+// FP64 iterations on 64-bit fixed point (lgf_kfx.cuh): links and G on the grid 2^-61, g
+// on 2^-62, packed parts and Re Tr on 2^-58.  start: from the stored links;
 // project: the end of the FP32 phase (links rebuilt on the input's orbit, phase
 // switched); finish: back to the stored FP64 links.  TF: precision of the transforms.
 struct FxExp;
@@ -102,13 +102,13 @@ bool fxt_fits(const Lat& d, const Shape& sh);
 FxtBuf fxt_carve(const Lat& d, void* p);
 void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const FxtBuf& b);
 cudaError_t fx_prepare(const Lat& d);
-void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, longlong2* U, longlong2* AH, long long* Fs,
-                     FxExp* fe);
-void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64, double2* G64,
-                       longlong2* U, longlong2* AH, long long* Fs, FxExp* fe, Ctl* ctl);
-void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, double2* U64, double2* G64, const Ctl* ctl,
-                      bool always);
-void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, double2* G, const longlong2* g, Ctl* ctl,
+void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
+                     longlong2* AH, long long* Fs, FxExp* fe);
+void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
+                       const double2* G64, longlong2* U, longlong2* G, longlong2* AH, long long* Fs, FxExp* fe, Ctl* ctl);
+void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
+                      const Ctl* ctl, bool always);
+void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, long long* Fs);
 template <typename TF>
 void launch_fx_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
