@@ -135,6 +135,7 @@ struct lgf_ctx {
     double* gl_D = nullptr;    // [5]
     double* wil_part = nullptr;  // plaquette partial sums, then the result
     int gen_precision = 64;      // arithmetic of the configuration generator's staples and draws
+    longlong2* genx = nullptr;   // [4][9][V]: fixed-point links of the FP64 generator
     float2* gen32 = nullptr;     // [4][6][V]: FP32 copy of the links for the FP32 generator's staples
 };
 
@@ -619,7 +620,7 @@ void free_all(lgf_ctx* c)
     if (c->exec) cudaGraphExecDestroy(c->exec);
     void* ptrs[] = {c->U64, c->G64, c->g64, c->U32, c->G32, c->g32, c->Fd, c->partials, c->ctl, c->ctl_stage,
                     c->hist, c->err, c->stage, c->tables, c->mult, c->AH64, c->Fs64, c->U32b, c->AH32, c->Fs32, c->dGp, c->dGud, c->dQ, c->dGgs, c->dFA, c->dFB,
-                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX};
+                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX, c->genx};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->host_ctl) cudaFreeHost(c->host_ctl);
@@ -1744,6 +1745,11 @@ int lgf_wilson_sweeps(lgf_ctx* c, double beta, unsigned long long seed, int firs
         if (!c->gen32) CKR(alloc((void**)&c->gen32, (size_t)24 * c->V * sizeof(float2)));
         launch_links_to_fp32(c->stream, c->lat, c->U64, c->gen32);
     }
+    const bool fixed = c->gen_precision == 64 && !c->wide && n_heatbath + n_overrelax > 0;
+    if (fixed) {
+        if (!c->genx) CKR(alloc((void**)&c->genx, (size_t)36 * c->V * sizeof(longlong2)));
+        launch_links_to_fx(c->stream, c->lat, c->U64, c->genx);
+    }
     // n_heatbath = 0: overrelaxation sweeps only
     const int rounds = n_heatbath > 0 ? n_heatbath : 1;
     for (int i = 0; i < rounds; i++) {
@@ -1751,10 +1757,14 @@ int lgf_wilson_sweeps(lgf_ctx* c, double beta, unsigned long long seed, int firs
         for (int mode = n_heatbath > 0 ? 0 : 1; mode < 1 + n_overrelax; mode++)
             for (int mu = 0; mu < 4; mu++)
                 for (int par = 0; par < 2; par++)
-                    launch_wilson(c->stream, c->lat, c->U64, c->gen32, mu, par, mode > 0, beta, seed, sweep,
-                                  c->gen_precision);
+                    if (fixed)
+                        launch_wilson_fx(c->stream, c->lat, c->genx, mu, par, mode > 0, beta, seed, sweep);
+                    else
+                        launch_wilson(c->stream, c->lat, c->U64, c->gen32, mu, par, mode > 0, beta, seed, sweep,
+                                      c->gen_precision);
         CK(cudaGetLastError());
     }
+    if (fixed) launch_links_from_fx(c->stream, c->lat, c->genx, c->U64);
     if (c->track) launch_identity_rows64(c->stream, c->V, c->G64);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->stream));

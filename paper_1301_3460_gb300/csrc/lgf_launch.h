@@ -162,6 +162,11 @@ void launch_gluon_bwd(cudaStream_t s, const Lat& d, const double2* U, const doub
 // and the mean plaquette (lgf_wilson.cu)
 void launch_wilson(cudaStream_t s, const Lat& d, double2* U, float2* U32, int mu, int parity, int overrelax,
                    double beta, unsigned long long seed, unsigned int sweep, int precision);
+// the same on fixed-point links UX [mu][9][V], converted once per call
+void launch_links_to_fx(cudaStream_t s, const Lat& d, const double2* U, longlong2* UX);
+void launch_links_from_fx(cudaStream_t s, const Lat& d, const longlong2* UX, double2* U);
+void launch_wilson_fx(cudaStream_t s, const Lat& d, longlong2* UX, int mu, int parity, int overrelax, double beta,
+                      unsigned long long seed, unsigned int sweep);
 void launch_links_to_fp32(cudaStream_t s, const Lat& d, const double2* U, float2* U32);
 void launch_unit_links(cudaStream_t s, const Lat& d, double2* U);
 int plaquette_blocks(int V);

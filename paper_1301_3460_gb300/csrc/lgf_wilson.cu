@@ -26,14 +26,19 @@
 // subgroup g reads draw 2a (y0) and, once accepted, 2a + 1 (direction); after
 // 512 failed attempts the subgroup is left unchanged.
 //
-// Every step is FP64.  Per link: 12 3x3 complex products for the staples (the
-// six of two SU(3) links with row 2 rebuilt instead of multiplied out), one for
-// W, the sampler's transcendental functions; the kernel is bound by the FP64
-// pipe.
+// Per link: 12 3x3 complex products for the staples (the six of two SU(3) links with
+// row 2 rebuilt instead of multiplied out), one for W, the rotations and the
+// sampler's transcendental functions.  In FP64 (k_wilson) the FP64 pipe bounds it (2
+// operations per clock and SM); by default the products, rotations and the
+// re-orthonormalisation run on 64-bit fixed point (k_wilson_fx, lgf_fx.cuh: finer
+// than FP64 for matrices bounded by 1), with the SU(2) elements and the sampler in
+// FP64.  Links outside the fixed-point range take the FP64 kernel.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "lgf_common.cuh"
+#include "lgf_fx.cuh"
+#include "lgf_kernels.cuh"
 #include "lgf_launch.h"
 
 namespace lgf {
@@ -349,6 +354,264 @@ __global__ void __launch_bounds__(kWilsonThreads) k_wilson(Lat d, double2* __res
     }
 }
 
+// ---------------------------------------------------------------- fixed-point generator
+
+// The links of a call on the grid 2^-61, all three rows: [mu][9][V] (the rows saved
+// from rebuilding, 144 integer products per staple, cost half as many bytes again).
+// Staples of up to six unit matrices and W are kept x 2^58 (range +-32).
+
+__global__ void k_links_to_fx(Lat d, const double2* __restrict__ U, longlong2* __restrict__ UX)
+{
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 4L * d.V) return;
+    const int mu = (int)(idx / d.V), s = (int)(idx - (long)mu * d.V);
+    cfx r[6];
+    cdig rd[6];
+#pragma unroll
+    for (int e = 0; e < 6; e++) {
+        const double2 v = U[(size_t)(mu * d.ne + e) * d.V + s];
+        r[e] = cfx{__double2ll_rn(v.x * 0x1p61), __double2ll_rn(v.y * 0x1p61)};
+        rd[e] = digits(r[e]);
+        stx(UX + (size_t)(mu * 9 + e) * d.V + s, r[e]);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; j++) stx(UX + (size_t)(mu * 9 + 6 + j) * d.V + s, fx_row2<3>(rd, rd + 3, j));
+}
+__global__ void k_links_from_fx(Lat d, const longlong2* __restrict__ UX, double2* __restrict__ U)
+{
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 4L * d.V) return;
+    const int mu = (int)(idx / d.V), s = (int)(idx - (long)mu * d.V);
+    cx<double> w[9];
+#pragma unroll
+    for (int e = 0; e < 6; e++) {
+        const cfx v = ldx(UX + (size_t)(mu * 9 + e) * d.V + s);
+        w[e] = mk<double>(fx2d(v.re, kFxBits), fx2d(v.im, kFxBits));
+    }
+    complete_row2(w, w + 6);
+    store_link<double>(U, d.V, d.ne, mu, s, w);
+}
+
+__device__ __forceinline__ void load9x(const longlong2* __restrict__ U, int V, int mu, int s, cfx* m)
+{
+#pragma unroll
+    for (int e = 0; e < 9; e++) m[e] = ldv<fx>(U + (size_t)(mu * 9 + e) * V + s);
+}
+
+// q = a b for SU(3) links a (rows 0,1 read), b; row 2 rebuilt
+__device__ __forceinline__ void fx_mm_su3(const longlong2* __restrict__ U, int V, int mua, int sa, int mub, int sb, cfx* q)
+{
+    cdig3 a[6], b[9];
+#pragma unroll
+    for (int e = 0; e < 6; e++) a[e] = with_sum(ldv<fx>(U + (size_t)(mua * 9 + e) * V + sa));
+#pragma unroll
+    for (int e = 0; e < 9; e++) b[e] = with_sum(ldv<fx>(U + (size_t)(mub * 9 + e) * V + sb));
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        q[j] = fx_mul<3>(a, b, j);
+        q[3 + j] = fx_mul<3>(a + 3, b, j);
+    }
+    cdig qd[6];
+#pragma unroll
+    for (int e = 0; e < 6; e++) qd[e] = digits(q[e]);
+#pragma unroll
+    for (int j = 0; j < 3; j++) q[6 + j] = fx_row2<3>(qd, qd + 3, j);
+}
+
+// staple sum of link (mu, s), x 2^58
+__device__ __forceinline__ void fx_staple_sum(const Lat& d, const longlong2* __restrict__ U, int mu, int s, const int* c,
+                                              cfx* A)
+{
+    const int V = d.V;
+#pragma unroll
+    for (int e = 0; e < 9; e++) A[e] = cfx{0, 0};
+    const int sp = site_shift(d, s, c[mu], mu, +1);
+#pragma unroll 1
+    for (int nu = 0; nu < 4; nu++) {
+        if (nu == mu) continue;
+        const int cn = nu == 0 ? c[0] : nu == 1 ? c[1] : nu == 2 ? c[2] : c[3];
+        // x + mu has the same nu coordinate as x
+        const int up = site_shift(d, s, cn, nu, +1), dn = site_shift(d, s, cn, nu, -1);
+        const int dnp = site_shift(d, sp, cn, nu, -1);
+        cfx q[9];
+        fx_mm_su3(U, V, nu, s, mu, up, q);  // U_nu(x) U_mu(x+nu)
+        {
+            // + U_nu(x+mu) q^dag
+            cdig3 qd[9];
+#pragma unroll
+            for (int e = 0; e < 9; e++) qd[e] = with_sum(q[e]);
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                cdig3 a[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) a[k] = with_diff(ldv<fx>(U + (size_t)(nu * 9 + 3 * i + k) * V + sp));
+#pragma unroll
+                for (int j = 0; j < 3; j++) A[3 * i + j] = A[3 * i + j] + fx_mul_dag<0>(a, qd + 3 * j);
+            }
+        }
+        fx_mm_su3(U, V, mu, dn, nu, dnp, q);  // U_mu(x-nu) U_nu(x+mu-nu)
+        {
+            // + q^dag U_nu(x-nu): conj(q_ki) b_kj = conj(q_ki conj(b_kj))
+            cdig3 qd[9];
+#pragma unroll
+            for (int e = 0; e < 9; e++) qd[e] = with_diff(q[e]);
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                cdig3 b[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) b[k] = with_sum(ldv<fx>(U + (size_t)(nu * 9 + 3 * k + j) * V + dn));
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                    const cdig3 a[3] = {qd[i], qd[3 + i], qd[6 + i]};
+                    const cfx t = fx_mul_dag<0>(a, b);
+                    A[3 * i + j] = A[3 * i + j] + cfx{t.re, -t.im};
+                }
+            }
+        }
+    }
+}
+
+// R = [[a, b], [-conj b, conj a]], x 2^61: a with its sum and difference, b likewise
+struct fx_su2 {
+    cdig3 as, ad, bs, bd;
+};
+// R00 x + R01 y (x, y with sums)
+template <int S> __device__ __forceinline__ cfx fx_rot0(const fx_su2& R, cdig3 x, cdig3 y)
+{
+    facc p = fmul<S>(R.as.re, x.re), q = fmul<S>(R.as.im, x.im), r = fmul<S>(R.as.s, x.s);
+    fmac(p, R.bs.re, y.re);
+    fmac(q, R.bs.im, y.im);
+    fmac(r, R.bs.s, y.s);
+    const fx pv = fval<S>(p), qv = fval<S>(q), rv = fval<S>(r);
+    return cfx{pv - qv, rv - pv - qv};
+}
+// R10 x + R11 y = conj(a) y - conj(b) x, with conj(u) v = (p + q, r - p + q), r = (Re u - Im u)(Re v + Im v)
+template <int S> __device__ __forceinline__ cfx fx_rot1(const fx_su2& R, cdig3 x, cdig3 y)
+{
+    facc p = fmul<S>(R.ad.re, y.re), q = fmul<S>(R.ad.im, y.im), r = fmul<S>(R.ad.s, y.s);
+    facc p2 = fmul<S>(R.bd.re, x.re), q2 = fmul<S>(R.bd.im, x.im), r2 = fmul<S>(R.bd.s, x.s);
+    const fx pv = fval<S>(p) - fval<S>(p2), qv = fval<S>(q) - fval<S>(q2), rv = fval<S>(r) - fval<S>(r2);
+    return cfx{pv + qv, rv - pv + qv};
+}
+
+// the SU(2) rotation of the block (wii, wij; wji, wjj) of W (x 2^58): R = Y V^dag (heat
+// bath) or (V^dag)^2; false where the block projects to zero
+template <int MODE>
+__device__ __forceinline__ bool fx_subgroup(cfx wii, cfx wij, cfx wji, cfx wjj, double beta23, uint32_t k0, uint32_t k1,
+                                            uint32_t link, uint32_t sweep, int sub, fx_su2& R)
+{
+    // r = (wii + conj wjj)/2, s = (wij - conj wji)/2: sums exact, x 2^59
+    const double rr = fx2d(wii.re + wjj.re, kFxSum + 1), ri = fx2d(wii.im - wjj.im, kFxSum + 1);
+    const double sr = fx2d(wij.re - wji.re, kFxSum + 1), si = fx2d(wij.im + wji.im, kFxSum + 1);
+    const double k2 = rr * rr + ri * ri + sr * sr + si * si;
+    if (!(k2 > 0)) return false;
+    const double ik = rsqrt(k2);
+    const C a = mk(rr * ik, ri * ik), b = mk(sr * ik, si * ik);  // V = [[a, b], [-conj b, conj a]]
+    C R00, R01;
+    if (MODE == 0) {
+        double y[4];
+        su2_draw(beta23 * (k2 * ik), k0, k1, link, sweep, sub, y);
+        // Y = y0 + i (y1 s1 + y2 s2 + y3 s3); V^dag = [[conj a, -b], [conj b, a]]
+        const C Y00 = mk(y[0], y[3]), Y01 = mk(y[2], y[1]);
+        R00 = cmac(cmul(Y00, conjg(a)), Y01, conjg(b));
+        R01 = cmac(cmul(Y00, mk(-b.re, -b.im)), Y01, a);
+    } else {
+        // (V^dag)^2: conj(a)^2 - |b|^2, -b (a + conj a)
+        R00 = mk(fma(a.re, a.re, -fma(a.im, a.im, norm2(b))), -2.0 * a.re * a.im);
+        R01 = b * (-2.0 * a.re);
+    }
+    bool bad = false;
+    const cfx x = cfx{d2fx<kFxBits>(R00.re, &bad), d2fx<kFxBits>(R00.im, &bad)};
+    const cfx y = cfx{d2fx<kFxBits>(R01.re, &bad), d2fx<kFxBits>(R01.im, &bad)};
+    R.as = with_sum(x);
+    R.ad = with_diff(x);
+    R.bs = with_sum(y);
+    R.bd = with_diff(y);
+    return true;
+}
+
+// Of W only what the later subgroups read is rotated (seven entries), of the link
+// rows 0,1 and, for the second subgroup, row 2.  32^4: see launch_wilson.
+template <int MODE>
+__global__ void __launch_bounds__(kWilsonThreads, 3) k_wilson_fx(Lat d, longlong2* __restrict__ U, int mu, int parity,
+                                                              double beta, uint32_t k0, uint32_t k1, uint32_t sweep)
+{
+    const int h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h >= (d.V >> 1)) return;
+    const int hx = d.L[0] >> 1;
+    int c[4];
+    int r = h / hx;
+    const int xh = h - r * hx;
+    c[1] = r % d.L[1];
+    r /= d.L[1];
+    c[2] = r % d.L[2];
+    c[3] = r / d.L[2];
+    c[0] = 2 * xh + ((parity + c[1] + c[2] + c[3]) & 1);
+    const int s = c[0] + d.stride[1] * c[1] + d.stride[2] * c[2] + d.stride[3] * c[3];
+    const int V = d.V;
+    cfx A[9], u[9], w[9];
+    fx_staple_sum(d, U, mu, s, c, A);
+    load9x(U, V, mu, s, u);
+    {
+        cdig3 Ad[9];
+#pragma unroll
+        for (int e = 0; e < 9; e++) Ad[e] = with_sum(A[e]);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const cdig3 ud[3] = {with_sum(u[3 * i]), with_sum(u[3 * i + 1]), with_sum(u[3 * i + 2])};
+#pragma unroll
+            for (int j = 0; j < 3; j++) w[3 * i + j] = fx_mul<3>(ud, Ad, j);
+        }
+    }
+    const uint32_t link = (uint32_t)mu * (uint32_t)V + (uint32_t)s;
+    const double beta23 = beta * (2.0 / 3.0);
+    fx_su2 R;
+    if (fx_subgroup<MODE>(w[0], w[1], w[3], w[4], beta23, k0, k1, link, sweep, 0, R)) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const cdig3 x = with_sum(w[j]), y = with_sum(w[3 + j]);
+            const cfx n = fx_rot0<3>(R, x, y);
+            if (j > 0) w[3 + j] = fx_rot1<3>(R, x, y);
+            w[j] = n;
+        }
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const cdig3 x = with_sum(u[j]), y = with_sum(u[3 + j]);
+            u[j] = fx_rot0<3>(R, x, y);
+            u[3 + j] = fx_rot1<3>(R, x, y);
+        }
+    }
+    if (fx_subgroup<MODE>(w[0], w[2], w[6], w[8], beta23, k0, k1, link, sweep, 1, R)) {
+#pragma unroll
+        for (int j = 1; j < 3; j++) w[6 + j] = fx_rot1<3>(R, with_sum(w[j]), with_sum(w[6 + j]));
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const cdig3 x = with_sum(u[j]), y = with_sum(u[6 + j]);
+            u[j] = fx_rot0<3>(R, x, y);
+            u[6 + j] = fx_rot1<3>(R, x, y);
+        }
+    }
+    if (fx_subgroup<MODE>(w[4], w[5], w[7], w[8], beta23, k0, k1, link, sweep, 2, R)) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) u[3 + j] = fx_rot0<3>(R, with_sum(u[3 + j]), with_sum(u[6 + j]));
+    }
+    // rows 0,1 orthonormalised, rounded to the grid 2^-53 (exact in FP64, so that a chain
+    // does not depend on how it is split into calls), row 2 rebuilt
+    cfx X[6], o[6];
+    cdig od[6];
+#pragma unroll
+    for (int e = 0; e < 6; e++) X[e] = cfx{(u[e].re + 1) >> 1, (u[e].im + 1) >> 1};
+    fx_gram_schmidt(X, 1, o, od);
+#pragma unroll
+    for (int e = 0; e < 6; e++) {
+        o[e] = cfx{((o[e].re + 256) >> 9) << 8, ((o[e].im + 256) >> 9) << 8};
+        od[e] = digits(o[e]);
+        stx(U + (size_t)(mu * 9 + e) * V + s, o[e]);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; j++) stx(U + (size_t)(mu * 9 + 6 + j) * V + s, fx_row2<3>(od, od + 3, j));
+}
+
 // ---------------------------------------------------------------- FP32 generator
 
 // The same update with the staples, W, the SU(2) draws and the rotation of the
@@ -581,6 +844,26 @@ int plaquette_blocks(int V)
 void launch_links_to_fp32(cudaStream_t s, const Lat& d, const double2* U, float2* U32)
 {
     k_links_to_fp32<<<(unsigned)((d.V + 255) / 256), 256, 0, s>>>(d, U, U32);
+}
+
+void launch_links_to_fx(cudaStream_t s, const Lat& d, const double2* U, longlong2* UX)
+{
+    k_links_to_fx<<<(unsigned)((4L * d.V + 255) / 256), 256, 0, s>>>(d, U, UX);
+}
+void launch_links_from_fx(cudaStream_t s, const Lat& d, const longlong2* UX, double2* U)
+{
+    k_links_from_fx<<<(unsigned)((4L * d.V + 255) / 256), 256, 0, s>>>(d, UX, U);
+}
+
+void launch_wilson_fx(cudaStream_t s, const Lat& d, longlong2* UX, int mu, int parity, int overrelax, double beta,
+                      unsigned long long seed, unsigned int sweep)
+{
+    const unsigned nb = (unsigned)((d.V / 2 + kWilsonThreads - 1) / kWilsonThreads);
+    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    if (overrelax)
+        k_wilson_fx<1><<<nb, kWilsonThreads, 0, s>>>(d, UX, mu, parity, beta, k0, k1, sweep);
+    else
+        k_wilson_fx<0><<<nb, kWilsonThreads, 0, s>>>(d, UX, mu, parity, beta, k0, k1, sweep);
 }
 
 void launch_wilson(cudaStream_t s, const Lat& d, double2* U, float2* U32, int mu, int parity, int overrelax,
