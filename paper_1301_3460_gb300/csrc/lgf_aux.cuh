@@ -3,6 +3,7 @@
 // check of input links, stand-alone stage kernels, and the precision switch of
 // the mixed mode (FP32 phase -> FP64 phase).
 #pragma once
+#include "lgf_fx.cuh"
 #include "lgf_kernels.cuh"
 
 namespace lgf {
@@ -22,107 +23,213 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double 
     atomicMax(p, (unsigned long long)__double_as_longlong(v));
 }
 
-// Interleaved [4][V][3][3] complex128 -> rows 0,1 planes of T; optional SU(3)
-// check of the full input matrix: err[0] = max |U U^dag - 1|, err[1] = max |det U - 1|,
-// err[2] = max error of the round trip through the 8-real form (ne = 4).
-template <typename T>
-static __global__ void k_pack_links(int V, int ne, const double* __restrict__ in, vec2_t<T>* __restrict__ U,
-                             unsigned long long* err, int validate)
+// Matrices cross the boundary as 144-byte records.  A block moves a run of kRecThreads
+// of them through shared memory, so that global memory sees whole lines (a thread
+// reading its own record takes 32 lines per load instruction); record t starts 144 t
+// bytes into the run, which 16-byte accesses of consecutive threads reach without bank
+// conflicts.  16-byte global accesses where the caller's array allows them.
+constexpr int kRecThreads = 128;
+__device__ __forceinline__ void records_in(const double* __restrict__ in, long first, int n, double2* sm)
 {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;  // link index mu*V + s
-    // squared errors, their square root taken once after the maximum (the square
-    // root is monotone and correctly rounded, so this is the maximum of the errors)
-    double e_unit = 0.0, e_det = 0.0, e_form = 0.0;
-    if (idx < 4L * V) {
-        const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
-        const double* p = in + idx * 18;  // 8-byte loads: the caller's array need not be 16-byte aligned
-        cx<double> m[9];
+    const double* p = in + first * 18;
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+        const double2* q = reinterpret_cast<const double2*>(p);
 #pragma unroll
-        for (int e = 0; e < 9; e++) m[e] = mk<double>(p[2 * e], p[2 * e + 1]);
-        if (ne == 4) {
-            // 8-real form; the check below also covers its round trip (the form
-            // cannot hold links with |u00| = 1, such as the unit matrix)
-            cx<T> w[9];
-#pragma unroll
-            for (int e = 0; e < 9; e++) w[e] = mk<T>((T)m[e].re, (T)m[e].im);
-            store_link<T>(U, V, 4, mu, s, w);
-            if (validate) {
-                cx<T> r[9];
-                rebuild8<T>(w[1], w[2], w[3], atan2(w[0].im, w[0].re), atan2(w[6].im, w[6].re), r);
-#pragma unroll
-                for (int e = 0; e < 9; e++) e_form = dmax_nan(e_form, (double)norm2(r[e] - w[e]));
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < 6; e++) {
-                vec2_t<T> v;
-                v.x = (T)m[e].re;
-                v.y = (T)m[e].im;
-                U[(size_t)(mu * ne + e) * V + s] = v;
-            }
+        for (int k = 0; k < 9; k++) {
+            const int i = threadIdx.x + k * kRecThreads;
+            if (i < 9 * n) sm[i] = __ldg(q + i);
         }
-        if (ne == 9) {
-            // row 2 stored as the rebuild from rows 0,1, as a 12-real load would give it
-            cx<T> r[9];
+    } else {
+        double* d = reinterpret_cast<double*>(sm);
 #pragma unroll
-            for (int e = 0; e < 6; e++) r[e] = mk<T>((T)m[e].re, (T)m[e].im);
-            complete_row2(r, r + 6);
-#pragma unroll
-            for (int e = 6; e < 9; e++) st<T>(U + (size_t)(mu * 9 + e) * V + s, r[e]);
-        }
-        if (validate) {
-            // U U^dag is Hermitian: its entries (i, j) with i <= j (the entry (j, i)
-            // is their conjugate up to the last rounding of one product)
-#pragma unroll
-            for (int i = 0; i < 3; i++)
-#pragma unroll
-                for (int j = i; j < 3; j++) {
-                    cx<double> acc = cmulc(m[3 * i], m[3 * j]);
-                    acc = cmacc(acc, m[3 * i + 1], m[3 * j + 1]);
-                    acc = cmacc(acc, m[3 * i + 2], m[3 * j + 2]);
-                    if (i == j) acc.re -= 1.0;
-                    e_unit = dmax_nan(e_unit, norm2(acc));
-                }
-            cx<double> r2[3];
-            complete_row2(m, r2);  // conj of the cofactor row: det = sum_j m2j conj(r2_j)
-            cx<double> det = cmulc(m[6], r2[0]);
-            det = cmacc(det, m[7], r2[1]);
-            det = cmacc(det, m[8], r2[2]);
-            det.re -= 1.0;
-            e_det = norm2(det);
-            if (!(e_det == e_det)) e_det = 1e300;
+        for (int k = 0; k < 18; k++) {
+            const int i = threadIdx.x + k * kRecThreads;
+            if (i < 18 * n) d[i] = __ldg(p + i);
         }
     }
-    if (validate) {
+    __syncthreads();
+}
+__device__ __forceinline__ void records_out(double* __restrict__ out, long first, int n, const double2* sm)
+{
+    __syncthreads();
+    double* p = out + first * 18;
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+        double2* q = reinterpret_cast<double2*>(p);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            e_unit = dmax_nan(e_unit, __shfl_down_sync(0xffffffffu, e_unit, o));
-            e_det = dmax_nan(e_det, __shfl_down_sync(0xffffffffu, e_det, o));
-            e_form = dmax_nan(e_form, __shfl_down_sync(0xffffffffu, e_form, o));
+        for (int k = 0; k < 9; k++) {
+            const int i = threadIdx.x + k * kRecThreads;
+            if (i < 9 * n) q[i] = sm[i];
         }
-        if ((threadIdx.x & 31) == 0) {
-            atomic_max_nonneg(err, sqrt(e_unit));
-            atomic_max_nonneg(err + 1, sqrt(e_det));
-            atomic_max_nonneg(err + 2, sqrt(e_form));
+    } else {
+        const double* d = reinterpret_cast<const double*>(sm);
+#pragma unroll
+        for (int k = 0; k < 18; k++) {
+            const int i = threadIdx.x + k * kRecThreads;
+            if (i < 18 * n) p[i] = d[i];
         }
     }
 }
 
-// [nmat][ne][V] planes -> interleaved [nmat][V][3][3] complex128 (row 2 rebuilt or read)
-template <typename T>
-static __global__ void k_unpack_su3(int V, int nmat, int ne, const vec2_t<T>* __restrict__ U, double* __restrict__ out)
+__device__ __forceinline__ float fx2f(fx v) { return fmaf((float)(int)(v >> 32), 0x1p32f, (float)(unsigned)v); }
+
+// Largest squared entry of U U^dag - 1 (its Hermitian half) and |det U - 1|^2, in FP64
+__device__ __forceinline__ void su3_errors64(const cx<double>* m, double& e_unit, double& e_det)
 {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long)nmat * V) return;
-    const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
-    cx<T> m[9];
-    load_link<T>(U, V, ne, mu, s, m);
-    double* p = out + idx * 18;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++) {
+            cx<double> acc = cmulc(m[3 * i], m[3 * j]);
+            acc = cmacc(acc, m[3 * i + 1], m[3 * j + 1]);
+            acc = cmacc(acc, m[3 * i + 2], m[3 * j + 2]);
+            if (i == j) acc.re -= 1.0;
+            e_unit = dmax_nan(e_unit, norm2(acc));
+        }
+    cx<double> r2[3];
+    complete_row2(m, r2);  // conj of the cofactor row: det = sum_j m2j conj(r2_j)
+    cx<double> det = cmulc(m[6], r2[0]);
+    det = cmacc(det, m[7], r2[1]);
+    det = cmacc(det, m[8], r2[2]);
+    det.re -= 1.0;
+    e_det = norm2(det);
+    if (!(e_det == e_det)) e_det = 1e300;
+}
+
+// The same on 64-bit fixed point (entries x 2^61: the products are exact to 1e-18, the
+// errors' squares taken in FP32: the bound is 1e-12).  Returns false when an entry is
+// larger than 1 + 2^-20 or not finite, or a row's norm above 1.5, which the products do
+// not cover and no SU(3) matrix has.
+__device__ __forceinline__ bool su3_errors_fx(const cx<double>* m, double& e_unit, double& e_det)
+{
+    cfx v[9];
+    bool bad = false;
 #pragma unroll
     for (int e = 0; e < 9; e++) {
-        p[2 * e] = (double)m[e].re;
-        p[2 * e + 1] = (double)m[e].im;
+        bad = bad || !(fabs(m[e].re) <= 1.0 + 0x1p-20) || !(fabs(m[e].im) <= 1.0 + 0x1p-20);
+        bool b = false;
+        v[e] = cfx{d2fx<kFxBits>(m[e].re, &b), d2fx<kFxBits>(m[e].im, &b)};
     }
+    cdig3 vs[9];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        float n = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const float x = (float)(int)(v[3 * i + k].re >> 32), y = (float)(int)(v[3 * i + k].im >> 32);
+            n = fmaf(x, x, fmaf(y, y, n));
+        }
+        bad = bad || !(n < 1.5f * 0x1p58f);
+    }
+    if (bad) return false;
+    float eu = 0.f;
+#pragma unroll
+    for (int e = 0; e < 9; e++) vs[e] = with_sum(v[e]);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        facc a = fmul<3>(vs[3 * i].re, vs[3 * i].re);
+        fmac(a, vs[3 * i].im, vs[3 * i].im);
+#pragma unroll
+        for (int k = 1; k < 3; k++) {
+            fmac(a, vs[3 * i + k].re, vs[3 * i + k].re);
+            fmac(a, vs[3 * i + k].im, vs[3 * i + k].im);
+        }
+        const float x = fx2f(fval<3>(a) - (1ll << kFxBits));
+        eu = fmaxf(eu, x * x);
+        const cdig3 ad[3] = {with_diff(v[3 * i]), with_diff(v[3 * i + 1]), with_diff(v[3 * i + 2])};
+#pragma unroll
+        for (int j = i + 1; j < 3; j++) {
+            const cfx t = fx_mul_dag<3>(ad, vs + 3 * j);
+            const float p = fx2f(t.re), q = fx2f(t.im);
+            eu = fmaxf(eu, fmaf(p, p, q * q));
+        }
+    }
+    cdig3 rs[3], ld[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        rs[j] = with_sum(fx_row2<3>(vs, vs + 3, j));
+        ld[j] = with_diff(v[6 + j]);
+    }
+    const cfx t = fx_mul_dag<3>(ld, rs);
+    const float p = fx2f(t.re - (1ll << kFxBits)), q = fx2f(t.im);
+    e_unit = (double)eu * 0x1p-122;
+    e_det = (double)fmaf(p, p, q * q) * 0x1p-122;
+    return true;
+}
+
+// Interleaved [4][V][3][3] complex128 -> the stored planes (ne entries per link), with the SU(3)
+// check of the full input matrix: err[0] = max |U U^dag - 1|, err[1] = max |det U - 1|,
+// err[2] = max error of the round trip through the 8-real form (ne = 4).
+// 32^4: 1.60 ms with the check in FP64 and a thread per record in global memory (its
+// FP64 work alone is 1 ms).
+static __global__ void __launch_bounds__(kRecThreads) k_pack_links(int V, int ne, const double* __restrict__ in,
+                                                                   double2* __restrict__ U, unsigned long long* err)
+{
+    __shared__ double2 rec[9 * kRecThreads];
+    const long first = (long)blockIdx.x * kRecThreads;  // link index mu*V + s
+    const int n = (int)(4L * V - first < kRecThreads ? 4L * V - first : kRecThreads);
+    records_in(in, first, n, rec);
+    // squared errors, their square root taken once after the maximum (the square
+    // root is monotone and correctly rounded, so this is the maximum of the errors)
+    double e_unit = 0.0, e_det = 0.0, e_form = 0.0;
+    if ((int)threadIdx.x < n) {
+        const long idx = first + threadIdx.x;
+        const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
+        cx<double> m[9];
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            const double2 v = rec[9 * threadIdx.x + e];
+            m[e] = mk<double>(v.x, v.y);
+        }
+        if (ne == 4) {
+            // 8-real form; the check below also covers its round trip (the form
+            // cannot hold links with |u00| = 1, such as the unit matrix)
+            store_link<double>(U, V, 4, mu, s, m);
+            cx<double> r[9];
+            rebuild8<double>(m[1], m[2], m[3], atan2(m[0].im, m[0].re), atan2(m[6].im, m[6].re), r);
+#pragma unroll
+            for (int e = 0; e < 9; e++) e_form = dmax_nan(e_form, norm2(r[e] - m[e]));
+        } else {
+#pragma unroll
+            for (int e = 0; e < 6; e++) st<double>(U + (size_t)(mu * ne + e) * V + s, m[e]);
+        }
+        if (ne == 9) {
+            // row 2 stored as the rebuild from rows 0,1, as a 12-real load would give it
+            cx<double> r[3];
+            complete_row2(m, r);
+#pragma unroll
+            for (int e = 0; e < 3; e++) st<double>(U + (size_t)(mu * 9 + 6 + e) * V + s, r[e]);
+        }
+        if (!su3_errors_fx(m, e_unit, e_det)) su3_errors64(m, e_unit, e_det);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        e_unit = dmax_nan(e_unit, __shfl_down_sync(0xffffffffu, e_unit, o));
+        e_det = dmax_nan(e_det, __shfl_down_sync(0xffffffffu, e_det, o));
+        if (ne == 4) e_form = dmax_nan(e_form, __shfl_down_sync(0xffffffffu, e_form, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomic_max_nonneg(err, sqrt(e_unit));
+        atomic_max_nonneg(err + 1, sqrt(e_det));
+        if (ne == 4) atomic_max_nonneg(err + 2, sqrt(e_form));
+    }
+}
+
+// [nmat][ne][V] planes -> interleaved [nmat][V][3][3] complex128 (row 2 rebuilt or read)
+static __global__ void __launch_bounds__(kRecThreads) k_unpack_su3(int V, int nmat, int ne, const double2* __restrict__ U,
+                                                                   double* __restrict__ out)
+{
+    __shared__ double2 rec[9 * kRecThreads];
+    const long total = (long)nmat * V, first = (long)blockIdx.x * kRecThreads;
+    const int n = (int)(total - first < kRecThreads ? total - first : kRecThreads);
+    if ((int)threadIdx.x < n) {
+        const long idx = first + threadIdx.x;
+        const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
+        cx<double> m[9];
+        load_link<double>(U, V, ne, mu, s, m);
+#pragma unroll
+        for (int e = 0; e < 9; e++) rec[9 * threadIdx.x + e] = make_double2(m[e].re, m[e].im);
+    }
+    records_out(out, first, n, rec);
 }
 
 template <typename T> __global__ void k_identity_rows(int V, vec2_t<T>* __restrict__ G)

@@ -20,7 +20,7 @@
 //   b4 (per site): G_M = T(G_Delta) - T(G_Delta)^dag;
 //                  G_U_mu(x) = G_U^direct + G_M(x+mu) - G_M(x); (row-2 rebuild)^T -> rows 0,1
 #pragma once
-#include "lgf_kernels.cuh"
+#include "lgf_aux.cuh"
 
 namespace lgf {
 
@@ -94,29 +94,34 @@ static __global__ void k_g_from_dt(int V, const double2* __restrict__ Fd, double
 }
 
 // [4][V][3][3] interleaved complex128 -> [4][9][V] planes (full matrices)
-static __global__ void k_pack_full(int V, const double* __restrict__ in, double2* __restrict__ out)
+static __global__ void __launch_bounds__(kRecThreads) k_pack_full(int V, const double* __restrict__ in,
+                                                                  double2* __restrict__ out)
 {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 4L * V) return;
+    __shared__ double2 rec[9 * kRecThreads];
+    const long first = (long)blockIdx.x * kRecThreads;
+    const int n = (int)(4L * V - first < kRecThreads ? 4L * V - first : kRecThreads);
+    records_in(in, first, n, rec);
+    if ((int)threadIdx.x >= n) return;
+    const long idx = first + threadIdx.x;
     const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
-    const double* p = in + idx * 18;
 #pragma unroll
-    for (int e = 0; e < 9; e++) out[(size_t)(mu * 9 + e) * V + s] = make_double2(p[2 * e], p[2 * e + 1]);
+    for (int e = 0; e < 9; e++) out[(size_t)(mu * 9 + e) * V + s] = rec[9 * threadIdx.x + e];
 }
 
 // [4][9][V] planes -> [4][V][3][3] interleaved complex128
-static __global__ void k_unpack_planes(int V, const double2* __restrict__ in, double* __restrict__ out)
+static __global__ void __launch_bounds__(kRecThreads) k_unpack_planes(int V, const double2* __restrict__ in,
+                                                                      double* __restrict__ out)
 {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 4L * V) return;
-    const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
-    double* p = out + idx * 18;
+    __shared__ double2 rec[9 * kRecThreads];
+    const long first = (long)blockIdx.x * kRecThreads;
+    const int n = (int)(4L * V - first < kRecThreads ? 4L * V - first : kRecThreads);
+    if ((int)threadIdx.x < n) {
+        const long idx = first + threadIdx.x;
+        const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
 #pragma unroll
-    for (int e = 0; e < 9; e++) {
-        const double2 v = in[(size_t)(mu * 9 + e) * V + s];
-        p[2 * e] = v.x;
-        p[2 * e + 1] = v.y;
+        for (int e = 0; e < 9; e++) rec[9 * threadIdx.x + e] = in[(size_t)(mu * 9 + e) * V + s];
     }
+    records_out(out, first, n, rec);
 }
 
 // ---------------------------------------------------------------- step backward

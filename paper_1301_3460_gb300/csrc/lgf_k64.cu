@@ -50,11 +50,11 @@ void launch_xyinv_g32_64(const Lat& d, const Shape& sh32, cudaStream_t s, const 
 
 void launch_pack_links64(cudaStream_t s, int V, int ne, const double* in, double2* U, unsigned long long* err)
 {
-    k_pack_links<double><<<blocks(4L * V, 256), 256, 0, s>>>(V, ne, in, U, err, 1);
+    k_pack_links<<<blocks(4L * V, kRecThreads), kRecThreads, 0, s>>>(V, ne, in, U, err);
 }
 void launch_unpack_su3_64(cudaStream_t s, int V, int nmat, int ne, const double2* U, double* out)
 {
-    k_unpack_su3<double><<<blocks((long)nmat * V, 256), 256, 0, s>>>(V, nmat, ne, U, out);
+    k_unpack_su3<<<blocks((long)nmat * V, kRecThreads), kRecThreads, 0, s>>>(V, nmat, ne, U, out);
 }
 void launch_identity_rows64(cudaStream_t s, int V, double2* G)
 {
@@ -115,11 +115,11 @@ void launch_g_from_dt(cudaStream_t s, int V, const double2* Fd, double2* g, doub
 }
 void launch_pack_full(cudaStream_t s, int V, const double* in, double2* out)
 {
-    k_pack_full<<<blocks(4L * V, 256), 256, 0, s>>>(V, in, out);
+    k_pack_full<<<blocks(4L * V, kRecThreads), kRecThreads, 0, s>>>(V, in, out);
 }
 void launch_unpack_planes(cudaStream_t s, int V, const double2* in, double* out)
 {
-    k_unpack_planes<<<blocks(4L * V, 256), 256, 0, s>>>(V, in, out);
+    k_unpack_planes<<<blocks(4L * V, kRecThreads), kRecThreads, 0, s>>>(V, in, out);
 }
 void launch_step_bwd(cudaStream_t s, const Lat& d, const double2* U, const double2* g, const double2* Fdt,
                      double2* Gp, double2* Gud, double2* Ggs, double2* Q, double alpha, double2* FA, double2* FB)
