@@ -99,13 +99,16 @@ __device__ __forceinline__ void su3_errors64(const cx<double>* m, double& e_unit
 // errors' squares taken in FP32: the bound is 1e-12).  Returns false when an entry is
 // larger than 1 + 2^-20 or not finite, or a row's norm above 1.5, which the products do
 // not cover and no SU(3) matrix has.
-__device__ __forceinline__ bool su3_errors_fx(const cx<double>* m, double& e_unit, double& e_det)
+// e_unit, e_det in units of 2^-122.
+__device__ __forceinline__ bool su3_errors_fx(const cx<double>* m, float& e_unit, float& e_det)
 {
     cfx v[9];
     bool bad = false;
 #pragma unroll
     for (int e = 0; e < 9; e++) {
-        bad = bad || !(fabs(m[e].re) <= 1.0 + 0x1p-20) || !(fabs(m[e].im) <= 1.0 + 0x1p-20);
+        // |x| >= 1 + 2^-20, infinities and NaN among them, by the high word
+        bad = bad || ((unsigned)__double2hiint(m[e].re) & 0x7fffffffu) > 0x3ff00000u ||
+              ((unsigned)__double2hiint(m[e].im) & 0x7fffffffu) > 0x3ff00000u;
         bool b = false;
         v[e] = cfx{d2fx<kFxBits>(m[e].re, &b), d2fx<kFxBits>(m[e].im, &b)};
     }
@@ -151,8 +154,8 @@ __device__ __forceinline__ bool su3_errors_fx(const cx<double>* m, double& e_uni
     }
     const cfx t = fx_mul_dag<3>(ld, rs);
     const float p = fx2f(t.re - (1ll << kFxBits)), q = fx2f(t.im);
-    e_unit = (double)eu * 0x1p-122;
-    e_det = (double)fmaf(p, p, q * q) * 0x1p-122;
+    e_unit = eu;
+    e_det = fmaf(p, p, q * q);
     return true;
 }
 
@@ -169,8 +172,9 @@ static __global__ void __launch_bounds__(kRecThreads) k_pack_links(int V, int ne
     const int n = (int)(4L * V - first < kRecThreads ? 4L * V - first : kRecThreads);
     records_in(in, first, n, rec);
     // squared errors, their square root taken once after the maximum (the square
-    // root is monotone and correctly rounded, so this is the maximum of the errors)
-    double e_unit = 0.0, e_det = 0.0, e_form = 0.0;
+    // root is monotone, so this is the maximum of the errors)
+    double e_form = 0.0;
+    float eu = 0.f, ed = 0.f;
     if ((int)threadIdx.x < n) {
         const long idx = first + threadIdx.x;
         const int mu = (int)(idx / V), s = (int)(idx - (long)mu * V);
@@ -199,18 +203,24 @@ static __global__ void __launch_bounds__(kRecThreads) k_pack_links(int V, int ne
 #pragma unroll
             for (int e = 0; e < 3; e++) st<double>(U + (size_t)(mu * 9 + 6 + e) * V + s, r[e]);
         }
-        if (!su3_errors_fx(m, e_unit, e_det)) su3_errors64(m, e_unit, e_det);
+        if (!su3_errors_fx(m, eu, ed)) {
+            double u64 = 0.0, d64 = 0.0;
+            su3_errors64(m, u64, d64);
+            atomic_max_nonneg(err, sqrt(u64));
+            atomic_max_nonneg(err + 1, sqrt(d64));
+        }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        e_unit = dmax_nan(e_unit, __shfl_down_sync(0xffffffffu, e_unit, o));
-        e_det = dmax_nan(e_det, __shfl_down_sync(0xffffffffu, e_det, o));
-        if (ne == 4) e_form = dmax_nan(e_form, __shfl_down_sync(0xffffffffu, e_form, o));
-    }
+    // non-negative floats order like their bit patterns
+    eu = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(eu)));
+    ed = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ed)));
     if ((threadIdx.x & 31) == 0) {
-        atomic_max_nonneg(err, sqrt(e_unit));
-        atomic_max_nonneg(err + 1, sqrt(e_det));
-        if (ne == 4) atomic_max_nonneg(err + 2, sqrt(e_form));
+        atomic_max_nonneg(err, (double)(sqrtf(eu) * 0x1p-61f));
+        atomic_max_nonneg(err + 1, (double)(sqrtf(ed) * 0x1p-61f));
+    }
+    if (ne == 4) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e_form = dmax_nan(e_form, __shfl_down_sync(0xffffffffu, e_form, o));
+        if ((threadIdx.x & 31) == 0) atomic_max_nonneg(err + 2, sqrt(e_form));
     }
 }
 

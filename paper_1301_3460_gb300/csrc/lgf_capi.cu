@@ -195,21 +195,22 @@ bool use_fxt(const lgf_ctx* c)
 
 // Delta, theta and F of the FP64 loop's links with the forward x,y transform: in
 // FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
-void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist)
+// (h: the loop's condition, for the fixed-point forms to decide about; 0: none)
+void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist, cudaGraphConditionalHandle h = 0)
 {
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
     float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
     const bool f32 = c->accel32 && !c->plain;
     if (use_fxt(c)) {
         launch_fxt_delta(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), as_fx(Fd), c->fxt, c->partials, ctl,
-                         hist);
+                         hist, h);
     } else if (!c->wide) {
         if (f32)
             launch_fx_delta<float>(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), Fd32, c->partials, ctl, hist,
-                                   true);
+                                   true, h);
         else
             launch_fx_delta<double>(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), Fd, c->partials, ctl, hist,
-                                    !c->plain);
+                                    !c->plain, h);
     } else if (f32) {
         launch_delta64_f32(c->lat, c->sh64, s, c->AH64, c->Fs64, Fd32, c->partials, ctl, hist);
     } else {
@@ -270,7 +271,7 @@ void launch_finish64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 
 // one FP64 iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, update,
 // Delta+FFT(x,y)
-void launch_body64(lgf_ctx* c, cudaStream_t s)
+void launch_body64(lgf_ctx* c, cudaStream_t s, cudaGraphConditionalHandle h)
 {
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
     if (!c->plain) {
@@ -282,7 +283,7 @@ void launch_body64(lgf_ctx* c, cudaStream_t s)
         launch_build_g<double>(c->lat, s, Fd, c->g64, c->ctl);
     }
     launch_update64(c, s, c->ctl);
-    launch_delta64(c, s, c->ctl, c->hist);
+    launch_delta64(c, s, c->ctl, c->hist, h);
 }
 
 // one FP32-phase iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, then
@@ -368,15 +369,22 @@ int add_while(cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps, cudaGraph_t
     return LGF_OK;
 }
 
-// FP64 loop: one iteration per body run
+// FP64 loop: two iterations per body run, the Delta kernel of each deciding about the
+// loop (every kernel of the second returns at once when the first ends it): 8^4, 40 us
+// per iteration with one and a control kernel, see launch_body64
 int add_loop64(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps)
 {
     cudaGraph_t body;
     cudaGraphConditionalHandle h;
     CKR(add_while(graph, deps, &body, &h));
     CK(cudaStreamBeginCaptureToGraph(c->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    launch_body64(c, c->cap);
-    launch_loop_ctl(c->cap, c->ctl, h);
+    if (!c->wide) {
+        launch_body64(c, c->cap, h);
+        launch_body64(c, c->cap, h);
+    } else {
+        launch_body64(c, c->cap, 0);
+        launch_loop_ctl(c->cap, c->ctl, h);
+    }
     CK(cudaGetLastError());
     cudaGraph_t out;
     CK(cudaStreamEndCapture(c->cap, &out));
@@ -742,7 +750,7 @@ template <typename T> int time_shape(lgf_ctx* c, const Shape& sh, int which, flo
             if constexpr (sizeof(T) == 8) {
                 if (use_fxt(c)) {
                     launch_fxt_delta(c->lat, sh, s, as_fx(c->AH64), as_fx(c->Fs64), as_fx(reinterpret_cast<double2*>(c->Fd)),
-                                     c->fxt, c->partials, c->ctl_stage, nullptr);
+                                     c->fxt, c->partials, c->ctl_stage, nullptr, 0);
                     launch_fxt_xyinv_g(c->lat, sh, s, as_fx(reinterpret_cast<double2*>(c->Fd)), as_fx(c->g64), c->fxt, c->ctl_stage);
                     continue;
                 }

@@ -167,12 +167,15 @@ template <int LMAX>
 __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delta_fxt(
     Lat d, const longlong2* __restrict__ AH, const fx* __restrict__ Fs, longlong2* __restrict__ Fd,
     const longlong2* __restrict__ tw, int* __restrict__ pexp, FxExp* fe, double* __restrict__ partials, Ctl* ctl,
-    double2* hist)
+    double2* hist, cudaGraphConditionalHandle h)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
     __shared__ unsigned s_or[3];
-    if (ld_flag(&ctl->phase_done)) return;
+    if (ld_flag(&ctl->phase_done)) {
+        end_loop(h);
+        return;
+    }
     if (threadIdx.x < 3) s_or[threadIdx.x] = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2 = kExpNone;
     __syncthreads();
@@ -189,7 +192,7 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delt
         }
     });
     block_or(o, s_or);
-    reduce_theta_F(th, fsum, partials, ctl, hist, V);
+    reduce_theta_F(th, fsum, partials, ctl, hist, V, h);
     longlong2* out = Fd + plane * P;
     int E = -kFxSum;
 #pragma unroll 1

@@ -194,33 +194,52 @@ __device__ __forceinline__ void plane_y_lines(const Lat& d, const vec2_t<T>* src
 
 constexpr int kMaxThreads = 512;  // block size bound of every plane-tiled kernel
 
-__device__ __forceinline__ double block_sum(double v, double* scratch /* kMaxThreads/32 */)
+// sums of two values over the block in a fixed order, valid in thread 0
+__device__ __forceinline__ double2 block_sum2(double2 v, double2* scratch /* kMaxThreads/32 */)
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+    }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __syncthreads();
     if (lane == 0) scratch[w] = v;
     __syncthreads();
-    double r = 0;
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int i = 0; i < nw; i++) r += scratch[i];
+    if (w == 0) {
+        v = lane < (int)(blockDim.x >> 5) ? scratch[lane] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int o = kMaxThreads / 64; o > 0; o >>= 1) {
+            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+        }
     }
-    return r;  // valid in thread 0
+    return v;
+}
+
+// Whether the device loop around this Delta goes on; a hard bound on its runs makes
+// it finite whatever the state says.
+__device__ __forceinline__ bool loop_goes_on(Ctl* ctl, unsigned int bound)
+{
+    const unsigned int n = ctl->body_runs + 1u;
+    ctl->body_runs = n;
+    const unsigned int cap = ctl->loop_bound;
+    return !ld_flag(&ctl->phase_done) && n < bound && n < (unsigned int)ctl->max_iter + 2u && (cap == 0u || n < cap);
 }
 
 // Per-block partial sums of theta and F, then the last block to finish sums
-// the partials in block order (deterministic) and updates the loop state.
-static __device__ void reduce_theta_F(double th, double f, double* __restrict__ partials, Ctl* ctl, double2* hist, int V)
+// the partials in block order (deterministic) and updates the loop state; with the
+// handle h of the loop's condition it also decides whether the loop goes on (a
+// kernel of its own for that costs a launch in every iteration).
+static __device__ void reduce_theta_F(double th, double f, double* __restrict__ partials, Ctl* ctl, double2* hist, int V,
+                                      cudaGraphConditionalHandle h = 0)
 {
-    __shared__ double scratch[kMaxThreads / 32];
+    __shared__ double2 scratch[kMaxThreads / 32];
     __shared__ int am_last;
-    double bt = block_sum(th, scratch);
-    double bf = block_sum(f, scratch);
+    const double2 bs = block_sum2(make_double2(th, f), scratch);
     if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = bt;
-        partials[2 * blockIdx.x + 1] = bf;
+        partials[2 * blockIdx.x] = bs.x;
+        partials[2 * blockIdx.x + 1] = bs.y;
         __threadfence();
         unsigned int tk = atomicAdd(&ctl->ticket, 1u);
         am_last = (tk == gridDim.x - 1);
@@ -228,13 +247,13 @@ static __device__ void reduce_theta_F(double th, double f, double* __restrict__ 
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    double a = 0, b = 0;
+    double2 ab = make_double2(0.0, 0.0);
     for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        a += __ldcg(partials + 2 * i);
-        b += __ldcg(partials + 2 * i + 1);
+        ab.x += __ldcg(partials + 2 * i);
+        ab.y += __ldcg(partials + 2 * i + 1);
     }
-    a = block_sum(a, scratch);
-    b = block_sum(b, scratch);
+    ab = block_sum2(ab, scratch);
+    const double a = ab.x, b = ab.y;
     if (threadIdx.x == 0) {
         // fixed-point links cannot hold the NaN of a g that is not finite
         const double nan = ld_flag(&ctl->bad) ? __hiloint2double(0x7ff80000, 0) : 0.0;
@@ -267,8 +286,18 @@ static __device__ void reduce_theta_F(double th, double f, double* __restrict__ 
             }
         }
         ctl->ticket = 0u;
+        if (h != 0) {
+            const bool go = loop_goes_on(ctl, 0x7fffffffu);
+            if (!go) ctl->phase_done = 1;  // stops the body's second iteration too
+            cudaGraphSetConditional(h, go ? 1u : 0u);
+        }
         __threadfence();
     }
+}
+// a Delta kernel that finds its loop over ends it (a loop runs its body at least once)
+__device__ __forceinline__ void end_loop(cudaGraphConditionalHandle h)
+{
+    if (h != 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
 }
 
 // ---------------------------------------------------------------- link loads
@@ -1098,17 +1127,10 @@ __global__ void __launch_bounds__(256) k_delta_links(Lat d, const vec2_t<T>* __r
 
 // ---------------------------------------------------------------- loop control
 
-// Last node of the while-loop body: keep looping while the running phase has
-// not met its stop condition; a hard bound on body runs makes the loop finite
-// whatever the state says.
+// Last node of a while-loop body whose Delta kernel does not decide about the loop
 static __global__ void k_loop_ctl(Ctl* ctl, cudaGraphConditionalHandle h, unsigned int bound)
 {
-    unsigned int n = ctl->body_runs + 1u;
-    ctl->body_runs = n;
-    const unsigned int cap = ctl->loop_bound;
-    const int cont = !ld_flag(&ctl->phase_done) && n < bound && n < (unsigned int)ctl->max_iter + 2u &&
-                     (cap == 0u || n < cap);
-    cudaGraphSetConditional(h, cont ? 1u : 0u);
+    cudaGraphSetConditional(h, loop_goes_on(ctl, bound) ? 1u : 0u);
 }
 
 }  // namespace lgf

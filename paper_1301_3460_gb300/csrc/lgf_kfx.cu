@@ -63,13 +63,13 @@ static int fxt_threads(int nt, size_t smem, bool lines32)
 }
 
 void launch_fxt_delta(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* AH, const fx* Fs, longlong2* Fd,
-                      const FxtBuf& b, double* partials, Ctl* ctl, double2* hist)
+                      const FxtBuf& b, double* partials, Ctl* ctl, double2* hist, cudaGraphConditionalHandle h)
 {
     const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
     if (small_plane<double>(d))
-        k_delta_fxt<32><<<d.nplanes, fxt_threads(sh.nt_xy, sm, true), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
+        k_delta_fxt<32><<<d.nplanes, fxt_threads(sh.nt_xy, sm, true), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist, h);
     else
-        k_delta_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist);
+        k_delta_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist, h);
 }
 void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl)
 {
@@ -109,23 +109,29 @@ void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const lo
 {
     k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl, always ? 1 : 0);
 }
+// A thread per link while three blocks of 32 sites on every SM hold the lattice twice
+// over.
+constexpr int kUpdSmallV = 32768;
 void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, fx* Fs)
 {
-    k_update_fx<<<blocks(d.V, kUpdThreads), kUpdThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+    if (d.V <= kUpdSmallV)
+        k_update_fx_small<<<blocks(d.V, 32), kUpdSmallThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+    else
+        k_update_fx<<<blocks(d.V, kUpdThreads), kUpdThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
 }
 
 template <typename TF>
 void launch_fx_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const fx* Fs,
-                     vec2_t<TF>* Fd, double* partials, Ctl* ctl, double2* hist, bool fft)
+                     vec2_t<TF>* Fd, double* partials, Ctl* ctl, double2* hist, bool fft, cudaGraphConditionalHandle h)
 {
     const size_t sm = plane_smem_bytes(d, sizeof(vec2_t<TF>));
     if (!fft)
-        k_delta_fx<false, 128, TF><<<d.nplanes, sh64.nt_xy, 0, s>>>(d, AH, Fs, Fd, partials, ctl, hist);
+        k_delta_fx<false, 128, TF><<<d.nplanes, sh64.nt_xy, 0, s>>>(d, AH, Fs, Fd, partials, ctl, hist, h);
     else if (small_plane<double>(d))
-        k_delta_fx<true, 32, TF><<<d.nplanes, sh64.nt_xy, sm, s>>>(d, AH, Fs, Fd, partials, ctl, hist);
+        k_delta_fx<true, 32, TF><<<d.nplanes, sh64.nt_xy, sm, s>>>(d, AH, Fs, Fd, partials, ctl, hist, h);
     else
-        k_delta_fx<true, 128, TF><<<d.nplanes, sh64.nt_xy, sm, s>>>(d, AH, Fs, Fd, partials, ctl, hist);
+        k_delta_fx<true, 128, TF><<<d.nplanes, sh64.nt_xy, sm, s>>>(d, AH, Fs, Fd, partials, ctl, hist, h);
 }
 
 template <typename TF>
@@ -150,9 +156,9 @@ void launch_check_range(const Lat& d, cudaStream_t s, const double2* U64, int* w
 }
 
 template void launch_fx_delta<double>(const Lat&, const Shape&, cudaStream_t, const longlong2*, const fx*, double2*,
-                                      double*, Ctl*, double2*, bool);
+                                      double*, Ctl*, double2*, bool, cudaGraphConditionalHandle);
 template void launch_fx_delta<float>(const Lat&, const Shape&, cudaStream_t, const longlong2*, const fx*, float2*,
-                                     double*, Ctl*, double2*, bool);
+                                     double*, Ctl*, double2*, bool, cudaGraphConditionalHandle);
 template void launch_fx_xyinv_g<double>(const Lat&, const Shape&, cudaStream_t, const double2*, longlong2*,
                                         const Ctl*);
 template void launch_fx_xyinv_g<float>(const Lat&, const Shape&, cudaStream_t, const float2*, longlong2*, const Ctl*);

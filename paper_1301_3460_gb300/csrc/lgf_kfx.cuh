@@ -224,6 +224,63 @@ static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, long
     }
 }
 
+// The same with a thread per link, a warp per direction of 32 sites and a fifth warp for
+// G: for lattices that leave most of the chip idle with a thread per site, whose four
+// links then follow one another (8^4: 14 us a launch against 9).
+constexpr int kUpdSmallThreads = 160;
+static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
+    Lat d, longlong2* __restrict__ U, longlong2* __restrict__ G, const longlong2* __restrict__ g, Ctl* ctl,
+    longlong2* __restrict__ AH, fx* __restrict__ Fs)
+{
+    __shared__ fx retr[4][32];
+    if (ld_flag(&ctl->phase_done)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->iter += 1;
+        if (ctl->phase == 0) ctl->iter_phase0 += 1;
+    }
+    const int V = d.V, mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = blockIdx.x * 32 + lane;
+    if (s < V) {
+        cdig3 gx[6];
+#pragma unroll
+        for (int e = 0; e < 6; e++) gx[e] = with_sum(ldx(g + (size_t)e * V + s));
+        if (mu < 4) {
+            int c[4];
+            site_coords(d, s, c);
+            const int sn = site_shift(d, s, mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3], mu, +1);
+            cfx u[9], w[6], gn[9];
+            longlong2 part[3];
+#pragma unroll
+            for (int e = 0; e < 6; e++) u[e] = ldv<fx>(U + (size_t)(mu * 6 + e) * V + s);
+#pragma unroll
+            for (int k = 0; k < 3; k++) part[k] = AH[(size_t)(mu * 4 + 1 + k) * V + s];
+#pragma unroll
+            for (int e = 0; e < 9; e++) gn[e] = ldx(g + (size_t)e * V + sn);
+            cdig3 A[6];
+            {
+                cdig3 ud[9];
+#pragma unroll
+                for (int e = 0; e < 6; e++) ud[e] = with_sum(u[e]);
+                fx_row2_from_part(u, ud, part, u + 6);
+#pragma unroll
+                for (int e = 6; e < 9; e++) ud[e] = with_sum(u[e]);
+                fx_left(gx, ud, A);
+            }
+            fx_right(A, [&](int e) { return gn[e]; }, w);
+            fx f = 0;
+            fx_store_link(U, AH, V, mu, s, w, f);
+            retr[mu][lane] = f;
+        } else if (G != nullptr) {
+            cfx m[6];
+#pragma unroll
+            for (int e = 0; e < 6; e++) m[e] = ldv<fx>(G + (size_t)e * V + s);
+            fx_gauge_accumulate(G, V, s, gx, m);
+        }
+    }
+    __syncthreads();
+    if (mu == 0 && s < V) Fs[s] = retr[0][lane] + retr[1][lane] + retr[2][lane] + retr[3][lane];
+}
+
 // magnitude exponents of the integer transform's fields (lgf_fxt.cuh)
 constexpr int kExpNone = -(1 << 28);
 struct FxExp {
@@ -396,11 +453,14 @@ __device__ __forceinline__ void fx_delta_plane(const Lat& d, const longlong2* __
 template <bool FFT, int LMAX, typename TF>
 __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double, LMAX>) k_delta_fx(
     Lat d, const longlong2* __restrict__ AH, const fx* __restrict__ Fs, vec2_t<TF>* __restrict__ Fd,
-    double* __restrict__ partials, Ctl* ctl, double2* hist)
+    double* __restrict__ partials, Ctl* ctl, double2* hist, cudaGraphConditionalHandle h)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     vec2_t<TF>* sm = reinterpret_cast<vec2_t<TF>*>(smem_raw);
-    if (ld_flag(&ctl->phase_done)) return;
+    if (ld_flag(&ctl->phase_done)) {
+        end_loop(h);
+        return;
+    }
     const int V = d.V, Lx = d.L[0], s0 = blockIdx.x * d.P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
     double th = 0.0, fsum = 0.0;
@@ -411,7 +471,7 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
             else st<TF>(Fd + (size_t)k * V + s0 + xy, to_tf<TF>(D[k]));
         }
     });
-    reduce_theta_F(th, fsum, partials, ctl, hist, V);
+    reduce_theta_F(th, fsum, partials, ctl, hist, V, h);
     if (FFT) {
         __syncthreads();
         tile_x_lines<TF, false, LMAX>(d, sm);

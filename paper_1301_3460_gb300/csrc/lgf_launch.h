@@ -83,7 +83,8 @@ void launch_xyinv_g32_64(const Lat& d, const Shape& sh32, cudaStream_t s, const 
 // FP64 iterations on 64-bit fixed point (lgf_kfx.cuh): links and G on the grid 2^-61, g
 // on 2^-62, packed parts and Re Tr on 2^-58.  start: from the stored links;
 // project: the end of the FP32 phase (links rebuilt on the input's orbit, phase
-// switched); finish: back to the stored FP64 links.  TF: precision of the transforms.
+// switched); finish: back to the stored FP64 links.  TF: precision of the transforms.  h:
+// condition of the loop that the Delta kernel decides about (0: none).
 struct FxExp;
 // buffers of the integer transform (lgf_fxt.cuh): multipliers and exponents, carved
 // from fxt_bytes(d) of device memory
@@ -112,14 +113,15 @@ void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, 
                       longlong2* AH, long long* Fs);
 template <typename TF>
 void launch_fx_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
-                     vec2_t<TF>* Fd, double* partials, Ctl* ctl, double2* hist, bool fft);
+                     vec2_t<TF>* Fd, double* partials, Ctl* ctl, double2* hist, bool fft, cudaGraphConditionalHandle h);
 template <typename TF>
 void launch_fx_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const vec2_t<TF>* Fd, longlong2* g,
                        const Ctl* ctl);
 // the iteration's transforms on integers: Delta + x,y forward; z,t with the
 // multiplier; x,y inverse + g
 void launch_fxt_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
-                      longlong2* Fd, const FxtBuf& b, double* partials, Ctl* ctl, double2* hist);
+                      longlong2* Fd, const FxtBuf& b, double* partials, Ctl* ctl, double2* hist,
+                      cudaGraphConditionalHandle h);
 void launch_fxt_zt(const Lat& d, const Shape& sh64, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl);
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* Fd, longlong2* g,
                         const FxtBuf& b, const Ctl* ctl);
