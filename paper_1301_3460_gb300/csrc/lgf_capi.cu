@@ -127,7 +127,7 @@ struct lgf_ctx {
     double2* dGp = nullptr;   // [4][9][V] cotangent in / out
     double2* dGud = nullptr;  // [4][9][V]
     double2* dQ = nullptr;    // [4][9][V]
-    double2* dGgs = nullptr;  // [6][V]
+    double2* dGgs = nullptr;  // [4][6][V] (the FP64 kernels use [6][V])
     double2* dFA = nullptr;   // [4][V]
     double2* dFB = nullptr;   // [4][V]
     double2* gl_part = nullptr;
@@ -856,7 +856,7 @@ int ensure_diff(lgf_ctx* c)
     CKR(alloc((void**)&c->dGp, 36 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dGud, 36 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dQ, 36 * Vs * sizeof(double2)));
-    CKR(alloc((void**)&c->dGgs, 6 * Vs * sizeof(double2)));
+    CKR(alloc((void**)&c->dGgs, 24 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dFA, 4 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dFB, 4 * Vs * sizeof(double2)));
     return LGF_OK;
@@ -1674,19 +1674,36 @@ int lgf_step_bwd(lgf_ctx* c, double alpha, const double* gU_out, double* gU_in)
     CKR(reset_stage_ctl(c, alpha));
     cudaStream_t s = c->stream;
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
-    // forward of the step on the stored links, up to g and the spatial Delta~
-    launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
-    launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, Fd, c->partials, c->ctl_stage, nullptr, true);
-    launch_zt<double>(c->lat, c->sh64, c->tb, s, Fd, c->ctl_stage);
-    launch_xy_fft<double>(c->lat, c->sh64, c->tb, s, Fd, true);
-    launch_g_from_dt(s, c->V, Fd, c->g64, alpha);
-    // backward
-    launch_pack_full(s, c->V, gU_out, c->dGp);
-    launch_step_bwd(s, c->lat, c->U64, c->g64, Fd, c->dGp, c->dGud, c->dGgs, c->dQ, alpha, c->dFA, c->dFB);
-    for (double2* F : {c->dFA, c->dFB}) {
-        launch_xy_fft<double>(c->lat, c->sh64, c->tb, s, F, false);
-        launch_zt<double>(c->lat, c->sh64, c->tb, s, F, c->ctl_stage);
-        launch_xy_fft<double>(c->lat, c->sh64, c->tb, s, F, true);
+    // forward of the step on the stored links, up to g and the spatial Delta~, and the
+    // backward up to the accelerator; by the kernels lgf_fix runs, or all in FP64
+    const bool fixed = !c->wide && !c->sh64.zt_tma && fxt_fits(c->lat, c->sh64);
+    if (fixed) {
+        longlong2 *work = as_fx(Fd), *gX = as_fx(c->g64);
+        double2* Dt = c->AH64 + 4 * (size_t)c->V;  // the parts are not read after Delta
+        launch_fx_start(c->lat, s, c->U64, nullptr, c->UX, nullptr, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
+        launch_fxt_delta(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), work, c->fxt, c->partials, c->ctl_stage,
+                         nullptr, 0);
+        launch_fxt_zt(c->lat, c->sh64, s, work, c->fxt, c->ctl_stage);
+        launch_fxt_xyinv_g(c->lat, c->sh64, s, work, gX, c->fxt, c->ctl_stage, Dt);
+        launch_pack_full(s, c->V, gU_out, c->dGp);
+        launch_fx_step_bwd(c->lat, s, c->UX, gX, Dt, c->dGp, c->dGud, c->dGgs, c->dQ, alpha, c->dFA, c->dFB);
+        // six fields: four in dFA, two in dFB
+        CK(fxt_clear_bad(c->fxt, s));
+        launch_fxt_accel(c->lat, c->sh64, s, c->dFA, c->dFA, work, 4, c->fxt, c->ctl_stage);
+        launch_fxt_accel(c->lat, c->sh64, s, c->dFB, c->dFB, work, 2, c->fxt, c->ctl_stage);
+    } else {
+        launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
+        launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, Fd, c->partials, c->ctl_stage, nullptr, true);
+        launch_zt<double>(c->lat, c->sh64, c->tb, s, Fd, c->ctl_stage);
+        launch_xy_fft<double>(c->lat, c->sh64, c->tb, s, Fd, true);
+        launch_g_from_dt(s, c->V, Fd, c->g64, alpha);
+        launch_pack_full(s, c->V, gU_out, c->dGp);
+        launch_step_bwd(s, c->lat, c->U64, c->g64, Fd, c->dGp, c->dGud, c->dGgs, c->dQ, alpha, c->dFA, c->dFB);
+        for (double2* F : {c->dFA, c->dFB}) {
+            launch_xy_fft<double>(c->lat, c->sh64, c->tb, s, F, false);
+            launch_zt<double>(c->lat, c->sh64, c->tb, s, F, c->ctl_stage);
+            launch_xy_fft<double>(c->lat, c->sh64, c->tb, s, F, true);
+        }
     }
     launch_bwd_delta(s, c->lat, c->U64, c->dFA, c->dFB, c->dGud, c->dGp);
     launch_unpack_planes(s, c->V, c->dGp, gU_in);

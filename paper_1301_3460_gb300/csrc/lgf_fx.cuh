@@ -168,6 +168,30 @@ template <int S, typename D> __device__ __forceinline__ cfx fx_row2(const D* r0,
     return fx_det2c<S>(r0[a], r1[b], r0[b], r1[a]);
 }
 
+// the same for any q, through zeros, subnormals and infinity where v 2^-q lies there
+__device__ __forceinline__ double fx2d_safe(fx v, int q)
+{
+    const double y = __ll2double_rn(v);
+    const int hi = __double2hiint(y), e = ((hi >> 20) & 0x7ff) - q;
+    if (v == 0) return 0.0;
+    if (e <= 0 || e >= 0x7ff) return scalbn(y, -q);
+    return __hiloint2double(hi - (q << 20), __double2loint(y));
+}
+
+// x 2^(60-e) of a double |x| < 2^e, rounded toward zero; zero for what is not finite
+__device__ __forceinline__ fx d2fx_rel(double x, int e)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7ffu);
+    const unsigned mh = 0x80000000u | ((hi & 0xfffffu) << 11) | (lo >> 21), ml = lo << 11;
+    const unsigned long long m = ((unsigned long long)mh << 32) | ml;  // 2^(ex-1023) -> 2^63
+    const int r = 1023 + 3 + e - ex;                                   // 2^e -> 2^60
+    unsigned long long v = (r >= 0 && r < 64) ? m >> r : 0ull;
+    if (ex == 0 || ex == 0x7ff) v = 0;
+    const fx s = -(fx)(hi >> 31);
+    return ((fx)v ^ s) - s;
+}
+
 // ---------------------------------------------------------------- Gram-Schmidt
 
 // Rows 0,1 of g = reunit(X), X = 1 + A with A anti-Hermitian, on integers: X comes

@@ -161,40 +161,15 @@ __device__ __forceinline__ void fx_lines(int len, int nlines, const longlong2* _
 
 __device__ __forceinline__ cfx swapped(longlong2 v) { return cfx{v.y, v.x}; }
 
-// Delta (as k_delta_fx), theta and F, then the forward transform along x and y.
-// tw: roots of unity of the four lengths, one after the other.
+// The forward transform along x and y of nf fields of a plane in the tile (values x
+// 2^E0, their bits in s_or[0], zeroed s_or[1..2]) to out; returns the result's exponent,
+// its bits in s_or[2] after the caller's next barrier.
 template <int LMAX>
-__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delta_fxt(
-    Lat d, const longlong2* __restrict__ AH, const fx* __restrict__ Fs, longlong2* __restrict__ Fd,
-    const longlong2* __restrict__ tw, int* __restrict__ pexp, FxExp* fe, double* __restrict__ partials, Ctl* ctl,
-    double2* hist, cudaGraphConditionalHandle h)
+__device__ __forceinline__ int fx_plane_fwd(const Lat& d, longlong2* sm, longlong2* out, const longlong2* __restrict__ tw,
+                                            unsigned* s_or, int E, int nf)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or[3];
-    if (ld_flag(&ctl->phase_done)) {
-        end_loop(h);
-        return;
-    }
-    if (threadIdx.x < 3) s_or[threadIdx.x] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2 = kExpNone;
-    __syncthreads();
-    const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1];
-    const int plane = blockIdx.x;
+    const int V = d.V, Lx = d.L[0], Ly = d.L[1];
     const int rsx = plane_rsx(d), fs = plane_fs(d);
-    double th = 0.0, fsum = 0.0;
-    unsigned o = 0;
-    fx_delta_plane(d, AH, Fs, plane, th, fsum, [&](int xy, int x, int y, const cfx* raw, const cx<double>*) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            or_bits(o, raw[k]);
-            st<fx>(sm + k * fs + y * rsx + x, raw[k]);
-        }
-    });
-    block_or(o, s_or);
-    reduce_theta_F(th, fsum, partials, ctl, hist, V, h);
-    longlong2* out = Fd + plane * P;
-    int E = -kFxSum;
 #pragma unroll 1
     for (int pass = 0; pass < 2; pass++) {
         __syncthreads();
@@ -205,13 +180,13 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delt
         const int l = sh > 0 ? sh : 0;
         const RShift rs = rshift(1 - (sh < 0 ? sh : 0));
         E += rs.r - l;
-        o = 0;
+        unsigned o = 0;
         auto line = [&](int ln) {
             const int f = (int)fdiv((unsigned)ln, pass ? d.dLx : d.dLy), c = ln - f * (pass ? Lx : Ly);
             return sm + f * fs + (pass ? c : c * rsx);
         };
         fx_lines<LMAX, false>(
-            len, pass ? 4 * Lx : 4 * Ly, tw + (pass ? Lx : 0),
+            len, pass ? nf * Lx : nf * Ly, tw + (pass ? Lx : 0),
             [&](int ln) {
                 const longlong2* p = line(ln);
                 return [=](int e) {
@@ -239,6 +214,42 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delt
             });
         block_or(o, s_or + pass + 1);
     }
+    return E;
+}
+
+// Delta (as k_delta_fx), theta and F, then the forward transform along x and y.
+// tw: roots of unity of the four lengths, one after the other.
+template <int LMAX>
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delta_fxt(
+    Lat d, const longlong2* __restrict__ AH, const fx* __restrict__ Fs, longlong2* __restrict__ Fd,
+    const longlong2* __restrict__ tw, int* __restrict__ pexp, FxExp* fe, double* __restrict__ partials, Ctl* ctl,
+    double2* hist, cudaGraphConditionalHandle h)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
+    __shared__ unsigned s_or[3];
+    if (ld_flag(&ctl->phase_done)) {
+        end_loop(h);
+        return;
+    }
+    if (threadIdx.x < 3) s_or[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2 = kExpNone;
+    __syncthreads();
+    const int P = d.P, V = d.V;
+    const int plane = blockIdx.x;
+    const int rsx = plane_rsx(d), fs = plane_fs(d);
+    double th = 0.0, fsum = 0.0;
+    unsigned o = 0;
+    fx_delta_plane(d, AH, Fs, plane, th, fsum, [&](int xy, int x, int y, const cfx* raw, const cx<double>*) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            or_bits(o, raw[k]);
+            st<fx>(sm + k * fs + y * rsx + x, raw[k]);
+        }
+    });
+    block_or(o, s_or);
+    reduce_theta_F(th, fsum, partials, ctl, hist, V, h);
+    const int E = fx_plane_fwd<LMAX>(d, sm, Fd + plane * P, tw, s_or, -kFxSum, 4);
     __syncthreads();
     if (threadIdx.x == 0) {
         pexp[plane] = E;
@@ -420,28 +431,20 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_zt_f
     }
 }
 
-// inverse along y and x, then g = reunit(1 + alpha/2 Delta~) stored in fixed point, by
-// the integer Gram-Schmidt (in FP64 where alpha/2 Delta~ exceeds 16: far beyond any
-// step that converges).  xs: log2 of the pencils' width.
+// The inverse transform along y and x of nf fields of plane p into the tile; returns the
+// exponent, the values' bits in s_or[1] (zeroed s_or[0..1] on entry; barriers inside).
 template <int LMAX>
-__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
-    Lat d, int xs, const longlong2* __restrict__ Fd, longlong2* __restrict__ g, const Ctl* ctl,
-    const longlong2* __restrict__ tw, const int* __restrict__ bexp, FxExp* fe)
+__device__ __forceinline__ int fx_plane_inv(const Lat& d, int xs, const longlong2* __restrict__ Fd, longlong2* sm,
+                                            const longlong2* __restrict__ tw, const int* __restrict__ bexp,
+                                            const FxExp* fe, unsigned* s_or, int plane, int nf)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or[2];
-    if (ld_flag(&ctl->phase_done)) return;
-    if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
-    const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1];
-    const int s0 = blockIdx.x * P;
+    const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1], s0 = plane * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
     const int nxc = Lx >> xs;
     int E = __ldg(&fe->amax2) - fx_bits_rt(Ly) - 1;
     // the plane, aligned to B + 1 bits of the largest pencil
     block_copy<4, longlong2>(
-        4 * P,
+        nf * P,
         [&](int i) {
             const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P;
             return Fd[s0 + f * V + xy];
@@ -465,7 +468,7 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
             return sm + f * fs + (pass ? c * rsx : c);
         };
         fx_lines<LMAX, true>(
-            len, pass ? 4 * Ly : 4 * Lx, tw + (pass ? 0 : Lx),
+            len, pass ? nf * Ly : nf * Lx, tw + (pass ? 0 : Lx),
             [&](int ln) {
                 const longlong2* p = line(ln);
                 return [=](int e) { return apply(rs, swapped(p[e * estr])); };
@@ -489,6 +492,38 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
         block_or(o, s_or + pass);
     }
     __syncthreads();
+    return E;
+}
+
+// inverse along y and x, then g = reunit(1 + alpha/2 Delta~) stored in fixed point, by
+// the integer Gram-Schmidt (in FP64 where alpha/2 Delta~ exceeds 16: far beyond any
+// step that converges).  xs: log2 of the pencils' width.  Dt (may be null) receives
+// Delta~ itself, packed, in FP64.
+template <int LMAX>
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyinv_fxt(
+    Lat d, int xs, const longlong2* __restrict__ Fd, longlong2* __restrict__ g, const Ctl* ctl,
+    const longlong2* __restrict__ tw, const int* __restrict__ bexp, FxExp* fe, double2* __restrict__ Dt)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
+    __shared__ unsigned s_or[2];
+    if (ld_flag(&ctl->phase_done)) return;
+    if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
+    const int P = d.P, V = d.V, Lx = d.L[0];
+    const int s0 = blockIdx.x * P;
+    const int rsx = plane_rsx(d), fs = plane_fs(d);
+    const int E = fx_plane_inv<LMAX>(d, xs, Fd, sm, tw, bexp, fe, s_or, blockIdx.x, 4);
+    if (Dt != nullptr)
+        for (int xy = threadIdx.x; xy < P; xy += blockDim.x) {
+            const int y = (int)fdiv((unsigned)xy, d.dLx), i = y * rsx + (xy - y * Lx);
+#pragma unroll
+            for (int f = 0; f < 4; f++) {
+                const longlong2 v = sm[f * fs + i];
+                const double k = f == 3 ? 2.0 / 3.0 : 1.0;
+                Dt[(size_t)f * V + s0 + xy] = make_double2(fx2d(v.x, -E) * k, fx2d(v.y, -E) * k);
+            }
+        }
     // |alpha/2 Delta~| <= alpha/2 2^(E + top) < 2^(q-1); ha = alpha/2 = hm 2^(he-62) exactly
     const double ha = 0.5 * ctl->alpha;
     const int he = ilogb(ha) + 1;
@@ -550,6 +585,86 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
         X[5] = mk<double>(h * __ll2double_rn(f2.re), h * __ll2double_rn(f2.im));
         gram_schmidt01(X, gm);
         store_g<fx>(g, V, s0 + xy, gm, ctl);
+    }
+}
+
+// ---------------------------------------------------------------- FP64 fields through the transform
+
+// The accelerator on nf packed fields in FP64 that are not a Delta (a cotangent): to
+// integers relative to each plane's largest value and forward along x and y; after
+// k_zt_fxt, back.  A value that is not finite sets *bad, which makes every result NaN,
+// as an FP64 transform would.
+template <int LMAX>
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyfwd_fxt(
+    Lat d, const double2* __restrict__ in, longlong2* __restrict__ Fd, int nf, const longlong2* __restrict__ tw,
+    int* __restrict__ pexp, FxExp* fe)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
+    __shared__ unsigned s_or[3], s_top;
+    if (threadIdx.x < 3) s_or[threadIdx.x] = 0u;
+    if (threadIdx.x == 3) s_top = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2 = kExpNone;
+    __syncthreads();
+    const int P = d.P, Lx = d.L[0], s0 = blockIdx.x * P;
+    const int rsx = plane_rsx(d), fs = plane_fs(d);
+    auto at = [&](int i) {
+        const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P, y = (int)fdiv((unsigned)xy, d.dLx);
+        return f * fs + y * rsx + (xy - y * Lx);
+    };
+    // the doubles into the tile, their largest exponent
+    unsigned top = 0;
+    block_copy<4, double2>(
+        nf * P,
+        [&](int i) {
+            const int f = (int)fdiv((unsigned)i, d.dP);
+            return __ldg(in + (size_t)f * d.V + s0 + (i - f * P));
+        },
+        [&](int i, double2 v) {
+            top = max(top, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+            reinterpret_cast<double2*>(sm)[at(i)] = v;
+        });
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
+    __syncthreads();
+    const int e = (int)(s_top >> 20) - 1022;  // every |x| < 2^e
+    if (e > 1024 && threadIdx.x == 0) fe->bad = 1;
+    // x 2^(60-e) (a value in place of its double: the same thread, the same slot)
+    unsigned o = 0;
+    for (int i = threadIdx.x; i < nf * P; i += blockDim.x) {
+        const double2 v = reinterpret_cast<const double2*>(sm)[at(i)];
+        const cfx w = cfx{d2fx_rel(v.x, e), d2fx_rel(v.y, e)};
+        or_bits(o, w);
+        st<fx>(sm + at(i), w);
+    }
+    block_or(o, s_or);
+    const int E = fx_plane_fwd<LMAX>(d, sm, Fd + s0, tw, s_or, e - 60, nf);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        pexp[blockIdx.x] = E;
+        atomicMax(&fe->amax1, E + align_top(s_or[2], d.L[2]));
+    }
+}
+
+template <int LMAX>
+__global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyback_fxt(
+    Lat d, int xs, const longlong2* __restrict__ Fd, double2* __restrict__ out, int nf, const longlong2* __restrict__ tw,
+    const int* __restrict__ bexp, FxExp* fe)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
+    __shared__ unsigned s_or[2];
+    if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
+    const int P = d.P, Lx = d.L[0], s0 = blockIdx.x * P;
+    const int rsx = plane_rsx(d), fs = plane_fs(d);
+    const int E = fx_plane_inv<LMAX>(d, xs, Fd, sm, tw, bexp, fe, s_or, blockIdx.x, nf);
+    const double nan = __hiloint2double(0x7ff80000, 0);
+    const bool bad = ld_flag(&fe->bad) != 0;
+    for (int i = threadIdx.x; i < nf * P; i += blockDim.x) {
+        const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P, y = (int)fdiv((unsigned)xy, d.dLx);
+        const longlong2 v = sm[f * fs + y * rsx + (xy - y * Lx)];
+        out[(size_t)f * d.V + s0 + xy] = bad ? make_double2(nan, nan) : make_double2(fx2d_safe(v.x, -E), fx2d_safe(v.y, -E));
     }
 }
 

@@ -1,6 +1,6 @@
 // The FP64 iterations on 64-bit fixed point: launchers of lgf_kfx.cuh and the g
 // builders that store a fixed-point g.
-#include "lgf_fxt.cuh"
+#include "lgf_fxdiff.cuh"
 #include "lgf_launch_impl.cuh"
 
 namespace lgf {
@@ -29,6 +29,10 @@ cudaError_t fx_prepare(const Lat& d)
     if ((e = allow_max_smem(k_zt_fxt<32>, optin))) return e;
     if ((e = allow_max_smem(k_zt_fxt<128>, optin))) return e;
     if ((e = allow_max_smem(k_xyinv_fxt<32>, optin))) return e;
+    if ((e = allow_max_smem(k_xyfwd_fxt<32>, optin))) return e;
+    if ((e = allow_max_smem(k_xyfwd_fxt<128>, optin))) return e;
+    if ((e = allow_max_smem(k_xyback_fxt<32>, optin))) return e;
+    if ((e = allow_max_smem(k_xyback_fxt<128>, optin))) return e;
     return allow_max_smem(k_xyinv_fxt<128>, optin);
 }
 
@@ -71,25 +75,25 @@ void launch_fxt_delta(const Lat& d, const Shape& sh, cudaStream_t s, const longl
     else
         k_delta_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist, h);
 }
-void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl)
+void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl, int nf)
 {
     const size_t sm = fxt_pencil_smem(d, sh.xw);
-    const dim3 grid(d.L[0] / sh.xw, d.L[1], 4);
+    const dim3 grid(d.L[0] / sh.xw, d.L[1], nf);
     if (short_zt_lines(d))
         k_zt_fxt<32><<<grid, fxt_threads(sh.nt_zt, sm, true), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
     else
         k_zt_fxt<128><<<grid, fxt_threads(sh.nt_zt, sm, false), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
 }
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* Fd, longlong2* g,
-                        const FxtBuf& b, const Ctl* ctl)
+                        const FxtBuf& b, const Ctl* ctl, double2* Dt)
 {
     const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
     int xs = 0;
     while ((1 << xs) < sh.xw) xs++;
     if (small_plane<double>(d))
-        k_xyinv_fxt<32><<<d.nplanes, fxt_threads(sh.nt_xy, sm, true), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
+        k_xyinv_fxt<32><<<d.nplanes, fxt_threads(sh.nt_xy, sm, true), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe, Dt);
     else
-        k_xyinv_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe);
+        k_xyinv_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe, Dt);
 }
 
 void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
@@ -109,6 +113,33 @@ void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const lo
 {
     k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl, always ? 1 : 0);
 }
+void launch_fxt_accel(const Lat& d, const Shape& sh, cudaStream_t s, const double2* in, double2* out, longlong2* work,
+                      int nf, const FxtBuf& b, const Ctl* ctl)
+{
+    const size_t sm = plane_smem_bytes(d, sizeof(longlong2));
+    int xs = 0;
+    while ((1 << xs) < sh.xw) xs++;
+    const bool small = small_plane<double>(d);
+    const int nt = fxt_threads(sh.nt_xy, sm, small);
+    if (small)
+        k_xyfwd_fxt<32><<<d.nplanes, nt, sm, s>>>(d, in, work, nf, b.tw, b.pexp, b.fe);
+    else
+        k_xyfwd_fxt<128><<<d.nplanes, nt, sm, s>>>(d, in, work, nf, b.tw, b.pexp, b.fe);
+    launch_fxt_zt(d, sh, s, work, b, ctl, nf);
+    if (small)
+        k_xyback_fxt<32><<<d.nplanes, nt, sm, s>>>(d, xs, work, out, nf, b.tw, b.bexp, b.fe);
+    else
+        k_xyback_fxt<128><<<d.nplanes, nt, sm, s>>>(d, xs, work, out, nf, b.tw, b.bexp, b.fe);
+}
+cudaError_t fxt_clear_bad(const FxtBuf& b, cudaStream_t s) { return cudaMemsetAsync(&b.fe->bad, 0, sizeof(int), s); }
+
+void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* g, const double2* Fdt,
+                        const double2* Gp, double2* Gud, double2* Ggm, double2* Q, double alpha, double2* FA, double2* FB)
+{
+    k_bwd_update_fx<<<dim3(blocks(d.V, 128), 4), 128, 0, s>>>(d, U, g, Gp, Gud, Ggm, Q);
+    k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Ggm, 4, Q, alpha, FA, FB);
+}
+
 // A thread per link while three blocks of 32 sites on every SM hold the lattice twice
 // over.
 constexpr int kUpdSmallV = 32768;

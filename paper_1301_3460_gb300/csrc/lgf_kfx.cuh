@@ -286,6 +286,8 @@ constexpr int kExpNone = -(1 << 28);
 struct FxExp {
     int amax1;  // over the planes, after the Delta kernel (reset at the start of a loop and by the g builder)
     int amax2;  // over the pencils, after the accelerator (reset by the Delta kernel)
+    int bad;    // a field of FP64 values was not finite (k_xyfwd_fxt; reset before it)
+    int pad;
 };
 
 // Start of a loop: the links' rows 0,1 (and G's) on the grid, rounded to nearest, with

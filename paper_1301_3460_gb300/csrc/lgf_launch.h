@@ -122,9 +122,18 @@ void launch_fx_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const vec2
 void launch_fxt_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
                       longlong2* Fd, const FxtBuf& b, double* partials, Ctl* ctl, double2* hist,
                       cudaGraphConditionalHandle h);
-void launch_fxt_zt(const Lat& d, const Shape& sh64, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl);
+void launch_fxt_zt(const Lat& d, const Shape& sh64, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl,
+                   int nf = 4);
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* Fd, longlong2* g,
-                        const FxtBuf& b, const Ctl* ctl);
+                        const FxtBuf& b, const Ctl* ctl, double2* Dt = nullptr);
+// the accelerator on nf packed FP64 fields (any values: a cotangent), in -> out, through
+// the integer fields work; fxt_clear_bad before the first of several
+cudaError_t fxt_clear_bad(const FxtBuf& b, cudaStream_t s);
+void launch_fxt_accel(const Lat& d, const Shape& sh64, cudaStream_t s, const double2* in, double2* out, longlong2* work,
+                      int nf, const FxtBuf& b, const Ctl* ctl);
+// k_bwd_update on fixed point and the Gram-Schmidt's derivative; Ggm: [4][6][V]
+void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* g, const double2* Fdt,
+                        const double2* Gp, double2* Gud, double2* Ggm, double2* Q, double alpha, double2* FA, double2* FB);
 void launch_fx_build_g(const Lat& d, cudaStream_t s, const double2* Fd, longlong2* g, const Ctl* ctl);
 // *wide set when a stored link is not within 1e-3 of SU(3)
 void launch_check_range(const Lat& d, cudaStream_t s, const double2* U64, int* wide);
