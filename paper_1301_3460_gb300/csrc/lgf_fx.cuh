@@ -290,6 +290,37 @@ __device__ __forceinline__ void fx_gram_schmidt(const cfx* X, int q, cfx* r, cdi
     }
 }
 
+// x 2^(61-q) of a float |x| < 2^(q-1), toward zero
+__device__ __forceinline__ fx f2fx(float x, int q)
+{
+    const unsigned u = __float_as_uint(x);
+    const int e = (int)((u >> 23) & 0xffu), r = e - 89 - q;  // 24-bit mantissa times 2^(e-150)
+    const fx m = e ? (fx)((u & 0x7fffffu) | 0x800000u) : 0;
+    const fx v = r >= 0 ? m << r : m >> (r < -63 ? 63 : -r);
+    const fx s = -(fx)(u >> 31);
+    return (v ^ s) - s;
+}
+// The float nearest to v 2^-62.  *safe is cleared when a value within tol (x 2^62) of v
+// may round to another float: v lies that close to the midpoint of two floats.
+__device__ __forceinline__ float g2f(fx v, unsigned long long tol, bool* safe)
+{
+    const fx s = v >> 63;
+    unsigned long long a = (unsigned long long)((v ^ s) - s);
+    const int lz = __clzll((long long)a);
+    if (lz > 40) {  // zero, or too few bits to tell
+        *safe = false;
+        return 0.f;
+    }
+    a <<= lz;
+    // 24 leading bits kept, 40 dropped; distance of the dropped part from one half
+    const long long d = (long long)(a & ((1ull << 40) - 1)) - (1ll << 39);
+    const unsigned long long t = tol << lz;
+    if ((unsigned long long)(d < 0 ? -d : d) <= t || (t >> lz) != tol) *safe = false;
+    const unsigned m = (unsigned)(a >> 40) + (d > 0 ? 1u : 0u);  // 2^23 <= m <= 2^24
+    const float f = (float)m * __int_as_float((127 - 22 - lz) << 23);
+    return s ? -f : f;
+}
+
 __device__ __forceinline__ cfx ldx(const longlong2* p)
 {
     const longlong2 v = __ldg(p);
