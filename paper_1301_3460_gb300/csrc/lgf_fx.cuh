@@ -169,12 +169,14 @@ template <int S, typename D> __device__ __forceinline__ cfx fx_row2(const D* r0,
 }
 
 // the same for any q, through zeros, subnormals and infinity where v 2^-q lies there
+// (out of line: inlined, its FP64 operations are issued for every value)
+static __device__ __noinline__ double fx2d_far(fx v, int q) { return scalbn(__ll2double_rn(v), -q); }
 __device__ __forceinline__ double fx2d_safe(fx v, int q)
 {
     const double y = __ll2double_rn(v);
     const int hi = __double2hiint(y), e = ((hi >> 20) & 0x7ff) - q;
     if (v == 0) return 0.0;
-    if (e <= 0 || e >= 0x7ff) return scalbn(y, -q);
+    if (e <= 0 || e >= 0x7ff) return fx2d_far(v, q);
     return __hiloint2double(hi - (q << 20), __double2loint(y));
 }
 

@@ -47,7 +47,8 @@ template <int S> __device__ __forceinline__ cfx fx_dag2(cdig3 a0, cdig3 b0, cdig
 // g x 2^62 of the forward pass.  Writes the direct cotangent of U (Gud), the link's
 // parts of G_g(x) (Ggm, rows 0,1) and of G_g(x+mu) (Q), in FP64.  32^4: 4.00 ms in FP64
 // (2000 operations per site at 2 per clock and SM).
-static __global__ void __launch_bounds__(128, 3) k_bwd_update_fx(Lat d, const longlong2* __restrict__ U,
+template <int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2* __restrict__ U,
                                                                  const longlong2* __restrict__ g,
                                                                  const double2* __restrict__ Gp,
                                                                  double2* __restrict__ Gud, double2* __restrict__ Ggm,

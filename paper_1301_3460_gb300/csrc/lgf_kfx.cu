@@ -136,7 +136,7 @@ cudaError_t fxt_clear_bad(const FxtBuf& b, cudaStream_t s) { return cudaMemsetAs
 void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* g, const double2* Fdt,
                         const double2* Gp, double2* Gud, double2* Ggm, double2* Q, double alpha, double2* FA, double2* FB)
 {
-    k_bwd_update_fx<<<dim3(blocks(d.V, 128), 4), 128, 0, s>>>(d, U, g, Gp, Gud, Ggm, Q);
+    k_bwd_update_fx<128, 3><<<dim3(blocks(d.V, 128), 4), 128, 0, s>>>(d, U, g, Gp, Gud, Ggm, Q);
     k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Ggm, 4, Q, alpha, FA, FB);
 }
 

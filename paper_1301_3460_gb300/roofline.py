@@ -5,7 +5,8 @@ Per lattice site and per launch, counting each unique array element once
 multiplies/adds (an FMA is 2), with the FFT at the conventional 5 N log2 N per
 complex transform of length N.
 
-FP64 path, per site (V sites per launch):
+FP64 iterations, per site (V sites per launch; 64-bit fixed point moves the same bytes
+as FP64 would, and the flops are those of the FP64 formulas):
   delta_xyfft   reads the packed anti-Hermitian parts of the four links (4 x 4
                 complex) and their Re Tr sum, writes the four packed Delta
                 fields: 256 + 8 + 64 B.  Flops: Delta as 16 complex differences
@@ -16,8 +17,10 @@ FP64 path, per site (V sites per launch):
                 (2 x 4 x 5 log2(Lz Lt)) + scale (8).
   xyifft_g      reads the 4 fields, writes g (full 3x3): 64 + 144 B.  Flops:
                 inverse x,y FFT (4 x 5 log2(Lx Ly)) + Gram-Schmidt and row 2 (134).
-  update        reads links, g, G; writes links, G, the packed anti-Hermitian
-                parts and Re Tr: 384 + 144 + 96 + 384 + 96 + 256 + 8 B.  Flops:
+  update        reads links, three entries of each packed part (row 2 of the links),
+                g, G; writes links, G, the packed anti-Hermitian
+                parts and Re Tr: 384 + 192 + 144 + 96 + 384 + 96 + 256 + 8 B (FP32: row 2
+                is rebuilt, no parts read).  Flops:
                 per link row-2 rebuild (42), two 2x3 by 3x3 complex products
                 (2 x 132), row 2 of the result (42), packing (12), Re Tr (2);
                 G: rebuild (42) + one product (132).
@@ -49,7 +52,8 @@ complex multiplies, 18 complex adds) and 216 when accumulated into a sum:
   total                                                         3514
 The sampler's transcendental functions (heat bath) are not counted.  Bytes: a
 launch reads about the whole link field (7/8 of it) and writes V/2 links, far
-below what the FP64 pipe takes to do the arithmetic: the kernel is ALU-bound.
+below what the arithmetic takes (integer products, lgf_wilson.cu): the kernel is
+ALU-bound.
 """
 from __future__ import annotations
 
@@ -77,14 +81,14 @@ def per_site(dims, precision: int = 64, fused32: bool = False, accel32: bool = F
             "delta_xyfft": dict(bytes=256 + 8 + 32, flops=64 + 21 + 4 * 5 * lxy),
             "zt_fft_accel": dict(bytes=32 + 32, flops=2 * 4 * 5 * lzt + 8),
             "xyifft_g": dict(bytes=32 + 144, flops=4 * 5 * lxy + 134),
-            "update": dict(bytes=384 + 144 + 96 + 384 + 96 + 256 + 8,
+            "update": dict(bytes=384 + 192 + 144 + 96 + 384 + 96 + 256 + 8,
                            flops=4 * (42 + 2 * 132 + 42 + 12 + 2) + 42 + 132),
         }
     return {
         "delta_xyfft": dict(bytes=(256 + 8 + 64) * w, flops=64 + 21 + 4 * 5 * lxy),
         "zt_fft_accel": dict(bytes=(64 + 64) * w + (8 if precision == 64 else 0), flops=2 * 4 * 5 * lzt + 8),
         "xyifft_g": dict(bytes=(64 + 144) * w, flops=4 * 5 * lxy + 134),
-        "update": dict(bytes=(384 + 144 + 96 + 384 + 96 + 256 + 8) * w,
+        "update": dict(bytes=(384 + (192 if precision == 64 else 0) + 144 + 96 + 384 + 96 + 256 + 8) * w,
                        flops=4 * (42 + 2 * 132 + 42 + 12 + 2) + 42 + 132),
     }
 
