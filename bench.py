@@ -211,6 +211,14 @@ def traffic_record(kernel, dims, precision):
     return float(v) if v is not None else None
 
 
+def hbm_peak_gbs():
+    """Copy bandwidth of the GPU (GB/s) and where the figure is from."""
+    try:
+        return float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"]), "measured copy"
+    except (OSError, ValueError, KeyError):
+        return 6800.0, "earlier measurement of a copy on a GB300"
+
+
 # ---------------------------------------------------------------- arms
 
 def run_reference(args, dims):
@@ -732,10 +740,7 @@ def run_ours(args, dims):
     traffic = traffic_record(kern, dims, 64)
     # The FP64 iterations run on 64-bit integers, so the FP64 pipe bounds nothing; the
     # kernels' bound is HBM (measured copy rate where the record exists).
-    try:
-        hbm_peak, hbm_src = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"]), "measured copy"
-    except (OSError, ValueError, KeyError):
-        hbm_peak, hbm_src = 6800.0, "earlier measurement of a copy on a GB300"
+    hbm_peak, hbm_src = hbm_peak_gbs()
     roof = {"bound": "hbm", "kernel": kern, "achieved": byts / sec / 1e9, "peak": hbm_peak, "unit": "GB/s",
             "frac": byts / sec / 1e9 / hbm_peak, "traffic": traffic, "peak_source": hbm_src,
             "flops_gflops": flops / sec / 1e9, "fp64_peak_gflops": FP64_PEAK_GFLOPS}
@@ -748,7 +753,7 @@ def run_ours(args, dims):
     kernels["fp64_iteration_ms"] = sum(ms.values())
     # the metric's "% of HBM peak": algorithmic bytes of one whole FP64 iteration at the measured rate
     try:
-        hbm = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"])
+        hbm = hbm_peak_gbs()[0]
         it_bytes = roofline.per_iteration(dims, 64)["bytes"]
         hbm_iter = {"bytes_per_iteration": it_bytes, "achieved_gbs": it_bytes * value / 1e9, "peak_gbs": hbm,
                     "frac": it_bytes * value / 1e9 / hbm,
@@ -1094,7 +1099,7 @@ def run_kernels(args, dims):
     from paper_1301_3460_gb300 import inputs, lgf, roofline
 
     V = int(np.prod(dims))
-    hbm = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"])
+    hbm = hbm_peak_gbs()[0]
     U = inputs.rough_gauge_field_cuda(dims, 0.3, 77)
     out = {"metric": "iteration kernels, median ms per launch", "dims": list(dims), "autotuned": not args.no_autotune}
     with lgf.Lattice(dims, mixed=True) as lat:

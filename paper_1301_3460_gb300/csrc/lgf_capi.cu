@@ -837,7 +837,11 @@ int autotune_ctx(lgf_ctx* c)
 {
     if (!c->have_links) return LGF_ERR_STATE;
     CKR(reset_stage_ctl(c, 0.08));
-    launch_start64(c, c->stream);
+    // the inputs of the Delta kernel that is timed: fixed-point parts, or FP64 ones
+    if (use_fxt(c))
+        launch_start64(c, c->stream);
+    else
+        launch_ah_init<double>(c->lat, c->stream, c->U64, c->AH64, c->Fs64);
     CKR(autotune_prec<double>(c));
     if (c->mixed) {
         launch_mixed_prep(c->stream, c->V, c->lat.ne, c->U64, c->U32, c->G32, c->ctl_stage);
