@@ -163,7 +163,7 @@ __device__ __forceinline__ bool su3_errors_fx(const cx<double>* m, float& e_unit
 // check of the full input matrix: err[0] = max |U U^dag - 1|, err[1] = max |det U - 1|,
 // err[2] = max error of the round trip through the 8-real form (ne = 4).
 // 32^4: 1.60 ms with the check in FP64 and a thread per record in global memory (its
-// FP64 work alone is 1 ms).
+// FP64 work alone is 1 ms), 0.31 ms like this.
 static __global__ void __launch_bounds__(kRecThreads) k_pack_links(int V, int ne, const double* __restrict__ in,
                                                                    double2* __restrict__ U, unsigned long long* err)
 {

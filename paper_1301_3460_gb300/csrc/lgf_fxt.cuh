@@ -9,7 +9,12 @@
 // points): 80 registers and 24 warps per SM, and 3 to 5 thousand instructions per
 // kernel.  Whole 32-point lines in registers, as the FP64 kernels have them, take 168
 // registers and 12,000 unrolled instructions in the z,t kernel and wait for
-// instruction fetches (32^4: 178/220/215 us against the figures at the kernels).
+// instruction fetches.  32^4, Delta + x,y / z,t / x,y inverse + g: 372 / 426 / 379 us in
+// FP64 (bound by the FP64 pipe), 178 / 220 / 215 us with whole integer lines, 136 / 124
+// / 106 us like this (the last with the integer Gram-Schmidt, 174 us without).  What
+// is left (ncu): Delta waits for its 32 loads per site (33% of the warps, issue 30%),
+// z,t issues 44% of the time with 16 warps per SM (its tile and multipliers), the g
+// builder 53%.
 // In place, frequency k of a line lands on position (k mod A) B + k / A; the fields
 // stay in that order between the kernels, the multiplier table is laid out in it,
 // and the inverse (B-point, twiddles, A-point) takes it back.  An inverse runs the

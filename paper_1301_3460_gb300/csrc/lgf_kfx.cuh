@@ -130,8 +130,10 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // wait out the loads.  Each direction's inputs are therefore copied to slots in shared
 // memory of the thread's own (no barrier) one direction ahead: the link and its part as
 // soon as the current ones are in registers, g(x+mu) as soon as it has been used; g(x)
-// waits in shared memory too.  32^4, with G: 447 us with loads where they are used (455
-// with G in FP64), 323 us like this; without G 357 and 281 us.
+// waits in shared memory too.  32^4, with G: 1630 us in FP64 (924 operations per site at
+// 2 per clock and SM), 406 us on integers with loads where they are used, 315 us like
+// this (77% of the HBM rate); without G 357 and 281 us.  G in FP64 beside the integer
+// products is slower (441 against 406 us): it comes at the end of every thread.
 constexpr int kUpdThreads = 128;
 static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, longlong2* __restrict__ U,
                                                                      longlong2* __restrict__ G,
