@@ -58,12 +58,14 @@ typedef enum {
 } lgf_status;
 
 /* creation flags */
-#define LGF_FP64 0        /* every step in FP64 */
+#define LGF_FP64 0        /* every step at FP64 accuracy or better (64-bit fixed point inside the loop,
+                             FP64 links, G, theta and F at the boundary) */
 #define LGF_MIXED 1       /* FP32 Delta/FFT/update until theta < switch_tol, then FP64 (see lgf_set_switch_tol) */
 #define LGF_NO_GAUGE 2    /* do not accumulate G (lgf_get_gauge then fails); FP64 mode only */
 #define LGF_LINKS18 8     /* keep row 2 of each FP64 link in memory (18 reals) instead of rebuilding it on
                              every load (12 reals): the same values (row 2 is stored as the rebuild from
-                             rows 0,1), 50% more link bytes, fewer FP64 operations per update */
+                             rows 0,1), 50% more link bytes.  A running fix keeps its own form of the
+                             links, so these two flags cost or save only where links are read or stored */
 #define LGF_LINKS8 16     /* keep each FP64 link in its 8-real form (u01, u02, u10 and the phases of u00 and
                              u20; the rest rebuilt from unitarity and det = 1 on every load): a third of the
                              12-real bytes, two sqrt, two sincos and a division more per load, two atan2 per
@@ -297,7 +299,7 @@ int lgf_get_shape(lgf_ctx* ctx, int precision, int* shape_out);
  * independent FMA chains of n_iter steps per thread over 8 blocks of 256 threads
  * per SM, timed with CUDA events after a short warm-up launch; *gflops counts
  * an FMA as two flops, *ms (may be NULL) is the launch time.  The FP64 rate is
- * the arithmetic ceiling of the FP64 iteration kernels.  Allocates a small
+ * the arithmetic ceiling of kernels that compute in FP64.  Allocates a small
  * output buffer; blocks until done.
  */
 int lgf_probe_fma(int precision, int n_iter, double* gflops, double* ms);
@@ -481,9 +483,10 @@ int lgf_plaquette(lgf_ctx* ctx, double* P);
  * sweeps keep current, uniforms from the top 24 bits of the same Philox words);
  * the links stay FP64 in memory, rows 0,1 of each re-orthonormalised in FP64
  * after its update.  A chain of its own, with the Wilson action's equilibrium up
- * to FP32 rounding, about 15x faster on GB300, where FP64 arithmetic runs at 1/64
- * of the FP32 rate (32^4: 1.30 against 19.6 ms per heat-bath sweep; the copy
- * takes 4 V x 48 bytes of device memory); the FP64 generator is the one that
+ * to FP32 rounding, 4 to 7x faster on GB300 (32^4: 1.30 against 8.8 ms per
+ * heat-bath sweep, 0.99 against 3.8 ms per overrelaxation sweep; the copy takes
+ * 4 V x 48 bytes of device memory, the fixed-point links of the FP64 generator
+ * 4 V x 144); the FP64 generator is the one that
  * matches the reference to rounding.
  */
 int lgf_set_generator_precision(lgf_ctx* ctx, int bits);

