@@ -532,8 +532,10 @@ __device__ __forceinline__ bool fx_subgroup(cfx wii, cfx wij, cfx wji, cfx wjj, 
 
 // Of W only what the later subgroups read is rotated (seven entries), of the link
 // rows 0,1 and, for the second subgroup, row 2.  Sweeps at 32^4: overrelaxation 14.4 ms
-// in FP64, 3.8 ms like this (integer products); heat bath 19.6 and 8.8 ms (the FP64
-// sampler is most of it).
+// in FP64, 3.8 ms like this (integer products); heat bath 19.6 and 8.8 ms (what it
+// takes beyond the overrelaxation is the sampler).  Attempts are not what costs there:
+// passing over those that FP32 rules out, and one direction per warp after the loop,
+// left the sweep at 8.3 ms under the profiler, as without.
 template <int MODE>
 __global__ void __launch_bounds__(kWilsonThreads, 3) k_wilson_fx(Lat d, longlong2* __restrict__ U, int mu, int parity,
                                                               double beta, uint32_t k0, uint32_t k1, uint32_t sweep)
