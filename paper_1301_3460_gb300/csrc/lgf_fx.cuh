@@ -302,6 +302,15 @@ __device__ __forceinline__ fx f2fx(float x, int q)
     const fx s = -(fx)(u >> 31);
     return (v ^ s) - s;
 }
+// How far (x 2^62) an entry v of g may lie from the FP64 code's: the integer rows' error,
+// about 2^-53, and 2^-46 of the entry or of the largest |alpha/2 Delta~| of the site (mx, x
+// 2^(61-q)), eight times the FP64 code's bound.  The second is shifted down from where it
+// stands: x 2^62 it does not fit a word from 2 on.
+__host__ __device__ __forceinline__ unsigned long long g2f_tol(fx v, fx mx, int q)
+{
+    const fx a = (v < 0 ? -v : v) >> 46, b = mx >> (45 - q);
+    return (unsigned long long)((1ll << (8 + q)) + (a > b ? a : b));
+}
 // The float nearest to v 2^-62.  *safe is cleared when a value within tol (x 2^62) of v
 // may round to another float: v lies that close to the midpoint of two floats.
 __device__ __forceinline__ float g2f(fx v, unsigned long long tol, bool* safe)
@@ -321,6 +330,34 @@ __device__ __forceinline__ float g2f(fx v, unsigned long long tol, bool* safe)
     const unsigned m = (unsigned)(a >> 40) + (d > 0 ? 1u : 0u);  // 2^23 <= m <= 2^24
     const float f = (float)m * __int_as_float((127 - 22 - lz) << 23);
     return s ? -f : f;
+}
+
+// Rows 0,1 of g x 2^62 (r, digits rd) of FP32 fields alpha/2 Delta~ (packed as the
+// transforms have them) of at most mx < 16 in magnitude; returns q.
+__device__ __forceinline__ int fx_rows_of(float2 f0, float2 f1, float2 f2, float2 f3, float mx, cfx* r, cdig* rd)
+{
+    const int q = max(1, (int)(__float_as_uint(mx) >> 23) - 125);  // |v| < 2^(q-1)
+    const fx one = 1ll << (61 - q);
+    cfx X[6];
+    X[0] = cfx{one, f2fx(f3.x, q)};
+    X[1] = cfx{f2fx(f0.x, q), f2fx(f0.y, q)};
+    X[2] = cfx{f2fx(f1.x, q), f2fx(f1.y, q)};
+    X[3] = cfx{-X[1].re, X[1].im};  // -conj(Delta01)
+    X[4] = cfx{one, f2fx(f3.y, q)};
+    X[5] = cfx{f2fx(f2.x, q), f2fx(f2.y, q)};
+    fx_gram_schmidt(X, q, r, rd);
+    return q;
+}
+// The rows as the floats that the FP64 Gram-Schmidt of the same fields rounds to; false
+// where that cannot be told.
+__device__ __forceinline__ bool fx_rows_to_float(const cfx* r, float mx, int q, cx<float>* gs)
+{
+    bool safe = true;
+    const fx m = f2fx(mx, q);
+#pragma unroll
+    for (int e = 0; e < 6; e++)
+        gs[e] = cx<float>{g2f(r[e].re, g2f_tol(r[e].re, m, q), &safe), g2f(r[e].im, g2f_tol(r[e].im, m, q), &safe)};
+    return safe;
 }
 
 __device__ __forceinline__ cfx ldx(const longlong2* p)

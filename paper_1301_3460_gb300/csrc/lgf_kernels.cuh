@@ -742,26 +742,17 @@ __device__ __forceinline__ void xyinv_g_plane(const Lat& d, const vec2_t<T>* __r
             // builder: 137 us against 68).  An FP32 g has to be the FP64 result rounded, bit
             // for bit (one other bit sends the FP32 phase to other roundings everywhere and
             // to links turned by another 1e-8): the integer rows decide where no float
-            // midpoint lies within both errors, about 2^-53 of one for the integers and
-            // 2^-46 of the row's scale, eight times the FP64 code's bound, else the site
-            // is done in FP64, as are fields so small that this would be the rule.
+            // midpoint lies within both errors (g2f_tol), else the site is done in FP64, as
+            // are fields so small that this would be the rule.
             float sum = 0.f, mx = 0.f;
             for (float v : {f0.x, f0.y, f1.x, f1.y, f2.x, f2.y, f3.x, f3.y}) {
                 sum += fabsf(v);
                 mx = fmaxf(mx, fabsf(v));
             }
             if (sum < 16.f && (std::is_same_v<TG, fx> || mx > 0x1p-18f)) {  // false for NaN
-                const int q = max(1, (int)(__float_as_uint(mx) >> 23) - 125);  // |v| < 2^(q-1)
-                const fx one = 1ll << (61 - q);
-                cfx Xi[6], r[6];
+                cfx r[6];
                 cdig rd[6];
-                Xi[0] = cfx{one, f2fx(f3.x, q)};
-                Xi[1] = cfx{f2fx(f0.x, q), f2fx(f0.y, q)};
-                Xi[2] = cfx{f2fx(f1.x, q), f2fx(f1.y, q)};
-                Xi[3] = cfx{-Xi[1].re, Xi[1].im};
-                Xi[4] = cfx{one, f2fx(f3.y, q)};
-                Xi[5] = cfx{f2fx(f2.x, q), f2fx(f2.y, q)};
-                fx_gram_schmidt(Xi, q, r, rd);
+                const int q = fx_rows_of(f0, f1, f2, f3, mx, r, rd);
                 if constexpr (std::is_same_v<TG, fx>) {
 #pragma unroll
                     for (int e = 0; e < 6; e++) stx(g + (size_t)e * V + s0 + xy, r[e]);
@@ -769,15 +760,8 @@ __device__ __forceinline__ void xyinv_g_plane(const Lat& d, const vec2_t<T>* __r
                     for (int j = 0; j < 3; j++) stx(g + (size_t)(6 + j) * V + s0 + xy, fx_row2<2>(rd, rd + 3, j));
                     continue;
                 } else {
-                    bool safe = true;
-                    const fx mxi = f2fx(mx, q) << (q + 1);
-                    auto tof = [&](fx v) {
-                        return g2f(v, (unsigned long long)((1ll << (8 + q)) + (max(v < 0 ? -v : v, mxi) >> 46)), &safe);
-                    };
                     cx<TG> gs[9];
-#pragma unroll
-                    for (int e = 0; e < 6; e++) gs[e] = mk<TG>(tof(r[e].re), tof(r[e].im));
-                    if (safe) {
+                    if (fx_rows_to_float(r, mx, q, gs)) {
                         complete_row2(gs, gs + 6);
 #pragma unroll
                         for (int e = 0; e < 9; e++) st<TG>(g + (size_t)e * V + s0 + xy, gs[e]);
