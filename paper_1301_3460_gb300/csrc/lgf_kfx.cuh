@@ -485,7 +485,9 @@ __global__ void __launch_bounds__(kTileMaxThreads<double>, kTileMinBlocks<double
 }
 
 // Whether every stored link is within 1e-3 of SU(3) (rows 0,1 orthonormal): the
-// range the fixed-point products are bounded for.  *wide counts the others.
+// range the fixed-point products are bounded for.  A stored row 2 (18-real form) has to be
+// the product of rows 0,1 to rounding as well (2^-50; its own error in FP64 is below
+// 2^-51): the loop keeps rows 0,1 only.  *wide is set by any other link.
 static __global__ void k_check_range(Lat d, const double2* __restrict__ U64, int* wide)
 {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -500,7 +502,20 @@ static __global__ void k_check_range(Lat d, const double2* __restrict__ U64, int
     cx<float> ip = cmulc(r[3], r[0]);
     ip = cmacc(ip, r[4], r[1]);
     ip = cmacc(ip, r[5], r[2]);
-    const bool ok = fabsf(n0 - 1.f) < 1e-3f && fabsf(n1 - 1.f) < 1e-3f && norm2(ip) < 1e-6f;
+    bool ok = fabsf(n0 - 1.f) < 1e-3f && fabsf(n1 - 1.f) < 1e-3f && norm2(ip) < 1e-6f;
+    if (d.ne == 9 && ok) {
+        bool bad = false;
+        cdig rd[6];
+#pragma unroll
+        for (int e = 0; e < 6; e++) rd[e] = digits(cfx{d2fx<kFxBits>(u[e].re, &bad), d2fx<kFxBits>(u[e].im, &bad)});
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            ok = ok && fabs(u[6 + j].re) < 2.0 && fabs(u[6 + j].im) < 2.0;  // false for NaN
+            const cfx t = cfx{d2fx<kFxBits>(u[6 + j].re, &bad), d2fx<kFxBits>(u[6 + j].im, &bad)};
+            const cfx e = t - fx_row2<3>(rd, rd + 3, j);
+            ok = ok && llabs(e.re) <= 1ll << (kFxBits - 50) && llabs(e.im) <= 1ll << (kFxBits - 50);
+        }
+    }
     if (!ok) *wide = 1;
 }
 

@@ -135,7 +135,7 @@ void launch_fxt_accel(const Lat& d, const Shape& sh64, cudaStream_t s, const dou
 void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* g, const double2* Fdt,
                         const double2* Gp, double2* Gud, double2* Ggm, double2* Q, double alpha, double2* FA, double2* FB);
 void launch_fx_build_g(const Lat& d, cudaStream_t s, const double2* Fd, longlong2* g, const Ctl* ctl);
-// *wide set when a stored link is not within 1e-3 of SU(3)
+// *wide set when a stored link is not within 1e-3 of SU(3), or its stored row 2 not rows 0,1's
 void launch_check_range(const Lat& d, cudaStream_t s, const double2* U64, int* wide);
 
 // conversion, checking and mode-switch kernels (FP64 unit)

@@ -1,0 +1,46 @@
+"""What decides between the fixed-point and the FP64 kernels, and that neither answers for
+links that are not its own: snapshots with a row 2 of their own, links that stopped being
+finite, plain descent under the instrumentation, links that the generator has rewritten."""
+import numpy as np
+import pytest
+
+from paper_1301_3460_gb300 import inputs, lgf
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def dag(m):
+    return np.conj(np.swapaxes(m, -1, -2))
+
+
+def one_step(lat, L, alpha=0.08):
+    """rows 0,1 of the links after a step made of the FP64 stages"""
+    W = lat.get_links()
+    D, _, _ = lat.delta()
+    g = lat.build_g(lat.accelerate(D), alpha)
+    return np.stack([g @ W[mu] @ dag(g[inputs.neighbour(L, mu)]) for mu in range(4)])[..., :2, :]
+
+
+def test_snapshot_of_18_reals_keeps_its_row_2():
+    """Row 2 of an 18-real snapshot is read as it stands, also where rows 0,1 are SU(3)'s
+    and it is not their product.  1e-13: the parity tests' bound after a step."""
+    L = (8, 4, 6, 4)
+    V = int(np.prod(L))
+    U = inputs.rough_gauge_field(L, 0.4, 71)
+    with lgf.Lattice(L, links18=True) as lat:
+        lat.set_links(U)
+        snap = lat.save_links()
+        lat.fix(tol=0.0, max_iter=3)
+        want = lat.get_links()
+        lat.load_links(snap)  # a row 2 that is the product: the same kernels as after set_links
+        lat.fix(tol=0.0, max_iter=3)
+        assert np.array_equal(lat.get_links(), want)
+        for err in (1e-6, 1e-12):
+            odd = snap.clone().view(torch.float64).reshape(4, 9, V, 2)
+            odd[:, 6:] *= 1 + err
+            lat.load_links(odd.reshape(-1).view(torch.uint8))
+            assert np.max(np.abs(lat.get_links()[..., 2, :] - U[..., 2, :])) > err / 4
+            want2 = one_step(lat, L)
+            lat.fix(tol=0.0, max_iter=1)
+            assert np.max(np.abs(lat.get_links()[..., :2, :] - want2)) < 1e-13
