@@ -1447,7 +1447,9 @@ int lgf_time_kernels(lgf_ctx* c, double alpha, int n_iter, int precision, double
     if (rc != LGF_OK) return rc;
     if (precision == 64) {
         launch_finish64(c, s, c->ctl_stage);
+        CK(cudaMemcpyAsync(&c->host_ctl->bad, &c->ctl_stage->bad, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        if (c->host_ctl->bad) c->wide = true;  // the stored links are NaN now
     }
     CK(cudaGetLastError());
     // median over the iterations: a launch delayed by the host (the events bracket

@@ -44,3 +44,16 @@ def test_snapshot_of_18_reals_keeps_its_row_2():
             want2 = one_step(lat, L)
             lat.fix(tol=0.0, max_iter=1)
             assert np.max(np.abs(lat.get_links()[..., :2, :] - want2)) < 1e-13
+
+
+def test_links_lost_under_the_instrumentation_stay_lost():
+    """Kernels timed with a step that is not finite leave NaN links; a later fix says so."""
+    L = (4, 6, 4, 4)
+    U = inputs.rough_gauge_field(L, 0.3, 72)
+    with lgf.Lattice(L) as lat:
+        lat.set_links(U)
+        lat.time_kernels(alpha=float("inf"), n_iter=1)
+        assert np.isnan(lat.get_links()).any()
+        assert lat.fix(check=False)["status"] == lgf.LGF_ERR_NAN
+        lat.set_links(U)
+        assert lat.fix(max_iter=2000)["converged"]
