@@ -193,10 +193,10 @@ bool use_fxt(const lgf_ctx* c)
     return !c->wide && !c->plain && !c->accel32 && !c->sh64.zt_tma && fxt_fits(c->lat, c->sh64);
 }
 
-// Delta, theta and F of the FP64 loop's links with the forward x,y transform: in
-// FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
+// Delta, theta and F of the FP64 loop's links, with the forward x,y transform when
+// fft: in FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
 // (h: the loop's condition, for the fixed-point forms to decide about; 0: none)
-void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist, cudaGraphConditionalHandle h = 0)
+void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist, bool fft, cudaGraphConditionalHandle h = 0)
 {
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
     float2* Fd32 = reinterpret_cast<float2*>(c->Fd);
@@ -210,11 +210,11 @@ void launch_delta64(lgf_ctx* c, cudaStream_t s, Ctl* ctl, double2* hist, cudaGra
                                    true, h);
         else
             launch_fx_delta<double>(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), Fd, c->partials, ctl, hist,
-                                    !c->plain, h);
+                                    fft, h);
     } else if (f32) {
         launch_delta64_f32(c->lat, c->sh64, s, c->AH64, c->Fs64, Fd32, c->partials, ctl, hist);
     } else {
-        launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, Fd, c->partials, ctl, hist, !c->plain);
+        launch_delta<double>(c->lat, c->sh64, c->tb, s, c->AH64, c->Fs64, Fd, c->partials, ctl, hist, fft);
     }
 }
 
@@ -283,7 +283,7 @@ void launch_body64(lgf_ctx* c, cudaStream_t s, cudaGraphConditionalHandle h)
         launch_build_g<double>(c->lat, s, Fd, c->g64, c->ctl);
     }
     launch_update64(c, s, c->ctl);
-    launch_delta64(c, s, c->ctl, c->hist, h);
+    launch_delta64(c, s, c->ctl, c->hist, !c->plain, h);
 }
 
 // one FP32-phase iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, then
@@ -433,7 +433,7 @@ int append_fix(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps
         CKR(capture_begin(c, graph, deps));
         launch_start64(c, c->cap);
     }
-    launch_delta64(c, c->cap, c->ctl, c->hist);
+    launch_delta64(c, c->cap, c->ctl, c->hist, !c->plain);
     CKR(capture_end(c, deps));
     CKR(add_loop64(c, graph, deps));
     CKR(capture_begin(c, graph, deps));
@@ -1396,8 +1396,9 @@ int lgf_time_kernels(lgf_ctx* c, double alpha, int n_iter, int precision, double
     for (int it = 0; it < n_iter && rc == LGF_OK; it++) {
         cudaEventRecord(ev[0], s);
         if (precision == 64) {
-            // the kernels lgf_fix runs (the accelerator in FP32 when so set)
-            launch_delta64(c, s, c->ctl_stage, nullptr);
+            // the kernels lgf_fix runs (the accelerator in FP32 when so set), with the
+            // accelerator in plain contexts too
+            launch_delta64(c, s, c->ctl_stage, nullptr, true);
             cudaEventRecord(ev[1], s);
             launch_zt64(c, s, c->ctl_stage);
             cudaEventRecord(ev[2], s);

@@ -57,3 +57,18 @@ def test_links_lost_under_the_instrumentation_stay_lost():
         assert lat.fix(check=False)["status"] == lgf.LGF_ERR_NAN
         lat.set_links(U)
         assert lat.fix(max_iter=2000)["converged"]
+
+
+def test_kernels_timed_in_a_plain_context_are_the_accelerated_iteration():
+    """Instrumentation of a context without Fourier acceleration runs the four kernels it
+    names: the links move by an accelerated step."""
+    L = (6, 8, 4, 6)
+    U = inputs.rough_gauge_field(L, 0.3, 73)
+    with lgf.Lattice(L) as lat:
+        lat.set_links(U)
+        lat.fix(tol=0.0, max_iter=2)
+        want = lat.get_links()
+    with lgf.Lattice(L, accelerate=False) as lat:
+        lat.set_links(U)
+        lat.time_kernels(n_iter=2)
+        assert np.max(np.abs(lat.get_links() - want)) < 1e-13
