@@ -854,6 +854,21 @@ int autotune_ctx(lgf_ctx* c)
     return LGF_OK;
 }
 
+// Whether the stored links are outside the fixed-point range, by looking at them (waits
+// for the stream)
+int find_wide(lgf_ctx* c)
+{
+    int* wide = reinterpret_cast<int*>(c->err);
+    CK(cudaMemsetAsync(wide, 0, sizeof(int), c->stream));
+    launch_check_range(c->lat, c->stream, c->U64, wide);
+    CK(cudaGetLastError());
+    int h = 0;
+    CK(cudaMemcpyAsync(&h, wide, sizeof h, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    c->wide = h != 0;
+    return LGF_OK;
+}
+
 int ensure_diff(lgf_ctx* c)
 {
     if (c->dGp) return LGF_OK;
@@ -1192,16 +1207,8 @@ int lgf_load_links(lgf_ctx* c, const void* src)
 {
     if (!c || !src) return LGF_ERR_ARG;
     CK(cudaMemcpyAsync(c->U64, src, lgf_links_state_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
-    // a snapshot is not checked: whether its links are in the fixed-point range
-    int* wide = reinterpret_cast<int*>(c->err);
-    CK(cudaMemsetAsync(wide, 0, sizeof(int), c->stream));
-    launch_check_range(c->lat, c->stream, c->U64, wide);
     if (c->track) launch_identity_rows64(c->stream, c->V, c->G64);
-    CK(cudaGetLastError());
-    int h = 0;
-    CK(cudaMemcpyAsync(&h, wide, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    c->wide = h != 0;
+    CKR(find_wide(c));  // a snapshot is not checked
     c->have_links = true;
     return LGF_OK;
 }
@@ -1800,6 +1807,8 @@ int lgf_wilson_sweeps(lgf_ctx* c, double beta, unsigned long long seed, int firs
     if (fixed) launch_links_from_fx(c->stream, c->lat, c->genx, c->U64);
     if (c->track) launch_identity_rows64(c->stream, c->V, c->G64);
     CK(cudaGetLastError());
+    // a sweep rewrites every link into SU(3), whatever it was (unless it was not finite)
+    if (c->wide && n_heatbath + n_overrelax > 0) return find_wide(c);
     CK(cudaStreamSynchronize(c->stream));
     return LGF_OK;
 }

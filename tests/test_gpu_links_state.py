@@ -72,3 +72,25 @@ def test_kernels_timed_in_a_plain_context_are_the_accelerated_iteration():
         lat.set_links(U)
         lat.time_kernels(n_iter=2)
         assert np.max(np.abs(lat.get_links() - want)) < 1e-13
+
+
+@pytest.mark.parametrize("bits", [64, 32])
+def test_rewritten_links_take_the_fixed_point_kernels(bits):
+    """Sweeps rewrite every link into SU(3), so what follows them runs as after set_links,
+    bit for bit, also when the chain started from a snapshot of other matrices."""
+    L = (4, 6, 4, 8)
+    U = inputs.rough_gauge_field(L, 0.4, 74)
+    with lgf.Lattice(L) as lat, lgf.Lattice(L) as ref:
+        lat.set_generator_precision(bits)
+        lat.set_links(U)
+        lat.load_links((lat.save_links().view(torch.float64) * 1.5).view(torch.uint8))
+        lat.wilson_sweeps(6.0, 5, n_heatbath=1, n_overrelax=1)
+        ref.set_links(lat.get_links())
+        lat.fix(tol=0.0, max_iter=3)
+        ref.fix(tol=0.0, max_iter=3)
+        assert np.array_equal(lat.get_links(), ref.get_links())
+        # a chain that begins with links out of range is the FP64 generator's
+        lat.set_links(U)
+        lat.load_links((lat.save_links().view(torch.float64) * 1.5).view(torch.uint8))
+        lat.wilson_sweeps(6.0, 5, n_heatbath=0, n_overrelax=0)
+        assert np.max(np.abs(lat.get_links()[..., :2, :] - 1.5 * U[..., :2, :])) < 1e-14
