@@ -267,7 +267,9 @@ int lgf_time_kernels(lgf_ctx* ctx, double alpha, int n_iter, int precision, doub
  * sizes of the plane and pencil kernels, x-columns per z,t pencil and the z,t
  * kernel's form, see lgf_set_shape) for this lattice by
  * timing the candidates on the stored links; both precisions of a mixed
- * context.  The choice is cached for the process by extents and precision.
+ * context.  The choice is cached for the process by extents, precision and the
+ * kernels that the context's FP64 iterations run (integer transforms; FP32
+ * accelerator; FP64 transforms).  The integer transforms have one z,t form.
  * Needs lgf_set_links first (LGF_ERR_STATE otherwise).  Changes no result
  * beyond rounding.
  */
@@ -287,6 +289,7 @@ int lgf_autotune(lgf_ctx* ctx);
  * lgf_set_shape returns LGF_ERR_ARG for a shape the kernels cannot run
  * (including a form-1 shape whose buffers exceed shared memory); it waits for the
  * context's stream and replaces the captured loop.  lgf_autotune overwrites it.
+ * zt_form 1 in precision 64 takes the FP64 loop's transforms from integers to FP64.
  * lgf_get_shape writes {nt_xy, nt_zt, xw, zt_form, grid of form 1} to shape_out[5].
  * Every shape gives the same results up to rounding.
  */

@@ -82,6 +82,7 @@ struct lgf_ctx {
     Lat lat{};    // FP64 kernels (links with ne = 6 or 9 entries)
     Lat lat32{};  // FP32 kernels (always 6: rows 0,1)
     Shape sh64{}, sh32{};
+    bool zt_tma_asked = false;  // the FP64 z,t kernel's TMA form was asked for (lgf_set_shape)
     Tables tb{};
     // state
     double2* U64 = nullptr;
@@ -186,12 +187,12 @@ template <> const Shape& shape_of<float>(const lgf_ctx* c) { return c->sh32; }
 longlong2* as_fx(double2* p) { return reinterpret_cast<longlong2*>(p); }
 long long* as_fx(double* p) { return reinterpret_cast<long long*>(p); }
 
-// whether the FP64 loop's transforms run on integers: the default form (the
-// TMA-staged z,t kernel and the FP32 accelerator have their own)
-bool use_fxt(const lgf_ctx* c)
-{
-    return !c->wide && !c->plain && !c->accel32 && !c->sh64.zt_tma && fxt_fits(c->lat, c->sh64);
-}
+// whether FP64 transforms of the stored links' fields run on integers: the default form.
+// A caller may ask for the TMA-staged z,t kernel, which is FP64; that the autotuner once
+// preferred it for links out of the fixed-point range is no such wish.
+bool fxt_allowed(const lgf_ctx* c) { return !c->wide && !c->zt_tma_asked && fxt_fits(c->lat, c->sh64); }
+// the same for the FP64 loop (the FP32 accelerator and plain descent have their own kernels)
+bool use_fxt(const lgf_ctx* c) { return !c->plain && !c->accel32 && fxt_allowed(c); }
 
 // Delta, theta and F of the FP64 loop's links, with the forward x,y transform when
 // fft: in FP64, or in FP32 into the front half of Fd when the accelerator runs in FP32
@@ -720,11 +721,25 @@ int stage_fault(lgf_ctx* c)
 
 // ---------------------------------------------------------------- autotuner
 
-// Launch shapes of the plane-tiled kernels are chosen per lattice shape and
-// precision by timing the candidates on the context's own data; the choice is
-// kept for the process, so contexts of equal extents are tuned once.
+// Launch shapes of the plane-tiled kernels are chosen per lattice shape, precision
+// and kernel family by timing the candidates on the context's own data; the choice
+// is kept for the process, so contexts of equal extents that run the same kernels are
+// tuned once.
 std::mutex g_tune_mutex;
-std::map<std::array<int, 5>, Shape> g_tuned;
+std::map<std::array<int, 6>, Shape> g_tuned;
+
+// The kernels that an FP64 shape is for.  The integer transforms have one z,t form: the
+// TMA form of the FP64 transforms is not timed against it, because it would take Delta and
+// the g builder off the integers too (32^4: 1.4 against 0.68 ms per iteration).
+enum TuneFamily {
+    kTuneFx = 0,       // integer transforms
+    kTuneAccel32 = 1,  // Delta with FP32 transforms; z,t and g take the FP32 shape
+    kTuneFp64 = 2      // FP64 transforms: links out of the fixed-point range, plain descent
+};
+TuneFamily tune_family(const lgf_ctx* c)
+{
+    return c->wide || c->plain ? kTuneFp64 : c->accel32 ? kTuneAccel32 : kTuneFx;
+}
 
 template <typename T> Shape& shape_ref(lgf_ctx* c);
 template <> Shape& shape_ref<double>(lgf_ctx* c) { return c->sh64; }
@@ -749,7 +764,13 @@ template <typename T> int time_shape(lgf_ctx* c, const Shape& sh, int which, flo
             // the plane kernels of the precision's iteration: FP64 Delta + FFT(x,y) and
             // IFFT(x,y) + g; FP32 FFT(x,y) and IFFT(x,y) + g
             if constexpr (sizeof(T) == 8) {
-                if (use_fxt(c)) {
+                const TuneFamily fam = tune_family(c);
+                if (fam == kTuneAccel32) {
+                    launch_fx_delta<float>(c->lat, sh, s, as_fx(c->AH64), as_fx(c->Fs64), reinterpret_cast<float2*>(c->Fd),
+                                           c->partials, c->ctl_stage, nullptr, true, 0);
+                    continue;
+                }
+                if (fam == kTuneFx) {
                     launch_fxt_delta(c->lat, sh, s, as_fx(c->AH64), as_fx(c->Fs64), as_fx(reinterpret_cast<double2*>(c->Fd)),
                                      c->fxt, c->partials, c->ctl_stage, nullptr, 0);
                     launch_fxt_xyinv_g(c->lat, sh, s, as_fx(reinterpret_cast<double2*>(c->Fd)), as_fx(c->g64), c->fxt, c->ctl_stage);
@@ -765,7 +786,7 @@ template <typename T> int time_shape(lgf_ctx* c, const Shape& sh, int which, flo
             launch_xyinv_g<T>(lat_of<T>(c), sh, c->tb, s, Fd, g_of<T>(c), c->ctl_stage);
         } else {
             if constexpr (sizeof(T) == 8) {
-                if (use_fxt(c) && !sh.zt_tma && fxt_fits(c->lat, sh)) {
+                if (tune_family(c) == kTuneFx) {
                     launch_fxt_zt(c->lat, sh, s, as_fx(reinterpret_cast<double2*>(c->Fd)), c->fxt, c->ctl_stage);
                     continue;
                 }
@@ -791,7 +812,8 @@ template <typename T> int time_shape(lgf_ctx* c, const Shape& sh, int which, flo
 template <typename T> int autotune_prec(lgf_ctx* c)
 {
     const size_t elem = sizeof(vec2_t<T>);
-    std::array<int, 5> key = {c->L[0], c->L[1], c->L[2], c->L[3], (int)elem};
+    const TuneFamily fam = sizeof(T) == 8 ? tune_family(c) : kTuneFp64;
+    std::array<int, 6> key = {c->L[0], c->L[1], c->L[2], c->L[3], (int)elem, (int)fam};
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tuned.find(key);
@@ -801,6 +823,7 @@ template <typename T> int autotune_prec(lgf_ctx* c)
         }
     }
     Shape best = shape_ref<T>(c);
+    if (fam != kTuneFp64) best.zt_tma = best.zt_grid = 0;
     float best_xy = 1e30f, best_zt = 1e30f;
     const int nts[3] = {64, 128, 256};
     for (int nt : nts) {
@@ -813,11 +836,13 @@ template <typename T> int autotune_prec(lgf_ctx* c)
             best.nt_xy = cand.nt_xy;
         }
     }
-    for (int form = 0; form <= 1; form++)
+    const int forms = fam == kTuneFp64 ? 2 : fam == kTuneFx ? 1 : 0;
+    for (int form = 0; form < forms; form++)
         for (int nt : nts)
             for (int xw = 1; xw <= 16; xw <<= 1) {
                 Shape cand;
                 if (!make_shape(lat_of<T>(c), elem, best.nt_xy, nt, xw, &cand, form)) continue;
+                if (fam == kTuneFx && !fxt_fits(c->lat, cand)) continue;
                 float ms;
                 CKR(time_shape<T>(c, cand, 1, &ms));
                 if (ms < best_zt) {
@@ -839,11 +864,12 @@ int autotune_ctx(lgf_ctx* c)
     if (!c->have_links) return LGF_ERR_STATE;
     CKR(reset_stage_ctl(c, 0.08));
     // the inputs of the Delta kernel that is timed: fixed-point parts, or FP64 ones
-    if (use_fxt(c))
+    if (tune_family(c) != kTuneFp64)
         launch_start64(c, c->stream);
     else
         launch_ah_init<double>(c->lat, c->stream, c->U64, c->AH64, c->Fs64);
     CKR(autotune_prec<double>(c));
+    c->zt_tma_asked = false;
     if (c->mixed) {
         launch_mixed_prep(c->stream, c->V, c->lat.ne, c->U64, c->U32, c->G32, c->ctl_stage);
         launch_start32(c, c->stream, c->ctl_stage, nullptr);
@@ -1488,6 +1514,7 @@ int lgf_set_shape(lgf_ctx* c, int precision, int nt_xy, int nt_zt, int xw, int z
     if (!ok) return LGF_ERR_ARG;
     CK(cudaStreamSynchronize(c->stream));
     (precision == 64 ? c->sh64 : c->sh32) = sh;
+    if (precision == 64) c->zt_tma_asked = zt_form == 1;
     drop_graph(c);
     return LGF_OK;
 }
@@ -1576,7 +1603,10 @@ int lgf_batch_set_fp32_update(lgf_batch* b, int form)
 int lgf_batch_set_accel_precision(lgf_batch* b, int precision)
 {
     if (!b) return LGF_ERR_ARG;
-    for (lgf_ctx* c : b->ctx) CKR(lgf_set_accel_precision(c, precision));
+    for (lgf_ctx* c : b->ctx) {
+        if (c->accel32 != (precision == 32)) b->tuned = false;  // other kernels: shapes of their own
+        CKR(lgf_set_accel_precision(c, precision));
+    }
     CK(cudaStreamSynchronize(b->stream));
     if (b->exec) cudaGraphExecDestroy(b->exec);
     b->exec = nullptr;
@@ -1691,7 +1721,7 @@ int lgf_step_bwd(lgf_ctx* c, double alpha, const double* gU_out, double* gU_in)
     double2* Fd = reinterpret_cast<double2*>(c->Fd);
     // forward of the step on the stored links, up to g and the spatial Delta~, and the
     // backward up to the accelerator; by the kernels lgf_fix runs, or all in FP64
-    const bool fixed = !c->wide && !c->sh64.zt_tma && fxt_fits(c->lat, c->sh64);
+    const bool fixed = fxt_allowed(c);
     if (fixed) {
         longlong2 *work = as_fx(Fd), *gX = as_fx(c->g64);
         double2* Dt = c->AH64 + 4 * (size_t)c->V;  // the parts are not read after Delta
