@@ -360,6 +360,18 @@ __device__ __forceinline__ bool fx_rows_to_float(const cfx* r, float mx, int q, 
     return safe;
 }
 
+// v x 2^62, |v| <= 1, rounded to the nearest double (ties to even), x 2^61: at most 53
+// significant bits and none below 2^-61, so that the FP64 value is exact
+__device__ __forceinline__ fx fx_round_double(fx v)
+{
+    const fx s = v >> 63;
+    unsigned long long a = (unsigned long long)((v ^ s) - s);
+    const int n = max(1, 11 - __clzll((long long)a));  // bits to drop
+    a += (1ull << (n - 1)) - 1 + ((a >> n) & 1);
+    a = (a >> n) << (n - 1);
+    return ((fx)a ^ s) - s;
+}
+
 __device__ __forceinline__ cfx ldx(const longlong2* p)
 {
     const longlong2 v = __ldg(p);

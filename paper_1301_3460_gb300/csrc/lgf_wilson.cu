@@ -599,8 +599,10 @@ __global__ void __launch_bounds__(kWilsonThreads, 3) k_wilson_fx(Lat d, longlong
 #pragma unroll
         for (int j = 0; j < 3; j++) u[3 + j] = fx_rot0<3>(R, with_sum(u[3 + j]), with_sum(u[6 + j]));
     }
-    // rows 0,1 orthonormalised, rounded to the grid 2^-53 (exact in FP64, so that a chain
-    // does not depend on how it is split into calls), row 2 rebuilt
+    // rows 0,1 orthonormalised, rounded to the nearest double (exact in FP64, so that a
+    // chain does not depend on how it is split into calls), row 2 rebuilt.  Measured rms of
+    // <row 0, row 1>: 3.3e-17 for rough links, 1.4e-17 near 1; with every entry on the grid
+    // 2^-53 both are 6.4e-17.
     cfx X[6], o[6];
     cdig od[6];
 #pragma unroll
@@ -608,7 +610,7 @@ __global__ void __launch_bounds__(kWilsonThreads, 3) k_wilson_fx(Lat d, longlong
     fx_gram_schmidt(X, 1, o, od);
 #pragma unroll
     for (int e = 0; e < 6; e++) {
-        o[e] = cfx{((o[e].re + 256) >> 9) << 8, ((o[e].im + 256) >> 9) << 8};
+        o[e] = cfx{fx_round_double(o[e].re), fx_round_double(o[e].im)};
         od[e] = digits(o[e]);
         stx(U + (size_t)(mu * 9 + e) * V + s, o[e]);
     }

@@ -1,0 +1,30 @@
+"""Precision that the fixed-point kernels keep where values of different size meet."""
+import numpy as np
+import pytest
+
+from paper_1301_3460_gb300 import inputs, lgf
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def test_generated_links_are_rounded_to_the_nearest_double():
+    """A generated link is an SU(3) matrix rounded to doubles.  Per row the rounding errors are
+    half a unit of each entry's own last place: <row 0, row 1> of rough links is below 4.4e-17 rms
+    (6.4e-17 with every entry on the grid 2^-53), and an entry of 2^-8 to 2^-4 lies on a
+    multiple of 2^-53 with a chance of 1/8 at most."""
+    L = (8, 8, 8, 8)
+    with lgf.Lattice(L, track_gauge=False) as lat:
+        lat.set_links(inputs.rough_gauge_field(L, 0.4, 81))
+        lat.wilson_sweeps(6.0, 3, n_heatbath=1, n_overrelax=1)
+        U = lat.get_links()
+    r = U[..., :2, :]
+    x = np.stack((r.real, r.imag)).ravel()
+    x = x[(np.abs(x) > 2.0 ** -8) & (np.abs(x) < 2.0 ** -4)]
+    assert x.size > 1000
+    assert np.mean(x * 2.0 ** 53 % 1 == 0) < 0.15
+    w = r.astype(np.clongdouble)
+    ip = (w[..., 0, :].conj() * w[..., 1, :]).sum(-1)
+    assert float(np.sqrt(np.mean(np.abs(ip) ** 2))) < 5e-17
+    norm = (np.abs(w) ** 2).sum(-1) - 1
+    assert float(np.sqrt(np.mean(norm ** 2))) < 1e-16
