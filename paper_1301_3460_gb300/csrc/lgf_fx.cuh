@@ -366,9 +366,9 @@ __device__ __forceinline__ fx fx_round_double(fx v)
 {
     const fx s = v >> 63;
     unsigned long long a = (unsigned long long)((v ^ s) - s);
-    const int n = max(1, 11 - __clzll((long long)a));  // bits to drop
-    a += (1ull << (n - 1)) - 1 + ((a >> n) & 1);
-    a = (a >> n) << (n - 1);
+    const int n = max(1, 11 - __clz((int)(a >> 32)));  // bits to drop, all in the low word
+    a += (1u << (n - 1)) - 1u + (((unsigned)a >> n) & 1u);
+    a = (a & ~(unsigned long long)((1u << n) - 1u)) >> 1;
     return ((fx)a ^ s) - s;
 }
 
