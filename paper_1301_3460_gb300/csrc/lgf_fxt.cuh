@@ -32,6 +32,10 @@
 // the integer times 2^E; E is kept per xy-plane after the Delta kernel (pexp), per
 // z,t pencil after the accelerator (bexp), and the consumer aligns them to the
 // largest magnitude exponent of all planes (FxExp::amax1) or pencils (amax2).
+// The fields of a Delta share their exponents (the first of each array): they end in one g
+// on one grid, 2^-62, which is what a small field is known to there in any case.  The
+// fields of a cotangent keep exponents of their own (OWN), as FP64 keeps their scales:
+// colour components need not be of one size, and each ends in a gradient by itself.
 // Field 3 stays at 3/2 of its value (lgf_kfx.cuh) through the transform.
 #pragma once
 #include "lgf_kfx.cuh"
@@ -65,6 +69,12 @@ __device__ __forceinline__ void block_or(unsigned o, unsigned* s)
 {
     o = __reduce_or_sync(0xffffffffu, o);
     if ((threadIdx.x & 31) == 0 && o) atomicOr(s, o);
+}
+
+// OR into shared memory; the bits of most values are there after the first few
+__device__ __forceinline__ void or_into(unsigned* s, unsigned b)
+{
+    if (b & ~*reinterpret_cast<volatile unsigned*>(s)) atomicOr(s, b);
 }
 
 // Right shift by r >= 1, rounded to nearest, ties away from zero: a tie rule that
@@ -166,37 +176,49 @@ __device__ __forceinline__ void fx_lines(int len, int nlines, const longlong2* _
 
 __device__ __forceinline__ cfx swapped(longlong2 v) { return cfx{v.y, v.x}; }
 
-// The forward transform along x and y of nf fields of a plane in the tile (values x
-// 2^E0, their bits in s_or[0], zeroed s_or[1..2]) to out; returns the result's exponent,
-// its bits in s_or[2] after the caller's next barrier.
-template <int LMAX>
-__device__ __forceinline__ int fx_plane_fwd(const Lat& d, longlong2* sm, longlong2* out, const longlong2* __restrict__ tw,
-                                            unsigned* s_or, int E, int nf)
+// The shifts that bring values with the magnitude bits o to B + 1 bits before a shift by
+// one (Delta shrinks by orders of magnitude over a fix: a left shift in the first pass):
+// left by l, then right by r.
+struct FwdShift {
+    int l, r;
+};
+__device__ __forceinline__ FwdShift fwd_shift(unsigned o, int len)
+{
+    const int sh = fx_bits_rt(len) + 1 - top_bits(o);
+    return FwdShift{sh > 0 ? sh : 0, sh < 0 ? 1 - sh : 1};
+}
+
+// The forward transform along x and y of nf fields of a plane in the tile to out.  s_or:
+// [3][4] (a column per field, or the first for all): the values' bits before in the first
+// row, zeros in the others; the results' bits in the last after the caller's next barrier.
+template <int LMAX, bool OWN>
+__device__ __forceinline__ void fx_plane_fwd(const Lat& d, longlong2* sm, longlong2* out, const longlong2* __restrict__ tw,
+                                             unsigned* s_or, int nf)
 {
     const int V = d.V, Lx = d.L[0], Ly = d.L[1];
     const int rsx = plane_rsx(d), fs = plane_fs(d);
 #pragma unroll 1
     for (int pass = 0; pass < 2; pass++) {
         __syncthreads();
-        // x rows, then y columns, each to B + 1 bits before a shift by one (Delta shrinks
-        // by orders of magnitude over a fix: a left shift in the first pass)
+        // x rows, then y columns
         const int len = pass ? Ly : Lx, estr = pass ? rsx : 1;
-        const int sh = fx_bits_rt(len) + 1 - top_bits(s_or[pass]);
-        const int l = sh > 0 ? sh : 0;
-        const RShift rs = rshift(1 - (sh < 0 ? sh : 0));
-        E += rs.r - l;
+        const FwdShift sh0 = fwd_shift(s_or[4 * pass], len);
+        const RShift rs0 = rshift(sh0.r);
         unsigned o = 0;
+        auto field = [&](int ln) { return (int)fdiv((unsigned)ln, pass ? d.dLx : d.dLy); };
         auto line = [&](int ln) {
-            const int f = (int)fdiv((unsigned)ln, pass ? d.dLx : d.dLy), c = ln - f * (pass ? Lx : Ly);
+            const int f = field(ln), c = ln - f * (pass ? Lx : Ly);
             return sm + f * fs + (pass ? c : c * rsx);
         };
         fx_lines<LMAX, false>(
             len, pass ? nf * Lx : nf * Ly, tw + (pass ? Lx : 0),
             [&](int ln) {
                 const longlong2* p = line(ln);
+                const FwdShift sh = OWN ? fwd_shift(s_or[4 * pass + field(ln)], len) : sh0;
+                const RShift rs = OWN ? rshift(sh.r) : rs0;
                 return [=](int e) {
                     const cfx v = ldv<fx>(p + e * estr);
-                    return apply(rs, cfx{v.re << l, v.im << l});
+                    return apply(rs, cfx{v.re << sh.l, v.im << sh.l});
                 };
             },
             [&](int ln) {
@@ -207,19 +229,30 @@ __device__ __forceinline__ int fx_plane_fwd(const Lat& d, longlong2* sm, longlon
                 longlong2* p = line(ln);
                 return [=](int e, cfx v) { st<fx>(p + e * estr, v); };
             },
-            [&](int, auto, const cfx* v, auto N) {
+            [&](int ln, auto, const cfx* v, auto N) {
+                if constexpr (OWN) o = 0;
 #pragma unroll
                 for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
+                if constexpr (OWN) or_into(s_or + 4 * (pass + 1) + field(ln), o);
             },
             [&](int ln) {
-                const int f = (int)fdiv((unsigned)ln, pass ? d.dLx : d.dLy), c = ln - f * (pass ? Lx : Ly);
+                const int f = field(ln), c = ln - f * (pass ? Lx : Ly);
                 longlong2* p = pass ? out + (f * V + c) : sm + f * fs + c * rsx;
                 const int str = pass ? Lx : 1;
                 return [=](int e, cfx v) { st<fx>(p + e * str, v); };
             });
-        block_or(o, s_or + pass + 1);
+        if constexpr (!OWN) block_or(o, s_or + 4 * (pass + 1));
     }
-    return E;
+}
+// Field f's exponent of a transformed plane into pexp and amax1: s_or the column of its bits,
+// E its values' exponent before (after a barrier; a thread per field)
+__device__ __forceinline__ void fx_plane_exp(const Lat& d, const unsigned* s_or, int f, int E, int plane,
+                                             int* __restrict__ pexp, FxExp* fe)
+{
+    const FwdShift x = fwd_shift(s_or[0], d.L[0]), y = fwd_shift(s_or[4], d.L[1]);
+    E += x.r - x.l + y.r - y.l;
+    pexp[f * d.nplanes + plane] = E;
+    atomicMax(&fe->amax1[f], E + align_top(s_or[8], d.L[2]));
 }
 
 // Delta (as k_delta_fx), theta and F, then the forward transform along x and y.
@@ -232,13 +265,13 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delt
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or[3];
+    __shared__ unsigned s_or[12];
     if (ld_flag(&ctl->phase_done)) {
         end_loop(h);
         return;
     }
-    if (threadIdx.x < 3) s_or[threadIdx.x] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2 = kExpNone;
+    if (threadIdx.x < 12) s_or[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2[0] = kExpNone;
     __syncthreads();
     const int P = d.P, V = d.V;
     const int plane = blockIdx.x;
@@ -254,19 +287,17 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_delt
     });
     block_or(o, s_or);
     reduce_theta_F(th, fsum, partials, ctl, hist, V, h);
-    const int E = fx_plane_fwd<LMAX>(d, sm, Fd + plane * P, tw, s_or, -kFxSum, 4);
+    fx_plane_fwd<LMAX, false>(d, sm, Fd + plane * P, tw, s_or, 4);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        pexp[plane] = E;
-        atomicMax(&fe->amax1, E + align_top(s_or[2], d.L[2]));
-    }
+    if (threadIdx.x == 0) fx_plane_exp(d, s_or, 0, -kFxSum, plane, pexp, fe);
 }
 
 // z,t pencils (as k_zt): z forward, t forward and the accelerator, t inverse, z inverse
 // in the tile [t][kz][xi].  The multiplier p2max/(p2 V) of a t-line is kept as
 // integers mx (digits, x 2^62) times 2^me, the largest of the line in [1/2, 1); every
-// accelerated t-line has an exponent of its own (lexp).  Shared memory after the
-// tile: the pencil's multipliers, lexp and the lines' magnitude bits [kz][xi].
+// accelerated t-line has an exponent of its own (lexp).  own: 1 for fields with exponents
+// of their own, else 0.  Shared memory after the tile: the pencil's multipliers, lexp and
+// the lines' magnitude bits [kz][xi].
 inline size_t fxt_pencil_smem(const Lat& d, int xw)
 {
     return pencil_smem_bytes(d, xw, sizeof(longlong2)) + (size_t)xw * d.L[2] * 2 * sizeof(int);
@@ -276,7 +307,7 @@ template <int LMAX>
 __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_zt_fxt(
     Lat d, int xw, longlong2* __restrict__ Fd, const Ctl* ctl, const longlong2* __restrict__ tw,
     const fx* __restrict__ mx, const int* __restrict__ me, const int* __restrict__ pexp, int* __restrict__ bexp,
-    FxExp* fe)
+    FxExp* fe, int own)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
@@ -288,6 +319,7 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_zt_f
     const int xs = __ffs(xw) - 1;
     const int x0 = (int)blockIdx.x * xw, ky = (int)blockIdx.y;
     const int c0 = x0 + Lx * ky;
+    const int fo = own * (int)blockIdx.z;
     longlong2* g = Fd + (size_t)blockIdx.z * d.V + c0;
     fx* m64 = reinterpret_cast<fx*>(sm + Lt * rs);
     int* lexp = reinterpret_cast<int*>(m64 + xw * Lz * Lt);       // [kz][xi]
@@ -296,14 +328,14 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_zt_f
     if (threadIdx.x == 2) s_az = kExpNone;
     for (int i = threadIdx.x; i < xw * Lz; i += blockDim.x) lor[i] = 0u;
     // the planes' values, aligned to B + 1 bits of the largest, and the multipliers
-    int E = __ldg(&fe->amax1) - fx_bits_rt(Lz) - 1;
+    int E = __ldg(fe->amax1 + fo) - fx_bits_rt(Lz) - 1;
     {
         const FastDiv dz = d.dLz;
         block_copy<4, longlong2>(
             xw * Lz * Lt, [&](int i) { return g[(i & (xw - 1)) + P * (i >> xs)]; },
             [&](int i, longlong2 v) {
                 const int zt = i >> xs, t = (int)fdiv((unsigned)zt, dz), z = zt - t * Lz;
-                const int r = E - __ldg(pexp + zt);
+                const int r = E - __ldg(pexp + (fo * d.nplanes + zt));
                 const cfx w = r > 0 ? apply(rshift(r), cfx{v.x, v.y}) : cfx{v.x, v.y};
                 st<fx>(sm + t * rs + (z << xs) + (i & (xw - 1)), w);
             });
@@ -432,22 +464,24 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_zt_f
     __syncthreads();
     if (threadIdx.x == 0) {
         bexp[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = E;
-        atomicMax(&fe->amax2, E + align_top(s_or[1], d.L[1]));
+        atomicMax(&fe->amax2[fo], E + align_top(s_or[1], d.L[1]));
     }
 }
 
-// The inverse transform along y and x of nf fields of plane p into the tile; returns the
-// exponent, the values' bits in s_or[1] (zeroed s_or[0..1] on entry; barriers inside).
-template <int LMAX>
+// The inverse transform along y and x of nf fields of plane p into the tile.  Returns the
+// exponent, or with OWN leaves the fields' in s_E; the values' bits in the second row of
+// s_or ([2][4] as for fx_plane_fwd, zeroed on entry; barriers inside).
+template <int LMAX, bool OWN>
 __device__ __forceinline__ int fx_plane_inv(const Lat& d, int xs, const longlong2* __restrict__ Fd, longlong2* sm,
-                                            const longlong2* __restrict__ tw, const int* __restrict__ bexp,
-                                            const FxExp* fe, unsigned* s_or, int plane, int nf)
+                                             const longlong2* __restrict__ tw, const int* __restrict__ bexp,
+                                             const FxExp* fe, unsigned* s_or, int* s_E, int plane, int nf)
 {
     const int P = d.P, V = d.V, Lx = d.L[0], Ly = d.L[1], s0 = plane * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
     const int nxc = Lx >> xs;
-    int E = __ldg(&fe->amax2) - fx_bits_rt(Ly) - 1;
-    // the plane, aligned to B + 1 bits of the largest pencil
+    // the plane, aligned to B + 1 bits of the largest pencil: of each field, or of all
+    int E = __ldg(fe->amax2) - fx_bits_rt(Ly) - 1;
+    auto start = [&](int f) { return OWN ? __ldg(fe->amax2 + f) - fx_bits_rt(Ly) - 1 : E; };
     block_copy<4, longlong2>(
         nf * P,
         [&](int i) {
@@ -456,7 +490,7 @@ __device__ __forceinline__ int fx_plane_inv(const Lat& d, int xs, const longlong
         },
         [&](int i, longlong2 v) {
             const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P, y = (int)fdiv((unsigned)xy, d.dLx), x = xy - y * Lx;
-            const int r = E - __ldg(bexp + (f * Ly + y) * nxc + (x >> xs));
+            const int r = start(f) - __ldg(bexp + (f * Ly + y) * nxc + (x >> xs));
             const cfx w = r > 0 ? apply(rshift(r), cfx{v.x, v.y}) : cfx{v.x, v.y};
             st<fx>(sm + (f * fs + y * rsx + x), w);
         });
@@ -465,17 +499,21 @@ __device__ __forceinline__ int fx_plane_inv(const Lat& d, int xs, const longlong
         __syncthreads();
         // y columns, then x rows
         const int len = pass ? Lx : Ly, estr = pass ? 1 : rsx;
-        const RShift rs = rshift(pass ? top_bits(s_or[0]) - fx_bits_rt(Lx) : 1);
-        E += rs.r;
+        auto shift = [&](int f) { return rshift(pass ? top_bits(s_or[OWN ? f : 0]) - fx_bits_rt(Lx) : 1); };
+        const RShift rs0 = shift(0);
+        if (!OWN) E += rs0.r;
+        else if (pass && threadIdx.x < 4) s_E[threadIdx.x] = start((int)threadIdx.x) + 1 + shift((int)threadIdx.x).r;
         unsigned o = 0;
+        auto field = [&](int ln) { return (int)fdiv((unsigned)ln, pass ? d.dLy : d.dLx); };
         auto line = [&](int ln) {
-            const int f = (int)fdiv((unsigned)ln, pass ? d.dLy : d.dLx), c = ln - f * (pass ? Ly : Lx);
+            const int f = field(ln), c = ln - f * (pass ? Ly : Lx);
             return sm + f * fs + (pass ? c * rsx : c);
         };
         fx_lines<LMAX, true>(
             len, pass ? nf * Ly : nf * Lx, tw + (pass ? 0 : Lx),
             [&](int ln) {
                 const longlong2* p = line(ln);
+                const RShift rs = OWN ? shift(field(ln)) : rs0;
                 return [=](int e) { return apply(rs, swapped(p[e * estr])); };
             },
             [&](int ln) {
@@ -486,15 +524,17 @@ __device__ __forceinline__ int fx_plane_inv(const Lat& d, int xs, const longlong
                 longlong2* p = line(ln);
                 return [=](int e, cfx v) { st<fx>(p + e * estr, v); };
             },
-            [&](int, auto, const cfx* v, auto N) {
+            [&](int ln, auto, const cfx* v, auto N) {
+                if constexpr (OWN) o = 0;
 #pragma unroll
                 for (int j = 0; j < decltype(N)::value; j++) or_bits(o, v[j]);
+                if constexpr (OWN) or_into(s_or + 4 * pass + field(ln), o);
             },
             [&](int ln) {
                 longlong2* p = line(ln);
                 return [=](int e, cfx v) { p[e * estr] = make_longlong2(v.im, v.re); };
             });
-        block_or(o, s_or + pass);
+        if constexpr (!OWN) block_or(o, s_or + 4 * pass);
     }
     __syncthreads();
     return E;
@@ -511,14 +551,14 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or[2];
+    __shared__ unsigned s_or[8];
     if (ld_flag(&ctl->phase_done)) return;
-    if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
+    if (threadIdx.x < 8) s_or[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 4) fe->amax1[threadIdx.x] = kExpNone;
     const int P = d.P, V = d.V, Lx = d.L[0];
     const int s0 = blockIdx.x * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
-    const int E = fx_plane_inv<LMAX>(d, xs, Fd, sm, tw, bexp, fe, s_or, blockIdx.x, 4);
+    const int E = fx_plane_inv<LMAX, false>(d, xs, Fd, sm, tw, bexp, fe, s_or, nullptr, blockIdx.x, 4);
     if (Dt != nullptr)
         for (int xy = threadIdx.x; xy < P; xy += blockDim.x) {
             const int y = (int)fdiv((unsigned)xy, d.dLx), i = y * rsx + (xy - y * Lx);
@@ -532,7 +572,7 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
     // |alpha/2 Delta~| <= alpha/2 2^(E + top) < 2^(q-1); ha = alpha/2 = hm 2^(he-62) exactly
     const double ha = 0.5 * ctl->alpha;
     const int he = ilogb(ha) + 1;
-    const int q = max(1, he + E + top_bits(s_or[1]) + 1);
+    const int q = max(1, he + E + top_bits(s_or[4]) + 1);
     if (ha < 1e30 && q <= 5) {
         // X x 2^(61-q) = f hm 2^(he - 62 + E + 61 - q)
         const dig hm = digits(__double2ll_rn(scalbn(ha, 62 - he)));
@@ -596,7 +636,7 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyin
 // ---------------------------------------------------------------- FP64 fields through the transform
 
 // The accelerator on nf packed fields in FP64 that are not a Delta (a cotangent): to
-// integers relative to each plane's largest value and forward along x and y; after
+// integers relative to each field's largest value in the plane and forward along x and y; after
 // k_zt_fxt, back.  A value that is not finite sets *bad, which makes every result NaN,
 // as an FP64 transform would.
 template <int LMAX>
@@ -606,10 +646,10 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyfw
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or[3], s_top;
-    if (threadIdx.x < 3) s_or[threadIdx.x] = 0u;
-    if (threadIdx.x == 3) s_top = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax2 = kExpNone;
+    __shared__ unsigned s_or[12], s_top[4];
+    if (threadIdx.x < 12) s_or[threadIdx.x] = 0u;
+    if (threadIdx.x < 4) s_top[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 4) fe->amax2[threadIdx.x] = kExpNone;
     __syncthreads();
     const int P = d.P, Lx = d.L[0], s0 = blockIdx.x * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
@@ -617,8 +657,7 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyfw
         const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P, y = (int)fdiv((unsigned)xy, d.dLx);
         return f * fs + y * rsx + (xy - y * Lx);
     };
-    // the doubles into the tile, their largest exponent
-    unsigned top = 0;
+    // the doubles into the tile, each field's largest exponent
     block_copy<4, double2>(
         nf * P,
         [&](int i) {
@@ -626,29 +665,28 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyfw
             return __ldg(in + (size_t)f * d.V + s0 + (i - f * P));
         },
         [&](int i, double2 v) {
-            top = max(top, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+            unsigned* t = s_top + (int)fdiv((unsigned)i, d.dP);
+            const unsigned top = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+            if (top > *reinterpret_cast<volatile unsigned*>(t)) atomicMax(t, top);
             reinterpret_cast<double2*>(sm)[at(i)] = v;
         });
-    top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
     __syncthreads();
-    const int e = (int)(s_top >> 20) - 1022;  // every |x| < 2^e
-    if (e > 1024 && threadIdx.x == 0) fe->bad = 1;
+    auto exponent = [&](int f) { return (int)(s_top[f] >> 20) - 1022; };  // every |x| of the field < 2^e
+    if (threadIdx.x < 4 && exponent((int)threadIdx.x) > 1024) fe->bad = 1;
     // x 2^(60-e) (a value in place of its double: the same thread, the same slot)
-    unsigned o = 0;
     for (int i = threadIdx.x; i < nf * P; i += blockDim.x) {
+        const int f = (int)fdiv((unsigned)i, d.dP), e = exponent(f);
         const double2 v = reinterpret_cast<const double2*>(sm)[at(i)];
         const cfx w = cfx{d2fx_rel(v.x, e), d2fx_rel(v.y, e)};
+        unsigned o = 0;
         or_bits(o, w);
+        or_into(s_or + f, o);
         st<fx>(sm + at(i), w);
     }
-    block_or(o, s_or);
-    const int E = fx_plane_fwd<LMAX>(d, sm, Fd + s0, tw, s_or, e - 60, nf);
+    fx_plane_fwd<LMAX, true>(d, sm, Fd + s0, tw, s_or, nf);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        pexp[blockIdx.x] = E;
-        atomicMax(&fe->amax1, E + align_top(s_or[2], d.L[2]));
-    }
+    if ((int)threadIdx.x < nf)
+        fx_plane_exp(d, s_or + threadIdx.x, (int)threadIdx.x, exponent((int)threadIdx.x) - 60, blockIdx.x, pexp, fe);
 }
 
 template <int LMAX>
@@ -658,18 +696,19 @@ __global__ void __launch_bounds__(kFxtThreads<LMAX>, kFxtMinBlocks<LMAX>) k_xyba
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     longlong2* sm = reinterpret_cast<longlong2*>(smem_raw);
-    __shared__ unsigned s_or[2];
-    if (threadIdx.x < 2) s_or[threadIdx.x] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) fe->amax1 = kExpNone;
+    __shared__ unsigned s_or[8];
+    __shared__ int s_E[4];
+    if (threadIdx.x < 8) s_or[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 4) fe->amax1[threadIdx.x] = kExpNone;
     const int P = d.P, Lx = d.L[0], s0 = blockIdx.x * P;
     const int rsx = plane_rsx(d), fs = plane_fs(d);
-    const int E = fx_plane_inv<LMAX>(d, xs, Fd, sm, tw, bexp, fe, s_or, blockIdx.x, nf);
+    fx_plane_inv<LMAX, true>(d, xs, Fd, sm, tw, bexp, fe, s_or, s_E, blockIdx.x, nf);
     const double nan = __hiloint2double(0x7ff80000, 0);
     const bool bad = ld_flag(&fe->bad) != 0;
     for (int i = threadIdx.x; i < nf * P; i += blockDim.x) {
         const int f = (int)fdiv((unsigned)i, d.dP), xy = i - f * P, y = (int)fdiv((unsigned)xy, d.dLx);
         const longlong2 v = sm[f * fs + y * rsx + (xy - y * Lx)];
-        out[(size_t)f * d.V + s0 + xy] = bad ? make_double2(nan, nan) : make_double2(fx2d_safe(v.x, -E), fx2d_safe(v.y, -E));
+        out[(size_t)f * d.V + s0 + xy] = bad ? make_double2(nan, nan) : make_double2(fx2d_safe(v.x, -s_E[f]), fx2d_safe(v.y, -s_E[f]));
     }
 }
 

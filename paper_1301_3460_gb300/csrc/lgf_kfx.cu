@@ -40,7 +40,7 @@ bool fxt_fits(const Lat& d, const Shape& sh) { return fxt_pencil_smem(d, sh.xw) 
 
 size_t fxt_bytes(const Lat& d)
 {
-    return sizeof(FxExp) + ((size_t)d.nplanes + 4 * (size_t)d.P + (size_t)d.P * d.L[2]) * sizeof(int) +
+    return sizeof(FxExp) + (4 * (size_t)d.nplanes + 4 * (size_t)d.P + (size_t)d.P * d.L[2]) * sizeof(int) +
            (size_t)d.V * sizeof(fx) + (size_t)(d.L[0] + d.L[1] + d.L[2] + d.L[3]) * sizeof(longlong2);
 }
 FxtBuf fxt_carve(const Lat& d, void* p)
@@ -50,7 +50,7 @@ FxtBuf fxt_carve(const Lat& d, void* p)
     b.mx = reinterpret_cast<fx*>(b.tw + d.L[0] + d.L[1] + d.L[2] + d.L[3]);
     b.fe = reinterpret_cast<FxExp*>(b.mx + d.V);
     b.pexp = reinterpret_cast<int*>(b.fe + 1);
-    b.bexp = b.pexp + d.nplanes;
+    b.bexp = b.pexp + 4 * (size_t)d.nplanes;
     b.me = b.bexp + 4 * (size_t)d.P;
     return b;
 }
@@ -75,14 +75,14 @@ void launch_fxt_delta(const Lat& d, const Shape& sh, cudaStream_t s, const longl
     else
         k_delta_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, AH, Fs, Fd, b.tw, b.pexp, b.fe, partials, ctl, hist, h);
 }
-void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl, int nf)
+void launch_fxt_zt(const Lat& d, const Shape& sh, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl, int nf, int own)
 {
     const size_t sm = fxt_pencil_smem(d, sh.xw);
     const dim3 grid(d.L[0] / sh.xw, d.L[1], nf);
     if (short_zt_lines(d))
-        k_zt_fxt<32><<<grid, fxt_threads(sh.nt_zt, sm, true), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
+        k_zt_fxt<32><<<grid, fxt_threads(sh.nt_zt, sm, true), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe, own);
     else
-        k_zt_fxt<128><<<grid, fxt_threads(sh.nt_zt, sm, false), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe);
+        k_zt_fxt<128><<<grid, fxt_threads(sh.nt_zt, sm, false), sm, s>>>(d, sh.xw, Fd, ctl, b.tw, b.mx, b.me, b.pexp, b.bexp, b.fe, own);
 }
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const longlong2* Fd, longlong2* g,
                         const FxtBuf& b, const Ctl* ctl, double2* Dt)
@@ -125,7 +125,7 @@ void launch_fxt_accel(const Lat& d, const Shape& sh, cudaStream_t s, const doubl
         k_xyfwd_fxt<32><<<d.nplanes, nt, sm, s>>>(d, in, work, nf, b.tw, b.pexp, b.fe);
     else
         k_xyfwd_fxt<128><<<d.nplanes, nt, sm, s>>>(d, in, work, nf, b.tw, b.pexp, b.fe);
-    launch_fxt_zt(d, sh, s, work, b, ctl, nf);
+    launch_fxt_zt(d, sh, s, work, b, ctl, nf, 1);
     if (small)
         k_xyback_fxt<32><<<d.nplanes, nt, sm, s>>>(d, xs, work, out, nf, b.tw, b.bexp, b.fe);
     else

@@ -283,13 +283,13 @@ static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
     if (mu == 0 && s < V) Fs[s] = retr[0][lane] + retr[1][lane] + retr[2][lane] + retr[3][lane];
 }
 
-// magnitude exponents of the integer transform's fields (lgf_fxt.cuh)
+// magnitude exponents of the integer transform's four fields (lgf_fxt.cuh)
 constexpr int kExpNone = -(1 << 28);
-struct FxExp {
-    int amax1;  // over the planes, after the Delta kernel (reset at the start of a loop and by the g builder)
-    int amax2;  // over the pencils, after the accelerator (reset by the Delta kernel)
-    int bad;    // a field of FP64 values was not finite (k_xyfwd_fxt; reset before it)
-    int pad;
+struct __align__(16) FxExp {
+    int amax1[4];  // over the planes, after the Delta kernel (reset at the start of a loop and by the g builder)
+    int amax2[4];  // over the pencils, after the accelerator (reset by the Delta kernel)
+    int bad;       // a field of FP64 values was not finite (k_xyfwd_fxt; reset before it)
+    int pad[3];
 };
 
 // Start of a loop: the links' rows 0,1 (and G's) on the grid, rounded to nearest, with
@@ -301,7 +301,7 @@ static __global__ void __launch_bounds__(128) k_fx_start(Lat d, const double2* _
 {
     const int V = d.V;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s == 0) fe->amax1 = kExpNone;
+    if (s < 4) fe->amax1[s] = kExpNone;
     if (s >= V) return;
     fx f = 0;
 #pragma unroll 1
@@ -335,7 +335,7 @@ static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2*
     if (ld_flag(&ctl->nan_seen)) return;
     const int V = d.V;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s == 0) fe->amax1 = kExpNone;
+    if (s < 4) fe->amax1[s] = kExpNone;
     if (s >= V) return;
     int c[4];
     site_coords(d, s, c);

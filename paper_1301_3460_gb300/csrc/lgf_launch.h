@@ -92,8 +92,8 @@ struct FxtBuf {
     longlong2* tw = nullptr;  // [Lx + Ly + Lz + Lt] roots of unity
     long long* mx = nullptr;  // [V]
     FxExp* fe = nullptr;
-    int* pexp = nullptr;      // [planes]
-    int* bexp = nullptr;      // [pencils], at most 4 P
+    int* pexp = nullptr;      // [field][plane]
+    int* bexp = nullptr;      // [field][pencil], at most 4 P
     int* me = nullptr;        // [t-lines]
 };
 size_t fxt_bytes(const Lat& d);
@@ -118,12 +118,12 @@ template <typename TF>
 void launch_fx_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const vec2_t<TF>* Fd, longlong2* g,
                        const Ctl* ctl);
 // the iteration's transforms on integers: Delta + x,y forward; z,t with the
-// multiplier; x,y inverse + g
+// multiplier (own: every field has exponents of its own); x,y inverse + g
 void launch_fxt_delta(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* AH, const long long* Fs,
                       longlong2* Fd, const FxtBuf& b, double* partials, Ctl* ctl, double2* hist,
                       cudaGraphConditionalHandle h);
 void launch_fxt_zt(const Lat& d, const Shape& sh64, cudaStream_t s, longlong2* Fd, const FxtBuf& b, const Ctl* ctl,
-                   int nf = 4);
+                   int nf = 4, int own = 0);
 void launch_fxt_xyinv_g(const Lat& d, const Shape& sh64, cudaStream_t s, const longlong2* Fd, longlong2* g,
                         const FxtBuf& b, const Ctl* ctl, double2* Dt = nullptr);
 // the accelerator on nf packed FP64 fields (any values: a cotangent), in -> out, through

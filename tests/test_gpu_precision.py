@@ -28,3 +28,28 @@ def test_generated_links_are_rounded_to_the_nearest_double():
     assert float(np.sqrt(np.mean(np.abs(ip) ** 2))) < 5e-17
     norm = (np.abs(w) ** 2).sum(-1) - 1
     assert float(np.sqrt(np.mean(norm ** 2))) < 1e-16
+
+
+def _unit_with_cotangent(lat, V, big, small):
+    """step_bwd at unit links (g = 1, so that colour components do not mix there): component
+    01 of size big on even sites, 02 of size small on odd ones"""
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    r = torch.randn((4, V, 2), dtype=torch.complex128, device="cuda", generator=gen)
+    ct = torch.zeros((4, V, 3, 3), dtype=torch.complex128, device="cuda")
+    ct[:, ::2, 0, 1] = big * r[:, ::2, 0]
+    ct[:, 1::2, 0, 2] = small * r[:, 1::2, 1]
+    lat.set_unit_links()
+    return lat.step_bwd(ct)
+
+
+@pytest.mark.parametrize("L", [(8, 8, 8, 8), (12, 6, 4, 48)])
+def test_fields_of_different_size_keep_their_own_precision(L):
+    """The backward step is linear and at unit links colour components stay apart, so a
+    component gets what it gets alone, to its own rounding, however large another is: a few
+    units of 2^-52 of its largest value, 64 covers the transforms' lengths."""
+    V = int(np.prod(L))
+    with lgf.Lattice(L, track_gauge=False) as lat:
+        alone = _unit_with_cotangent(lat, V, 0.0, 1e-6)[..., 0, 2]
+        both = _unit_with_cotangent(lat, V, 1.0, 1e-6)
+        assert float(both[..., 0, 1].abs().max()) > 0.1
+        assert float((both[..., 0, 2] - alone).abs().max()) < 64 * 2.0 ** -52 * float(alone.abs().max())
