@@ -180,16 +180,17 @@ __device__ __forceinline__ double fx2d_safe(fx v, int q)
     return __hiloint2double(hi - (q << 20), __double2loint(y));
 }
 
-// x 2^(60-e) of a double |x| < 2^e, rounded toward zero; zero for what is not finite
+// x 2^(60-e) of a double |x| < 2^e (e >= -1022), rounded toward zero; zero for what is not
+// finite.  Subnormals count: no leading one, the exponent of the smallest normal numbers.
 __device__ __forceinline__ fx d2fx_rel(double x, int e)
 {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     const int ex = (int)((hi >> 20) & 0x7ffu);
-    const unsigned mh = 0x80000000u | ((hi & 0xfffffu) << 11) | (lo >> 21), ml = lo << 11;
+    const unsigned mh = (ex ? 0x80000000u : 0u) | ((hi & 0xfffffu) << 11) | (lo >> 21), ml = lo << 11;
     const unsigned long long m = ((unsigned long long)mh << 32) | ml;  // 2^(ex-1023) -> 2^63
-    const int r = 1023 + 3 + e - ex;                                   // 2^e -> 2^60
+    const int r = 1023 + 3 + e - max(ex, 1);                           // 2^e -> 2^60
     unsigned long long v = (r >= 0 && r < 64) ? m >> r : 0ull;
-    if (ex == 0 || ex == 0x7ff) v = 0;
+    if (ex == 0x7ff) v = 0;
     const fx s = -(fx)(hi >> 31);
     return ((fx)v ^ s) - s;
 }

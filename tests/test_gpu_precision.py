@@ -53,3 +53,19 @@ def test_fields_of_different_size_keep_their_own_precision(L):
         both = _unit_with_cotangent(lat, V, 1.0, 1e-6)
         assert float(both[..., 0, 1].abs().max()) > 0.1
         assert float((both[..., 0, 2] - alone).abs().max()) < 64 * 2.0 ** -52 * float(alone.abs().max())
+
+
+def test_subnormal_cotangents_count():
+    """Cotangents in the subnormal range go through like others: with 2^-1074 as their last
+    place and values near 2^-1040 each is known to 2^-35, and the step's sums multiply that by
+    no more than a few hundred."""
+    L = (6, 8, 4, 4)
+    V = int(np.prod(L))
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    ct = torch.randn((4, V, 3, 3), dtype=torch.complex128, device="cuda", generator=gen)
+    with lgf.Lattice(L, track_gauge=False) as lat:
+        lat.set_links(inputs.rough_gauge_field(L, 0.3, 82))
+        one = lat.step_bwd(ct)
+        tiny = lat.step_bwd(torch.view_as_complex(torch.view_as_real(ct) * 2.0 ** -1040))
+        back = torch.view_as_complex(torch.view_as_real(tiny) * 2.0 ** 1000 * 2.0 ** 40)
+    assert float((back - one).abs().max()) < 2.0 ** -26 * float(one.abs().max())
