@@ -311,7 +311,7 @@ def run_ours(args, dims):
     # then the graph of lgf_fix (packed parts and Delta of the input, then per loop
     # pass the z,t kernel, the inverse x,y + g kernel, the update, Delta and the
     # loop control)
-    launches = sum(2 + 3 + 4 * max(r["iters"], 1) for r in info)
+    launches = sum(2 + 4 + 4 * max(r["iters"], 1) for r in info)
     ttt = {}
     for k, r in enumerate(info):
         ttt.setdefault(str(EPS[k % len(EPS)]), dict(iters=r["iters"], ms=1000 * per_step[k], F=r["F"],

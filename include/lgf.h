@@ -488,9 +488,8 @@ int lgf_plaquette(lgf_ctx* ctx, double* P);
  * after its update.  A chain of its own, with the Wilson action's equilibrium up
  * to FP32 rounding, 4 to 7x faster on GB300 (32^4: 1.30 against 8.8 ms per
  * heat-bath sweep, 0.99 against 3.8 ms per overrelaxation sweep; the copy takes
- * 4 V x 48 bytes of device memory, the fixed-point links of the FP64 generator
- * 4 V x 144); the FP64 generator is the one that
- * matches the reference to rounding.
+ * 4 V x 48 bytes of device memory, the FP64 generator none); the FP64 generator is
+ * the one that matches the reference to rounding.
  */
 int lgf_set_generator_precision(lgf_ctx* ctx, int bits);
 

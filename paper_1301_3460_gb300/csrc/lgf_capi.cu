@@ -100,8 +100,9 @@ struct lgf_ctx {
     unsigned* gu_sync = nullptr;  // its queue, epoch and per-plane flags
     // FP64 iterations run on 64-bit fixed point (lgf_kfx.cuh) while the stored links
     // are within its range; `wide` links (a snapshot of anything else) take the FP64
-    // kernels.  g64, AH64 and Fs64 hold the fixed-point g, parts and Re Tr meanwhile.
-    longlong2* UX = nullptr;  // [4][6][V]
+    // kernels.  g64, AH64 and Fs64 hold the fixed-point g, parts and Re Tr meanwhile, U64 and
+    // G64 (mixed: U32 with U32b, and AH32) the fixed-point links and G.
+    longlong2* UX = nullptr;  // [4][nx][V]
     longlong2* GX = nullptr;  // [6][V]
     bool wide = false, graph_wide = false;
     FxtBuf fxt{};             // the integer transform's tables and exponents (in mult)
@@ -128,7 +129,7 @@ struct lgf_ctx {
     double2* dGp = nullptr;   // [4][9][V] cotangent in / out
     double2* dGud = nullptr;  // [4][9][V]
     double2* dQ = nullptr;    // [4][9][V]
-    double2* dGgs = nullptr;  // [4][6][V] (the FP64 kernels use [6][V])
+    double2* dGgs = nullptr;  // [6][V]
     double2* dFA = nullptr;   // [4][V]
     double2* dFB = nullptr;   // [4][V]
     double2* gl_part = nullptr;
@@ -136,7 +137,6 @@ struct lgf_ctx {
     double* gl_D = nullptr;    // [5]
     double* wil_part = nullptr;  // plaquette partial sums, then the result
     int gen_precision = 64;      // arithmetic of the configuration generator's staples and draws
-    longlong2* genx = nullptr;   // [4][9][V]: fixed-point links of the FP64 generator
     float2* gen32 = nullptr;     // [4][6][V]: FP32 copy of the links for the FP32 generator's staples
 };
 
@@ -257,17 +257,22 @@ void launch_update64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
         launch_update<double>(c->lat, s, c->U64, c->G64, c->g64, ctl, c->AH64, c->Fs64);
 }
 
-// start of an FP64 loop on the stored links (without Delta), and its end
+// start of an FP64 loop on the stored links (without Delta), what comes between the first
+// Delta and the first update, and the loop's end
 void launch_start64(lgf_ctx* c, cudaStream_t s)
 {
     if (!c->wide)
-        launch_fx_start(c->lat, s, c->U64, c->G64, c->UX, c->GX, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
+        launch_fx_start(c->lat, s, as_fx(c->U64), as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
     else
         launch_ah_init<double>(c->lat, s, c->U64, c->AH64, c->Fs64);
 }
+void launch_enter64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
+{
+    if (!c->wide) launch_fx_enter(c->lat, s, as_fx(c->U64), as_fx(c->G64), c->UX, c->GX, ctl);
+}
 void launch_finish64(lgf_ctx* c, cudaStream_t s, Ctl* ctl)
 {
-    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->GX, c->U64, c->G64, ctl, c->mixed);
+    if (!c->wide) launch_fx_finish(c->lat, s, c->UX, c->GX, c->U64, c->G64, ctl);
 }
 
 // one FP64 iteration after Delta: FFT(z,t)+scale+IFFT(t,z), IFFT(x,y)+g, update,
@@ -435,6 +440,7 @@ int append_fix(lgf_ctx* c, cudaGraph_t graph, std::vector<cudaGraphNode_t>& deps
         launch_start64(c, c->cap);
     }
     launch_delta64(c, c->cap, c->ctl, c->hist, !c->plain);
+    if (!c->mixed) launch_enter64(c, c->cap, c->ctl);  // mixed: the projection has done it
     CKR(capture_end(c, deps));
     CKR(add_loop64(c, graph, deps));
     CKR(capture_begin(c, graph, deps));
@@ -575,6 +581,7 @@ int create_impl(const int dims[4], int flags, lgf_ctx* c)
     d.nplanes = dims[2] * dims[3];
     lat_set_divisors(d);
     d.ne = (flags & LGF_LINKS18) ? 9 : (flags & LGF_LINKS8) ? 4 : 6;
+    d.nx = c->mixed ? 6 : std::max(d.ne, 6);
     c->lat32 = d;
     c->lat32.ne = 6;
     if (!pick_shape(d, sizeof(double2), 4, &c->sh64)) return LGF_ERR_UNSUPPORTED_DIMS;
@@ -588,19 +595,26 @@ int create_impl(const int dims[4], int flags, lgf_ctx* c)
     if (c->mixed) CK(prepare_kernels<float>(d, c->sh32));
 
     const size_t Vs = (size_t)c->V;
-    CKR(alloc((void**)&c->U64, (size_t)4 * d.ne * Vs * sizeof(double2)));
+    // Links, g and packed parts in one piece.  Without an FP32 phase the fixed-point links of
+    // a running loop take the FP64 links' place; those of the generator, 36 entries per
+    // site, reach over g into the parts.
+    const size_t nu = (size_t)4 * (c->mixed ? d.ne : d.nx);
+    CKR(alloc((void**)&c->U64, (nu + 9 + 16) * Vs * sizeof(double2)));
+    c->g64 = c->U64 + nu * Vs;
+    c->AH64 = c->g64 + 9 * Vs;
     if (c->track) CKR(alloc((void**)&c->G64, 6 * Vs * sizeof(double2)));
-    CKR(alloc((void**)&c->g64, 9 * Vs * sizeof(double2)));
     CKR(alloc(&c->Fd, 4 * Vs * sizeof(double2)));
-    CKR(alloc((void**)&c->AH64, 16 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->Fs64, Vs * sizeof(double)));
     CK(fx_prepare(d));
-    CKR(alloc((void**)&c->UX, (c->track ? 30 : 24) * Vs * sizeof(longlong2)));
-    if (c->track) c->GX = c->UX + 24 * Vs;
+    c->UX = as_fx(c->U64);
+    c->GX = as_fx(c->G64);
     if (c->mixed) {
-        CKR(alloc((void**)&c->U32, 24 * Vs * sizeof(float2)));
-        CKR(alloc((void**)&c->U32b, 24 * Vs * sizeof(float2)));
+        // the FP32 phase's links and parts, idle in the FP64 phase, are the place there
+        CKR(alloc((void**)&c->U32, 48 * Vs * sizeof(float2)));
+        c->U32b = c->U32 + 24 * Vs;
         CKR(alloc((void**)&c->AH32, 16 * Vs * sizeof(float2)));
+        c->UX = reinterpret_cast<longlong2*>(c->U32);
+        c->GX = reinterpret_cast<longlong2*>(c->AH32);
         CKR(alloc((void**)&c->Fs32, Vs * sizeof(float)));
         CKR(alloc((void**)&c->G32, 6 * Vs * sizeof(float2)));
         CKR(alloc((void**)&c->g32, 9 * Vs * sizeof(float2)));
@@ -628,9 +642,9 @@ int create_impl(const int dims[4], int flags, lgf_ctx* c)
 void free_all(lgf_ctx* c)
 {
     if (c->exec) cudaGraphExecDestroy(c->exec);
-    void* ptrs[] = {c->U64, c->G64, c->g64, c->U32, c->G32, c->g32, c->Fd, c->partials, c->ctl, c->ctl_stage,
-                    c->hist, c->err, c->stage, c->tables, c->mult, c->AH64, c->Fs64, c->U32b, c->AH32, c->Fs32, c->dGp, c->dGud, c->dQ, c->dGgs, c->dFA, c->dFB,
-                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync, c->UX, c->genx};
+    void* ptrs[] = {c->U64, c->G64, c->U32, c->G32, c->g32, c->Fd, c->partials, c->ctl, c->ctl_stage,
+                    c->hist, c->err, c->stage, c->tables, c->mult, c->Fs64, c->AH32, c->Fs32, c->dGp, c->dGud, c->dQ, c->dGgs, c->dFA, c->dFB,
+                    c->gl_part, c->gl_At, c->gl_D, c->wil_part, c->gen32, c->gu_sync};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->host_ctl) cudaFreeHost(c->host_ctl);
@@ -902,7 +916,7 @@ int ensure_diff(lgf_ctx* c)
     CKR(alloc((void**)&c->dGp, 36 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dGud, 36 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dQ, 36 * Vs * sizeof(double2)));
-    CKR(alloc((void**)&c->dGgs, 24 * Vs * sizeof(double2)));
+    CKR(alloc((void**)&c->dGgs, 6 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dFA, 4 * Vs * sizeof(double2)));
     CKR(alloc((void**)&c->dFB, 4 * Vs * sizeof(double2)));
     return LGF_OK;
@@ -1425,6 +1439,7 @@ int lgf_time_kernels(lgf_ctx* c, double alpha, int n_iter, int precision, double
         launch_start32(c, s, c->ctl_stage, nullptr);
     } else {
         launch_start64(c, s);
+        launch_enter64(c, s, c->ctl_stage);
     }
     for (int it = 0; it < n_iter && rc == LGF_OK; it++) {
         cudaEventRecord(ev[0], s);
@@ -1725,13 +1740,13 @@ int lgf_step_bwd(lgf_ctx* c, double alpha, const double* gU_out, double* gU_in)
     if (fixed) {
         longlong2 *work = as_fx(Fd), *gX = as_fx(c->g64);
         double2* Dt = c->AH64 + 4 * (size_t)c->V;  // the parts are not read after Delta
-        launch_fx_start(c->lat, s, c->U64, nullptr, c->UX, nullptr, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
+        launch_fx_start_bwd(c->lat, s, c->U64, c->dGud, as_fx(c->AH64), as_fx(c->Fs64), c->fxt.fe);
         launch_fxt_delta(c->lat, c->sh64, s, as_fx(c->AH64), as_fx(c->Fs64), work, c->fxt, c->partials, c->ctl_stage,
                          nullptr, 0);
         launch_fxt_zt(c->lat, c->sh64, s, work, c->fxt, c->ctl_stage);
         launch_fxt_xyinv_g(c->lat, c->sh64, s, work, gX, c->fxt, c->ctl_stage, Dt);
         launch_pack_full(s, c->V, gU_out, c->dGp);
-        launch_fx_step_bwd(c->lat, s, c->UX, gX, Dt, c->dGp, c->dGud, c->dGgs, c->dQ, alpha, c->dFA, c->dFB);
+        launch_fx_step_bwd(c->lat, s, gX, Dt, c->dGp, c->dGud, c->dQ, alpha, c->dFA, c->dFB);
         // six fields: four in dFA, two in dFB
         CK(fxt_clear_bad(c->fxt, s));
         launch_fxt_accel(c->lat, c->sh64, s, c->dFA, c->dFA, work, 4, c->fxt, c->ctl_stage);
@@ -1816,10 +1831,8 @@ int lgf_wilson_sweeps(lgf_ctx* c, double beta, unsigned long long seed, int firs
         launch_links_to_fp32(c->stream, c->lat, c->U64, c->gen32);
     }
     const bool fixed = c->gen_precision == 64 && !c->wide && n_heatbath + n_overrelax > 0;
-    if (fixed) {
-        if (!c->genx) CKR(alloc((void**)&c->genx, (size_t)36 * c->V * sizeof(longlong2)));
-        launch_links_to_fx(c->stream, c->lat, c->U64, c->genx);
-    }
+    // fixed-point links with all rows: over the stored ones, g and the packed parts
+    if (fixed) launch_links_to_fx(c->stream, c->lat, c->U64);
     // n_heatbath = 0: overrelaxation sweeps only
     const int rounds = n_heatbath > 0 ? n_heatbath : 1;
     for (int i = 0; i < rounds; i++) {
@@ -1828,13 +1841,13 @@ int lgf_wilson_sweeps(lgf_ctx* c, double beta, unsigned long long seed, int firs
             for (int mu = 0; mu < 4; mu++)
                 for (int par = 0; par < 2; par++)
                     if (fixed)
-                        launch_wilson_fx(c->stream, c->lat, c->genx, mu, par, mode > 0, beta, seed, sweep);
+                        launch_wilson_fx(c->stream, c->lat, as_fx(c->U64), mu, par, mode > 0, beta, seed, sweep);
                     else
                         launch_wilson(c->stream, c->lat, c->U64, c->gen32, mu, par, mode > 0, beta, seed, sweep,
                                       c->gen_precision);
         CK(cudaGetLastError());
     }
-    if (fixed) launch_links_from_fx(c->stream, c->lat, c->genx, c->U64);
+    if (fixed) launch_links_from_fx(c->stream, c->lat, c->U64);
     if (c->track) launch_identity_rows64(c->stream, c->V, c->G64);
     CK(cudaGetLastError());
     // a sweep rewrites every link into SU(3), whatever it was (unless it was not finite)

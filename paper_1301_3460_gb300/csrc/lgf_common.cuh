@@ -205,6 +205,8 @@ struct Lat {
     int ne;        // complex entries stored per link: 6 (rows 0,1; row 2 rebuilt on load),
                    // 9 (row 2 kept as written, the rebuild done once when stored) or
                    // 4 (the 8-real form, FP64 only: u01, u02, u10, phases of u00 and u20)
+    int nx;        // 16-byte entries from one link to the next in the fixed-point links (6, or
+                   // 9 where these take the place of 18-real FP64 links)
     FastDiv dLx, dLy, dP, dLz;  // division by Lx, Ly, Lx*Ly and Lz
 };
 
@@ -262,6 +264,7 @@ struct Ctl {
     int stall_near;        // ... or after this many once theta_best < near_floor
     double near_floor;
     int bad;               // an entry of g was not finite (fixed-point iterations): theta and F become NaN
+    int fixed_form;        // the links (and G) are in their fixed-point form: the end of the loop brings them back
     int fault;             // a kernel gave up waiting for its own asynchronous copies (loop stopped)
 };
 

@@ -232,9 +232,9 @@ static __global__ void __launch_bounds__(128) k_bwd_update(Lat d, const double2*
 
 // b2: one thread per site.  G_g -> Gram-Schmidt backward -> G_Dt rows 0,1,
 // written as six fields into FA (fields 00,01,02,10) and FB (11,12,0,0).
-// nself: the parts of G_g's rows 0,1 in Ggs ([nself][6][V]: one, or one per direction).
+// nself: the parts of G_g's rows 0,1 in Ggs, stride planes apart (one, or one per direction).
 static __global__ void k_bwd_reunit(Lat d, const double2* __restrict__ Fdt, const double2* __restrict__ Ggs, int nself,
-                                    const double2* __restrict__ Q, double alpha, double2* __restrict__ FA,
+                                    int stride, const double2* __restrict__ Q, double alpha, double2* __restrict__ FA,
                                     double2* __restrict__ FB)
 {
     const int V = d.V;
@@ -247,7 +247,7 @@ static __global__ void k_bwd_reunit(Lat d, const double2* __restrict__ Fdt, cons
     for (int e = 0; e < 6; e++) Gg[e] = ld<double>(Ggs + (size_t)e * V + s);
     for (int m = 1; m < nself; m++)
 #pragma unroll
-        for (int e = 0; e < 6; e++) Gg[e] = Gg[e] + ld<double>(Ggs + (size_t)(6 * m + e) * V + s);
+        for (int e = 0; e < 6; e++) Gg[e] = Gg[e] + ld<double>(Ggs + (size_t)(stride * m + e) * V + s);
 #pragma unroll
     for (int e = 6; e < 9; e++) Gg[e] = mk<double>(0, 0);
 #pragma unroll

@@ -43,17 +43,19 @@ template <int S> __device__ __forceinline__ cfx fx_dag2(cdig3 a0, cdig3 b0, cdig
     return cfx{pv + qv, rv - pv + qv};  // conj(a) b = (p + q, r - p + q), r = (Re a - Im a)(Re b + Im b)
 }
 
-// b1 of lgf_diff.cuh, one thread per link (mu = blockIdx.y).  UX, gX: links x 2^61 and
-// g x 2^62 of the forward pass.  Writes the direct cotangent of U (Gud), the link's
-// parts of G_g(x) (Ggm, rows 0,1) and of G_g(x+mu) (Q), in FP64.  32^4: 4.00 ms in FP64
-// (2000 operations per site at 2 per clock and SM), 1.46 ms like this (5000 integer
-// products per site; 12 warps per SM at 168 registers, 16 at 128 take 1.7 ms).
+// b1 of lgf_diff.cuh, one thread per link (mu = blockIdx.y).  gX: g x 2^62 of the forward
+// pass.  Gp, Gud: [4][9][V].  On entry Gp holds the cotangent of the new links and the first
+// six slots of a link in Gud the link itself, x 2^61; on exit Gud holds the direct cotangent
+// of U and the first six slots of Gp the link's parts of G_g(x) (rows 0,1).  Q: the
+// link's parts of G_g(x+mu).  In FP64 (Gud and Gp are read and written by the link's own
+// thread only, and read as what they hold).  The nine components of a cotangent share one scale:
+// their errors are 2^-57 of the largest of them, where FP64's are 2^-53 of the largest
+// term of each sum.  32^4: 4.00 ms in FP64 (2000 operations per site at 2 per clock and
+// SM), 1.46 ms like this (5000 integer products per site; 12 warps per SM at 168
+// registers, 16 at 128 take 1.7 ms).
 template <int NT, int MB>
-__global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2* __restrict__ U,
-                                                                 const longlong2* __restrict__ g,
-                                                                 const double2* __restrict__ Gp,
-                                                                 double2* __restrict__ Gud, double2* __restrict__ Ggm,
-                                                                 double2* __restrict__ Q)
+__global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2* __restrict__ g, double2* Gp, double2* Gud,
+                                                          double2* __restrict__ Q)
 {
     const int V = d.V, mu = blockIdx.y;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2
     unsigned top = 0;
 #pragma unroll
     for (int e = 0; e < 9; e++) {
-        gp[e] = __ldg(Gp + (size_t)(mu * 9 + e) * V + s);
+        gp[e] = Gp[(size_t)(mu * 9 + e) * V + s];
         top = max(top, max((unsigned)__double2hiint(gp[e].x) & 0x7fffffffu, (unsigned)__double2hiint(gp[e].y) & 0x7fffffffu));
     }
     const int ex = (int)(top >> 20) - 1022 + 3;  // components below 2^57
@@ -81,13 +83,18 @@ __global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2
     auto put = [&](double2* p, cfx v) {
         *p = bad ? make_double2(nan, nan) : make_double2(fx2d_safe(v.re, 60 - ex), fx2d_safe(v.im, 60 - ex));
     };
+    // an entry of the link
+    auto link = [&](int e) {
+        const double2 v = Gud[(size_t)(mu * 9 + e) * V + s];
+        return cfx{__double_as_longlong(v.x), __double_as_longlong(v.y)};
+    };
     cdig3 gx[6], Vr[6];  // Vr = rows 0,1 of g(x) U (x 2^61)
 #pragma unroll
     for (int e = 0; e < 6; e++) gx[e] = with_sum(ldx(g + (size_t)e * V + s));
     {
         cdig3 ud[9];
 #pragma unroll
-        for (int e = 0; e < 6; e++) ud[e] = with_sum(ldx(U + (size_t)(mu * 6 + e) * V + s));
+        for (int e = 0; e < 6; e++) ud[e] = with_sum(link(e));
 #pragma unroll
         for (int j = 0; j < 3; j++) ud[6 + j] = with_sum(fx_row2<3>(ud, ud + 3, j));
         cfx t[6];
@@ -139,6 +146,22 @@ __global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2
             for (int b = 0; b < 3; b++)
                 put(Q + (size_t)(mu * 9 + 3 * a + b) * V + s, fx_dag2<3>(Gd[a], Vr[b], Gd[3 + a], Vr[3 + b]));
     }
+    // G_g(x) rows 0,1 += Y U^dag
+    {
+        cdig3 Yd[6], ud[9];
+#pragma unroll
+        for (int e = 0; e < 6; e++) {
+            Yd[e] = with_diff(Y[e]);
+            ud[e] = with_sum(link(e));
+        }
+#pragma unroll
+        for (int j = 0; j < 3; j++) ud[6 + j] = with_sum(fx_row2<3>(ud, ud + 3, j));
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            put(Gp + (size_t)(mu * 9 + j) * V + s, fx_mul_dag<3>(Yd, ud + 3 * j));
+            put(Gp + (size_t)(mu * 9 + 3 + j) * V + s, fx_mul_dag<3>(Yd + 3, ud + 3 * j));
+        }
+    }
     // G_U^direct = (rows 0,1 of g)^dag Y
     {
         cdig3 Ys[6];
@@ -151,22 +174,6 @@ __global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2
 #pragma unroll
             for (int b = 0; b < 3; b++)
                 put(Gud + (size_t)(mu * 9 + 3 * a + b) * V + s, fx_dag2<2>(a0, Ys[b], a1, Ys[3 + b]));
-        }
-    }
-    // G_g(x) rows 0,1 += Y U^dag
-    {
-        cdig3 Yd[6], ud[9];
-#pragma unroll
-        for (int e = 0; e < 6; e++) {
-            Yd[e] = with_diff(Y[e]);
-            ud[e] = with_sum(ldx(U + (size_t)(mu * 6 + e) * V + s));
-        }
-#pragma unroll
-        for (int j = 0; j < 3; j++) ud[6 + j] = with_sum(fx_row2<3>(ud, ud + 3, j));
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            put(Ggm + (size_t)(mu * 6 + j) * V + s, fx_mul_dag<3>(Yd, ud + 3 * j));
-            put(Ggm + (size_t)(mu * 6 + 3 + j) * V + s, fx_mul_dag<3>(Yd + 3, ud + 3 * j));
         }
     }
 }

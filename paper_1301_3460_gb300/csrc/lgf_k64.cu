@@ -125,7 +125,7 @@ void launch_step_bwd(cudaStream_t s, const Lat& d, const double2* U, const doubl
                      double2* Gp, double2* Gud, double2* Ggs, double2* Q, double alpha, double2* FA, double2* FB)
 {
     k_bwd_update<<<blocks(d.V, 128), 128, 0, s>>>(d, U, g, Gp, Gud, Ggs, Q);
-    k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Ggs, 1, Q, alpha, FA, FB);
+    k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Ggs, 1, 6, Q, alpha, FA, FB);
 }
 void launch_bwd_delta(cudaStream_t s, const Lat& d, const double2* U, const double2* FA, const double2* FB,
                       const double2* Gud, double2* Gin)

@@ -96,10 +96,21 @@ void launch_fxt_xyinv_g(const Lat& d, const Shape& sh, cudaStream_t s, const lon
         k_xyinv_fxt<128><<<d.nplanes, fxt_threads(sh.nt_xy, sm, false), sm, s>>>(d, xs, Fd, g, ctl, b.tw, b.bexp, b.fe, Dt);
 }
 
-void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
-                     longlong2* AH, fx* Fs, FxExp* fe)
+void launch_fx_start(const Lat& d, cudaStream_t s, const longlong2* U64, longlong2* AH, fx* Fs, FxExp* fe)
 {
-    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, U, G, AH, Fs, fe);
+    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, nullptr, AH, Fs, fe);
+}
+void launch_fx_start_bwd(const Lat& d, cudaStream_t s, const double2* U64, double2* Gud, longlong2* AH, fx* Fs, FxExp* fe)
+{
+    Lat dx = d;
+    dx.nx = 9;  // the links on the grid wait in the slots of their cotangents
+    k_fx_start<<<blocks(d.V, 128), 128, 0, s>>>(dx, reinterpret_cast<const longlong2*>(U64),
+                                                reinterpret_cast<longlong2*>(Gud), AH, Fs, fe);
+}
+void launch_fx_enter(const Lat& d, cudaStream_t s, const longlong2* U64, const longlong2* G64, longlong2* U, longlong2* G,
+                     Ctl* ctl)
+{
+    k_fx_enter<<<blocks(d.V, 128), 128, 0, s>>>(d, U64, G64, U, G, ctl);
 }
 void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
                        const double2* G64, longlong2* U, longlong2* G, longlong2* AH, fx* Fs, FxExp* fe, Ctl* ctl)
@@ -109,9 +120,9 @@ void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2*
     k_phase_switch<<<1, 1, 0, s>>>(ctl);
 }
 void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
-                      const Ctl* ctl, bool always)
+                      const Ctl* ctl)
 {
-    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl, always ? 1 : 0);
+    k_fx_finish<<<blocks(d.V, 128), 128, 0, s>>>(d, U, G, U64, G64, ctl);
 }
 void launch_fxt_accel(const Lat& d, const Shape& sh, cudaStream_t s, const double2* in, double2* out, longlong2* work,
                       int nf, const FxtBuf& b, const Ctl* ctl)
@@ -133,11 +144,11 @@ void launch_fxt_accel(const Lat& d, const Shape& sh, cudaStream_t s, const doubl
 }
 cudaError_t fxt_clear_bad(const FxtBuf& b, cudaStream_t s) { return cudaMemsetAsync(&b.fe->bad, 0, sizeof(int), s); }
 
-void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* g, const double2* Fdt,
-                        const double2* Gp, double2* Gud, double2* Ggm, double2* Q, double alpha, double2* FA, double2* FB)
+void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* g, const double2* Fdt, double2* Gp, double2* Gud,
+                        double2* Q, double alpha, double2* FA, double2* FB)
 {
-    k_bwd_update_fx<128, 3><<<dim3(blocks(d.V, 128), 4), 128, 0, s>>>(d, U, g, Gp, Gud, Ggm, Q);
-    k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Ggm, 4, Q, alpha, FA, FB);
+    k_bwd_update_fx<128, 3><<<dim3(blocks(d.V, 128), 4), 128, 0, s>>>(d, g, Gp, Gud, Q);
+    k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Gp, 4, 9, Q, alpha, FA, FB);
 }
 
 // A thread per link while three blocks of 32 sites on every SM hold the lattice twice

@@ -1,8 +1,11 @@
 // The FP64 iterations on 64-bit fixed point (lgf_fx.cuh): start and end of a
 // loop, the update and the Delta stencil.  Arrays of a loop:
-//   UX   [mu=4][6][V]  rows 0,1 of every link, x 2^61 (whatever form the
-//                      context stores its FP64 links in)
-//   GX   [6][V]        rows 0,1 of G, x 2^61 (null: not tracked)
+//   UX   [mu=4][nx][V] rows 0,1 of every link, x 2^61, in the first six planes of
+//                      each direction (whatever form the context stores its FP64 links
+//                      in).  Without an FP32 phase they take the FP64 links' place while
+//                      the loop runs (nx is 9 over 18-real links, else 6), with one the
+//                      idle FP32 links' place: no memory of their own
+//   GX   [6][V]        rows 0,1 of G, x 2^61 (null: not tracked), likewise
 //   gX   [9][V]        g, x 2^62
 //   AHX  [mu=4][4][V]  packed anti-Hermitian parts of the links, x 2^58; the
 //                      fourth entry holds 2 Im w00 - Im w11 - Im w22 and 2 Im w11
@@ -79,14 +82,14 @@ template <typename GB> __device__ __forceinline__ void fx_right(const cdig3* A, 
 }
 
 // stores link (mu, s) and its packed part
-__device__ __forceinline__ void fx_store_link(longlong2* __restrict__ U, longlong2* __restrict__ AH, int V, int mu,
+__device__ __forceinline__ void fx_store_link(longlong2* __restrict__ U, longlong2* __restrict__ AH, int V, int nx, int mu,
                                               int s, const cfx* w, fx& f)
 {
     cdig wd[6];
 #pragma unroll
     for (int e = 0; e < 6; e++) {
         wd[e] = digits(w[e]);
-        stx(U + (size_t)(mu * 6 + e) * V + s, w[e]);
+        stx(U + (size_t)(mu * nx + e) * V + s, w[e]);
     }
     cfx a[4];
     fx_ah(w, wd, a, f);
@@ -160,7 +163,7 @@ static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, long
     }
     auto fetch_u = [&](int mu) {
 #pragma unroll
-        for (int e = 0; e < 6; e++) cp_async16<false>(su + e * NT, U + (size_t)(mu * 6 + e) * V + s);
+        for (int e = 0; e < 6; e++) cp_async16<false>(su + e * NT, U + (size_t)(mu * d.nx + e) * V + s);
 #pragma unroll
         for (int k = 0; k < 3; k++) cp_async16<false>(su + (6 + k) * NT, AH + (size_t)(mu * 4 + 1 + k) * V + s);
     };
@@ -212,7 +215,7 @@ static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, long
         fx_right(A, [&](int e) { return ldv<fx>(sn + e * NT); }, w);
         if (mu < 3) fetch_g(mu == 0 ? nb[1] : mu == 1 ? nb[2] : nb[3]);
         cp_async_commit();
-        fx_store_link(U, AH, V, mu, s, w, f);
+        fx_store_link(U, AH, V, d.nx, mu, s, w, f);
     }
     Fs[s] = f;
     if (G != nullptr) {
@@ -253,7 +256,7 @@ static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
             cfx u[9], w[6], gn[9];
             longlong2 part[3];
 #pragma unroll
-            for (int e = 0; e < 6; e++) u[e] = ldv<fx>(U + (size_t)(mu * 6 + e) * V + s);
+            for (int e = 0; e < 6; e++) u[e] = ldv<fx>(U + (size_t)(mu * d.nx + e) * V + s);
 #pragma unroll
             for (int k = 0; k < 3; k++) part[k] = AH[(size_t)(mu * 4 + 1 + k) * V + s];
 #pragma unroll
@@ -270,7 +273,7 @@ static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
             }
             fx_right(A, [&](int e) { return gn[e]; }, w);
             fx f = 0;
-            fx_store_link(U, AH, V, mu, s, w, f);
+            fx_store_link(U, AH, V, d.nx, mu, s, w, f);
             retr[mu][lane] = f;
         } else if (G != nullptr) {
             cfx m[6];
@@ -292,11 +295,32 @@ struct __align__(16) FxExp {
     int pad[3];
 };
 
-// Start of a loop: the links' rows 0,1 (and G's) on the grid, rounded to nearest, with
-// the links' packed parts and Re Tr.
-static __global__ void __launch_bounds__(128) k_fx_start(Lat d, const double2* __restrict__ U64,
-                                                         const double2* __restrict__ G64, longlong2* __restrict__ U,
-                                                         longlong2* __restrict__ G, longlong2* __restrict__ AH,
+// An FP64 link's rows 0,1 on the grid, rounded to nearest.  U64 may be the place that the
+// fixed-point links go to, so it is read as integers (no read-only loads).
+__device__ __forceinline__ void fx_rows_of_link(const longlong2* U64, int V, int ne, int mu, int s, cfx* w)
+{
+    const longlong2* p = U64 + (size_t)mu * ne * V + s;
+    auto get = [&](int e) {
+        const longlong2 v = p[(size_t)e * V];
+        return mk<double>(__longlong_as_double(v.x), __longlong_as_double(v.y));
+    };
+    cx<double> u[9];
+    if (ne == 4) {
+        const cx<double> th = get(3);
+        rebuild8<double>(get(0), get(1), get(2), th.re, th.im, u);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 6; e++) u[e] = get(e);
+    }
+#pragma unroll
+    for (int e = 0; e < 6; e++) w[e] = cfx{d2fx_rn<kFxBits>(u[e].re), d2fx_rn<kFxBits>(u[e].im)};
+}
+
+// Start of a loop: the packed parts and Re Tr of the links on the grid.  The links stay what
+// they are until there is an update to make (k_fx_enter).  U (may be null): a place of its
+// own for the links on the grid.
+static __global__ void __launch_bounds__(128) k_fx_start(Lat d, const longlong2* __restrict__ U64,
+                                                         longlong2* __restrict__ U, longlong2* __restrict__ AH,
                                                          fx* __restrict__ Fs, FxExp* fe)
 {
     const int V = d.V;
@@ -306,19 +330,47 @@ static __global__ void __launch_bounds__(128) k_fx_start(Lat d, const double2* _
     fx f = 0;
 #pragma unroll 1
     for (int mu = 0; mu < 4; mu++) {
-        cx<double> u[9];
-        load_link<double>(U64, V, d.ne, mu, s, u);
-        cfx w[6];
+        cfx w[6], a[4];
+        cdig wd[6];
+        fx_rows_of_link(U64, V, d.ne, mu, s, w);
 #pragma unroll
-        for (int e = 0; e < 6; e++) w[e] = cfx{__double2ll_rn(u[e].re * 0x1p61), __double2ll_rn(u[e].im * 0x1p61)};
-        fx_store_link(U, AH, V, mu, s, w, f);
+        for (int e = 0; e < 6; e++) wd[e] = digits(w[e]);
+        if (U != nullptr) {
+#pragma unroll
+            for (int e = 0; e < 6; e++) stx(U + (size_t)(mu * d.nx + e) * V + s, w[e]);
+        }
+        fx_ah(w, wd, a, f);
+#pragma unroll
+        for (int k = 0; k < 4; k++) stx(AH + (size_t)(mu * 4 + k) * V + s, a[k]);
     }
     Fs[s] = f;
+}
+
+// Before the first update: links and G to their fixed-point form, which may lie where the
+// FP64 ones do (nx >= ne: from the last direction down, no link is overwritten before it is
+// read, all by the site's own thread).  When the loop makes no update the stored links
+// stay as they are.
+static __global__ void __launch_bounds__(128) k_fx_enter(Lat d, const longlong2* U64, const longlong2* G64, longlong2* U,
+                                                         longlong2* G, Ctl* ctl)
+{
+    if (ld_flag(&ctl->phase_done)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->fixed_form = 1;
+    const int V = d.V;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= V) return;
+#pragma unroll 1
+    for (int mu = 3; mu >= 0; mu--) {
+        cfx w[6];
+        fx_rows_of_link(U64, V, d.ne, mu, s, w);
+#pragma unroll
+        for (int e = 0; e < 6; e++) stx(U + (size_t)(mu * d.nx + e) * V + s, w[e]);
+    }
     if (G != nullptr) {
 #pragma unroll
         for (int e = 0; e < 6; e++) {
-            const double2 v = G64[(size_t)e * V + s];
-            stx(G + (size_t)e * V + s, cfx{__double2ll_rn(v.x * 0x1p61), __double2ll_rn(v.y * 0x1p61)});
+            const longlong2 v = G64[(size_t)e * V + s];
+            stx(G + (size_t)e * V + s,
+                cfx{d2fx_rn<kFxBits>(__longlong_as_double(v.x)), d2fx_rn<kFxBits>(__longlong_as_double(v.y))});
         }
     }
 }
@@ -335,6 +387,7 @@ static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2*
     if (ld_flag(&ctl->nan_seen)) return;
     const int V = d.V;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s == 0) const_cast<Ctl*>(ctl)->fixed_form = 1;
     if (s < 4) fe->amax1[s] = kExpNone;
     if (s >= V) return;
     int c[4];
@@ -365,7 +418,7 @@ static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2*
             fx_left(gx, ud, A);
         }
         fx_right(A, [&](int e) { return load_gs(sn, e); }, w);
-        fx_store_link(U, AH, V, mu, s, w, f);
+        fx_store_link(U, AH, V, d.nx, mu, s, w, f);
     }
     Fs[s] = f;
     if (G != nullptr) {
@@ -380,17 +433,14 @@ static __global__ void __launch_bounds__(128) k_fx_project(Lat d, const double2*
     if (bad) const_cast<Ctl*>(ctl)->bad = 1;
 }
 
-// End of a loop: links and G back to FP64 in the context's form (NaN when an entry of g
-// was not finite).  Nothing is written when no update was made (always: the start's
-// links are not the stored ones, mixed mode), nor after a NaN in the FP32 phase.
-static __global__ void __launch_bounds__(128) k_fx_finish(Lat d, const longlong2* __restrict__ U,
-                                                          const longlong2* __restrict__ G,
-                                                          double2* __restrict__ U64, double2* __restrict__ G64,
-                                                          const Ctl* ctl, int always)
+// End of a loop that took the links to their fixed-point form: links and G back to FP64 in
+// the context's form, which may lie in the same place (ne <= nx: from the first direction
+// up), NaN when an entry of g was not finite.
+static __global__ void __launch_bounds__(128) k_fx_finish(Lat d, const longlong2* U, const longlong2* G, double2* U64,
+                                                          double2* G64, const Ctl* ctl)
 {
+    if (!ld_flag(&ctl->fixed_form)) return;
     const bool bad = ld_flag(&ctl->bad) != 0;
-    if (ld_flag(&ctl->nan_seen) && !bad) return;
-    if (!always && ld_flag(&ctl->iter) == 0) return;
     const int V = d.V;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= V) return;
@@ -400,13 +450,20 @@ static __global__ void __launch_bounds__(128) k_fx_finish(Lat d, const longlong2
     for (int mu = 0; mu < 4; mu++) {
         cx<double> w[9];
 #pragma unroll
-        for (int e = 0; e < 6; e++) w[e] = back(ldx(U + (size_t)(mu * 6 + e) * V + s));
+        for (int e = 0; e < 6; e++) w[e] = back(ldv<fx>(U + (size_t)(mu * d.nx + e) * V + s));
         if (d.ne != 6) complete_row2(w, w + 6);
+        // the loads above come first whatever types the two views of the place have
+        asm volatile("" ::: "memory");
         store_link<double>(U64, V, d.ne, mu, s, w);
+        asm volatile("" ::: "memory");
     }
     if (G != nullptr) {
+        cx<double> m[6];
 #pragma unroll
-        for (int e = 0; e < 6; e++) st<double>(G64 + (size_t)e * V + s, back(ldx(G + (size_t)e * V + s)));
+        for (int e = 0; e < 6; e++) m[e] = back(ldv<fx>(G + (size_t)e * V + s));
+        asm volatile("" ::: "memory");
+#pragma unroll
+        for (int e = 0; e < 6; e++) st<double>(G64 + (size_t)e * V + s, m[e]);
     }
 }
 

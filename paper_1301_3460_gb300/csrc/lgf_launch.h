@@ -81,10 +81,12 @@ void launch_xyinv_g32_64(const Lat& d, const Shape& sh32, cudaStream_t s, const 
                          const Ctl* ctl);
 
 // FP64 iterations on 64-bit fixed point (lgf_kfx.cuh): links and G on the grid 2^-61, g
-// on 2^-62, packed parts and Re Tr on 2^-58.  start: from the stored links;
-// project: the end of the FP32 phase (links rebuilt on the input's orbit, phase
-// switched); finish: back to the stored FP64 links.  TF: precision of the transforms.  h:
-// condition of the loop that the Delta kernel decides about (0: none).
+// on 2^-62, packed parts and Re Tr on 2^-58.  start: parts and Re Tr of the stored
+// links (start_bwd: and the links on the grid in the slots of their cotangents, for
+// launch_fx_step_bwd); enter: the stored links (and G) to the grid, in place or elsewhere,
+// when the loop goes on; project: the end of the FP32 phase (links rebuilt on the
+// input's orbit, phase switched); finish: back to the stored FP64 links.  TF: precision
+// of the transforms.  h: condition of the loop that the Delta kernel decides about (0: none).
 struct FxExp;
 // buffers of the integer transform (lgf_fxt.cuh): multipliers and exponents, carved
 // from fxt_bytes(d) of device memory
@@ -103,12 +105,15 @@ bool fxt_fits(const Lat& d, const Shape& sh);
 FxtBuf fxt_carve(const Lat& d, void* p);
 void launch_fxt_tables(const Lat& d, cudaStream_t s, const double* m64, const FxtBuf& b);
 cudaError_t fx_prepare(const Lat& d);
-void launch_fx_start(const Lat& d, cudaStream_t s, const double2* U64, const double2* G64, longlong2* U, longlong2* G,
-                     longlong2* AH, long long* Fs, FxExp* fe);
+void launch_fx_start(const Lat& d, cudaStream_t s, const longlong2* U64, longlong2* AH, long long* Fs, FxExp* fe);
+void launch_fx_start_bwd(const Lat& d, cudaStream_t s, const double2* U64, double2* Gud, longlong2* AH, long long* Fs,
+                         FxExp* fe);
+void launch_fx_enter(const Lat& d, cudaStream_t s, const longlong2* U64, const longlong2* G64, longlong2* U, longlong2* G,
+                     Ctl* ctl);
 void launch_fx_project(const Lat& d, cudaStream_t s, const float2* G32, double2* Gs, const double2* U64,
                        const double2* G64, longlong2* U, longlong2* G, longlong2* AH, long long* Fs, FxExp* fe, Ctl* ctl);
 void launch_fx_finish(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* G, double2* U64, double2* G64,
-                      const Ctl* ctl, bool always);
+                      const Ctl* ctl);
 void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, long long* Fs);
 template <typename TF>
@@ -131,9 +136,10 @@ void launch_fxt_xyinv_g(const Lat& d, const Shape& sh64, cudaStream_t s, const l
 cudaError_t fxt_clear_bad(const FxtBuf& b, cudaStream_t s);
 void launch_fxt_accel(const Lat& d, const Shape& sh64, cudaStream_t s, const double2* in, double2* out, longlong2* work,
                       int nf, const FxtBuf& b, const Ctl* ctl);
-// k_bwd_update on fixed point and the Gram-Schmidt's derivative; Ggm: [4][6][V]
-void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* U, const longlong2* g, const double2* Fdt,
-                        const double2* Gp, double2* Gud, double2* Ggm, double2* Q, double alpha, double2* FA, double2* FB);
+// k_bwd_update on fixed point and the Gram-Schmidt's derivative; Gp is used up, Gud holds the
+// links on entry
+void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* g, const double2* Fdt, double2* Gp, double2* Gud,
+                        double2* Q, double alpha, double2* FA, double2* FB);
 void launch_fx_build_g(const Lat& d, cudaStream_t s, const double2* Fd, longlong2* g, const Ctl* ctl);
 // *wide set when a stored link is not within 1e-3 of SU(3), or its stored row 2 not rows 0,1's
 void launch_check_range(const Lat& d, cudaStream_t s, const double2* U64, int* wide);
@@ -173,9 +179,10 @@ void launch_gluon_bwd(cudaStream_t s, const Lat& d, const double2* U, const doub
 // and the mean plaquette (lgf_wilson.cu)
 void launch_wilson(cudaStream_t s, const Lat& d, double2* U, float2* U32, int mu, int parity, int overrelax,
                    double beta, unsigned long long seed, unsigned int sweep, int precision);
-// the same on fixed-point links UX [mu][9][V], converted once per call
-void launch_links_to_fx(cudaStream_t s, const Lat& d, const double2* U, longlong2* UX);
-void launch_links_from_fx(cudaStream_t s, const Lat& d, const longlong2* UX, double2* U);
+// the same on fixed-point links, converted once per call: [mu][9][V] from U on, where 36 V
+// entries have to be free
+void launch_links_to_fx(cudaStream_t s, const Lat& d, double2* U);
+void launch_links_from_fx(cudaStream_t s, const Lat& d, double2* U);
 void launch_wilson_fx(cudaStream_t s, const Lat& d, longlong2* UX, int mu, int parity, int overrelax, double beta,
                       unsigned long long seed, unsigned int sweep);
 void launch_links_to_fp32(cudaStream_t s, const Lat& d, const double2* U, float2* U32);

@@ -359,37 +359,48 @@ __global__ void __launch_bounds__(kWilsonThreads) k_wilson(Lat d, double2* __res
 // The links of a call on the grid 2^-61, all three rows: [mu][9][V] (the rows saved
 // from rebuilding, 144 integer products per staple, cost half as many bytes again).
 // Staples of up to six unit matrices and W are kept x 2^58 (range +-32).
+// They begin where the FP64 links do and reach into the idle arrays behind them: a thread
+// converts the four links of its site, the last direction first on the way in (nothing is
+// overwritten before it is read) and the first one first on the way back.
 
-__global__ void k_links_to_fx(Lat d, const double2* __restrict__ U, longlong2* __restrict__ UX)
+__global__ void k_links_to_fx(Lat d, const longlong2* U, longlong2* UX)
 {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 4L * d.V) return;
-    const int mu = (int)(idx / d.V), s = (int)(idx - (long)mu * d.V);
-    cfx r[6];
-    cdig rd[6];
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= d.V) return;
+#pragma unroll 1
+    for (int mu = 3; mu >= 0; mu--) {
+        cfx r[6];
+        cdig rd[6];
 #pragma unroll
-    for (int e = 0; e < 6; e++) {
-        const double2 v = U[(size_t)(mu * d.ne + e) * d.V + s];
-        r[e] = cfx{__double2ll_rn(v.x * 0x1p61), __double2ll_rn(v.y * 0x1p61)};
-        rd[e] = digits(r[e]);
-        stx(UX + (size_t)(mu * 9 + e) * d.V + s, r[e]);
+        for (int e = 0; e < 6; e++) {
+            const longlong2 v = U[(size_t)(mu * d.ne + e) * d.V + s];
+            r[e] = cfx{d2fx_rn<kFxBits>(__longlong_as_double(v.x)), d2fx_rn<kFxBits>(__longlong_as_double(v.y))};
+            rd[e] = digits(r[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 6; e++) stx(UX + (size_t)(mu * 9 + e) * d.V + s, r[e]);
+#pragma unroll
+        for (int j = 0; j < 3; j++) stx(UX + (size_t)(mu * 9 + 6 + j) * d.V + s, fx_row2<3>(rd, rd + 3, j));
     }
-#pragma unroll
-    for (int j = 0; j < 3; j++) stx(UX + (size_t)(mu * 9 + 6 + j) * d.V + s, fx_row2<3>(rd, rd + 3, j));
 }
-__global__ void k_links_from_fx(Lat d, const longlong2* __restrict__ UX, double2* __restrict__ U)
+__global__ void k_links_from_fx(Lat d, const longlong2* UX, double2* U)
 {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 4L * d.V) return;
-    const int mu = (int)(idx / d.V), s = (int)(idx - (long)mu * d.V);
-    cx<double> w[9];
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= d.V) return;
+#pragma unroll 1
+    for (int mu = 0; mu < 4; mu++) {
+        cx<double> w[9];
 #pragma unroll
-    for (int e = 0; e < 6; e++) {
-        const cfx v = ldx(UX + (size_t)(mu * 9 + e) * d.V + s);
-        w[e] = mk<double>(fx2d(v.re, kFxBits), fx2d(v.im, kFxBits));
+        for (int e = 0; e < 6; e++) {
+            const cfx v = ldv<fx>(UX + (size_t)(mu * 9 + e) * d.V + s);
+            w[e] = mk<double>(fx2d(v.re, kFxBits), fx2d(v.im, kFxBits));
+        }
+        if (d.ne == 9) complete_row2(w, w + 6);
+        // the loads come first whatever types the two views of the place have
+        asm volatile("" ::: "memory");
+        store_link<double>(U, d.V, d.ne, mu, s, w);
+        asm volatile("" ::: "memory");
     }
-    complete_row2(w, w + 6);
-    store_link<double>(U, d.V, d.ne, mu, s, w);
 }
 
 __device__ __forceinline__ void load9x(const longlong2* __restrict__ U, int V, int mu, int s, cfx* m)
@@ -852,13 +863,14 @@ void launch_links_to_fp32(cudaStream_t s, const Lat& d, const double2* U, float2
     k_links_to_fp32<<<(unsigned)((d.V + 255) / 256), 256, 0, s>>>(d, U, U32);
 }
 
-void launch_links_to_fx(cudaStream_t s, const Lat& d, const double2* U, longlong2* UX)
+void launch_links_to_fx(cudaStream_t s, const Lat& d, double2* U)
 {
-    k_links_to_fx<<<(unsigned)((4L * d.V + 255) / 256), 256, 0, s>>>(d, U, UX);
+    longlong2* X = reinterpret_cast<longlong2*>(U);
+    k_links_to_fx<<<(unsigned)((d.V + 127) / 128), 128, 0, s>>>(d, X, X);
 }
-void launch_links_from_fx(cudaStream_t s, const Lat& d, const longlong2* UX, double2* U)
+void launch_links_from_fx(cudaStream_t s, const Lat& d, double2* U)
 {
-    k_links_from_fx<<<(unsigned)((4L * d.V + 255) / 256), 256, 0, s>>>(d, UX, U);
+    k_links_from_fx<<<(unsigned)((d.V + 127) / 128), 128, 0, s>>>(d, reinterpret_cast<const longlong2*>(U), U);
 }
 
 void launch_wilson_fx(cudaStream_t s, const Lat& d, longlong2* UX, int mu, int parity, int overrelax, double beta,
