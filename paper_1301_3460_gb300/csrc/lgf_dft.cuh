@@ -234,7 +234,9 @@ template <typename T, bool INV> __host__ __device__ __forceinline__ cx<T> mul_ni
 // Transforms of integers (T = fx): values of up to 2^62 in magnitude, roots x 2^62
 // in digits (lgf_fx.cuh), every product rounded to nearest.  Against the doubles'
 // relative 2^-53 the absolute error of one product is 2^-1 or less, so a line
-// scaled to fill 57 bits keeps more precision than FP64 arithmetic does.
+// scaled to fill 57 bits keeps more precision than FP64 arithmetic does.  The kernels
+// run the forward codelets only (lgf_fxt.cuh: an inverse exchanges real and imaginary
+// part); the inverse ones complete the set and are checked with them on the host.
 
 // root x 2^62 -> digits (a value of exactly 2^62 is exact in its high digit)
 __host__ __device__ constexpr dig xdigits(fx v)
@@ -453,30 +455,13 @@ template <typename T, int L, int NL = line_lanes<T>(L)> __host__ __device__ __fo
 // tau < T, chosen among T compile-time constants
 template <typename T, int L, int Tl, int E, bool INV> __host__ __device__ __forceinline__ cx<T> lane_root(int tau)
 {
-    if constexpr (std::is_same_v<T, fx>) {
-        cx<fx> w = cx<fx>{1ll << 62, 0};  // x 2^62
-        sfor<1, Tl>([&](auto t) {
-            constexpr int m = imod(t.value * E * (384 / L), 384);
-            constexpr fx c = cos384x(m), sn = INV ? sin384x(m) : -sin384x(m);
-            if (tau == t.value) w = cx<fx>{c, sn};
-        });
-        return w;
-    } else {
-        cx<T> w = cx<T>{(T)1, (T)0};
-        sfor<1, Tl>([&](auto t) {
-            constexpr int m = imod(t.value * E * (384 / L), 384);
-            constexpr T c = (T)cos384(m), sn = (T)(INV ? sin384(m) : -sin384(m));
-            if (tau == t.value) w = cx<T>{c, sn};
-        });
-        return w;
-    }
-}
-
-// v times a root from lane_root
-template <typename T> __host__ __device__ __forceinline__ cx<T> mul_root(cx<T> v, cx<T> w)
-{
-    if constexpr (std::is_same_v<T, fx>) return xcmul(digits(w.re), digits(w.im), digits(-w.im), v);
-    else return cmul(v, w);
+    cx<T> w = cx<T>{(T)1, (T)0};
+    sfor<1, Tl>([&](auto t) {
+        constexpr int m = imod(t.value * E * (384 / L), 384);
+        constexpr T c = (T)cos384(m), sn = (T)(INV ? sin384(m) : -sin384(m));
+        if (tau == t.value) w = cx<T>{c, sn};
+    });
+    return w;
 }
 
 // steps 1-2 of the forward line transform in one lane (step 1 alone for T = 1)
@@ -486,7 +471,7 @@ __host__ __device__ __forceinline__ void line_fwd_local(cx<T>* v, int tau)
     constexpr int Tl = NL, R = L / Tl;
     dft<T, R, false>(v);
     if constexpr (Tl > 1) {
-        sfor<1, R>([&](auto r) { v[r.value] = mul_root<T>(v[r.value], lane_root<T, L, Tl, r.value, false>(tau)); });
+        sfor<1, R>([&](auto r) { v[r.value] = cmul(v[r.value], lane_root<T, L, Tl, r.value, false>(tau)); });
     }
 }
 
@@ -496,7 +481,7 @@ __host__ __device__ __forceinline__ void line_inv_local(cx<T>* v, int tau)
 {
     constexpr int Tl = NL, R = L / Tl;
     if constexpr (Tl > 1) {
-        sfor<1, R>([&](auto r) { v[r.value] = mul_root<T>(v[r.value], lane_root<T, L, Tl, r.value, true>(tau)); });
+        sfor<1, R>([&](auto r) { v[r.value] = cmul(v[r.value], lane_root<T, L, Tl, r.value, true>(tau)); });
     }
     dft<T, R, true>(v);
 }
@@ -518,8 +503,6 @@ __host__ __device__ __forceinline__ float sflip(float x, unsigned m)
     return m ? -x : x;
 #endif
 }
-
-__host__ __device__ __forceinline__ fx sflip(fx x, unsigned m) { return m ? -x : x; }
 
 // One radix-2 stage across lanes for lane bit h, o the partner lane's value
 // (partner tau ^ h).  Forward (decimation in frequency): the low lane keeps
@@ -558,7 +541,7 @@ template <typename T, int R, bool INV> __host__ __device__ __forceinline__ void 
     } else if (h == 4) {
         const cx<T> w = lane_root<T, 8, 4, 1, INV>((tau & 4) ? (tau & 3) : 0);
 #pragma unroll
-        for (int r = 0; r < R; r++) v[r] = mul_root<T>(v[r], w);
+        for (int r = 0; r < R; r++) v[r] = cmul(v[r], w);
     }
 }
 
