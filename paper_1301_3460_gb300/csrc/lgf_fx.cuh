@@ -1,8 +1,8 @@
 // 64-bit fixed-point arithmetic of the FP64 iterations.
 //
-// GB300 issues 2 FP64 operations per clock and SM but 63 mad.wide.s32 (32 x 32
-// -> 64 bits with a 64-bit accumulator; both measured on the device), and the
-// entries of SU(3) matrices are bounded by 1.  The matrix products of the FP64
+// GB300 issues 2 FP64 operations per clock and SM but 24 to 32 mad.wide.s32 (32 x 32
+// -> 64 bits with a 64-bit accumulator, operands from distinct registers; both measured
+// on the device), and the entries of SU(3) matrices are bounded by 1.  The matrix products of the FP64
 // iterations therefore run on 64-bit integers: links and G hold a real x as
 // x 2^61 (range +-4, resolution 4.3e-19; FP64 resolves 1.1e-16 near 1), g as x 2^62.
 //
@@ -21,8 +21,10 @@
 // rows of norm <= 1 the six digits h of a row sum to at most sqrt(6) 2^(p-32)
 // and |l| <= 2^31, so |m| <= sqrt(6) (2^61 + 2^60) < 2^63 for p = 62, q = 61.
 //
-// Sums of packed anti-Hermitian parts use the grid 2^-58 (range +-32; eight links'
-// parts reach 27.4); adding them is exact and needs no FP64 operation.
+// Sums of packed anti-Hermitian parts use the grid 2^-58 (range +-32); adding them is
+// exact and needs no FP64 operation.  The largest entry of a part is 2 Im w00 - Im w11
+// - Im w22: at most 2 sin a + 2 sin(a/2) = 3.520 (phases a = 1.872, -a/2, -a/2), so eight
+// links reach 28.2.
 #pragma once
 #include "lgf_common.cuh"
 
@@ -166,6 +168,14 @@ template <int S, typename D> __device__ __forceinline__ cfx fx_row2(const D* r0,
 {
     const int a = j == 0 ? 1 : j == 1 ? 2 : 0, b = j == 0 ? 2 : j == 1 ? 0 : 1;
     return fx_det2c<S>(r0[a], r1[b], r0[b], r1[a]);
+}
+
+// the double nearest to v 2^-q
+__device__ __forceinline__ double fx2d(fx v, int q)
+{
+    const double y = __ll2double_rn(v);
+    const int hi = __double2hiint(y) - (q << 20);
+    return v == 0 ? 0.0 : __hiloint2double(hi, __double2loint(y));
 }
 
 // the same for any q, through zeros, subnormals and infinity where v 2^-q lies there
@@ -421,14 +431,6 @@ template <int Q> __device__ __forceinline__ fx d2fx_rn(double x)
     }
     const fx s = -(fx)(hi >> 31);
     return ((fx)v ^ s) - s;
-}
-
-// the double nearest to v 2^-q
-__device__ __forceinline__ double fx2d(fx v, int q)
-{
-    const double y = __ll2double_rn(v);
-    const int hi = __double2hiint(y) - (q << 20);
-    return v == 0 ? 0.0 : __hiloint2double(hi, __double2loint(y));
 }
 
 }  // namespace lgf

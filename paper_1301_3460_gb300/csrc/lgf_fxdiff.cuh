@@ -51,7 +51,7 @@ template <int S> __device__ __forceinline__ cfx fx_dag2(cdig3 a0, cdig3 b0, cdig
 // thread only, and read as what they hold).  The nine components of a cotangent share one scale:
 // their errors are 2^-57 of the largest of them, where FP64's are 2^-53 of the largest
 // term of each sum.  32^4: 4.00 ms in FP64 (2000 operations per site at 2 per clock and
-// SM), 1.46 ms like this (5000 integer products per site; 12 warps per SM at 168
+// SM), 1.50 ms like this (5000 integer products per site; 12 warps per SM at 168
 // registers, 16 at 128 take 1.7 ms).
 template <int NT, int MB>
 __global__ void __launch_bounds__(NT, MB) k_bwd_update_fx(Lat d, const longlong2* __restrict__ g, double2* Gp, double2* Gud,

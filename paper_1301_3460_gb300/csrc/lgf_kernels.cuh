@@ -739,7 +739,7 @@ __device__ __forceinline__ void xyinv_g_plane(const Lat& d, const vec2_t<T>* __r
         if constexpr (sizeof(T) == 4 && !std::is_same_v<TG, double>) {
             // The integer Gram-Schmidt (lgf_fx.cuh) while every |alpha/2 Delta~| < 16.  In
             // FP64 its 56 operations per site bound the kernel (32^4, the FP32 phase's g
-            // builder: 137 us against 68).  An FP32 g has to be the FP64 result rounded, bit
+            // builder: 137 us against 88).  An FP32 g has to be the FP64 result rounded, bit
             // for bit (one other bit sends the FP32 phase to other roundings everywhere and
             // to links turned by another 1e-8): the integer rows decide where no float
             // midpoint lies within both errors (g2f_tol), else the site is done in FP64, as

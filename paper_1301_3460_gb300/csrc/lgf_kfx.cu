@@ -151,9 +151,11 @@ void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* g, const 
     k_bwd_reunit<<<blocks(d.V, 256), 256, 0, s>>>(d, Fdt, Gp, 4, 9, Q, alpha, FA, FB);
 }
 
-// A thread per link while three blocks of 32 sites on every SM hold the lattice twice
-// over.
-constexpr int kUpdSmallV = 32768;
+// A thread per link while its blocks of 32 sites, three to an SM, run in two rounds on the
+// chip's 152 SMs.  With G, us a launch, a thread per link / per site: 4,096 sites 8.2 / 14.3,
+// 8,192 10.2 / 14.3, 16,384 14.3 / 14.3, 20,736 15.4 / 18.4, 27,648 16.4 / 18.4, 32,768 19.5 to
+// 20.5 / 18.4, 36,864 20.5 / 18.4, 49,152 26.6 / 24.6, 131,072 63.5 / 49.2.
+constexpr int kUpdSmallV = 2 * 152 * 3 * 32;
 void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, fx* Fs)
 {
