@@ -156,13 +156,22 @@ void launch_fx_step_bwd(const Lat& d, cudaStream_t s, const longlong2* g, const 
 // 8,192 10.2 / 14.3, 16,384 14.3 / 14.3, 20,736 15.4 / 18.4, 27,648 16.4 / 18.4, 32,768 19.5 to
 // 20.5 / 18.4, 36,864 20.5 / 18.4, 49,152 26.6 / 24.6, 131,072 63.5 / 49.2.
 constexpr int kUpdSmallV = 2 * 152 * 3 * 32;
+template <int NX>
+static void launch_fx_update_nx(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
+                                longlong2* AH, fx* Fs)
+{
+    if (d.V <= kUpdSmallV)
+        k_update_fx_small<NX><<<blocks(d.V, 32), kUpdSmallThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+    else
+        k_update_fx<NX><<<blocks(d.V, kUpdThreads), kUpdThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+}
 void launch_fx_update(const Lat& d, cudaStream_t s, longlong2* U, longlong2* G, const longlong2* g, Ctl* ctl,
                       longlong2* AH, fx* Fs)
 {
-    if (d.V <= kUpdSmallV)
-        k_update_fx_small<<<blocks(d.V, 32), kUpdSmallThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+    if (d.nx == 9)
+        launch_fx_update_nx<9>(d, s, U, G, g, ctl, AH, Fs);
     else
-        k_update_fx<<<blocks(d.V, kUpdThreads), kUpdThreads, 0, s>>>(d, U, G, g, ctl, AH, Fs);
+        launch_fx_update_nx<6>(d, s, U, G, g, ctl, AH, Fs);
 }
 
 template <typename TF>

@@ -137,11 +137,12 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // 2 per clock and SM), 406 us on integers with loads where they are used, 315 us like
 // this (77% of the HBM rate); without G 357 and 281 us.  G in FP64 beside the integer
 // products is slower (441 against 406 us): it comes at the end of every thread.
+// NX: the links' nx as a constant (as an argument it costs 0.7%: 1558 -> 1571 us at 48^4).
 constexpr int kUpdThreads = 128;
-static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, longlong2* __restrict__ U,
-                                                                     longlong2* __restrict__ G,
-                                                                     const longlong2* __restrict__ g, Ctl* ctl,
-                                                                     longlong2* __restrict__ AH, fx* __restrict__ Fs)
+template <int NX>
+__global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, longlong2* __restrict__ U, longlong2* __restrict__ G,
+                                                              const longlong2* __restrict__ g, Ctl* ctl,
+                                                              longlong2* __restrict__ AH, fx* __restrict__ Fs)
 {
     __shared__ longlong2 slots[24 * kUpdThreads];  // per thread: link and part (9), g(x+mu) (9), rows 0,1 of g(x) (6)
     constexpr int NT = kUpdThreads;
@@ -163,7 +164,7 @@ static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, long
     }
     auto fetch_u = [&](int mu) {
 #pragma unroll
-        for (int e = 0; e < 6; e++) cp_async16<false>(su + e * NT, U + (size_t)(mu * d.nx + e) * V + s);
+        for (int e = 0; e < 6; e++) cp_async16<false>(su + e * NT, U + (size_t)(mu * NX + e) * V + s);
 #pragma unroll
         for (int k = 0; k < 3; k++) cp_async16<false>(su + (6 + k) * NT, AH + (size_t)(mu * 4 + 1 + k) * V + s);
     };
@@ -215,7 +216,7 @@ static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, long
         fx_right(A, [&](int e) { return ldv<fx>(sn + e * NT); }, w);
         if (mu < 3) fetch_g(mu == 0 ? nb[1] : mu == 1 ? nb[2] : nb[3]);
         cp_async_commit();
-        fx_store_link(U, AH, V, d.nx, mu, s, w, f);
+        fx_store_link(U, AH, V, NX, mu, s, w, f);
     }
     Fs[s] = f;
     if (G != nullptr) {
@@ -233,7 +234,8 @@ static __global__ void __launch_bounds__(kUpdThreads, 4) k_update_fx(Lat d, long
 // G: for lattices that leave most of the chip idle with a thread per site, whose four
 // links then follow one another (8^4: 14 us a launch against 9).
 constexpr int kUpdSmallThreads = 160;
-static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
+template <int NX>
+__global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
     Lat d, longlong2* __restrict__ U, longlong2* __restrict__ G, const longlong2* __restrict__ g, Ctl* ctl,
     longlong2* __restrict__ AH, fx* __restrict__ Fs)
 {
@@ -256,7 +258,7 @@ static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
             cfx u[9], w[6], gn[9];
             longlong2 part[3];
 #pragma unroll
-            for (int e = 0; e < 6; e++) u[e] = ldv<fx>(U + (size_t)(mu * d.nx + e) * V + s);
+            for (int e = 0; e < 6; e++) u[e] = ldv<fx>(U + (size_t)(mu * NX + e) * V + s);
 #pragma unroll
             for (int k = 0; k < 3; k++) part[k] = AH[(size_t)(mu * 4 + 1 + k) * V + s];
 #pragma unroll
@@ -273,7 +275,7 @@ static __global__ void __launch_bounds__(kUpdSmallThreads, 3) k_update_fx_small(
             }
             fx_right(A, [&](int e) { return gn[e]; }, w);
             fx f = 0;
-            fx_store_link(U, AH, V, d.nx, mu, s, w, f);
+            fx_store_link(U, AH, V, NX, mu, s, w, f);
             retr[mu][lane] = f;
         } else if (G != nullptr) {
             cfx m[6];
